@@ -308,10 +308,10 @@ voldor_status voldor_probe_bounded_wait(long long polls, long long* cycles);
  * Batching and tuning of many windows (no counterpart in the paper).
  * ------------------------------------------------------------------------- */
 
-/* Autotunes the dense-scoring tile shape of one window: hypotheses per thread
- * (2, 4 or 8, i.e. 512, 1024 or 2048 hypotheses per block, 3, 2 or 1 blocks
- * per SM) and pixel chunks (1, 2, 4
- * or 8 waves of resident blocks), timing each candidate with CUDA events on
+/* Autotunes the dense-scoring shape of one window: the hypotheses a thread
+ * takes from tensor memory at a time (2, 4 or 8) and the pixel chunks (at
+ * most 1, 2, 4 or 8 work items, chunk x 128 hypotheses, per SM), timing each
+ * candidate with CUDA events on
  * the window's own frame-1 hypotheses and records. Keeps the fastest;
  * discards captured graphs that used another shape. Overwrites the stage
  * buffers (hypotheses, records), not the state (poses, depth, W, k).

@@ -9,6 +9,7 @@
 // instructions of the geometry (this GPU's FP64 rate is a small fraction of
 // its FP32 rate).
 #include "df32.cuh"
+#include "score_ops.cuh"
 #include "voldor_internal.cuh"
 
 namespace vd {
@@ -26,7 +27,7 @@ namespace vd {
 // offset.
 // ---------------------------------------------------------------------------
 struct PrepGeo {
-    DF Px, Py, Pz, u, v;
+    DF Px, Py, Pz, iz, u, v;       // iz = 1 / Pz (set for t > 1 where Pz > 0)
     bool valid;
 };
 
@@ -62,9 +63,9 @@ __device__ __forceinline__ PrepGeo prep_geometry(const DevParams& p, const DF* C
     }
     g.valid = df_gt0(g.Pz);
     if (g.valid && t > 1) {
-        const DF iz = df_div(df_of(1.f), g.Pz);
-        g.u = df_add(df_mul(df_mul(fx, g.Px), iz), cx);
-        g.v = df_add(df_mul(df_mul(fy, g.Py), iz), cy);
+        g.iz = df_div(df_of(1.f), g.Pz);
+        g.u = df_add(df_mul(df_mul(fx, g.Px), g.iz), cx);
+        g.v = df_add(df_mul(df_mul(fy, g.Py), g.iz), cy);
     }
     g.valid = g.valid && df_ge(g.u, 0.f) && df_le(g.u, small_int_to_float(p.W - 1)) && df_ge(g.v, 0.f) &&
               df_le(g.v, small_int_to_float(p.H - 1));
@@ -122,13 +123,18 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
         *s.prep_done = 0u;
         *s.p3p_claims = 0;
         *s.p3p_done = 0ull;
+        *s.sc_wild = 0;
     }
 }
 
 __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevState s, int t)
 {
-    __shared__ DF C[12];
+    __shared__ DF C[12], T0[12];
     __shared__ int warp_sum[kPixThreads / 32];
+    if (threadIdx.x < 12) {
+        const float* c = s.poses_df + 24 * (t - 1) + 2 * threadIdx.x;
+        T0[threadIdx.x] = DF{c[0], c[1]};
+    }
     load_cum_df(s, t, C);
     const int base = s.pix_block_count[blockIdx.x];      // this block's offset (set by the count pass)
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -157,22 +163,47 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevStat
         const DF fvd = df_add(gv0, df_mul(df_sub(gv1, gv0), ay));
         const DF ifx{p.kdf[8], p.kdf[9]};
         const float fu = df_to_float(fud), fv = df_to_float(fvd);
-        const float ut = df_to_float(df_mul(fud, ifx)), vt = df_to_float(df_mul(fvd, ifx));
-        const DF iz = df_div(df_of(1.f), g.Pz);
+        const DF ut = df_mul(fud, ifx), vt = df_mul(fvd, ifx);
+        const DF iz = t == 1 ? df_div(df_of(1.f), g.Pz) : g.iz;
         const float n = sqrtf(fmaf(fu, fu, fv * fv));
         const float fx2 = df_to_float(df_mul(DF{p.kdf[0], p.kdf[1]}, DF{p.kdf[0], p.kdf[1]}));
-        PixRec r;
-        r.a = make_float4(df_to_float(df_mul(g.Px, iz)), df_to_float(df_mul(df_mul(g.Py, iz), p.fy_over_fx)),
-                          df_to_float(iz), ut);
+        // features of the projection (score_ops.cuh), in float-float
+        const DF xn = df_mul(g.Px, iz), yu = df_mul(g.Py, iz), yn = df_mul(yu, p.fy_over_fx);
+        const DF X = df_add(xn, ut), Y = df_add(yn, vt);
+        // a = (T_t - I) p at the current pose: a_z0, U0 = X a_z0 - a_x0 + ut, V0 alike
+        auto row = [&](int r) {
+            const DF e0 = r == 0 ? df_add(T0[0], -1.f) : T0[4 * r], e1 = r == 1 ? df_add(T0[5], -1.f) : T0[4 * r + 1];
+            const DF e2 = r == 2 ? df_add(T0[10], -1.f) : T0[4 * r + 2];
+            return df_add(df_add(df_mul(e0, xn), df_mul(e1, yu)), df_add(e2, df_mul(T0[4 * r + 3], iz)));
+        };
+        const DF az0 = row(2);
+        const DF U0 = df_add(df_sub(df_mul(X, az0), row(0)), ut);
+        const DF V0 = df_add(df_sub(df_mul(Y, az0), df_mul(row(1), p.fy_over_fx)), vt);
+        __align__(16) __nv_bfloat16 o[kScPixCols];
+        const DF up{1.f, (float)(kScUntruncate - 1.0)};
+        const Slice3 fs[3] = {slice3(xn), slice3(yn), slice3(iz)};
+        pixel_block_s(fs, slice3(df_mul(az0, up)), o);
+        const Slice3 fu4[4] = {slice3(df_mul(X, xn)), slice3(df_mul(X, yn)), slice3(df_mul(X, iz)), slice3(X)};
+        pixel_block_x(fu4, slice3(df_mul(U0, up)), fs, o + 32);
+        const Slice3 fv4[4] = {slice3(df_mul(Y, xn)), slice3(df_mul(Y, yn)), slice3(df_mul(Y, iz)), slice3(Y)};
+        pixel_block_x(fv4, slice3(df_mul(V0, up)), fs, o + 64);
+        const int i = base + rank;
+        unsigned char* d = s.sc_pix + (size_t)(i / kScTilePix) * kScTileBytes + ((i % kScTilePix) / 8) * 128 + (i % 8) * 16;
+#pragma unroll
+        for (int q = 0; q < kScPixCols / 8; ++q)
+            *reinterpret_cast<uint4*>(d + q * (kScTilePix * 16)) = *reinterpret_cast<const uint4*>(o + 8 * q);
+        float4 cst;
         if (p.residual == VOLDOR_RESIDUAL_GAUSSIAN) {
             const GaussConst gc = gauss_const(p, n);
-            r.b = make_float4(vt, fx2 * gc.inv_alpha, -gc.x_mu * gc.inv_alpha, 0.f);
+            cst = make_float4(fx2 * gc.inv_alpha, -gc.x_mu * gc.inv_alpha, 0.f, 0.f);
         } else {
             const FiskConst fc = fisk_const(p, n);
-            r.b = make_float4(vt, fc.beta, fc.beta * (p.log2_fx2 - fc.log2_alpha), fx2 * fc.mu_over_beta);
+            cst = make_float4(fc.beta, fc.beta * (p.log2_fx2 - fc.log2_alpha), fx2 * fc.mu_over_beta, 0.f);
+            s.sc_xmu[i] = fminf(fmaxf(p.lambda2 * n * n, p.x_min), p.x_max) / fx2;
         }
-        r.c = make_float4(s.wmap[(size_t)(t - 1) * N + j], 0.f, 0.f, 0.f);
-        s.pix[base + rank] = r;
+        cst.w = s.wmap[(size_t)(t - 1) * N + j];
+        s.sc_cst[i] = cst;
+        if (!(fabsf(xn.hi) < kScWild && fabsf(yn.hi) < kScWild && fabsf(iz.hi) < kScWild)) atomicOr(s.sc_wild, 1);
     }
 }
 

@@ -7,6 +7,7 @@
 #include <cooperative_groups.h>
 
 #include "df32.cuh"
+#include "score_ops.cuh"
 #include "voldor_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -606,7 +607,7 @@ __device__ void se3_exp_vec(const double* p6, double* Rt)
 
 // One thread per (group, solution slot), so that each thread's FP64 chain is
 // a single se(3) logarithm.
-__global__ void k_hyp_write(DevParams p, DevState s)
+__global__ void k_hyp_write(DevParams p, DevState s, int t)
 {
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= groups_solved(p, s) * kMaxSols) return;
@@ -617,16 +618,23 @@ __global__ void k_hyp_write(DevParams p, DevState s)
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};
     const double* Rt = s.grp_sols + ((size_t)g * kMaxSols + i) * 12;
+    const double* T0 = s.poses + 12 * (t - 1);
     double* oR = s.hyp_Rt + (size_t)h * 12;
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) oR[r * 3 + c] = Rt[r * 4 + c];
-        oR[9 + r] = Rt[r * 4 + 3];
-    }
     float* f = s.hyp_f32 + (size_t)h * 12;
+    double e[12], e0[12];
     for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) f[r * 3 + c] = (float)(sc[r] * (Rt[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c]);
-        f[9 + r] = (float)(sc[r] * Rt[r * 4 + 3]);
+        for (int c = 0; c < 3; ++c) {
+            oR[r * 3 + c] = Rt[r * 4 + c];
+            e[r * 3 + c] = sc[r] * (Rt[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
+            e0[r * 3 + c] = sc[r] * (T0[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
+            f[r * 3 + c] = (float)e[r * 3 + c];
+        }
+        oR[9 + r] = Rt[r * 4 + 3];
+        e[9 + r] = sc[r] * Rt[r * 4 + 3];
+        e0[9 + r] = sc[r] * T0[r * 4 + 3];
+        f[9 + r] = (float)e[9 + r];
     }
+    if (write_hyp_operand(s.sc_hyp, h, e, e0)) atomicOr(s.sc_wild, 1);
     s.hyp_w[h] = s.grp_weight[g];
     s.hyp_info[(size_t)h * 2 + 0] = g;
     s.hyp_info[(size_t)h * 2 + 1] = i;
@@ -660,15 +668,15 @@ void launch_hyp_log(const DevParams& p, const DevState& s, cudaStream_t st)
     k_hyp_log<<<(p.S + 127) / 128, 128, 0, st>>>(p, s);
 }
 
-void launch_hyp_collect(const DevParams& p, const DevState& s, cudaStream_t st)
+void launch_hyp_collect(const DevParams& p, const DevState& s, int t, cudaStream_t st)
 {
     k_hyp_scan<<<1, 1024, 0, st>>>(p, s);
     // sized for the budget; threads past the solved prefix return at once
-    k_hyp_write<<<(p.G * kMaxSols + 127) / 128, 128, 0, st>>>(p, s);
+    k_hyp_write<<<(p.G * kMaxSols + 127) / 128, 128, 0, st>>>(p, s, t);
 }
 
 // Scoring form of caller-given hypotheses already copied to hyp_Rt.
-__global__ void k_hyp_from_rt(DevParams p, DevState s, int n)
+__global__ void k_hyp_from_rt(DevParams p, DevState s, int t, int n)
 {
     const int h = blockIdx.x * blockDim.x + threadIdx.x;
     if (h == 0) *s.n_hyp = n;
@@ -676,16 +684,25 @@ __global__ void k_hyp_from_rt(DevParams p, DevState s, int n)
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};
     const double* R = s.hyp_Rt + (size_t)h * 12;
+    const double* T0 = s.poses + 12 * (t - 1);
     float* f = s.hyp_f32 + (size_t)h * 12;
+    double e[12], e0[12];
     for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) f[r * 3 + c] = (float)(sc[r] * (R[r * 3 + c] - (r == c ? 1.0 : 0.0)) / sc[c]);
-        f[9 + r] = (float)(sc[r] * R[9 + r]);
+        for (int c = 0; c < 3; ++c) {
+            e[r * 3 + c] = sc[r] * (R[r * 3 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
+            e0[r * 3 + c] = sc[r] * (T0[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
+            f[r * 3 + c] = (float)e[r * 3 + c];
+        }
+        e[9 + r] = sc[r] * R[9 + r];
+        e0[9 + r] = sc[r] * T0[r * 4 + 3];
+        f[9 + r] = (float)e[9 + r];
     }
+    if (write_hyp_operand(s.sc_hyp, h, e, e0)) atomicOr(s.sc_wild, 1);
 }
 
-void score_hyps_from_host(const DevParams& p, const DevState& s, int n, cudaStream_t st)
+void score_hyps_from_host(const DevParams& p, const DevState& s, int t, int n, cudaStream_t st)
 {
-    k_hyp_from_rt<<<(n + 127) / 128 + 1, 128, 0, st>>>(p, s, n);
+    k_hyp_from_rt<<<(n + 127) / 128 + 1, 128, 0, st>>>(p, s, t, n);
 }
 
 // ---------------------------------------------------------------------------

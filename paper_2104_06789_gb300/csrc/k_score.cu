@@ -3,28 +3,17 @@
 // over the pixels whose pi_{t-1} is valid -- the MIE criterion of Eq. 10 with
 // the pose as the free variable (Eq. 9's MLE form as the ablation variant).
 //
-// Per pair, with the pixel record (xb, yb2, w, ut, vt, beta, beta_k, Cp, wq)
-// and the hypothesis in scaled form (E, tt):
-//   a    = E (xb, yb2, 1) + tt w                (camera-t point / z_{t-1} - p)
-//   r_u  = (a_x - xb a_z) / (1 + a_z) - ut      (residual / fx, no cancellation
-//   r_v  = (a_y - yb2 a_z) / (1 + a_z) - vt      against the pixel position)
+// Per (hypothesis, pixel) pair, with the scaled form (E, tt) of the hypothesis
+// and the pixel's normalised coordinates, inverse depth and flow over fx:
+//   a_z, U, V               three contractions (score_ops.cuh)
+//   r_u  = U / (1 + a_z), r_v = V / (1 + a_z)          (residual / fx)
 //   xs   = r_u^2 + r_v^2, clamped to [xs_min, xs_max]  (squared residual / fx^2)
 //   s    = beta log2(xs) + beta_k               (log2 of (x/alpha)^beta)
 //   r    = Cp xs (2^s + 2 + 2^-s)               (= mu / rho, Eqs. 3-4, 7)
 //   ell  = -log1p(r); behind camera t (1 + a_z <= 0) rho := mu, ell = -log 2.
-// SFU work: rcp, lg2, ex2, ex2, lg2 (for r >= 1/8); log1p(r) for r < 1/8 is a
-// polynomial on the FMA pipe, because lg2 near 1 has only absolute accuracy.
-//
-// The FP32 add / mul / fma work runs on packed pairs: two hypotheses share a
-// 64-bit register pair and one .f32x2 instruction does both lanes, which
-// halves the issue slots of the FMA-pipe work (the pipe still does 128 lane
-// operations per SM clock: after the SFU it is this kernel's second limit).
-// Each thread carries 1 pair (2 hypotheses, three 256-thread blocks per SM:
-// the default shape), 2 pairs (4 hypotheses, two blocks per SM) or 4 pairs
-// (8 hypotheses, one block per SM); the pixel
-// loop is software-pipelined over two consecutive pixels; pixel records are
-// bulk-copied into shared memory tile by tile and expanded there into both
-// lanes; sums are FP32 per 256-pixel tile, then FP64.
+// The contractions run on the tensor cores (tcgen05, BF16 slices, FP32
+// accumulation in tensor memory); the rest is FP32 on packed pairs of
+// hypotheses (.f32x2), with the SFU's rcp, lg2 and ex2.
 #include <cmath>
 #include <mutex>
 #include <type_traits>
@@ -32,6 +21,8 @@
 
 #include <algorithm>
 
+#include "score_ops.cuh"
+#include "tc.cuh"
 #include "voldor_internal.cuh"
 
 namespace vd {
@@ -109,51 +100,9 @@ __device__ __forceinline__ float pair_term2(const HypF& h, const float4 a, const
     return v;
 }
 
-// Bulk-copy staging of pixel-record tiles: one thread issues
-// cp.async.bulk (global -> shared) completing on an mbarrier per ring slot;
-// every thread waits on the slot's phase with a bounded try_wait.
-constexpr int kTilePix = 256;                       // records per tile (12 KB)
-constexpr int kStages = 2;
-constexpr long long kWaitLimit = 1ll << 26;        // bounded spin on an mbarrier phase
-
-__device__ __forceinline__ uint32_t smem_u32(const void* ptr)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(ptr));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n .reg .pred P;\n mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n selp.u32 %0, 1, 0, P;\n}"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long limit = kWaitLimit)
-{
-    for (long long i = 0; i < limit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
 
 // ---------------------------------------------------------------------------
-// Packed pair arithmetic (.f32x2) and the packed pair term.
+// Packed pair arithmetic (.f32x2).
 // ---------------------------------------------------------------------------
 typedef unsigned long long f2;      // {lo, hi} FP32 lanes
 
@@ -177,6 +126,8 @@ __device__ __forceinline__ float f2_hi(f2 v)
     asm("mov.b64 {_, %0}, %1;" : "=f"(hi) : "l"(v));
     return hi;
 }
+
+__device__ __forceinline__ f2 f2_both(float v) { return f2_pack(v, v); }
 
 __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
 {
@@ -208,297 +159,445 @@ __device__ __forceinline__ f2 f2_mul(f2 a, f2 b)
 
 __device__ __forceinline__ f2 f2_lg2(f2 v) { return f2_pack(mufu_lg2(f2_lo(v)), mufu_lg2(f2_hi(v))); }
 
-// c >= 0 ? a : b, one instruction per lane
-__device__ __forceinline__ float slct(float a, float b, float c)
-{
-    float d;
-    asm("slct.f32.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
-// A hypothesis pair in packed form: the rows of a_x and a_y negated, a_z as is.
-struct HypX2 {
-    f2 x0, x1, x2, xt, y0, y1, y2, yt, z0, z1, z2, zt;
+// ---------------------------------------------------------------------------
+// Terms of P hypothesis pairs against the lane's pixel, added to acc.
+// ---------------------------------------------------------------------------
+struct PixConst {
+    f2 beta, beta_k, Cp, wq;
+    float xmu;                       // x_mu / fx^2: the squared residual at which rho = mu
 };
 
-// Pixel record expanded in shared memory: each field in both lanes.
-struct PixX2 {
-    f2 xb, yb2, w, ut, vt, beta, beta_k, Cp, wq, pad;
-};
-static_assert(sizeof(PixX2) == 80, "PixX2 is five 16-byte words");
-
-
-// log2(1 + r) (MIE) or log2(r) (MLE), r = mu / rho, of two hypotheses against
-// one pixel, with the checks of pair_term2<true>; the residual's sign is
-// flipped (it is squared). kGauss: the Gaussian residual model, r = 2^s with
-// s = xs fx^2 / alpha - x_mu / alpha (record fields beta, beta_k), and
-// log2(1 + 2^s) = max(s, 0) + log2(1 + 2^-|s|).
-//
-// The term is computed in two halves so that the tile loop can overlap the
-// second half of one pixel with the first half of the next: the front
-// (projection, reciprocal, squared residual and, under the Fisk model, its
-// log2) leaves u = Cp xs, s and -(1 + a_z); the back (the exponentials, the
-// log1p and the selects) finishes the term.
-struct PairMid {
-    f2 u, s, nden;
-};
-
-template <bool kGauss>
-__device__ __forceinline__ PairMid pair_front(const HypX2& h, const PixX2& q, float xs_min, float xs_max)
+// The polynomial of log2_1p_pos for r < 1/8.
+__device__ __forceinline__ f2 log2_1p_small(f2 r)
 {
-    const f2 nax = f2_fma(h.x0, q.xb, f2_fma(h.x1, q.yb2, f2_fma(h.xt, q.w, h.x2)));   // -a_x
-    const f2 nay = f2_fma(h.y0, q.xb, f2_fma(h.y1, q.yb2, f2_fma(h.yt, q.w, h.y2)));   // -a_y
-    const f2 az = f2_fma(h.z0, q.xb, f2_fma(h.z1, q.yb2, f2_fma(h.zt, q.w, h.z2)));
-    const f2 mu = f2_fma(q.xb, az, nax);         // xb a_z - a_x
-    const f2 mv = f2_fma(q.yb2, az, nay);
-    const f2 nden = f2_sub(f2_pack(-1.f, -1.f), az);                     // -(1 + a_z), exactly
-    const f2 rd = f2_pack(mufu_rcp(-f2_lo(nden)), mufu_rcp(-f2_hi(nden)));
-    const f2 ru = f2_fma(mu, rd, q.ut);          // -(residual u) / fx
-    const f2 rv = f2_fma(mv, rd, q.vt);
-    f2 xs = f2_fma(ru, ru, f2_mul(rv, rv));
-    xs = f2_pack(fminf(fmaxf(f2_lo(xs), xs_min), xs_max), fminf(fmaxf(f2_hi(xs), xs_min), xs_max));
-    if (kGauss) return PairMid{xs, f2_fma(q.beta, xs, q.beta_k), nden};       // s = log2(mu / rho)
-    return PairMid{f2_mul(q.Cp, xs), f2_fma(q.beta, f2_lg2(xs), q.beta_k), nden};
+    f2 p = f2_fma(r, f2_both(kL1pC3), f2_both(kL1pC2));
+    p = f2_fma(r, p, f2_both(kL1pC1));
+    p = f2_fma(r, p, f2_both(kL1pC0));
+    return f2_mul(r, p);
 }
 
-template <bool kMLE, bool kGauss>
-__device__ __forceinline__ f2 pair_back(const PairMid& m)
+// log2(1 + r) from that polynomial (`small`) or, for r >= 1/8, lg2 of r1 = 1 + r; the
+// lg2 is predicated, so a warp whose 32 pixels all lie below issues none.
+__device__ __forceinline__ float lg2_if_large(float small, float r, float r1)
 {
-    const f2 ONE = f2_pack(1.f, 1.f), TWO = f2_pack(2.f, 2.f);
-    const f2 nden = m.nden;
-    const float behind = kMLE ? 0.f : 1.f;       // 1 + a_z <= 0: rho := mu
-    if (kGauss) {
-        const float g0 = f2_lo(m.s), g1 = f2_hi(m.s);
-        if (kMLE) return f2_pack(slct(behind, g0, f2_lo(nden)), slct(behind, g1, f2_hi(nden)));
-        const f2 e = f2_pack(mufu_ex2(-fabsf(g0)), mufu_ex2(-fabsf(g1)));
-        f2 ps = f2_fma(e, f2_pack(kL1pC3, kL1pC3), f2_pack(kL1pC2, kL1pC2));
-        ps = f2_fma(e, ps, f2_pack(kL1pC1, kL1pC1));
-        ps = f2_fma(e, ps, f2_pack(kL1pC0, kL1pC0));
-        const f2 small = f2_mul(e, ps);
-        const f2 big = f2_lg2(f2_add(e, ONE));
-        const f2 d = f2_add(e, f2_pack(-kL1pMax, -kL1pMax));
-        const float v0 = fmaxf(g0, 0.f) + slct(f2_lo(big), f2_lo(small), f2_lo(d));
-        const float v1 = fmaxf(g1, 0.f) + slct(f2_hi(big), f2_hi(small), f2_hi(d));
-        return f2_pack(slct(behind, v0, f2_lo(nden)), slct(behind, v1, f2_hi(nden)));
-    }
-    const float s0 = f2_lo(m.s), s1 = f2_hi(m.s);
-    const f2 ep = f2_pack(mufu_ex2(s0), mufu_ex2(s1)), en = f2_pack(mufu_ex2(-s0), mufu_ex2(-s1));
-    const f2 r = f2_mul(m.u, f2_add(ep, f2_add(en, TWO)));
-    if (kMLE) {
-        const f2 v = f2_lg2(r);
-        return f2_pack(slct(behind, f2_lo(v), f2_lo(nden)), slct(behind, f2_hi(v), f2_hi(nden)));
-    }
-    f2 ps = f2_fma(r, f2_pack(kL1pC3, kL1pC3), f2_pack(kL1pC2, kL1pC2));
-    ps = f2_fma(r, ps, f2_pack(kL1pC1, kL1pC1));
-    ps = f2_fma(r, ps, f2_pack(kL1pC0, kL1pC0));
-    const f2 small = f2_mul(r, ps);
-    const f2 big = f2_lg2(f2_add(r, ONE));
-    const f2 d = f2_add(r, f2_pack(-kL1pMax, -kL1pMax));
-    const float v0 = slct(f2_lo(big), f2_lo(small), f2_lo(d)), v1 = slct(f2_hi(big), f2_hi(small), f2_hi(d));
-    return f2_pack(slct(behind, v0, f2_lo(nden)), slct(behind, v1, f2_hi(nden)));
+    static_assert(kL1pMax == 0.125f, "the literal below");
+    asm("{\n .reg .pred p;\n setp.ge.f32 p, %1, 0f3E000000;\n @p lg2.approx.ftz.f32 %0, %2;\n}"
+        : "+f"(small) : "f"(r), "f"(r1));
+    return small;
 }
 
-// One shared-memory tile against the first NS hypothesis pairs of the thread,
-// software-pipelined over the pixels: the front half of pixel q is issued
-// beside the back half of pixel q - 1 (independent chains), and each pixel's
-// term is added to the accumulator in pixel order as before.
-template <int NS, bool MLE, bool GAUSS>
-__device__ __forceinline__ void score_tile(const HypX2* hy, const PixX2* xt, int cnt, float xs_min, float xs_max,
-                                           f2* facc)
+// U, V and a_z of P pairs against the lane's pixel. One reciprocal serves the two
+// lanes of a pair, 1 / d0 = d1 / (d0 d1), d = 1 + a_z: a nonzero d is at least 2^-25
+// in size (the spacing of a_z near -1), so adding 2^-40 moves no d beyond its own
+// rounding and keeps an exact 0 from spoiling its partner; above, kWild frames (the
+// only ones where |d| may reach 2^62) take a reciprocal per lane. Behind the
+// camera (d <= 0) rho := mu. The loops over P keep P independent chains side by
+// side for the in-order issue.
+template <int P, bool kMLE, bool kGauss, bool kWild>
+__device__ __forceinline__ void score_pairs(const uint32_t* U, const uint32_t* V, const uint32_t* Z, const PixConst& q,
+                                            float xs_min, float xs_max, f2* acc)
 {
-    if (cnt <= 0) return;
-    PairMid m[NS];
-    f2 wq = xt[0].wq;
+    auto at = [](const uint32_t* v, int i) { return f2_pack(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])); };
+    f2 nden[P];                                           // -(1 + a_z)
 #pragma unroll
-    for (int k = 0; k < NS; ++k) m[k] = pair_front<GAUSS>(hy[k], xt[0], xs_min, xs_max);
-    for (int q = 1; q < cnt; ++q) {
-        const PixX2 px = xt[q];
-        PairMid n[NS];
+    for (int i = 0; i < P; ++i) nden[i] = f2_sub(f2_both(-1.f), at(Z, i));
+    f2 xs[P], s[P], v[P];
 #pragma unroll
-        for (int k = 0; k < NS; ++k) n[k] = pair_front<GAUSS>(hy[k], px, xs_min, xs_max);
-#pragma unroll
-        for (int k = 0; k < NS; ++k) {
-            facc[k] = f2_fma(wq, pair_back<MLE, GAUSS>(m[k]), facc[k]);
-            m[k] = n[k];
+    for (int i = 0; i < P; ++i) {
+        f2 rd;                                            // -1 / (1 + a_z): squared below
+        if (kWild) {
+            rd = f2_pack(mufu_rcp(f2_lo(nden[i])), mufu_rcp(f2_hi(nden[i])));
+        } else {
+            const f2 d = f2_add(nden[i], f2_both(9.094947e-13f));
+            const float inv = mufu_rcp(f2_lo(d) * f2_hi(d));
+            rd = f2_pack(inv * f2_hi(d), inv * f2_lo(d));
         }
-        wq = px.wq;
+        const f2 ru = f2_mul(at(U, i), rd), rv = f2_mul(at(V, i), rd);
+        const f2 x = f2_fma(ru, ru, f2_mul(rv, rv));
+        float x0 = fminf(fmaxf(f2_lo(x), xs_min), xs_max), x1 = fminf(fmaxf(f2_hi(x), xs_min), xs_max);
+        if (!kGauss && !kMLE) {
+            x0 = f2_lo(nden[i]) >= 0.f ? q.xmu : x0;
+            x1 = f2_hi(nden[i]) >= 0.f ? q.xmu : x1;
+        }
+        xs[i] = f2_pack(x0, x1);
     }
 #pragma unroll
-    for (int k = 0; k < NS; ++k) facc[k] = f2_fma(wq, pair_back<MLE, GAUSS>(m[k]), facc[k]);
+    for (int i = 0; i < P; ++i) s[i] = f2_fma(q.beta, kGauss ? xs[i] : f2_lg2(xs[i]), q.beta_k);
+    if (kGauss) {
+        // log2(mu / rho) = s; log2(1 + 2^s) = max(s, 0) + log2(1 + 2^-|s|)
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            v[i] = s[i];
+            if (!kMLE) {
+                const float g0 = f2_lo(s[i]), g1 = f2_hi(s[i]);
+                const f2 e = f2_pack(mufu_ex2(-fabsf(g0)), mufu_ex2(-fabsf(g1)));
+                const f2 sm = log2_1p_small(e), e1 = f2_add(e, f2_both(1.f));
+                v[i] = f2_add(f2_pack(fmaxf(g0, 0.f), fmaxf(g1, 0.f)),
+                              f2_pack(lg2_if_large(f2_lo(sm), f2_lo(e), f2_lo(e1)), lg2_if_large(f2_hi(sm), f2_hi(e), f2_hi(e1))));
+            }
+        }
+    } else {
+        f2 r[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            const float s0 = f2_lo(s[i]), s1 = f2_hi(s[i]);
+            const f2 ep = f2_pack(mufu_ex2(s0), mufu_ex2(s1)), en = f2_pack(mufu_ex2(-s0), mufu_ex2(-s1));
+            r[i] = f2_mul(f2_mul(q.Cp, xs[i]), f2_add(ep, f2_add(en, f2_both(2.f))));
+        }
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            if (kMLE) {
+                v[i] = f2_lg2(r[i]);
+            } else {
+                const f2 sm = log2_1p_small(r[i]), r1 = f2_add(r[i], f2_both(1.f));
+                v[i] = f2_pack(lg2_if_large(f2_lo(sm), f2_lo(r[i]), f2_lo(r1)), lg2_if_large(f2_hi(sm), f2_hi(r[i]), f2_hi(r1)));
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        if (kGauss || kMLE) {
+            constexpr float behind = kMLE ? 0.f : 1.f;
+            v[i] = f2_pack(f2_lo(nden[i]) >= 0.f ? behind : f2_lo(v[i]), f2_hi(nden[i]) >= 0.f ? behind : f2_hi(v[i]));
+        }
+        acc[i] = f2_fma(q.wq, v[i], acc[i]);
+    }
 }
 
-// SLOTS hypothesis pairs per thread; MINB resident blocks per SM. A block
-// scores a tile of 2 * SLOTS * 256 hypotheses against one chunk of the pixel
-// records. The tile is cut into groups of 64 consecutive hypotheses, and warp
-// slot k of a warp holds one group, lane l taking hypotheses 2l and 2l + 1 of
-// it. A full tile needs every warp slot (16 groups for SLOTS = 2): warp w holds
-// groups w * SLOTS .. w * SLOTS + SLOTS - 1 and scores every pixel of the
-// chunk. The last, partial tile of a frame needs only u = ceil(m / 64) groups
-// for its m hypotheses, i.e. wpg = ceil(u / SLOTS) warps; the block's warps
-// then form P = 8 / wpg teams of wpg warps, team j scoring the same groups on
-// the j-th of P equal parts of every pixel tile, and the teams' sums are added
-// in team order at the end. So a partial tile costs about m / 1024 of a full
-// one instead of a whole 512-hypothesis slot per started slot. The autotuner
-// picks among the instances.
-template <int SLOTS, int MINB, bool MLE, bool GAUSS>
-__global__ void __launch_bounds__(kScoreThreads, MINB) k_score(DevParams p, DevState s, int log_idx)
+// NC consecutive TMEM columns of the warp's 32 lanes.
+template <int NC>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r);
+
+template <>
+__device__ __forceinline__ void tmem_ld<2>(uint32_t taddr, uint32_t* r)
 {
-    constexpr int HPT = 2 * SLOTS;
-    constexpr int kWarps = kScoreThreads / 32;
-    const int n_hyp = *s.n_hyp;
-    const int n_pix = *s.pix_count;
-    if (log_idx >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+}
+
+template <>
+__device__ __forceinline__ void tmem_ld<4>(uint32_t taddr, uint32_t* r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
+}
+
+template <>
+__device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t* r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// Bounded wait on an mbarrier phase: false (and *bad set, if given) on expiry or
+// when another role of the CTA already gave up. The loop is out of line: the
+// first try nearly always succeeds, and the hot loop holds only that.
+constexpr long long kWaitLimit = 1ll << 26;
+
+__device__ __noinline__ bool score_wait_loop(uint32_t bar, uint32_t parity, volatile int* bad, long long limit)
+{
+    for (long long i = 0; i < limit; ++i) {
+        if (tc_try_wait(bar, parity)) return true;
+        if ((i & 1023) == 1023 && bad && *bad) return false;
+    }
+    if (bad) *bad = 1;
+    return false;
+}
+
+__device__ __forceinline__ bool score_wait(uint32_t bar, uint32_t parity, volatile int* bad)
+{
+    return tc_try_wait(bar, parity) || score_wait_loop(bar, parity, bad, kWaitLimit);
+}
+
+// ---------------------------------------------------------------------------
+// The scoring kernel: one persistent CTA per SM over work items (pixel chunk,
+// group of 128 hypotheses), chunk-major so that the CTAs running at one time
+// share the pixel tiles in L2. Warp roles:
+//   warp 16, one lane: bulk copies of an item's hypothesis operand (40 KB, two
+//     buffers) and pixel tiles (128 pixels, 24 KB, kScSlots slots);
+//   warp 17, one lane: per tile and stage of 32 hypotheses six MMAs of M = 128
+//     pixels, K = 16 (N = 96: S by US, VS, ZS; N = 32: U by XU, V by XV) into one of
+//     five TMEM buffers of 96 columns U, V, a_z;
+//   warps 0-15: warp w takes the 32 pixels of TMEM lane quarter w % 4 and stage
+//     w / 4 of the group, kL hypotheses at a time: one pixel per lane, the
+//     hypotheses packed in pairs. Four warp groups and five buffers: a group's
+//     next tile is computed while it works on this one. A lane's sums over its pixels
+//     are FP32 over at most kScFlush tiles, then added across lanes and from
+//     there on in FP64; the four quarters' sums are added in order.
+//
+// What bounds it. Per SM sub-partition and 64 pairs (one warp instruction of
+// packed pairs) the Fisk / MIE term costs 56 cycles of SFU time (half an rcp, one
+// lg2, two ex2 per pair, one lg2 where r >= 1/8; rcp and lg2 take 8 cycles per
+// warp, ex2 4) and 49 issue slots, of which the 17 packed instructions hold the
+// dispatch port two cycles each; it runs in 73 cycles, the SFU 77 % busy, the
+// tensor pipe 10 %. With the contractions in FP32 on the CUDA cores the term
+// needed 28 packed instructions and five shared-memory loads per pixel and was
+// bound by dispatch: 88 cycles. 8192 hypotheses x 465,750 pixels: 4.38 -> 3.64 ms.
+// Measured and not kept: 8 or 12 compute warps with more registers (101 and 91
+// cycles against 88 with 16 at the first version), all arithmetic scalar (79
+// against 73), two 64-hypothesis buffers (76), lg2(1 + r) as a polynomial on the
+// FMA pipe (115 in the FP32 kernel), and a shortened register share for the two
+// issuing warps (setmaxnreg; 95).
+// ---------------------------------------------------------------------------
+constexpr int kScWarps = 16;                              // compute warps
+constexpr int kScThreads = (kScWarps + 2) * 32;
+constexpr int kScSlots = 3;
+constexpr int kScFlush = 64;                              // tiles summed in FP32 per lane: 64 terms, then 4 lanes
+constexpr int kScHypOff = kScSlots * kScTileBytes;
+constexpr int kScBarOff = kScHypOff + 2 * kScGroupBytes;
+constexpr int kScRedOff = kScBarOff + 256;
+constexpr int kScSmemBytes = kScRedOff + 2 * 4 * kScGroupHyps * 8;
+constexpr int kScStageCols = 3 * kScStageHyps;            // TMEM columns of a buffer
+constexpr int kScBufs = 5;
+constexpr int kScTmemCols = 512;                          // the buffers' 480, rounded up to a power of two
+
+struct ScItem {
+    int t0, cnt, hyps;                                    // first tile, tiles, hypotheses
+};
+
+template <int kL, bool kMLE, bool kGauss>
+__global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s, int log_idx)
+{
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const uint32_t sb = smem_addr(smem), ring = sb, hyp_s = sb + kScHypOff, bars = sb + kScBarOff;
+    const uint32_t full = bars, empty = full + 8 * kScSlots, hfull = empty + 8 * kScSlots, hempty = hfull + 16;
+    const uint32_t afull = hempty + 16, aempty = afull + 8 * kScBufs, done = aempty + 8 * kScBufs;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kScBarOff + 200);
+    volatile int& bad = *reinterpret_cast<volatile int*>(smem + kScBarOff + 204);
+    double* red = reinterpret_cast<double*>(smem + kScRedOff);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n_hyp = *s.n_hyp, n_pix = *s.pix_count;
+    if (log_idx >= 0 && blockIdx.x == 0 && threadIdx.x == 0) {
         s.score_log[2 * log_idx] = n_hyp;
         s.score_log[2 * log_idx + 1] = n_pix;
     }
-    // tile-major block order: the partial last hypothesis tile's (lighter)
-    // blocks are scheduled after every full tile's, so they fill the last wave
-    const int blk = blockIdx.x + gridDim.x * blockIdx.y;
-    const int n_chunks = gridDim.y, chunk = blk % n_chunks;
-    const int tile0 = (blk / n_chunks) * (kScoreThreads * HPT);
-    if (tile0 >= n_hyp) return;
-    const long long lo = (long long)n_pix * chunk / n_chunks;
-    const long long hi = (long long)n_pix * (chunk + 1) / n_chunks;
-    const int n_tiles = (int)((hi - lo + kTilePix - 1) / kTilePix);
-
-    // work split (block-uniform; warp-uniform per warp)
-    const int m = min(n_hyp - tile0, kScoreThreads * HPT);
-    const int u = (m + 63) / 64;                       // hypothesis groups of this tile
-    const int wpg = (u + SLOTS - 1) / SLOTS;           // warps per team
-    const int P = kWarps / wpg;                        // teams
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int team = warp / wpg, wg = warp - team * wpg;
-    const int nsw = team < P ? max(0, min(SLOTS, u - wg * SLOTS)) : 0;   // this warp's groups
-
-    __shared__ __align__(128) float4 tile[kStages][kTilePix * 3];
-    __shared__ __align__(16) PixX2 xt[kTilePix];
-    __shared__ __align__(8) uint64_t full[kStages];
-    __shared__ int timed_out;
-    const float4* gpix = reinterpret_cast<const float4*>(s.pix);
-    auto issue = [&](int it) {
-        const long long j0 = lo + (long long)it * kTilePix;
-        const int cnt = (int)min((long long)kTilePix, hi - j0);
-        const uint32_t bytes = (uint32_t)cnt * (uint32_t)sizeof(PixRec);
-        uint64_t* bar = &full[it % kStages];
-        mbar_expect_tx(bar, bytes);
-        bulk_g2s(&tile[it % kStages][0], gpix + 3 * j0, bytes, bar);
+    const int n_tiles = (n_pix + kScTilePix - 1) / kScTilePix;
+    const int n_groups = (n_hyp + kScGroupHyps - 1) / kScGroupHyps, n_chunks = s.n_chunks;
+    const int n_items = n_groups * n_chunks;
+    if (blockIdx.x >= n_items) return;
+    auto item = [&](int u) {
+        const int chunk = u / n_groups, group = u % n_groups;
+        ScItem w;
+        w.t0 = (int)((long long)n_tiles * chunk / n_chunks);
+        w.cnt = (int)((long long)n_tiles * (chunk + 1) / n_chunks) - w.t0;
+        w.hyps = min(kScGroupHyps, n_hyp - group * kScGroupHyps);
+        return w;
     };
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) mbar_init(&full[i], 1);
+        for (int i = 0; i < kScSlots; ++i) {
+            tc_mbar_init(full + 8 * i, 1);
+            tc_mbar_init(empty + 8 * i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            tc_mbar_init(hfull + 8 * i, 1);
+            tc_mbar_init(hempty + 8 * i, 1);
+        }
+        for (int i = 0; i < kScBufs; ++i) {
+            tc_mbar_init(afull + 8 * i, 1);
+            tc_mbar_init(aempty + 8 * i, kScWarps / kScGroupStages);
+        }
+        tc_mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        timed_out = 0;
+        bad = 0;
     }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
+                     "r"((uint32_t)kScTmemCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int i = 0; i < kStages && i < n_tiles; ++i) issue(i);
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
 
-    // hypothesis of slot k, lane half v: tile0 + (wg * SLOTS + k) * 64 + 2 * lane + v
-    const int hbase = tile0 + wg * SLOTS * 64 + 2 * lane;
-    HypX2 hy[SLOTS];
-    {
-#pragma unroll
-        for (int k = 0; k < SLOTS; ++k) {
-            HypF a[2];
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int h = hbase + k * 64 + v;
-                const float* f = s.hyp_f32 + (size_t)min(h, n_hyp - 1) * 12;
-                a[v] = HypF{f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8], f[9], f[10], f[11]};
+    if (warp == kScWarps) {
+        if (lane == 0) {
+            // loader: n counts tiles, w work items (those with pixels)
+            uint32_t n = 0, w = 0;
+            for (int u = blockIdx.x; u < n_items && !bad; u += gridDim.x) {
+                const ScItem it = item(u);
+                if (it.cnt == 0) continue;
+                const uint32_t hb = w & 1, bytes = (it.hyps + kScStageHyps - 1) / kScStageHyps * kScStageBytes;
+                if (w >= 2 && !score_wait(hempty + 8 * hb, ((w >> 1) - 1) & 1, &bad)) break;
+                tc_expect_tx(hfull + 8 * hb, bytes);
+                tc_bulk_g2s(hyp_s + hb * kScGroupBytes, s.sc_hyp + (size_t)(u % n_groups) * kScGroupBytes, bytes, hfull + 8 * hb);
+                ++w;
+                for (int k = 0; k < it.cnt && !bad; ++k, ++n) {
+                    const uint32_t slot = n % kScSlots;
+                    if (n >= kScSlots && !score_wait(empty + 8 * slot, ((n / kScSlots) - 1) & 1, &bad)) break;
+                    tc_expect_tx(full + 8 * slot, kScTileBytes);
+                    tc_bulk_g2s(ring + slot * kScTileBytes, s.sc_pix + (size_t)(it.t0 + k) * kScTileBytes, kScTileBytes, full + 8 * slot);
+                }
             }
-            hy[k] = HypX2{f2_pack(-a[0].e0, -a[1].e0), f2_pack(-a[0].e1, -a[1].e1), f2_pack(-a[0].e2, -a[1].e2),
-                          f2_pack(-a[0].t0, -a[1].t0), f2_pack(-a[0].e3, -a[1].e3), f2_pack(-a[0].e4, -a[1].e4),
-                          f2_pack(-a[0].e5, -a[1].e5), f2_pack(-a[0].t1, -a[1].t1), f2_pack(a[0].e6, a[1].e6),
-                          f2_pack(a[0].e7, a[1].e7), f2_pack(a[0].e8, a[1].e8), f2_pack(a[0].t2, a[1].t2)};
+            // the last copies may still be landing when another role gave up
+            for (uint32_t j = n > kScSlots ? n - kScSlots : 0; j < n; ++j)
+                score_wait(full + 8 * (j % kScSlots), (j / kScSlots) & 1, nullptr);
+            for (uint32_t j = w > 2 ? w - 2 : 0; j < w; ++j) score_wait(hfull + 8 * (j & 1), (j >> 1) & 1, nullptr);
+        }
+    } else if (warp == kScWarps + 1) {
+        if (lane == 0) {
+            // MMA issuer: m counts stages (stage m in TMEM buffer m % kScBufs)
+            constexpr uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kScTilePix >> 4) << 24);
+            constexpr uint32_t idS = id | ((uint32_t)(3 * kScStageHyps >> 3) << 17), idX = id | ((uint32_t)(kScStageHyps >> 3) << 17);
+            constexpr uint32_t kA = kScTilePix * 16;                   // bytes of a column block of A
+            uint32_t n = 0, w = 0, m = 0;
+            for (int u = blockIdx.x; u < n_items && !bad; u += gridDim.x) {
+                const ScItem it = item(u);
+                if (it.cnt == 0) continue;
+                const uint32_t hb = w & 1;
+                if (!score_wait(hfull + 8 * hb, (w >> 1) & 1, &bad)) break;
+                const int stages = (it.hyps + kScStageHyps - 1) / kScStageHyps;
+                for (int k = 0; k < it.cnt && !bad; ++k, ++n) {
+                    const uint32_t slot = n % kScSlots, a = ring + slot * kScTileBytes;
+                    if (!score_wait(full + 8 * slot, (n / kScSlots) & 1, &bad)) break;
+                    for (int st = 0; st < stages; ++st, ++m) {
+                        const uint32_t tb = m % kScBufs;
+                        if (m >= kScBufs && !score_wait(aempty + 8 * tb, ((m / kScBufs) - 1) & 1, &bad)) break;
+                        tc_fence_after();
+                        const uint32_t b = hyp_s + hb * kScGroupBytes + st * kScStageBytes, d = tmem + tb * kScStageCols;
+                        // column blocks of A: S at 0, U at 4, V at 8; each block's small products are in its
+                        // first two column blocks, the large ones of U and V in the last two of U and V
+                        auto mma_s = [&](int half, uint32_t acc) {
+                            tc_mma(d, tc_desc(a + 2 * half * kA, kA, 128), tc_desc(b + 2 * half * kScHypSBlock, kScHypSBlock, 128), idS, acc);
+                        };
+                        auto mma_x = [&](int v, int half) {
+                            tc_mma(d + v * kScStageHyps, tc_desc(a + (4 + 4 * v + 2 * half) * kA, kA, 128),
+                                   tc_desc(b + (v ? kScHypVOff : kScHypUOff) + 2 * half * kScHypXBlock, kScHypXBlock, 128), idX, 1u);
+                        };
+                        mma_s(0, 0u);
+                        mma_s(1, 1u);
+                        mma_x(0, 0);
+                        mma_x(1, 0);
+                        mma_x(0, 1);
+                        mma_x(1, 1);
+                        tc_commit(afull + 8 * tb);
+                    }
+                    if (bad) break;
+                    tc_commit(empty + 8 * slot);
+                }
+                if (bad) break;
+                tc_commit(hempty + 8 * hb);
+                ++w;
+            }
+            tc_commit(done);                  // arrives once every MMA issued above has completed
+            score_wait(done, 0, nullptr);
+        }
+    } else {
+        const int quarter = warp & 3, wg = warp >> 2;
+        const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16);
+        const float xs_min = p.xs_min, xs_max = p.xs_max;
+        const bool wild = *s.sc_wild != 0;
+        uint32_t tb = 0, phase = 0;                          // TMEM buffer of the next tile's stage 0 and its phase
+        int buf = 0;
+        bool go = true;
+        f2 acc[kScStageHyps / 2];
+        // tiles [t0, t1) of `stages` stages: the lane's pixel of each against the warp's 32 hypotheses
+        auto tiles = [&](auto is_wild, int t0, int t1, int stages) {
+            constexpr bool kWild = decltype(is_wild)::value;
+            int j = t0 * kScTilePix + quarter * 32 + lane;
+            // a lane past the last pixel: weight 0 and a finite term (whatever its operand row holds)
+            float4 cst;
+            float xmu;
+            auto load_const = [&]() {
+                const bool in = j < n_pix;
+                cst = in ? __ldg(s.sc_cst + j) : make_float4(0.f, 0.f, 1.f, 0.f);
+                xmu = in ? __ldg(s.sc_xmu + j) : 1.f;
+            };
+            load_const();
+            for (int t = t0; t < t1; ++t) {
+                const PixConst q{f2_both(cst.x), f2_both(cst.y), f2_both(cst.z), f2_both(cst.w), xmu};
+                j += kScTilePix;
+                load_const();
+                // every lane polls; the warp proceeds only together (tcgen05.ld is warp-wide)
+                const uint32_t b = tb + wg, bw = b >= kScBufs, buf8 = 8 * (b - bw * kScBufs);
+                go = __all_sync(0xffffffffu, score_wait(afull + buf8, phase ^ bw, &bad));
+                if (!go) return;
+                tc_fence_after();
+                const uint32_t cols = tlane + buf8 * (kScStageCols / 8);
+                tb += stages;
+                if (tb >= kScBufs) {
+                    tb -= kScBufs;
+                    phase ^= 1u;
+                }
+#pragma unroll
+                for (int part = 0; part < kScStageHyps / kL; ++part) {
+                    uint32_t U[kL], V[kL], Z[kL];
+                    tmem_ld<kL>(cols + part * kL, U);
+                    tmem_ld<kL>(cols + part * kL + kScStageHyps, V);
+                    tmem_ld<kL>(cols + part * kL + 2 * kScStageHyps, Z);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (part == kScStageHyps / kL - 1) {      // the warp's columns are in registers
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) tc_arrive(aempty + buf8);
+                    }
+                    score_pairs<kL / 2, kMLE, kGauss, kWild>(U, V, Z, q, xs_min, xs_max, &acc[part * (kL / 2)]);
+                }
+            }
+        };
+        // every warp passes every item's barrier, also after a wait gave up (go stays false)
+        for (int u = blockIdx.x; u < n_items; u += gridDim.x) {
+            const ScItem it = item(u);
+            double tot = 0.0;
+            const int stages = (it.hyps + kScStageHyps - 1) / kScStageHyps;
+            if (wg >= stages) {                              // nothing of this group for the warp: keep count of the buffers
+                const uint32_t b = tb + (uint32_t)(it.cnt * stages);
+                phase ^= (b / kScBufs) & 1u;
+                tb = b % kScBufs;
+            }
+            for (int k0 = 0; k0 < it.cnt && wg < stages && go; k0 += kScFlush) {
+                const int k1 = min(k0 + kScFlush, it.cnt);
+#pragma unroll
+                for (int i = 0; i < kScStageHyps / 2; ++i) acc[i] = 0ull;
+                if (wild) tiles(std::true_type{}, it.t0 + k0, it.t0 + k1, stages);
+                else tiles(std::false_type{}, it.t0 + k0, it.t0 + k1, stages);
+                // sums over the warp's 32 lanes: at each step a lane keeps half of its values and
+                // adds the partner's, so lane l ends with the sum of value l (FP32 over 4 lanes, then FP64)
+                float f[32];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    f[2 * i] = f2_lo(acc[i]);
+                    f[2 * i + 1] = f2_hi(acc[i]);
+                }
+#pragma unroll
+                for (int o = 16, m = 16; o >= 8; o >>= 1, m >>= 1)
+#pragma unroll
+                    for (int i = 0; i < m; ++i) {
+                        const bool up = (lane & o) != 0;
+                        const float send = up ? f[i] : f[i + m], keep = up ? f[i + m] : f[i];
+                        f[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                double d[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) d[i] = (double)f[i];
+#pragma unroll
+                for (int o = 4, m = 4; o >= 1; o >>= 1, m >>= 1)
+#pragma unroll
+                    for (int i = 0; i < m; ++i) {
+                        const bool up = (lane & o) != 0;
+                        const double send = up ? d[i] : d[i + m], keep = up ? d[i + m] : d[i];
+                        d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                tot += d[0];
+            }
+            red[(buf * 4 + quarter) * kScGroupHyps + wg * kScStageHyps + lane] = tot;
+            asm volatile("bar.sync 1, %0;" ::"n"(kScWarps * 32) : "memory");
+            const int h = threadIdx.x;
+            if (h < it.hyps) {
+                const double* r = red + buf * 4 * kScGroupHyps + h;
+                const double v = ((r[0] + r[kScGroupHyps]) + r[2 * kScGroupHyps]) + r[3 * kScGroupHyps];
+                s.partial[(size_t)(u / n_groups) * p.S + (u % n_groups) * kScGroupHyps + h] = -v * 0.69314718055994531;
+            }
+            buf ^= 1;          // the next item's sums go to the other buffer, so one barrier per item suffices
         }
     }
-    double acc[HPT];
-#pragma unroll
-    for (int i = 0; i < HPT; ++i) acc[i] = 0.0;
-    const float xs_min = p.xs_min, xs_max = p.xs_max;
-
-    // the tile loop; TEAMS = false is the full-tile case (one team, every
-    // pixel), kept as its own copy so that it carries no team state
-    int it = 0;
-    auto run = [&](auto teams) {
-        constexpr bool TEAMS = decltype(teams)::value;
-        for (; it < n_tiles; ++it) {
-            const int slot = it % kStages;
-            if (!mbar_wait_bounded(&full[slot], (uint32_t)((it / kStages) & 1))) atomicExch(&timed_out, 1);
-            const int cnt = (int)min((long long)kTilePix, hi - (lo + (long long)it * kTilePix));
-            if ((int)threadIdx.x < cnt) {
-                // expand record threadIdx.x into both lanes (a timed-out tile's
-                // contents are never used)
-                const float4* r = &tile[slot][3 * threadIdx.x];
-                const float4 a = r[0], b = r[1];
-                const float wq = r[2].x;
-                float4* x = reinterpret_cast<float4*>(&xt[threadIdx.x]);
-                x[0] = make_float4(a.x, a.x, a.y, a.y);
-                x[1] = make_float4(a.z, a.z, a.w, a.w);
-                x[2] = make_float4(b.x, b.x, b.y, b.y);
-                x[3] = make_float4(b.z, b.z, b.w, b.w);
-                x[4] = make_float4(wq, wq, 0.f, 0.f);
-            }
-            __syncthreads();                       // tile expanded; the raw slot is free
-            if (timed_out) break;
-            if (threadIdx.x == 0 && it + kStages < n_tiles) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                issue(it + kStages);
-            }
-            // this team's part of the tile
-            const int q0 = TEAMS ? cnt * team / P : 0, q1 = TEAMS ? cnt * (team + 1) / P : cnt;
-            f2 facc[SLOTS];
-#pragma unroll
-            for (int k = 0; k < SLOTS; ++k) facc[k] = 0ull;
-            if (nsw >= SLOTS) score_tile<SLOTS, MLE, GAUSS>(hy, xt + q0, q1 - q0, xs_min, xs_max, facc);
-            else if (SLOTS > 3 && nsw == 3) score_tile<(SLOTS > 3 ? 3 : 1), MLE, GAUSS>(hy, xt + q0, q1 - q0, xs_min, xs_max, facc);
-            else if (SLOTS > 2 && nsw == 2) score_tile<(SLOTS > 2 ? 2 : 1), MLE, GAUSS>(hy, xt + q0, q1 - q0, xs_min, xs_max, facc);
-            else if (nsw == 1) score_tile<1, MLE, GAUSS>(hy, xt + q0, q1 - q0, xs_min, xs_max, facc);
-#pragma unroll
-            for (int k = 0; k < SLOTS; ++k) {
-                acc[2 * k] += (double)f2_lo(facc[k]);
-                acc[2 * k + 1] += (double)f2_hi(facc[k]);
-            }
-            __syncthreads();                       // every thread is done with the expanded tile
-        }
-    };
-    if (P == 1) run(std::false_type{});
-    else run(std::true_type{});
-    if (timed_out) {
-        // drain the copies this block issued (bounded) before leaving
-        if (threadIdx.x == 0) {
-            for (int j = it; j < n_tiles && j < it + kStages; ++j)
-                mbar_wait_bounded(&full[j % kStages], (uint32_t)((j / kStages) & 1));
-            atomicOr(s.status + 3, kStatusTimeout);
-        }
-        return;
-    }
-    const int S = p.S;
-    if (P == 1) {
-        if (team == 0) {                               // warps past the one team scored nothing
-#pragma unroll
-            for (int i = 0; i < HPT; ++i) {
-                const int h = hbase + (i >> 1) * 64 + (i & 1);
-                if (h < n_hyp) s.partial[(size_t)chunk * S + h] = -acc[i] * 0.69314718055994531;
-            }
-        }
-        return;
-    }
-    // teams: sums per (team, hypothesis of the tile) in the expanded-tile
-    // buffer (free after the loop's last barrier; P * wpg * SLOTS * 64 <=
-    // 8 * SLOTS * 64 doubles fit in it), then added in team order
-    double* red = reinterpret_cast<double*>(xt);
-    const int span = wpg * SLOTS * 64;                 // hypotheses a team covers (>= m)
-    static_assert(kWarps * SLOTS * 64 * sizeof(double) <= sizeof(PixX2) * kTilePix, "team sums fit");
-    if (team < P) {
-#pragma unroll
-        for (int i = 0; i < HPT; ++i) red[team * span + (hbase - tile0) + (i >> 1) * 64 + (i & 1)] = acc[i];
-    }
+    tc_fence_before();
     __syncthreads();
-    for (int i = threadIdx.x; i < m; i += kScoreThreads) {
-        double t = 0.0;
-        for (int j = 0; j < P; ++j) t += red[j * span + i];
-        s.partial[(size_t)chunk * S + tile0 + i] = -t * 0.69314718055994531;
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kScTmemCols));
     }
+    if (threadIdx.x == 0 && bad) atomicOr(s.status + 3, kStatusTimeout);
 }
 
 // L_h = sum over the chunks' partials (natural-log units) in a fixed order:
@@ -553,46 +652,75 @@ static int num_sms()
     return g_num_sms;
 }
 
-// Pixel chunks so that (hypothesis tiles x chunks) blocks fill `waves` waves
-// of the resident blocks of a tile shape.
-int score_chunks_for(int S, int N, int hpt, int waves)
+// Pixel chunks of at most `waves` work items (pixel chunk x group of 128
+// hypotheses) per SM: the count with the shortest schedule, rounds of items times
+// an item's tiles plus kItemTiles, the cost of starting and flushing an item in
+// tiles. Few items leave the last round partly empty, many pay that cost each time.
+int score_chunks_for(int S, int N, int waves)
 {
-    const int minb = hpt == 8 ? 1 : (hpt == 4 ? 2 : 3);
-    const int tiles = (S + kScoreThreads * hpt - 1) / (kScoreThreads * hpt);
-    int chunks = (num_sms() * minb * waves + tiles - 1) / tiles;
-    if (chunks > N) chunks = N;
-    return chunks < 1 ? 1 : chunks;
+    constexpr double kItemTiles = 1.5;
+    const int groups = (S + kScGroupHyps - 1) / kScGroupHyps, tiles = (N + kScTilePix - 1) / kScTilePix, sms = num_sms();
+    const int most = std::max(1, std::min(sms * waves / groups, tiles));
+    int best = most;
+    double best_cost = 1e300;
+    for (int c = 1; c <= most; ++c) {
+        const double cost = ((groups * (long long)c + sms - 1) / sms) * ((tiles + c - 1) / c + kItemTiles);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
 }
 
-int score_chunks(int S, int N) { return score_chunks_for(S, N, kScoreDefaultHpt, kScoreDefaultWaves); }
+int score_chunks(int S, int N) { return score_chunks_for(S, N, kScoreDefaultWaves); }
 
+// Largest chunk count a window accepts (and its partial sums are sized for).
 int score_chunks_max(int S, int N)
 {
-    const int a = score_chunks_for(S, N, 8, kTuneMaxWaves), b = score_chunks_for(S, N, 4, kTuneMaxWaves);
-    const int c = score_chunks_for(S, N, 2, kTuneMaxWaves);
-    return std::max(a, std::max(b, c));
+    const int groups = (S + kScGroupHyps - 1) / kScGroupHyps, px = (N + kScTilePix - 1) / kScTilePix;
+    int most = std::max(1, std::min(num_sms() * kTuneMaxWaves / groups, px));
+    for (int hpt = 2; hpt <= 8; hpt *= 2) {
+        const int tiles = (S + 256 * hpt - 1) / (256 * hpt), blocks = hpt == 8 ? 1 : (hpt == 4 ? 2 : 3);
+        most = std::max(most, std::min((num_sms() * blocks * kTuneMaxWaves + tiles - 1) / tiles, N));
+    }
+    return most;
 }
 
-template <int SLOTS, int MINB>
+template <int kL, bool kMLE, bool kGauss>
+static void launch_score_as(const DevParams& p, const DevState& s, int li, cudaStream_t st)
+{
+    // the dynamic shared-memory limit is raised once per device
+    constexpr int kMaxDevices = 64;
+    static std::mutex mutex;
+    static bool raised[kMaxDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (!raised[dev])
+            raised[dev] = cudaFuncSetAttribute(k_score<kL, kMLE, kGauss>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               kScSmemBytes) == cudaSuccess;
+    }
+    const long long items = (long long)((p.S + kScGroupHyps - 1) / kScGroupHyps) * s.n_chunks;
+    k_score<kL, kMLE, kGauss><<<(unsigned)std::min<long long>(items, num_sms()), kScThreads, kScSmemBytes, st>>>(p, s, li);
+}
+
+template <int kL>
 static void launch_score_shape(const DevParams& p, const DevState& s, int li, cudaStream_t st)
 {
-    dim3 grid((p.S + kScoreThreads * 2 * SLOTS - 1) / (kScoreThreads * 2 * SLOTS), s.n_chunks);
     const bool mle = p.criterion == VOLDOR_CRITERION_MLE, gauss = p.residual == VOLDOR_RESIDUAL_GAUSSIAN;
-    if (gauss) {
-        if (mle) k_score<SLOTS, MINB, true, true><<<grid, kScoreThreads, 0, st>>>(p, s, li);
-        else k_score<SLOTS, MINB, false, true><<<grid, kScoreThreads, 0, st>>>(p, s, li);
-    } else {
-        if (mle) k_score<SLOTS, MINB, true, false><<<grid, kScoreThreads, 0, st>>>(p, s, li);
-        else k_score<SLOTS, MINB, false, false><<<grid, kScoreThreads, 0, st>>>(p, s, li);
-    }
+    if (gauss && mle) launch_score_as<kL, true, true>(p, s, li, st);
+    else if (gauss) launch_score_as<kL, false, true>(p, s, li, st);
+    else if (mle) launch_score_as<kL, true, false>(p, s, li, st);
+    else launch_score_as<kL, false, false>(p, s, li, st);
 }
 
 void launch_score(const DevParams& p, const DevState& s, int log_idx, cudaStream_t st)
 {
     const int li = log_idx < kScoreLogMax ? log_idx : -1;
-    if (s.score_hpt == 4) launch_score_shape<2, 2>(p, s, li, st);
-    else if (s.score_hpt == 2) launch_score_shape<1, 3>(p, s, li, st);
-    else launch_score_shape<4, 1>(p, s, li, st);
+    if (s.score_hpt == 4) launch_score_shape<4>(p, s, li, st);
+    else if (s.score_hpt == 2) launch_score_shape<2>(p, s, li, st);
+    else launch_score_shape<8>(p, s, li, st);
 }
 
 void launch_score_reduce(const DevParams& p, const DevState& s, cudaStream_t st)
@@ -843,12 +971,12 @@ __global__ void k_wait_probe(long long polls, long long* out)
 {
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
+        tc_mbar_init(smem_addr(&bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     const long long t0 = clock64();
-    const bool done = mbar_wait_bounded(&bar, 0, polls);
+    const bool done = score_wait_loop(smem_addr(&bar), 0, nullptr, polls);
     const long long t1 = clock64();
     const int gave_up = __syncthreads_count(!done);
     if (threadIdx.x == 0) {

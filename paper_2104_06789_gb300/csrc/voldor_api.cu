@@ -9,6 +9,7 @@
 #include <new>
 #include <vector>
 
+#include "score_ops.cuh"
 #include "voldor_internal.cuh"
 
 using namespace vd;
@@ -145,7 +146,11 @@ size_t layout(voldor_ctx& c, char* base)
     s.iter = (int*)take(4);
     s.status = (int*)take(16);
     c.flag_dev = (int*)take(4);
-    s.pix = (PixRec*)take(N * sizeof(PixRec));
+    s.sc_pix = (unsigned char*)take((N + kScTilePix - 1) / kScTilePix * kScTileBytes);
+    s.sc_cst = (float4*)take(N * sizeof(float4));
+    s.sc_xmu = (float*)take(N * sizeof(float));
+    s.sc_hyp = (unsigned char*)take((S + kScGroupHyps - 1) / kScGroupHyps * kScGroupBytes);
+    s.sc_wild = (int*)take(4);
     s.pix_block_count = (int*)take(((N + kPixThreads - 1) / kPixThreads) * 4);
     s.prep_done = (unsigned*)take(4);
     s.pix_count = (int*)take(4);
@@ -238,7 +243,7 @@ bool enqueue_pose_update(voldor_ctx* c, int t, cudaEvent_t ev0, cudaEvent_t ev1,
     if (!cuda_ok(c, cudaEventRecord(c->ev_join, c->aux))) return false;
     launch_prep_write(p, s, t, st);
     if (!cuda_ok(c, cudaStreamWaitEvent(st, c->ev_join, 0))) return false;
-    launch_hyp_collect(p, s, st);
+    launch_hyp_collect(p, s, t, st);
     // the meanshift's form of the hypotheses (FP64 se(3) logarithms) is
     // computed beside the dense scoring
     if (!cuda_ok(c, cudaEventRecord(c->ev_fork2, st))) return false;
@@ -497,7 +502,7 @@ voldor_status voldor_bootstrap_epipolar(voldor_ctx* c, int n_samples, double bas
         c->epi_cap = n_samples;
     }
     EpiState e;
-    epi_layout(c->epi_base, n_samples, reinterpret_cast<float4*>(c->ds.pix), &e);
+    epi_layout(c->epi_base, n_samples, c->ds.sc_cst, &e);
     c->launches += launch_epipolar(c->dp, c->ds, e, baseline, c->stream);
     if (!launched(c)) return kCuda;
     c->epi_M = n_samples;
@@ -687,7 +692,7 @@ voldor_status voldor_score_hypotheses(voldor_ctx* c, int t, int n, const double*
     if (!cuda_ok(c, cudaMemcpyAsync(c->ds.hyp_Rt, h.data(), h.size() * 8, cudaMemcpyHostToDevice, c->stream))) return kCuda;
     launch_frame_setup(c->dp, c->ds, c->stream);
     launch_pose_prep(c->dp, c->ds, t, c->stream);
-    score_hyps_from_host(c->dp, c->ds, n, c->stream);
+    score_hyps_from_host(c->dp, c->ds, t, n, c->stream);
     launch_score(c->dp, c->ds, -1, c->stream);
     launch_score_reduce(c->dp, c->ds, c->stream);
     c->launches += 6;
@@ -744,7 +749,7 @@ static bool buffer_of(voldor_ctx* c, int which, void** dev, size_t* bytes, bool*
         case VOLDOR_BUF_EPI_REFINED: {
             if (!c->epi_base || c->epi_M < 1) return false;
             EpiState e;
-            epi_layout(c->epi_base, c->epi_M, reinterpret_cast<float4*>(c->ds.pix), &e);
+            epi_layout(c->epi_base, c->epi_M, c->ds.sc_cst, &e);
             const size_t M = (size_t)c->epi_M;
             if (which == VOLDOR_BUF_EPI_E) { *dev = e.E; *bytes = M * 9 * 8; }
             else if (which == VOLDOR_BUF_EPI_MEDIANS) { *dev = e.median; *bytes = M * 4; }
@@ -834,7 +839,7 @@ voldor_status voldor_autotune(voldor_ctx* c, int* hpt_out, int* chunks_out, floa
     launch_frame_setup(c->dp, c->ds, c->stream);
     launch_pose_prep(c->dp, c->ds, 1, c->stream);
     launch_p3p_groups(c->dp, c->ds, 1, c->stream);
-    launch_hyp_collect(c->dp, c->ds, c->stream);
+    launch_hyp_collect(c->dp, c->ds, 1, c->stream);
     if (!launched(c)) return kCuda;
     cudaEvent_t e0, e1;
     if (!cuda_ok(c, cudaEventCreate(&e0)) || !cuda_ok(c, cudaEventCreate(&e1))) return kCuda;
@@ -847,7 +852,7 @@ voldor_status voldor_autotune(voldor_ctx* c, int* hpt_out, int* chunks_out, floa
     for (int hi = 0; hi < 3 && ok; ++hi) {
         for (int wi = 0; wi < 4 && ok; ++wi) {
             c->ds.score_hpt = hpts[hi];
-            c->ds.n_chunks = score_chunks_for(c->params.hyps_per_frame, c->N, hpts[hi], waves[wi]);
+            c->ds.n_chunks = score_chunks_for(c->params.hyps_per_frame, c->N, waves[wi]);
             launch_score(c->dp, c->ds, -1, c->stream);            // warm-up
             float ms[3];
             for (int r = 0; r < 3 && ok; ++r) {

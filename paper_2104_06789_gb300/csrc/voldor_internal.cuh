@@ -16,8 +16,8 @@ constexpr int kMaxT = 16;
 constexpr int kMaxSols = 4;            // P3P has at most four solutions
 constexpr int kScoreThreads = 256;     // dense scoring block
 constexpr int kScoreHypsPerThread = 8;   // hypotheses per thread of the allocation-free scoring (ILP)
-constexpr int kScoreDefaultHpt = 2;      // a window's dense-scoring shape until autotuned: 2 hypotheses
-constexpr int kScoreDefaultWaves = 8;    // per thread, three blocks per SM, pixel chunks for 8 waves
+constexpr int kScoreDefaultHpt = 8;      // a window's dense-scoring shape until autotuned: 8 hypotheses at a time per
+constexpr int kScoreDefaultWaves = 8;    // thread, pixel chunks for 8 work items per SM
 constexpr int kScoreBlocksPerSM = 1;
 constexpr int kScoreHypsPerBlock = kScoreThreads * kScoreHypsPerThread;
 constexpr int kMeanshiftCtas = 8;      // thread-block cluster of the meanshift
@@ -64,17 +64,6 @@ __device__ __forceinline__ void pixel_xy(const DevParams& p, int j, int& x, int&
     y = (int)q;
 }
 
-// Per-pixel record of a frame for dense scoring (three float4 = 48 B).
-//  a = {xb, yb2, w, ut}: normalised coords x/z, (fy/fx) y/z, inverse depth 1/z
-//      in camera t-1, observed flow u / fx
-//  b = {vt, beta, beta_k, Cp}: observed flow v / fx, Fisk shape, beta *
-//      log2(fx^2 / alpha), mu / beta * fx^2; under the Gaussian residual
-//      model {vt, fx^2 / alpha, -x_mu / alpha, 0}
-//  c = {wq, 0, 0, 0}: rigidness weight W_t^j
-struct PixRec {
-    float4 a, b, c;
-};
-
 // Device state of a window (all pointers are device memory).
 struct DevState {
     const void* flows;        // [T][H][W] float2 or __half2
@@ -89,7 +78,13 @@ struct DevState {
     int* iter;                // [1] iteration counter k
     int* status;              // [4] n_hyp, seed, meanshift steps, status bits
     // dense scoring scratch
-    PixRec* pix;              // [N] compacted valid pixels of the current frame
+    unsigned char* sc_pix;    // tensor-core operand of the current frame's valid pixels, compacted in pixel order:
+                              // [ceil(N / 128)] tiles of 24 KB (score_ops.cuh)
+    float4* sc_cst;           // [N] their Fisk constants {beta, beta log2(fx^2 / alpha), fx^2 mu / beta, W}, under the
+                              // Gaussian model {fx^2 / alpha, -x_mu / alpha, 0, W}
+    float* sc_xmu;            // [N] their x_mu / fx^2 (Fisk)
+    unsigned char* sc_hyp;    // tensor-core operand of the hypotheses: [ceil(S / 128)] groups of 40 KB
+    int* sc_wild;             // [1] nonzero if a pixel or hypothesis of the frame is beyond kScWild
     int* pix_block_count;     // [ceil(N / kPixThreads)] valid pixels per block, then the blocks' record offsets
     unsigned* prep_done;      // [1] blocks of the count pass finished (0 between launches)
     int* pix_count;           // [1]
@@ -119,7 +114,7 @@ struct DevState {
     float* fb_fwd;            // [T][H][W] forward messages
     long long* score_log;     // [kScoreLogMax][2] (n_hyp, n_pix) of timed scoring launches
     int n_chunks;             // dense scoring pixel chunks
-    int score_hpt;            // dense scoring hypotheses per thread (2, 4 or 8)
+    int score_hpt;            // hypotheses a scoring thread takes from tensor memory at a time (2, 4 or 8)
 };
 
 // ---------------------------------------------------------------------------
@@ -278,7 +273,7 @@ void launch_pose_prep(const DevParams& p, const DevState& s, int t, cudaStream_t
 void launch_prep_count(const DevParams& p, const DevState& s, int t, cudaStream_t st);
 void launch_prep_write(const DevParams& p, const DevState& s, int t, cudaStream_t st);
 void launch_p3p_groups(const DevParams& p, const DevState& s, int t, cudaStream_t st);
-void launch_hyp_collect(const DevParams& p, const DevState& s, cudaStream_t st);
+void launch_hyp_collect(const DevParams& p, const DevState& s, int t, cudaStream_t st);
 void launch_hyp_log(const DevParams& p, const DevState& s, cudaStream_t st);
 void launch_score(const DevParams& p, const DevState& s, int log_idx, cudaStream_t st);
 void launch_score_reduce(const DevParams& p, const DevState& s, cudaStream_t st);
@@ -322,8 +317,8 @@ int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, do
 constexpr int kGroundScratchBytes = 4096 * 4 + 256;
 int launch_ground_scale(const DevParams& p, const DevState& s, double camera_height, double cos_tilt, double dmin,
                         double dmax, int apply, unsigned* hist, double* out, cudaStream_t st);
-int score_chunks_for(int S, int N, int hpt, int waves);
+int score_chunks_for(int S, int N, int waves);
 int score_chunks_max(int S, int N);
-void score_hyps_from_host(const DevParams& p, const DevState& s, int n, cudaStream_t st);
+void score_hyps_from_host(const DevParams& p, const DevState& s, int t, int n, cudaStream_t st);
 
 }  // namespace vd
