@@ -475,62 +475,6 @@ void launch_p3p_groups(const DevParams& p, const DevState& s, int t, cudaStream_
     k_p3p_groups<<<wave, 32, 0, st>>>(p, s, t);
 }
 
-// ---------------------------------------------------------------------------
-// Hypothesis collection: exclusive scan of the group solution counts (one
-// block), then one thread per group writes its solutions h = offset + i < S
-// with their scoring form and se(3) logarithm.
-// ---------------------------------------------------------------------------
-__global__ void k_hyp_scan(DevParams p, DevState s)
-{
-    __shared__ int wsum[32];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int G = groups_solved(p, s);
-    const int seg = (G + nt - 1) / nt;
-    const int g0 = min(tid * seg, G), g1 = min(g0 + seg, G);
-    // segments of a multiple of 4 counts start 16-byte aligned (the arrays are
-    // 256-byte aligned): read and write them four at a time
-    const bool vec = (seg & 3) == 0;
-    const int gv = vec ? g0 + ((g1 - g0) & ~3) : g0;
-    int local = 0;
-    for (int g = g0; g < gv; g += 4) {
-        const int4 c = *reinterpret_cast<const int4*>(s.grp_count + g);
-        local += c.x + c.y + c.z + c.w;
-    }
-    for (int g = gv; g < g1; ++g) local += s.grp_count[g];
-    // block exclusive scan of `local`
-    const int lane = tid & 31, warp = tid >> 5;
-    int incl = local;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = nt >> 5;
-        int v = lane < nw ? wsum[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += u;
-        }
-        if (lane < nw) wsum[lane] = v;
-    }
-    __syncthreads();
-    int off = incl - local + (warp > 0 ? wsum[warp - 1] : 0);
-    for (int g = g0; g < gv; g += 4) {
-        const int4 c = *reinterpret_cast<const int4*>(s.grp_count + g);
-        int4 o;
-        o.x = off; o.y = o.x + c.x; o.z = o.y + c.y; o.w = o.z + c.z;
-        *reinterpret_cast<int4*>(s.grp_offset + g) = o;
-        off = o.w + c.w;
-    }
-    for (int g = gv; g < g1; ++g) {
-        s.grp_offset[g] = off;
-        off += s.grp_count[g];
-    }
-    if (tid == nt - 1) *s.n_hyp = min(off, p.S);
-}
-
 // se(3) logarithm through the unit quaternion of R (Shepperd's selection):
 // phi = 2 atan2(|v|, w) v/|v|, rho = V^-1 t with
 // V^-1 = I - Phi/2 + (1 - (th/2) cot(th/2)) / th^2 Phi^2, where
@@ -605,35 +549,71 @@ __device__ void se3_exp_vec(const double* p6, double* Rt)
     Rt[11] = rho[2] + B * a[2] + C * b[2];
 }
 
-// One thread per (group, solution slot), so that each thread's FP64 chain is
-// a single se(3) logarithm.
-__global__ void k_hyp_write(DevParams p, DevState s, int t)
+// Hypothesis collection: one thread per (group, solution slot) writes its
+// solution h = offset + slot < S with its scoring form and tensor-core operand.
+// A block covers 32 groups and finds its offset itself, as the sum of all earlier
+// groups' counts: up to 24 KB of counts read from L2 per block take less time than
+// a scan kernel before this one (4 us and a launch per frame).
+constexpr int kHypGroups = 32;             // groups per block
+
+__global__ void __launch_bounds__(kHypGroups * kMaxSols) k_hyp_write(DevParams p, DevState s, int t)
 {
-    const int gi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gi >= groups_solved(p, s) * kMaxSols) return;
-    const int g = gi / kMaxSols, i = gi % kMaxSols;
-    if (i >= s.grp_count[g]) return;
-    const int h = s.grp_offset[g] + i;
-    if (h >= p.S) return;
+    __shared__ int wsum[kHypGroups * kMaxSols / 32], off_s[kHypGroups];
+    __shared__ double e0[12];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int G = groups_solved(p, s), g0 = blockIdx.x * kHypGroups;
+    if (g0 >= G && blockIdx.x > 0) return;
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};
+    if (tid < 12) {                                       // the frame's current pose in scaled form, {E, t}
+        const double* T0 = s.poses + 12 * (t - 1);
+        const int r = tid / 3, c = tid % 3;
+        e0[tid] = tid < 9 ? sc[r] * (T0[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c] : sc[tid - 9] * T0[(tid - 9) * 4 + 3];
+    }
+    int before = 0;
+    for (int i = tid; i < g0 / 4; i += blockDim.x) {
+        const int4 c = *reinterpret_cast<const int4*>(s.grp_count + 4 * i);
+        before += c.x + c.y + c.z + c.w;
+    }
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (lane == 0) wsum[tid >> 5] = before;
+    __syncthreads();
+    if (tid < 32) {
+        int base = 0;
+        for (int w = 0; w < kHypGroups * kMaxSols / 32; ++w) base += wsum[w];
+        const int c = g0 + tid < G ? s.grp_count[g0 + tid] : 0;
+        int incl = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        off_s[tid] = base + incl - c;
+        if (tid == 31 && g0 + kHypGroups >= G) *s.n_hyp = min(base + incl, p.S);   // the last block with groups
+    }
+    __syncthreads();
+    const int g = g0 + tid / kMaxSols, i = tid % kMaxSols;
+    if (g >= G || i >= s.grp_count[g]) return;
+    const int h = off_s[tid / kMaxSols] + i;
+    if (h >= p.S) return;
     const double* Rt = s.grp_sols + ((size_t)g * kMaxSols + i) * 12;
-    const double* T0 = s.poses + 12 * (t - 1);
     double* oR = s.hyp_Rt + (size_t)h * 12;
     float* f = s.hyp_f32 + (size_t)h * 12;
-    double e[12], e0[12];
+    double e[12];
     for (int r = 0; r < 3; ++r) {
         for (int c = 0; c < 3; ++c) {
             oR[r * 3 + c] = Rt[r * 4 + c];
-            e[r * 3 + c] = sc[r] * (Rt[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
-            e0[r * 3 + c] = sc[r] * (T0[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
-            f[r * 3 + c] = (float)e[r * 3 + c];
+            e[r * 3 + c] = Rt[r * 4 + c] - (r == c ? 1.0 : 0.0);
         }
         oR[9 + r] = Rt[r * 4 + 3];
-        e[9 + r] = sc[r] * Rt[r * 4 + 3];
-        e0[9 + r] = sc[r] * T0[r * 4 + 3];
-        f[9 + r] = (float)e[9 + r];
+        e[9 + r] = Rt[r * 4 + 3];
     }
+    if (q != 1.0) {                        // square pixels need no scaling, and FP64 divisions are long here
+        for (int r = 0; r < 3; ++r) {
+            for (int c = 0; c < 3; ++c) e[r * 3 + c] = sc[r] * e[r * 3 + c] / sc[c];
+            e[9 + r] = sc[r] * e[9 + r];
+        }
+    }
+    for (int c = 0; c < 12; ++c) f[c] = (float)e[c];
     if (write_hyp_operand(s.sc_hyp, h, e, e0)) atomicOr(s.sc_wild, 1);
     s.hyp_w[h] = s.grp_weight[g];
     s.hyp_info[(size_t)h * 2 + 0] = g;
@@ -670,9 +650,8 @@ void launch_hyp_log(const DevParams& p, const DevState& s, cudaStream_t st)
 
 void launch_hyp_collect(const DevParams& p, const DevState& s, int t, cudaStream_t st)
 {
-    k_hyp_scan<<<1, 1024, 0, st>>>(p, s);
-    // sized for the budget; threads past the solved prefix return at once
-    k_hyp_write<<<(p.G * kMaxSols + 127) / 128, 128, 0, st>>>(p, s, t);
+    // sized for the budget; blocks past the solved prefix return at once
+    k_hyp_write<<<(p.G + kHypGroups - 1) / kHypGroups, kHypGroups * kMaxSols, 0, st>>>(p, s, t);
 }
 
 // Scoring form of caller-given hypotheses already copied to hyp_Rt.
@@ -740,6 +719,39 @@ __device__ __forceinline__ long long score_key(double v)
     return b >= 0 ? b : (b ^ 0x7fffffffffffffffll);
 }
 
+// The frame tables after the pose update of frame t: C_t = T_t C_{t-1} and T_t in the
+// forms k_frame_setup writes, with the same operations (products and sums rounded
+// one by one, so the values are bit-identical to a set-up from scratch). One CTA,
+// after poses[t - 1] is written: a set-up kernel before every frame and stage cost
+// 5-8 us each, most of it the FP64 chain over all frames.
+__device__ void advance_frame_tables(const DevParams& p, const DevState& s, int t)
+{
+    __shared__ double T[12], C[12];
+    const int i = threadIdx.x;
+    __syncthreads();
+    if (i < 12) {
+        T[i] = s.poses[12 * (t - 1) + i];
+        C[i] = s.cum[12 * (t - 1) + i];
+    }
+    __syncthreads();
+    if (i >= 12) return;
+    const int r = i / 4, c = i % 4;
+    const double one = r == c ? 1.0 : 0.0;
+    const double av = T[i];
+    double cv = __dadd_rn(__dadd_rn(__dmul_rn(T[4 * r], C[c]), __dmul_rn(T[4 * r + 1], C[4 + c])),
+                          __dmul_rn(T[4 * r + 2], C[8 + c]));
+    if (c == 3) cv = __dadd_rn(cv, T[4 * r + 3]);
+    const float ah = (float)av, ch = (float)cv;
+    s.poses_df[24 * (t - 1) + 2 * i] = ah;
+    s.poses_df[24 * (t - 1) + 2 * i + 1] = (float)(av - (double)ah);
+    s.frames32[24 * (t - 1) + 12 + (c < 3 ? 3 * r + c : 9 + r)] = c < 3 ? (float)(av - one) : ah;
+    if (t == p.T) return;
+    s.cum[12 * t + i] = cv;
+    s.cum_df[24 * t + 2 * i] = ch;
+    s.cum_df[24 * t + 2 * i + 1] = (float)(cv - (double)ch);
+    s.frames32[24 * t + (c < 3 ? 3 * r + c : 9 + r)] = c < 3 ? (float)(cv - one) : ch;
+}
+
 __device__ __forceinline__ DF shfl_df(DF v, int src)
 {
     return DF{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
@@ -763,6 +775,7 @@ k_meanshift(DevParams p, DevState s, int t)
         if (rank == 0 && tid == 0) {
             s.status[0] = 0; s.status[1] = -1; s.status[2] = 0; s.status[3] += 1;
         }
+        if (rank == 0) advance_frame_tables(p, s, t);     // the pose stays, but C_{t-1} may have moved
         return;   // uniform over the cluster: every CTA reads the same n
     }
     // argmax of L (lowest index on ties; NaN never wins)
@@ -941,6 +954,7 @@ k_meanshift(DevParams p, DevState s, int t)
             se3_exp_vec(x, s.poses + 12 * (t - 1));
         }
     }
+    if (rank == 0) advance_frame_tables(p, s, t);
 }
 
 void launch_meanshift(const DevParams& p, const DevState& s, int t, cudaStream_t st)

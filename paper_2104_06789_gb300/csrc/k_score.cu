@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
     const uint32_t afull = hempty + 16, aempty = afull + 8 * kScBufs, done = aempty + 8 * kScBufs;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kScBarOff + 200);
     volatile int& bad = *reinterpret_cast<volatile int*>(smem + kScBarOff + 204);
+    volatile int& last = *reinterpret_cast<volatile int*>(smem + kScBarOff + 208);
     double* red = reinterpret_cast<double*>(smem + kScRedOff);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_hyp = *s.n_hyp, n_pix = *s.pix_count;
@@ -582,11 +583,34 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
             }
             red[(buf * 4 + quarter) * kScGroupHyps + wg * kScStageHyps + lane] = tot;
             asm volatile("bar.sync 1, %0;" ::"n"(kScWarps * 32) : "memory");
-            const int h = threadIdx.x;
-            if (h < it.hyps) {
-                const double* r = red + buf * 4 * kScGroupHyps + h;
-                const double v = ((r[0] + r[kScGroupHyps]) + r[2 * kScGroupHyps]) + r[3 * kScGroupHyps];
-                s.partial[(size_t)(u / n_groups) * p.S + (u % n_groups) * kScGroupHyps + h] = -v * 0.69314718055994531;
+            if (warp < kScGroupHyps / 32) {
+                const int h = threadIdx.x, chunk = u / n_groups, group = u % n_groups;
+                double* part = s.partial + group * kScGroupHyps + h;
+                if (h < it.hyps) {
+                    const double* r = red + buf * 4 * kScGroupHyps + h;
+                    const double v = ((r[0] + r[kScGroupHyps]) + r[2 * kScGroupHyps]) + r[3 * kScGroupHyps];
+                    part[(size_t)chunk * p.S] = -v * 0.69314718055994531;
+                }
+                // the CTA that finishes a group's last chunk adds the chunks in order (no CTA waits)
+                __threadfence();
+                asm volatile("bar.sync 2, %0;" ::"n"(kScGroupHyps) : "memory");
+                if (h == 0) last = atomicAdd(s.score_done + group, 1) == n_chunks - 1;
+                asm volatile("bar.sync 2, %0;" ::"n"(kScGroupHyps) : "memory");
+                if (last) {
+                    __threadfence();
+                    if (h == 0) s.score_done[group] = 0;
+                    if (h < it.hyps) {
+                        double v = 0.0;
+                        for (int c = 0; c < n_chunks; c += 8) {
+                            double a[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) a[i] = c + i < n_chunks ? __ldcg(part + (size_t)(c + i) * p.S) : 0.0;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) v += a[i];
+                        }
+                        s.scores[group * kScGroupHyps + h] = v;
+                    }
+                }
             }
             buf ^= 1;          // the next item's sums go to the other buffer, so one barrier per item suffices
         }
@@ -598,45 +622,6 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kScTmemCols));
     }
     if (threadIdx.x == 0 && bad) atomicOr(s.status + 3, kStatusTimeout);
-}
-
-// L_h = sum over the chunks' partials (natural-log units) in a fixed order:
-// 32 threads per hypothesis each add a contiguous range of chunks in chunk
-// order (loads issued four at a time, so a thread waits on memory about three
-// times rather than once per chunk), then their 32 sums are added in range
-// order (deterministic). A block covers 32 consecutive hypotheses, so every
-// warp's loads are 256 contiguous bytes.
-constexpr int kReduceSplit = 32;
-
-__global__ void __launch_bounds__(32 * kReduceSplit) k_score_reduce(DevParams p, DevState s)
-{
-    __shared__ double part[kReduceSplit][32];
-    const int hl = threadIdx.x & 31, q = threadIdx.x >> 5;
-    const int h = blockIdx.x * 32 + hl;
-    const int n_hyp = *s.n_hyp, nc = s.n_chunks;
-    const int c0 = nc * q / kReduceSplit, c1 = nc * (q + 1) / kReduceSplit;
-    double v = 0.0;
-    if (h < n_hyp) {
-        const double* src = s.partial + h;
-        const size_t S = (size_t)p.S;
-        int c = c0;
-        for (; c + 4 <= c1; c += 4) {
-            const double a0 = src[(size_t)c * S], a1 = src[(size_t)(c + 1) * S];
-            const double a2 = src[(size_t)(c + 2) * S], a3 = src[(size_t)(c + 3) * S];
-            v += a0;
-            v += a1;
-            v += a2;
-            v += a3;
-        }
-        for (; c < c1; ++c) v += src[(size_t)c * S];
-    }
-    part[q][hl] = v;
-    __syncthreads();
-    if (q == 0 && h < n_hyp) {
-        double t = 0.0;
-        for (int r = 0; r < kReduceSplit; ++r) t += part[r][hl];
-        s.scores[h] = t;
-    }
 }
 
 static int g_num_sms = 0;
@@ -721,11 +706,6 @@ void launch_score(const DevParams& p, const DevState& s, int log_idx, cudaStream
     if (s.score_hpt == 4) launch_score_shape<4>(p, s, li, st);
     else if (s.score_hpt == 2) launch_score_shape<2>(p, s, li, st);
     else launch_score_shape<8>(p, s, li, st);
-}
-
-void launch_score_reduce(const DevParams& p, const DevState& s, cudaStream_t st)
-{
-    k_score_reduce<<<(p.S + 31) / 32, 32 * kReduceSplit, 0, st>>>(p, s);
 }
 
 

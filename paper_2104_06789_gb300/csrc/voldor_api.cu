@@ -160,7 +160,6 @@ size_t layout(voldor_ctx& c, char* base)
     s.grp_sols = (double*)take(G * kMaxSols * 12 * 8);
     s.grp_weight = (double*)take(G * 8);
     s.grp_count = (int*)take(G * 4);
-    s.grp_offset = (int*)take(G * 4);
     s.n_hyp = (int*)take(4);
     s.hyp_Rt = (double*)take(S * 12 * 8);
     s.hyp_f32 = (float*)take(S * 12 * 4);
@@ -169,6 +168,7 @@ size_t layout(voldor_ctx& c, char* base)
     s.hyp_dp = (float*)take(S * 8 * 4);
     s.hyp_info = (long long*)take(S * 2 * 8);
     s.partial = (double*)take((size_t)chunks_max * S * 8);
+    s.score_done = (int*)take((S + kScGroupHyps - 1) / kScGroupHyps * 4);
     s.scores = (double*)take(S * 8);
     s.mie_prev_score = (float*)take(N * 4);
     s.mie_smp = (float*)take(N * 4);
@@ -227,13 +227,13 @@ voldor_status upload_flows(voldor_ctx* c, const void* flows, int on_device)
     return VOLDOR_OK;
 }
 
-// One pose update of frame t (iteration counter already set on the device).
+// One pose update of frame t (iteration counter and frame tables already set on
+// the device; it leaves the tables of frame t + 1 and T_t up to date).
 bool enqueue_pose_update(voldor_ctx* c, int t, cudaEvent_t ev0, cudaEvent_t ev1, int log_idx)
 {
     const DevParams& p = c->dp;
     const DevState& s = c->ds;
     cudaStream_t st = c->stream;
-    launch_frame_setup(p, s, st);
     launch_prep_count(p, s, t, st);
     // the minimal groups (drawn from the valid pixels the count pass listed)
     // and their P3P (FP64) run beside the write of the pixel records
@@ -254,15 +254,14 @@ bool enqueue_pose_update(voldor_ctx* c, int t, cudaEvent_t ev0, cudaEvent_t ev1,
     if (ev0 && !cuda_ok(c, cudaEventRecordWithFlags(ev0, st, cudaEventRecordExternal))) return false;
     launch_score(p, s, log_idx, st);
     if (ev1 && !cuda_ok(c, cudaEventRecordWithFlags(ev1, st, cudaEventRecordExternal))) return false;
-    launch_score_reduce(p, s, st);
     if (!cuda_ok(c, cudaStreamWaitEvent(st, c->ev_join2, 0))) return false;
     launch_meanshift(p, s, t, st);
     return launched(c);
 }
 
+// The per-pixel stages read the frame tables of all frames.
 bool enqueue_smooth(voldor_ctx* c)
 {
-    launch_frame_setup(c->dp, c->ds, c->stream);
     launch_emissions(c->dp, c->ds, c->ds.qs, c->stream);
     launch_forward_backward(c->dp, c->ds, c->stream);
     return launched(c);
@@ -270,14 +269,12 @@ bool enqueue_smooth(voldor_ctx* c)
 
 bool enqueue_depth(voldor_ctx* c)
 {
-    launch_frame_setup(c->dp, c->ds, c->stream);
     launch_mie(c->dp, c->ds, c->stream);
     return launched(c);
 }
 
 bool enqueue_rigidness(voldor_ctx* c)
 {
-    launch_frame_setup(c->dp, c->ds, c->stream);
     launch_emissions(c->dp, c->ds, c->ds.wmap, c->stream);
     return launched(c);
 }
@@ -331,6 +328,7 @@ bool ensure_graph(voldor_ctx* c, int n_iters, bool timing)
     cudaGraph_t g = nullptr;
     bool ok = cuda_ok(c, cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
     if (ok) {
+        launch_frame_setup(c->dp, c->ds, cap);      // once: the pose updates keep the tables
         for (int i = 0; i < n_iters && ok; ++i) ok = enqueue_iteration(c, i * c->T);
         cudaError_t ee = cudaStreamEndCapture(cap, &g);
         ok = ok && cuda_ok(c, ee);
@@ -669,6 +667,7 @@ voldor_status voldor_pose_update(voldor_ctx* c, int k, int t)
     if (!c->bootstrapped) return VOLDOR_ERR_NOT_BOOTSTRAPPED;
     if (!cuda_ok(c, cudaMemsetAsync(c->ds.status, 0, 16, c->stream))) return kCuda;
     launch_set_iteration(c->ds, k, c->stream);
+    launch_frame_setup(c->dp, c->ds, c->stream);
     if (!enqueue_pose_update(c, t, nullptr, nullptr, -1)) return kCuda;
     int st4[4];
     voldor_status rs = read_status_word(c, st4);
@@ -694,8 +693,7 @@ voldor_status voldor_score_hypotheses(voldor_ctx* c, int t, int n, const double*
     launch_pose_prep(c->dp, c->ds, t, c->stream);
     score_hyps_from_host(c->dp, c->ds, t, n, c->stream);
     launch_score(c->dp, c->ds, -1, c->stream);
-    launch_score_reduce(c->dp, c->ds, c->stream);
-    c->launches += 6;
+    c->launches += 5;
     if (!launched(c)) return kCuda;
     if (!cuda_ok(c, cudaMemcpyAsync(L, c->ds.scores, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream))) return kCuda;
     if (!cuda_ok(c, cudaStreamSynchronize(c->stream))) return kCuda;
@@ -708,6 +706,7 @@ voldor_status voldor_rigidness_smooth(voldor_ctx* c, int k)
     if (c->poisoned) return kCuda;
     if (!c->bootstrapped) return VOLDOR_ERR_NOT_BOOTSTRAPPED;
     launch_set_iteration(c->ds, k, c->stream);
+    launch_frame_setup(c->dp, c->ds, c->stream);
     return enqueue_smooth(c) ? VOLDOR_OK : kCuda;
 }
 
@@ -717,6 +716,7 @@ voldor_status voldor_depth_update(voldor_ctx* c, int k)
     if (c->poisoned) return kCuda;
     if (!c->bootstrapped) return VOLDOR_ERR_NOT_BOOTSTRAPPED;
     launch_set_iteration(c->ds, k, c->stream);
+    launch_frame_setup(c->dp, c->ds, c->stream);
     return enqueue_depth(c) ? VOLDOR_OK : kCuda;
 }
 
@@ -725,6 +725,7 @@ voldor_status voldor_rigidness_update(voldor_ctx* c)
     if (!c) return VOLDOR_ERR_INVALID_ARG;
     if (c->poisoned) return kCuda;
     if (!c->bootstrapped) return VOLDOR_ERR_NOT_BOOTSTRAPPED;
+    launch_frame_setup(c->dp, c->ds, c->stream);
     return enqueue_rigidness(c) ? VOLDOR_OK : kCuda;
 }
 

@@ -95,7 +95,6 @@ struct DevState {
     double* grp_sols;         // [G][4][12]
     double* grp_weight;       // [G]
     int* grp_count;           // [G]
-    int* grp_offset;          // [G]
     int* n_hyp;               // [1]
     double* hyp_Rt;           // [S][12]
     float* hyp_f32;           // [S][12] scoring form
@@ -104,6 +103,7 @@ struct DevState {
     float* hyp_dp;            // [S][8] meanshift scratch: p_h - p_seed (6), w_h, 0
     long long* hyp_info;      // [S][2]
     double* partial;          // [n_chunks][S]
+    int* score_done;          // [ceil(S / 128)] chunks scored per hypothesis group (0 between launches)
     double* scores;           // [S]
     // depth sweep
     float* mie_prev_score;    // [N]
@@ -276,7 +276,6 @@ void launch_p3p_groups(const DevParams& p, const DevState& s, int t, cudaStream_
 void launch_hyp_collect(const DevParams& p, const DevState& s, int t, cudaStream_t st);
 void launch_hyp_log(const DevParams& p, const DevState& s, cudaStream_t st);
 void launch_score(const DevParams& p, const DevState& s, int log_idx, cudaStream_t st);
-void launch_score_reduce(const DevParams& p, const DevState& s, cudaStream_t st);
 void launch_meanshift(const DevParams& p, const DevState& s, int t, cudaStream_t st);
 void launch_emissions(const DevParams& p, const DevState& s, float* out, cudaStream_t st);
 void launch_forward_backward(const DevParams& p, const DevState& s, cudaStream_t st);
