@@ -704,12 +704,6 @@ void score_hyps_from_host(const DevParams& p, const DevState& s, int t, int n, c
 // ---------------------------------------------------------------------------
 constexpr int kMsCached = 4;     // hypotheses per thread held in registers (all of them up to S = 8192)
 
-__device__ __forceinline__ float warp_sum_f(float v)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // Order-preserving integer key of a double: a < b iff key(a) < key(b) for
 // non-NaN values, -0 and +0 equal.
 __device__ __forceinline__ long long score_key(double v)
@@ -757,191 +751,154 @@ __device__ __forceinline__ DF shfl_df(DF v, int src)
     return DF{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
 }
 
-__global__ void __cluster_dims__(kMeanshiftCtas, 1, 1) __launch_bounds__(kMeanshiftThreads, 1)
-k_meanshift(DevParams p, DevState s, int t)
+// Sums of eight per-lane values over a warp: at each step a lane keeps half of its
+// values and adds the partner's, so lane l ends with the sum of value l / 4 (9 shuffles
+// instead of 5 per value). The pairs are those of an xor butterfly from 16 down to
+// 1, so each sum is bit-identical to it.
+__device__ __forceinline__ float warp_sum8(const float* a, int lane)
 {
-    cg::cluster_group cluster = cg::this_cluster();
-    const unsigned rank = cluster.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-    __shared__ float wred[32][8];
-    __shared__ float2 part[2][8];
-    __shared__ float xo_hi[6], xo_lo[6];      // x - p_seed, float-float
-    __shared__ float seed_hi[6], seed_lo[6];
-    __shared__ long long bkey[32];
-    __shared__ int bidx[32];
-    __shared__ int flag;
-    const int n = *s.n_hyp;
-    if (n == 0) {
-        if (rank == 0 && tid == 0) {
-            s.status[0] = 0; s.status[1] = -1; s.status[2] = 0; s.status[3] += 1;
-        }
-        if (rank == 0) advance_frame_tables(p, s, t);     // the pose stays, but C_{t-1} may have moved
-        return;   // uniform over the cluster: every CTA reads the same n
+    float v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool up = (lane & 16) != 0;
+        v[i] = (up ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + 4], 16);
     }
-    // argmax of L (lowest index on ties; NaN never wins)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const bool up = (lane & 8) != 0;
+        v[i] = (up ? v[i + 2] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + 2], 8);
+    }
+    const bool up = (lane & 4) != 0;
+    float r = (up ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    return r + __shfl_xor_sync(0xffffffffu, r, 1);
+}
+
+// Shared state of a meanshift CTA.
+struct MsShared {
+    float wred[32][8];                    // the warps' sums of the step
+    float2 part[2][8];                    // the CTA's sums, by step parity (cluster form)
+    float xo_hi[6], xo_lo[6];             // x - p_seed, float-float
+    float seed_hi[6], seed_lo[6];
+    long long bkey[32];
+    int bidx[32];
+    int flag;
+    float consts[3];
+};
+
+// argmax of L (lowest index on ties; NaN never wins), then the seed and the
+// constants into shared memory. Eight scores in flight per thread.
+__device__ __forceinline__ void ms_seed(const DevParams& p, const DevState& s, MsShared& m, int n)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
     long long bk = 0;
     int bi = 0x7fffffff;
-    for (int h = tid; h < n; h += blockDim.x) {
-        const double v = s.scores[h];
-        const long long raw = __double_as_longlong(v) & 0x7fffffffffffffffll;
-        if (raw > 0x7ff0000000000000ll) continue;                 // NaN
-        const long long k = score_key(v);
-        if (bi == 0x7fffffff || k > bk || (k == bk && h < bi)) { bk = k; bi = h; }
+    for (int h0 = tid; h0 < n; h0 += 8 * blockDim.x) {
+        double v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = h0 + i * (int)blockDim.x < n ? s.scores[h0 + i * blockDim.x] : NAN;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long raw = __double_as_longlong(v[i]) & 0x7fffffffffffffffll;
+            if (raw > 0x7ff0000000000000ll) continue;             // NaN
+            const long long k = score_key(v[i]);
+            if (bi == 0x7fffffff || k > bk) { bk = k; bi = h0 + i * blockDim.x; }   // increasing h: the first wins ties
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         const long long ok = __shfl_xor_sync(0xffffffffu, bk, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (oi != 0x7fffffff && (bi == 0x7fffffff || ok > bk || (ok == bk && oi < bi))) { bk = ok; bi = oi; }
     }
-    if (lane == 0) { bkey[warp] = bk; bidx[warp] = bi; }
+    if (lane == 0) { m.bkey[warp] = bk; m.bidx[warp] = bi; }
     __syncthreads();
-    if (tid == 0) {
-        long long k = bkey[0];
-        int i = bidx[0];
-        for (int w = 1; w < nwarp; ++w)
-            if (bidx[w] != 0x7fffffff && (i == 0x7fffffff || bkey[w] > k || (bkey[w] == k && bidx[w] < i))) {
-                k = bkey[w];
-                i = bidx[w];
-            }
-        if (i == 0x7fffffff) i = 0;
-        const float* ps = s.hyp_pw + (size_t)i * 16;
-        for (int c = 0; c < 6; ++c) {
-            seed_hi[c] = ps[c];
-            seed_lo[c] = ps[6 + c];
-            xo_hi[c] = 0.f;
-            xo_lo[c] = 0.f;
+    if (warp == 0) {
+        bk = lane < nwarp ? m.bkey[lane] : 0;
+        bi = lane < nwarp ? m.bidx[lane] : 0x7fffffff;
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long ok = __shfl_xor_sync(0xffffffffu, bk, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (oi != 0x7fffffff && (bi == 0x7fffffff || ok > bk || (ok == bk && oi < bi))) { bk = ok; bi = oi; }
         }
-        bidx[0] = i;
-        flag = 0;
-    }
-    __syncthreads();
-    const int seed = bidx[0];
-    // FP32 offsets of this CTA's hypotheses from the seed: a thread's first
-    // kMsCached stay in registers, the rest (S above kMsCached x the cluster's
-    // threads) go to global memory
-    const int stride = kMeanshiftCtas * blockDim.x, h0 = rank * blockDim.x + tid;
-    DF sd[6];
-    for (int c = 0; c < 6; ++c) sd[c] = DF{seed_hi[c], seed_lo[c]};
-    float4 r0[kMsCached], r1[kMsCached];
-#pragma unroll
-    for (int k = 0; k < kMsCached; ++k) { r0[k] = make_float4(0.f, 0.f, 0.f, 0.f); r1[k] = r0[k]; }
-    for (int h = h0, k = 0; h < n; h += stride, ++k) {
-        const float4* pw = reinterpret_cast<const float4*>(s.hyp_pw + (size_t)h * 16);
-        const float4 a = pw[0], b = pw[1], c2 = pw[2], d = pw[3];
-        const float ph[6] = {a.x, a.y, a.z, a.w, b.x, b.y}, pl[6] = {b.z, b.w, c2.x, c2.y, c2.z, c2.w};
-        float o[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) o[c] = df_to_float(df_sub(DF{ph[c], pl[c]}, sd[c]));
-        const float4 o0 = make_float4(o[0], o[1], o[2], o[3]);
-        const float4 o1 = make_float4(o[4], o[5], d.x, 0.f);
-        if (k < kMsCached) {
-#pragma unroll
-            for (int i = 0; i < kMsCached; ++i)
-                if (i == k) { r0[i] = o0; r1[i] = o1; }
-        } else {
-            float4* od = reinterpret_cast<float4*>(s.hyp_dp + (size_t)h * 8);
-            od[0] = o0;
-            od[1] = o1;
+        if (bi == 0x7fffffff) bi = 0;
+        if (lane < 6) {
+            const float* ps = s.hyp_pw + (size_t)bi * 16;
+            m.seed_hi[lane] = ps[lane];
+            m.seed_lo[lane] = ps[6 + lane];
+            m.xo_hi[lane] = 0.f;
+            m.xo_lo[lane] = 0.f;
         }
-    }
-    __shared__ float consts[3];
-    if (tid == 0) {
-        consts[0] = (float)(1.0 / p.sigma_t);
-        consts[1] = (float)(1.0 / p.sigma_r);
-        consts[2] = (float)p.ms_tol;
+        if (lane == 6) m.bidx[0] = bi;
+        if (lane == 7) m.flag = 0;
+    } else if (tid == 32) {
+        m.consts[0] = (float)(1.0 / p.sigma_t);
+        m.consts[1] = (float)(1.0 / p.sigma_r);
+        m.consts[2] = (float)p.ms_tol;
     }
     __syncthreads();
-    const float ivt = consts[0], ivr = consts[1], tol = consts[2];
+}
+
+// Offset of hypothesis h from the seed in FP32, its weight in o1.z.
+__device__ __forceinline__ void ms_offset(const DevState& s, const DF* sd, int h, float4& o0, float4& o1)
+{
+    const float4* pw = reinterpret_cast<const float4*>(s.hyp_pw + (size_t)h * 16);
+    const float4 a = pw[0], b = pw[1], c2 = pw[2], d = pw[3];
+    const float ph[6] = {a.x, a.y, a.z, a.w, b.x, b.y}, pl[6] = {b.z, b.w, c2.x, c2.y, c2.z, c2.w};
+    float o[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) o[c] = df_to_float(df_sub(DF{ph[c], pl[c]}, sd[c]));
+    o0 = make_float4(o[0], o[1], o[2], o[3]);
+    o1 = make_float4(o[4], o[5], d.x, 0.f);
+}
+
+// acc += w K(x - p) (1, p) for one offset.
+__device__ __forceinline__ void ms_add(const float* dx, float ivt, float ivr, const float4 q0, const float4 q1, float* acc)
+{
     const float mlog2e = -0.5f * 1.4426950408889634f;
-    int it = 0;
-    bool degenerate = false;
-    float prev_step = INFINITY;
-    for (; it < p.ms_max_iter; ++it) {
-        float dx[6];
-        for (int c = 0; c < 6; ++c) dx[c] = xo_hi[c] + xo_lo[c];
-        float acc[7] = {0, 0, 0, 0, 0, 0, 0};
-        // hypotheses in increasing h (the registers' first, then global memory)
-        auto add = [&](const float4 q0, const float4 q1) {
-            const float d0 = dx[0] - q0.x, d1 = dx[1] - q0.y, d2 = dx[2] - q0.z;
-            const float d3 = dx[3] - q0.w, d4 = dx[4] - q1.x, d5 = dx[5] - q1.y;
-            const float m = fmaf(d0 * d0 + d1 * d1 + d2 * d2, ivt, (d3 * d3 + d4 * d4 + d5 * d5) * ivr);
-            const float kw = q1.z * exp2f(mlog2e * m);
-            if (!(kw > 0.f)) return;       // zero weight (or a non-finite hypothesis) adds nothing
-            acc[0] += kw;
-            acc[1] = fmaf(kw, q0.x, acc[1]); acc[2] = fmaf(kw, q0.y, acc[2]); acc[3] = fmaf(kw, q0.z, acc[3]);
-            acc[4] = fmaf(kw, q0.w, acc[4]); acc[5] = fmaf(kw, q1.x, acc[5]); acc[6] = fmaf(kw, q1.y, acc[6]);
-        };
-#pragma unroll
-        for (int k = 0; k < kMsCached; ++k)
-            if (h0 + k * stride < n) add(r0[k], r1[k]);
-        for (int h = h0 + kMsCached * stride; h < n; h += stride) {
-            const float4* o = reinterpret_cast<const float4*>(s.hyp_dp + (size_t)h * 8);
-            add(o[0], o[1]);
-        }
-        // warp sums in FP32 (each lane holds at most 4 terms), then the CTA's
-        // warps in order as float-float
-        float accw[7];
-        for (int c = 0; c < 7; ++c) accw[c] = warp_sum_f(acc[c]);
-        if (lane == 0)
-            for (int c = 0; c < 7; ++c) wred[warp][c] = accw[c];
-        __syncthreads();
-        const int buf = it & 1;
-        if (tid < 7) {
-            DF v{0.f, 0.f};
-            for (int w = 0; w < nwarp; ++w) v = df_add(v, wred[w][tid]);
-            part[buf][tid] = make_float2(v.hi, v.lo);
-        }
-        cluster.sync();
-        if (warp == 0) {
-            // entry e = r * 7 + c (component c of rank r's sums, from distributed
-            // shared memory) is fetched by lane e % 32 into slot e / 32; lane
-            // c < 7 adds the entries of its component in rank order
-            static_assert(kMeanshiftCtas * 7 <= 64, "two entries per lane");
-            DF g[2] = {DF{0.f, 0.f}, DF{0.f, 0.f}};
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int e = lane + 32 * q;
-                if (e < kMeanshiftCtas * 7) {
-                    const float2 v = *cluster.map_shared_rank(&part[buf][e % 7], (unsigned)(e / 7));
-                    g[q] = DF{v.x, v.y};
-                }
-            }
-            DF tot{0.f, 0.f};
-            for (int r = 0; r < kMeanshiftCtas; ++r) {
-                const int e = r * 7 + (lane < 7 ? lane : 0);
-                const DF v0 = shfl_df(g[0], e & 31), v1 = shfl_df(g[1], e & 31);
-                tot = df_add(tot, e < 32 ? v0 : v1);
-            }
-            const DF t0 = shfl_df(tot, 0);
-            const bool mass = t0.hi > 0.f;
-            float dd = 0.f;
-            if (mass && lane >= 1 && lane < 7) {
-                const DF xn = df_div(tot, t0);                    // mean offset of component lane - 1
-                const DF xo{xo_hi[lane - 1], xo_lo[lane - 1]};
-                dd = df_to_float(df_sub(xn, xo));
-                dd *= dd;
-                xo_hi[lane - 1] = xn.hi;
-                xo_lo[lane - 1] = xn.lo;
-            }
-            float s2 = 0.f;
-            for (int c = 1; c < 7; ++c) s2 += __shfl_sync(0xffffffffu, dd, c);
-            if (lane == 0) {
-                if (!mass) {
-                    flag = (it == 0) ? 2 : 1;
-                } else {
-                    const float step = sqrtf(s2);
-                    flag = (step < tol || (step >= prev_step && step < 1e-7f)) ? 1 : 0;
-                    prev_step = step;
-                }
-            }
-        }
-        __syncthreads();
-        const int f = flag;
-        if (f == 2) { degenerate = true; break; }
-        if (f == 1) { ++it; break; }
+    const float d0 = dx[0] - q0.x, d1 = dx[1] - q0.y, d2 = dx[2] - q0.z;
+    const float d3 = dx[3] - q0.w, d4 = dx[4] - q1.x, d5 = dx[5] - q1.y;
+    const float m = fmaf(d0 * d0 + d1 * d1 + d2 * d2, ivt, (d3 * d3 + d4 * d4 + d5 * d5) * ivr);
+    const float kw = q1.z * exp2f(mlog2e * m);
+    if (!(kw > 0.f)) return;       // zero weight (or a non-finite hypothesis) adds nothing
+    acc[0] += kw;
+    acc[1] = fmaf(kw, q0.x, acc[1]); acc[2] = fmaf(kw, q0.y, acc[2]); acc[3] = fmaf(kw, q0.z, acc[3]);
+    acc[4] = fmaf(kw, q0.w, acc[4]); acc[5] = fmaf(kw, q1.x, acc[5]); acc[6] = fmaf(kw, q1.y, acc[6]);
+}
+
+// One warp finishes a step from the total (component c in lane c < 7): the new
+// state, and the flag 0 go on, 1 converged, 2 no mass at the first step.
+__device__ __forceinline__ void ms_finish(MsShared& m, DF tot, int lane, int it, float tol, float& prev_step)
+{
+    const DF t0 = shfl_df(tot, 0);
+    const bool mass = t0.hi > 0.f;
+    float dd = 0.f;
+    if (mass && lane >= 1 && lane < 7) {
+        const DF xn = df_div(tot, t0);                    // mean offset of component lane - 1
+        const DF xo{m.xo_hi[lane - 1], m.xo_lo[lane - 1]};
+        dd = df_to_float(df_sub(xn, xo));
+        dd *= dd;
+        m.xo_hi[lane - 1] = xn.hi;
+        m.xo_lo[lane - 1] = xn.lo;
     }
-    cluster.sync();   // no CTA leaves while another may still read its partials
-    if (rank == 0 && tid == 0) {
+    float s2 = 0.f;
+#pragma unroll
+    for (int c = 1; c < 7; ++c) s2 += __shfl_sync(0xffffffffu, dd, c);
+    if (lane == 0) {
+        if (!mass) {
+            m.flag = (it == 0) ? 2 : 1;
+        } else {
+            const float step = sqrtf(s2);
+            m.flag = (step < tol || (step >= prev_step && step < 1e-7f)) ? 1 : 0;
+            prev_step = step;
+        }
+    }
+}
+
+// Status words, the pose and the frame tables (one CTA).
+__device__ __forceinline__ void ms_result(const DevParams& p, const DevState& s, const MsShared& m, int t, int n, int seed,
+                                          int it, bool degenerate)
+{
+    if (threadIdx.x == 0) {
         s.status[0] = n;
         s.status[1] = seed;
         s.status[2] = it;
@@ -950,16 +907,163 @@ k_meanshift(DevParams p, DevState s, int t)
         } else {
             double x[6];
             for (int c = 0; c < 6; ++c)
-                x[c] = ((double)seed_hi[c] + (double)seed_lo[c]) + ((double)xo_hi[c] + (double)xo_lo[c]);
+                x[c] = ((double)m.seed_hi[c] + (double)m.seed_lo[c]) + ((double)m.xo_hi[c] + (double)m.xo_lo[c]);
             se3_exp_vec(x, s.poses + 12 * (t - 1));
         }
     }
-    if (rank == 0) advance_frame_tables(p, s, t);
+    advance_frame_tables(p, s, t);
 }
 
+__device__ __forceinline__ void ms_no_hypothesis(const DevParams& p, const DevState& s, int t)
+{
+    if (threadIdx.x == 0) {
+        s.status[0] = 0; s.status[1] = -1; s.status[2] = 0; s.status[3] += 1;
+    }
+    advance_frame_tables(p, s, t);        // the pose stays, but C_{t-1} may have moved
+}
+
+// A cluster of kMeanshiftCtas CTAs, hypothesis h in CTA (h / 256) % 8.
+__global__ void __cluster_dims__(kMeanshiftCtas, 1, 1) __launch_bounds__(kMeanshiftThreads, 1)
+k_meanshift(DevParams p, DevState s, int t)
+{
+    cg::cluster_group cluster = cg::this_cluster();
+    const unsigned rank = cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
+    __shared__ MsShared m;
+    const int n = *s.n_hyp;
+    if (n == 0) {
+        if (rank == 0) ms_no_hypothesis(p, s, t);
+        return;   // uniform over the cluster: every CTA reads the same n
+    }
+    ms_seed(p, s, m, n);
+    const int seed = m.bidx[0];
+    // FP32 offsets of this CTA's hypotheses from the seed: a thread's first
+    // kMsCached stay in registers, the rest (S above kMsCached x the cluster's
+    // threads) go to global memory
+    const int stride = kMeanshiftCtas * blockDim.x, h0 = rank * blockDim.x + tid;
+    DF sd[6];
+    for (int c = 0; c < 6; ++c) sd[c] = DF{m.seed_hi[c], m.seed_lo[c]};
+    float4 r0[kMsCached], r1[kMsCached];
+#pragma unroll
+    for (int k = 0; k < kMsCached; ++k) {
+        r0[k] = r1[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (h0 + k * stride < n) ms_offset(s, sd, h0 + k * stride, r0[k], r1[k]);
+    }
+    for (int h = h0 + kMsCached * stride; h < n; h += stride) {
+        float4* od = reinterpret_cast<float4*>(s.hyp_dp + (size_t)h * 8);
+        ms_offset(s, sd, h, od[0], od[1]);
+    }
+    const float ivt = m.consts[0], ivr = m.consts[1], tol = m.consts[2];
+    int it = 0;
+    bool degenerate = false;
+    float prev_step = INFINITY;
+    for (; it < p.ms_max_iter; ++it) {
+        float dx[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) dx[c] = m.xo_hi[c] + m.xo_lo[c];
+        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        // hypotheses in increasing h (the registers' first, then global memory)
+#pragma unroll
+        for (int k = 0; k < kMsCached; ++k)
+            if (h0 + k * stride < n) ms_add(dx, ivt, ivr, r0[k], r1[k], acc);
+        for (int h = h0 + kMsCached * stride; h < n; h += stride) {
+            const float4* o = reinterpret_cast<const float4*>(s.hyp_dp + (size_t)h * 8);
+            ms_add(dx, ivt, ivr, o[0], o[1], acc);
+        }
+        // warp sums in FP32 (each lane holds at most 4 terms), then the CTA's
+        // warps in order as float-float
+        const float ws = warp_sum8(acc, lane);
+        if ((lane & 3) == 0) m.wred[warp][lane >> 2] = ws;
+        __syncthreads();
+        const int buf = it & 1;
+        if (tid < 7) {
+            DF v{0.f, 0.f};
+            for (int w = 0; w < nwarp; ++w) v = df_add(v, m.wred[w][tid]);
+            m.part[buf][tid] = make_float2(v.hi, v.lo);
+        }
+        cluster.sync();
+        if (warp == 0) {
+            // lane c < 7 adds component c of the ranks' sums in rank order, all
+            // eight loads from distributed shared memory in flight at once
+            float2 g[kMeanshiftCtas];
+#pragma unroll
+            for (int r = 0; r < kMeanshiftCtas; ++r)
+                g[r] = lane < 7 ? *cluster.map_shared_rank(&m.part[buf][lane], (unsigned)r) : make_float2(0.f, 0.f);
+            DF tot{0.f, 0.f};
+#pragma unroll
+            for (int r = 0; r < kMeanshiftCtas; ++r) tot = df_add(tot, DF{g[r].x, g[r].y});
+            ms_finish(m, tot, lane, it, tol, prev_step);
+        }
+        __syncthreads();
+        const int f = m.flag;
+        if (f == 2) { degenerate = true; break; }
+        if (f == 1) { ++it; break; }
+    }
+    cluster.sync();   // no CTA leaves while another may still read its partials
+    if (rank == 0) ms_result(p, s, m, t, n, seed, it, degenerate);
+}
+
+// The same for at most 1024 hypotheses in one CTA, one hypothesis per thread: no
+// cluster barrier and no distributed shared memory in the step. The sums keep the
+// cluster form's order (eight warps of 256 hypotheses, then those groups), so the
+// result is bit-identical to it.
+constexpr int kMsBlockMax = 1024;
+
+__global__ void __launch_bounds__(kMsBlockMax, 1) k_meanshift_block(DevParams p, DevState s, int t)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, groups = blockDim.x / kMeanshiftThreads;
+    __shared__ MsShared m;
+    const int n = *s.n_hyp;
+    if (n == 0) {
+        ms_no_hypothesis(p, s, t);
+        return;
+    }
+    ms_seed(p, s, m, n);
+    const int seed = m.bidx[0];
+    DF sd[6];
+    for (int c = 0; c < 6; ++c) sd[c] = DF{m.seed_hi[c], m.seed_lo[c]};
+    float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
+    if (tid < n) ms_offset(s, sd, tid, r0, r1);
+    const float ivt = m.consts[0], ivr = m.consts[1], tol = m.consts[2];
+    int it = 0;
+    bool degenerate = false;
+    float prev_step = INFINITY;
+    for (; it < p.ms_max_iter; ++it) {
+        float dx[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) dx[c] = m.xo_hi[c] + m.xo_lo[c];
+        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (tid < n) ms_add(dx, ivt, ivr, r0, r1, acc);
+        const float ws = warp_sum8(acc, lane);
+        if ((lane & 3) == 0) m.wred[warp][lane >> 2] = ws;
+        __syncthreads();
+        if (warp == 0) {
+            // lane 8 g + c: component c of group g's eight warps in order, then the groups in order
+            const int g = lane >> 3, c = lane & 7;
+            DF v{0.f, 0.f};
+            if (g < groups)
+                for (int w = 0; w < 8; ++w) v = df_add(v, m.wred[8 * g + w][c]);
+            DF tot{0.f, 0.f};
+            for (int r = 0; r < groups; ++r) tot = df_add(tot, shfl_df(v, 8 * r + c));
+            ms_finish(m, tot, lane, it, tol, prev_step);
+        }
+        __syncthreads();
+        const int f = m.flag;
+        if (f == 2) { degenerate = true; break; }
+        if (f == 1) { ++it; break; }
+    }
+    ms_result(p, s, m, t, n, seed, it, degenerate);
+}
+
+// Up to 1024 hypotheses fit one CTA.
 void launch_meanshift(const DevParams& p, const DevState& s, int t, cudaStream_t st)
 {
-    k_meanshift<<<kMeanshiftCtas, kMeanshiftThreads, 0, st>>>(p, s, t);
+    if (p.S <= kMsBlockMax) {
+        const int threads = (p.S + kMeanshiftThreads - 1) / kMeanshiftThreads * kMeanshiftThreads;
+        k_meanshift_block<<<1, threads, 0, st>>>(p, s, t);
+    } else {
+        k_meanshift<<<kMeanshiftCtas, kMeanshiftThreads, 0, st>>>(p, s, t);
+    }
 }
 
 }  // namespace vd
