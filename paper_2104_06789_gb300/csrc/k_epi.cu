@@ -10,9 +10,11 @@
 //     essential matrices (eigen-decomposition of E^T E by Jacobi rotations),
 //     and a scoring form: the decomposition [t]x R with the smaller rotation,
 //     as Q = R - I and unit t in FP32.
-//  3. k_epi_hist / k_epi_select, three passes: the exact lower median of every
-//     sample's Sampson errors over all valid pixels by radix selection on the
-//     FP32 bit patterns (11 + 11 + 9 bits). The Sampson error is evaluated
+//  3. The exact lower median of every valid sample's Sampson errors over all valid
+//     pixels: k_epi_bracket brackets it from a regular subset of the pixels,
+//     k_epi_count counts the errors below the bracket and collects those inside
+//     it over all pixels, k_epi_median selects among these (and, should the bracket
+//     have missed, by radix passes over all pixels). The Sampson error is evaluated
 //     without cancellation: with m1 = m0 + d (d = flow / f, third component 0)
 //     and R m0 = m0 + Q m0, the epipolar residual is
 //         t . (m0 x d + (Q m0) x m1),
@@ -191,10 +193,8 @@ __device__ void scoring_form(const double* U, const double* V, float* f)
 // ---------------------------------------------------------------------------
 // 2. Minimal samples
 // ---------------------------------------------------------------------------
-__global__ void k_epi_samples(DevParams p, DevState s, EpiState e)
+__device__ void epi_sample(const DevParams& p, const DevState& s, const EpiState& e, int m)
 {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= e.M) return;
     int ok = 1, why = 1;
     long long j[8];
     for (int q = 0; q < 2; ++q) {
@@ -273,10 +273,50 @@ __global__ void k_epi_samples(DevParams p, DevState s, EpiState e)
     }
 }
 
+// The last block to finish lists the valid samples in order (the median passes
+// then work on full groups of them: of a fast forward motion's samples most hold a
+// pixel whose target leaves the image).
+__global__ void __launch_bounds__(kEpiSampleBlock) k_epi_samples(DevParams p, DevState s, EpiState e)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < e.M) {
+        epi_sample(p, s, e, m);
+        if (e.valid[m] <= 0) e.median[m] = __int_as_float(0x7f800000);
+    }
+    __threadfence();
+    __shared__ bool last;
+    __shared__ int wsum[kEpiSampleBlock / 32];
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(e.done, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int base = 0;
+    for (int m0 = 0; m0 < e.M; m0 += kEpiSampleBlock) {
+        const int i = m0 + threadIdx.x;
+        const bool ok = i < e.M && __ldcg(e.valid + i) > 0;
+        const unsigned bal = __ballot_sync(0xffffffffu, ok);
+        if (lane == 0) wsum[warp] = __popc(bal);
+        __syncthreads();
+        int before = base, all = 0;
+        for (int w = 0; w < kEpiSampleBlock / 32; ++w) {
+            if (w < warp) before += wsum[w];
+            all += wsum[w];
+        }
+        if (ok) e.list[before + __popc(bal & ((1u << lane) - 1u))] = i;
+        base += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *e.n_list = base;
+}
+
 // ---------------------------------------------------------------------------
 // 3. Sampson error (FP32, cancellation-free) and radix selection of the median
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float sampson32(const float* F, float4 r)
+// Numerator and denominator: the error is e2 / den, +inf where den is not positive
+// or the quotient no number.
+__device__ __forceinline__ void sampson_parts(const float* F, float4 r, float& e2, float& den)
 {
     const float m0x = r.x, m0y = r.y, dx = r.z, dy = r.w;
     const float m1x = m0x + dx, m1y = m0y + dy;
@@ -296,106 +336,274 @@ __device__ __forceinline__ float sampson32(const float* F, float4 r)
     const float w0 = fmaf(ty, 1.f, -tz * m1y), w1 = fmaf(tz, m1x, -tx), w2 = fmaf(tx, m1y, -ty * m1x);
     const float b0 = w0 + fmaf(F[0], w0, fmaf(F[3], w1, F[6] * w2));
     const float b1 = w1 + fmaf(F[1], w0, fmaf(F[4], w1, F[7] * w2));
-    const float den = fmaf(a0, a0, fmaf(a1, a1, fmaf(b0, b0, b1 * b1)));
-    const float d = e * e / den;
+    den = fmaf(a0, a0, fmaf(a1, a1, fmaf(b0, b0, b1 * b1)));
+    e2 = e * e;
+}
+
+__device__ __forceinline__ float sampson_ratio(float e2, float den)
+{
+    const float d = e2 / den;
     return (den > 0.f && d == d) ? d : __int_as_float(0x7f800000);
 }
 
-__device__ __forceinline__ int epi_digit(unsigned bits, int pass)
+__device__ __forceinline__ float sampson32(const float* F, float4 r)
 {
-    return pass == 0 ? (int)(bits >> 20) : pass == 1 ? (int)((bits >> 9) & 0x7ff) : (int)(bits & 0x1ff);
+    float e2, den;
+    sampson_parts(F, r, e2, den);
+    return sampson_ratio(e2, den);
 }
 
-__device__ __forceinline__ bool epi_prefix_match(unsigned bits, int pass, unsigned prefix)
+constexpr int kEpiPix = 4;                                   // pixels per thread of a work item
+constexpr int kEpiItemPix = kEpiThreads * kEpiPix;           // 1024
+// Loads a group's scoring forms; the samples of group g are list[8 g ...].
+__device__ __forceinline__ int epi_load_group(const EpiState& e, int g, int n, float (*F)[12], int* id)
 {
-    return pass == 0 || (pass == 1 ? (bits >> 20) == prefix : (bits >> 9) == prefix);
+    const int cnt = min(kEpiSamplesPerBlock, n - g * kEpiSamplesPerBlock);
+    if ((int)threadIdx.x < cnt * 12) {
+        const int sm = threadIdx.x / 12, q = threadIdx.x % 12, m = e.list[g * kEpiSamplesPerBlock + sm];
+        F[sm][q] = e.form[(size_t)m * 12 + q];
+        if (q == 0) id[sm] = m;
+    }
+    return cnt;
 }
 
-// grid (pixel chunks, M / 8); dynamic shared memory 8 x kEpiBins counters.
-__global__ void __launch_bounds__(kEpiThreads, 2) k_epi_hist(DevParams p, EpiState e, int pass)
+// The bin of a block's shared histogram that holds rank `rank`, and the rank inside
+// it (all threads get both); false if the counts do not reach the rank.
+__device__ __forceinline__ bool epi_pick(const unsigned* h, int bins, unsigned rank, unsigned* ws, unsigned& bin, unsigned& rest)
 {
-    extern __shared__ unsigned h[];
-    __shared__ float F[kEpiSamplesPerBlock][12];
-    __shared__ unsigned pre[kEpiSamplesPerBlock];
-    __shared__ int act[kEpiSamplesPerBlock];
-    const int m0 = blockIdx.y * kEpiSamplesPerBlock;
-    for (int i = threadIdx.x; i < kEpiSamplesPerBlock * kEpiBins; i += blockDim.x) h[i] = 0;
-    if (threadIdx.x < kEpiSamplesPerBlock * 12) {
-        const int sm = threadIdx.x / 12, q = threadIdx.x % 12;
-        F[sm][q] = (m0 + sm < e.M) ? e.form[(size_t)(m0 + sm) * 12 + q] : 0.f;
-    }
-    if (threadIdx.x < kEpiSamplesPerBlock) {
-        const int m = m0 + threadIdx.x;
-        act[threadIdx.x] = (m < e.M && e.valid[m] > 0) ? 1 : 0;
-        pre[threadIdx.x] = (m < e.M) ? e.prefix[m] : 0u;
-    }
-    __syncthreads();
-    const long long lo = (long long)p.N * blockIdx.x / gridDim.x;
-    const long long hi = (long long)p.N * (blockIdx.x + 1) / gridDim.x;
-    auto count = [&](const float4& r) {
-        if (r.x != r.x) return;                       // invalid pixel
-#pragma unroll
-        for (int sm = 0; sm < kEpiSamplesPerBlock; ++sm) {
-            if (!act[sm]) continue;
-            const unsigned bits = __float_as_uint(sampson32(F[sm], r));
-            if (!epi_prefix_match(bits, pass, pre[sm])) continue;
-            atomicAdd(&h[sm * kEpiBins + epi_digit(bits, pass)], 1u);
-        }
-    };
-    // two records in flight per thread
-    long long j = lo + threadIdx.x;
-    for (; j + blockDim.x < hi; j += 2 * blockDim.x) {
-        const float4 r0 = e.rec[j], r1 = e.rec[j + blockDim.x];
-        count(r0);
-        count(r1);
-    }
-    if (j < hi) count(e.rec[j]);
-    __syncthreads();
-    unsigned* g = e.hist + (size_t)pass * e.M * kEpiBins;
-    for (int i = threadIdx.x; i < kEpiSamplesPerBlock * kEpiBins; i += blockDim.x) {
-        const int sm = i / kEpiBins, b = i % kEpiBins;
-        if (m0 + sm < e.M && h[i]) atomicAdd(g + (size_t)(m0 + sm) * kEpiBins + b, h[i]);
-    }
-}
-
-// One warp per sample: the bin of this pass that holds the remaining rank.
-__global__ void k_epi_select(EpiState e, int pass)
-{
-    const int lane = threadIdx.x & 31;
-    const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (m >= e.M) return;
-    if (e.valid[m] <= 0 || e.info[2] == 0) {
-        if (lane == 0) e.median[m] = __int_as_float(0x7f800000);
-        return;
-    }
-    const unsigned rank = pass == 0 ? (unsigned)((e.info[2] - 1) / 2) : e.rank[m];
-    const unsigned* h = e.hist + ((size_t)pass * e.M + m) * kEpiBins;
-    const int nb = pass == 2 ? 512 : kEpiBins;
-    const int per = nb / 32;
+    __shared__ unsigned out[2];
+    const int per = (bins + blockDim.x - 1) / blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned mine = 0;
-    for (int i = 0; i < per; ++i) mine += h[lane * per + i];
+    for (int i = 0; i < per; ++i) {
+        const int b = threadIdx.x * per + i;
+        if (b < bins) mine += h[b];
+    }
     unsigned incl = mine;
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
     }
-    const unsigned excl = incl - mine;
-    const bool here = rank >= excl && rank < incl;
-    const unsigned ball = __ballot_sync(0xffffffffu, here);
-    if (!ball) {                                      // counts do not reach the rank: no valid value
-        if (lane == 0) e.median[m] = __int_as_float(0x7f800000);
+    if (lane == 31) ws[warp] = incl;
+    if (threadIdx.x == 0) out[0] = 0xffffffffu;
+    __syncthreads();
+    unsigned cum = incl - mine;
+    for (int w = 0; w < warp; ++w) cum += ws[w];
+    for (int i = 0; i < per; ++i) {
+        const int b = threadIdx.x * per + i;
+        const unsigned c = b < bins ? h[b] : 0u;
+        if (rank >= cum && rank < cum + c) { out[0] = (unsigned)b; out[1] = rank - cum; }
+        cum += c;
+    }
+    __syncthreads();
+    bin = out[0];
+    rest = out[1];
+    __syncthreads();
+    return bin != 0xffffffffu;
+}
+
+// Bracket of the median from a subset of the pixels, one block per valid sample:
+// one pixel of every `step`, at a place that varies (all pixels of a small image),
+// 16384 errors in registers at most; the subset's ranks four and a half standard
+// deviations of a binomial count below and above its median are selected exactly
+// by radix passes. Between them lie about 3.5 % of all errors; a bracket that
+// misses costs time (k_epi_median), not exactness. Bound by the latency of the
+// strided record loads and of the six scans between barriers.
+constexpr int kEpiSubThreads = 512, kEpiSubPer = 32;
+
+__global__ void __launch_bounds__(kEpiSubThreads, 2) k_epi_bracket(DevParams p, EpiState e)
+{
+    __shared__ unsigned h[2][kEpiBins], ws[kEpiSubThreads / 32];
+    __shared__ __align__(16) float F[12];
+    if ((int)blockIdx.x >= *e.n_list) return;
+    const int q = blockIdx.x;
+    if (threadIdx.x < 12) F[threadIdx.x] = e.form[(size_t)e.list[q] * 12 + threadIdx.x];
+    for (int i = threadIdx.x; i < kEpiBins; i += blockDim.x) h[0][i] = 0;
+    __syncthreads();
+    const int step = (p.N + kEpiSubThreads * kEpiSubPer - 1) / (kEpiSubThreads * kEpiSubPer), n_sub = p.N / step;
+    constexpr unsigned kNone = 0xffffffffu;
+    unsigned v[kEpiSubPer], mine = 0;
+#pragma unroll
+    for (int i = 0; i < kEpiSubPer; ++i) {
+        const int k = i * kEpiSubThreads + threadIdx.x;
+        v[i] = kNone;
+        if (k < n_sub) {
+            const float4 r = e.rec[(size_t)k * step + (unsigned)(k * 5) % (unsigned)step];
+            if (r.x == r.x) {
+                v[i] = __float_as_uint(sampson32(F, r));
+                ++mine;
+                atomicAdd(&h[0][v[i] >> 21], 1u);
+            }
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    __shared__ unsigned total_s;
+    if (threadIdx.x == 0) total_s = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicAdd(&total_s, mine);
+    __syncthreads();
+    const unsigned total = total_s;
+    if (total == 0) {
+        if (threadIdx.x == 0) e.lo[q] = e.hi[q] = 0u;
         return;
     }
-    const int L = __ffs(ball) - 1;
-    if (lane == L) {
-        unsigned cum = excl;
-        int b = lane * per;
-        for (; b < lane * per + per - 1 && cum + h[b] <= rank; ++b) cum += h[b];
-        const unsigned prefix = e.prefix[m];
-        if (pass == 0) { e.prefix[m] = (unsigned)b; e.rank[m] = rank - cum; }
-        else if (pass == 1) { e.prefix[m] = (prefix << 11) | (unsigned)b; e.rank[m] = rank - cum; }
-        else e.median[m] = __uint_as_float((prefix << 9) | (unsigned)b);
+    const float mid = 0.5f * (float)total, dev = step > 1 ? 2.25f * sqrtf((float)total) + 2.f : 1.f;
+    unsigned rank[2] = {mid > dev ? (unsigned)(mid - dev) : 0u, min((unsigned)(mid + dev), total - 1u)}, prefix[2];
+    for (int r = 0; r < 2; ++r) epi_pick(h[0], 1024, rank[r], ws, prefix[r], rank[r]);
+    for (int level = 0; level < 2; ++level) {
+        const int shift = level == 0 ? 10 : 0, top = level == 0 ? 21 : 10, bins = level == 0 ? 2048 : 1024;
+        for (int i = threadIdx.x; i < bins; i += blockDim.x) h[0][i] = h[1][i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kEpiSubPer; ++i)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (v[i] != kNone && (v[i] >> top) == prefix[r]) atomicAdd(&h[r][(v[i] >> shift) & (bins - 1)], 1u);
+        __syncthreads();
+        for (int r = 0; r < 2; ++r) {
+            unsigned bin;
+            epi_pick(h[r], bins, rank[r], ws, bin, rank[r]);
+            prefix[r] = (prefix[r] << (top - shift)) | bin;
+        }
     }
+    if (threadIdx.x == 0) {
+        e.lo[q] = prefix[0];
+        e.hi[q] = prefix[1] + 1u;
+    }
+}
+
+// One pass over all pixels: per sample, the errors below its bracket are counted
+// and those inside it collected. An error is compared without the division, e2
+// against the edge times den, unless it lies within 2^-20 of an edge or inside the
+// bracket (a few percent of the pairs); only then is the rounded quotient formed.
+// The 1e-30 keeps products that round as denormals out of the short way.
+// Four pixels per thread share a sample's form. What bounds it: the ~45 FP32
+// instructions of a pair. 512 samples over 1242 x 375 pixels: three radix passes
+// over all pixels, with a division and a shared-memory atomic per pair and pass,
+// took 735 us; bracket, count and selection take 45 + 157 + 18 us.
+__global__ void __launch_bounds__(kEpiThreads, 3) k_epi_count(DevParams p, EpiState e)
+{
+    __shared__ __align__(16) float F[kEpiSamplesPerBlock][12];
+    __shared__ int id[kEpiSamplesPerBlock];
+    __shared__ float edge[kEpiSamplesPerBlock][2];
+    __shared__ unsigned lo_s[kEpiSamplesPerBlock], hi_s[kEpiSamplesPerBlock], below[kEpiSamplesPerBlock];
+    __shared__ unsigned fill[kEpiSamplesPerBlock], base[kEpiSamplesPerBlock];
+    __shared__ unsigned found[kEpiSamplesPerBlock][kEpiItemPix];
+    const int n = *e.n_list, groups = (n + kEpiSamplesPerBlock - 1) / kEpiSamplesPerBlock;
+    const int chunks = (p.N + kEpiItemPix - 1) / kEpiItemPix, lane = threadIdx.x & 31;
+    for (int u = blockIdx.x; u < groups * chunks; u += gridDim.x) {
+        const int g = u / chunks, j0 = (u % chunks) * kEpiItemPix, q0 = g * kEpiSamplesPerBlock;
+        const int cnt = epi_load_group(e, g, n, F, id);
+        if ((int)threadIdx.x < cnt) {
+            lo_s[threadIdx.x] = e.lo[q0 + threadIdx.x];
+            hi_s[threadIdx.x] = e.hi[q0 + threadIdx.x];
+            edge[threadIdx.x][0] = __uint_as_float(lo_s[threadIdx.x]) * (1.f - 9.5367432e-7f);
+            edge[threadIdx.x][1] = __uint_as_float(hi_s[threadIdx.x]) * (1.f + 9.5367432e-7f);
+            below[threadIdx.x] = fill[threadIdx.x] = 0u;
+        }
+        __syncthreads();
+        float4 r[kEpiPix];
+#pragma unroll
+        for (int i = 0; i < kEpiPix; ++i) {
+            const int j = j0 + i * kEpiThreads + threadIdx.x;
+            r[i] = j < p.N ? e.rec[j] : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+        }
+        for (int sm = 0; sm < cnt; ++sm) {
+            float f[12];
+#pragma unroll
+            for (int i = 0; i < 12; ++i) f[i] = F[sm][i];
+            const float lo_m = edge[sm][0], hi_p = edge[sm][1];
+            unsigned less = 0;
+#pragma unroll
+            for (int i = 0; i < kEpiPix; ++i) {
+                float e2, den;
+                sampson_parts(f, r[i], e2, den);
+                if (e2 < fmaf(lo_m, den, -1e-30f)) {
+                    ++less;
+                } else if (!(e2 > fmaf(hi_p, den, 1e-30f)) && r[i].x == r[i].x) {
+                    const unsigned bits = __float_as_uint(sampson_ratio(e2, den));
+                    if (bits < lo_s[sm]) ++less;
+                    else if (bits < hi_s[sm]) found[sm][atomicAdd(&fill[sm], 1u)] = bits;
+                }
+            }
+            less = __reduce_add_sync(0xffffffffu, less);
+            if (lane == 0 && less) atomicAdd(&below[sm], less);
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < cnt) {
+            if (below[threadIdx.x]) atomicAdd(e.below + q0 + threadIdx.x, below[threadIdx.x]);
+            base[threadIdx.x] = fill[threadIdx.x] ? atomicAdd(e.inside + q0 + threadIdx.x, fill[threadIdx.x]) : 0u;
+        }
+        __syncthreads();
+        for (int sm = 0; sm < cnt; ++sm)
+            for (unsigned i = threadIdx.x; i < fill[sm]; i += blockDim.x)
+                if (base[sm] + i < (unsigned)e.cap && hi_s[sm] - lo_s[sm] > 1) e.found[(size_t)(q0 + sm) * e.cap + base[sm] + i] = found[sm][i];
+        __syncthreads();
+    }
+}
+
+// One block per valid sample: the exact median, rank (n - 1) / 2 of the valid
+// pixels' errors, among the collected ones (radix passes over the bracket's bit
+// patterns, 11 bits each; a bracket of one bit pattern is the median itself);
+// where they do not hold it, radix passes over all pixels (11 + 11 + 10 bits).
+constexpr int kEpiMedianThreads = 1024;
+
+__global__ void __launch_bounds__(kEpiMedianThreads, 2) k_epi_median(DevParams p, EpiState e)
+{
+    __shared__ unsigned h[kEpiBins], ws[kEpiMedianThreads / 32];
+    __shared__ __align__(16) float F[12];
+    if ((int)blockIdx.x >= *e.n_list) return;
+    const int q = blockIdx.x, m = e.list[q];
+    const long long nv = e.info[2];
+    if (nv == 0) {
+        if (threadIdx.x == 0) e.median[m] = __int_as_float(0x7f800000);
+        return;
+    }
+    const unsigned rank = (unsigned)((nv - 1) / 2), under = e.below[q], in = e.inside[q], lo = e.lo[q];
+    const unsigned span = e.hi[q] - lo;                                // at most 2^31
+    unsigned bits = 0, bin, rest;
+    bool ok = rank >= under && rank - under < in && (in <= (unsigned)e.cap || span == 1);
+    if (ok) {
+        const unsigned* v = e.found + (size_t)q * e.cap;
+        // levels of 11 bits from the top of the span
+        unsigned from = lo, width = span;
+        rest = rank - under;
+        while (width > 1 && ok) {
+            const int shift = max(0, 32 - __clz(width - 1) - 11);
+            for (int i = threadIdx.x; i < kEpiBins; i += blockDim.x) h[i] = 0;
+            __syncthreads();
+            for (unsigned i = threadIdx.x; i < in; i += blockDim.x) {
+                const unsigned o = v[i] - from;
+                if (o < width) atomicAdd(&h[o >> shift], 1u);
+            }
+            __syncthreads();
+            ok = epi_pick(h, kEpiBins, rest, ws, bin, rest);
+            from += bin << shift;
+            width = 1u << shift;
+        }
+        bits = from;
+    }
+    if (!ok) {
+        if (threadIdx.x < 12) F[threadIdx.x] = e.form[(size_t)m * 12 + threadIdx.x];
+        unsigned prefix = 0;
+        rest = rank;
+        ok = true;
+        for (int pass = 0; pass < 3 && ok; ++pass) {
+            const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0), width = pass == 2 ? 1024 : 2048;
+            for (int i = threadIdx.x; i < kEpiBins; i += blockDim.x) h[i] = 0;
+            __syncthreads();
+            for (int j = threadIdx.x; j < p.N; j += blockDim.x) {
+                const float4 r = e.rec[j];
+                if (r.x != r.x) continue;
+                const unsigned b = __float_as_uint(sampson32(F, r));
+                if (pass == 0 || (b >> (pass == 1 ? 21 : 10)) == prefix) atomicAdd(&h[(b >> shift) & (width - 1)], 1u);
+            }
+            __syncthreads();
+            ok = epi_pick(h, width, rest, ws, bin, rest);
+            prefix = pass == 0 ? bin : (prefix << (pass == 1 ? 11 : 10)) | bin;
+        }
+        bits = ok ? prefix : 0x7f800000u;
+    }
+    if (threadIdx.x == 0) e.median[m] = __uint_as_float(bits);
 }
 
 // ---------------------------------------------------------------------------
@@ -635,9 +843,13 @@ __global__ void k_epi_finish(EpiState e, double baseline)
 // ---------------------------------------------------------------------------
 static int epi_refine_blocks() { return 2 * 152; }
 
+// Collected errors a sample has room for: a sixteenth of the pixels (the bracket
+// holds a few percent), within these bounds.
+constexpr int kEpiCapMin = 4096, kEpiCapMax = 65536;
+
 // Carves the scratch for M samples out of `base` (which may be null to measure)
 // and returns the bytes it spans; every piece starts on a 256-byte boundary.
-size_t epi_layout(void* base, int M, float4* rec, EpiState* e)
+size_t epi_layout(void* base, int M, int N, float4* rec, EpiState* e)
 {
     const uintptr_t start = reinterpret_cast<uintptr_t>(base);
     size_t off = 0;
@@ -652,11 +864,21 @@ size_t epi_layout(void* base, int M, float4* rec, EpiState* e)
     e->E = static_cast<double*>(take((size_t)M * 9 * 8));
     e->UV = static_cast<double*>(take((size_t)M * 18 * 8));
     e->form = static_cast<float*>(take((size_t)M * 12 * 4));
-    e->hist = static_cast<unsigned*>(take((size_t)3 * M * kEpiBins * 4));
-    e->prefix = static_cast<unsigned*>(take((size_t)M * 4));
-    e->rank = static_cast<unsigned*>(take((size_t)M * 4));
-    e->median = static_cast<float*>(take((size_t)M * 4));
+    e->list = static_cast<int*>(take((size_t)M * 4));
+    e->lo = static_cast<unsigned*>(take((size_t)M * 4));
+    e->hi = static_cast<unsigned*>(take((size_t)M * 4));
+    e->cap = N / 16 < kEpiCapMin ? kEpiCapMin : (N / 16 > kEpiCapMax ? kEpiCapMax : N / 16);
+    e->found = static_cast<unsigned*>(take((size_t)M * e->cap * 4));
+    // zeroed together before every estimate: zero .. zero + zero_bytes
+    const size_t z0 = off;
+    e->zero = reinterpret_cast<void*>(start + off);
+    e->below = static_cast<unsigned*>(take((size_t)M * 4));
+    e->inside = static_cast<unsigned*>(take((size_t)M * 4));
+    e->n_list = static_cast<int*>(take(4));
+    e->done = static_cast<int*>(take(4));
     e->info = static_cast<long long*>(take(8 * 8));
+    e->zero_bytes = off - z0;
+    e->median = static_cast<float*>(take((size_t)M * 4));
     e->partial_blocks = epi_refine_blocks();
     e->partial = static_cast<double*>(take((size_t)e->partial_blocks * 46 * 8));
     e->refined = static_cast<double*>(take(27 * 8));
@@ -665,34 +887,23 @@ size_t epi_layout(void* base, int M, float4* rec, EpiState* e)
     return off;
 }
 
-size_t epi_scratch_bytes(int M)
+size_t epi_scratch_bytes(int M, int N)
 {
     EpiState e;
-    return epi_layout(nullptr, M, nullptr, &e);
+    return epi_layout(nullptr, M, N, nullptr, &e);
 }
 
 // Enqueues the whole estimate on st; returns the number of kernels launched.
 int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, double baseline, cudaStream_t st)
 {
-    static bool attr = false;
-    const int hist_smem = kEpiSamplesPerBlock * kEpiBins * 4;
-    if (!attr) {
-        cudaFuncSetAttribute(k_epi_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_smem);
-        attr = true;
-    }
     int k = 0;
-    cudaMemsetAsync(e.hist, 0, (size_t)3 * e.M * kEpiBins * 4, st);
-    cudaMemsetAsync(e.prefix, 0, (size_t)e.M * 4, st);
-    cudaMemsetAsync(e.info, 0, 8 * 8, st);
+    cudaMemsetAsync(e.zero, 0, e.zero_bytes, st);
     k_epi_records<<<(p.N + 255) / 256, 256, 0, st>>>(p, s, e); ++k;
     k_epi_samples<<<(e.M + kEpiSampleBlock - 1) / kEpiSampleBlock, kEpiSampleBlock, 0, st>>>(p, s, e); ++k;
-    const int groups = (e.M + kEpiSamplesPerBlock - 1) / kEpiSamplesPerBlock;
-    int chunks = (8 * 152 + groups - 1) / groups;
-    chunks = chunks < 1 ? 1 : (chunks > 1024 ? 1024 : chunks);
-    for (int pass = 0; pass < 3; ++pass) {
-        k_epi_hist<<<dim3(chunks, groups), kEpiThreads, hist_smem, st>>>(p, e, pass); ++k;
-        k_epi_select<<<(e.M + 7) / 8, 256, 0, st>>>(e, pass); ++k;
-    }
+    k_epi_bracket<<<e.M, kEpiSubThreads, 0, st>>>(p, e); ++k;
+    // persistent blocks: the number of valid samples is known on the device only
+    k_epi_count<<<3 * 152, kEpiThreads, 0, st>>>(p, e); ++k;
+    k_epi_median<<<e.M, kEpiMedianThreads, 0, st>>>(p, e); ++k;
     k_epi_argmin<<<1, 1024, 0, st>>>(e); ++k;
     k_epi_refine_accum<<<e.partial_blocks, kEpiThreads, 0, st>>>(p, s, e); ++k;
     k_epi_refine_solve<<<1, 64, 0, st>>>(e); ++k;

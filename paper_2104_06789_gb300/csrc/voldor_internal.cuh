@@ -297,9 +297,17 @@ struct EpiState {
     double* E;                // [M][9] projected essential matrix
     double* UV;               // [M][18] U, V (row-major, det +1)
     float* form;              // [M][12] Q = R - I (9), t (3)
-    unsigned* hist;           // [3][M][kEpiBins]
-    unsigned* prefix;         // [M] bits selected so far
-    unsigned* rank;           // [M] remaining rank
+    int* list;                // [M] the valid samples in order
+    unsigned* lo;             // [M] bracket of the i-th valid sample's median, as bit patterns [lo, hi)
+    unsigned* hi;
+    int cap;                  // collected errors per sample
+    unsigned* found;          // [M][cap] errors inside the bracket
+    void* zero;               // what follows down to info, zeroed before an estimate
+    size_t zero_bytes;
+    unsigned* below;          // [M] errors below the bracket
+    unsigned* inside;         // [M] errors inside it
+    int* n_list;              // [1] valid samples
+    int* done;                // [1] blocks of the sample kernel done
     float* median;            // [M]
     long long* info;          // [8]: chosen, candidate, n_valid, n_inliers, count[4]
     double* partial;          // [blocks][46] A^T A partials (45) + inlier count
@@ -308,8 +316,8 @@ struct EpiState {
     double* T1;               // [12]
     int partial_blocks;
 };
-size_t epi_scratch_bytes(int M);
-size_t epi_layout(void* base, int M, float4* rec, EpiState* e);
+size_t epi_scratch_bytes(int M, int N);
+size_t epi_layout(void* base, int M, int N, float4* rec, EpiState* e);
 int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, double baseline, cudaStream_t st);
 // Ground-plane scale: hist [4096] and out [3] are device scratch; returns the
 // number of kernels launched.
