@@ -3,7 +3,7 @@
 //
 //  1. k_epi_records: per pixel, the calibrated correspondence of X_1 as
 //     {m0x, m0y, u/fx, v/fy} (FP32), m0 = K^-1 [x y 1]; NaN marks a pixel whose
-//     flow target leaves I_1 (tested in FP64).
+//     flow target leaves I_1 (the test and the values are those of FP64).
 //  2. k_epi_samples: one thread per minimal sample: 8 Philox-drawn pixels,
 //     the 8-point essential matrix (null vector of the 8 x 9 system by Gaussian
 //     elimination with complete pivoting, FP64), its projection onto the
@@ -41,33 +41,65 @@ constexpr int kEpiThreads = 256;
 // ---------------------------------------------------------------------------
 // 1. Records (and the count of valid pixels into info[2])
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool epi_target_inside(const DevParams& p, const DevState& s, int j)
+// 0 <= i + f <= last with the sum rounded to FP64, as the samples test it. A sum of
+// an integer and an FP32 number keeps its sign when it is rounded, and one that is
+// at most `last` stays so; what FP32 leaves open is an f just above last - i.
+__device__ __forceinline__ bool target_inside(int i, float f, int last)
 {
-    const float2 f = load_flow(s.flows, p.flow_f16, (size_t)j);
-    const double u = (double)(j % p.W) + (double)f.x, v = (double)(j / p.W) + (double)f.y;
-    return u >= 0.0 && u <= (double)(p.W - 1) && v >= 0.0 && v <= (double)(p.H - 1);
+    const float c = (float)(last - i);
+    if (!(f >= -(float)i)) return false;
+    if (f <= c) return true;
+    return f <= c + 1.f && (double)i + (double)f <= (double)last;
 }
 
-__global__ void k_epi_records(DevParams p, DevState s, EpiState e)
+// (float)((double)f / fd) without an FP64 division where the FP32 result is beyond
+// doubt: f times the float-float reciprocal has a relative error below 2^-43.
+__device__ __forceinline__ float quotient32(float f, float inv_hi, float inv_lo, double fd)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int cnt = __syncthreads_count(j < p.N && epi_target_inside(p, s, j));
-    if (threadIdx.x == 0 && cnt) atomicAdd(reinterpret_cast<unsigned long long*>(e.info + 2), (unsigned long long)cnt);
-    if (j >= p.N) return;
-    const int x = j % p.W, y = j / p.W;
-    const float2 f = load_flow(s.flows, p.flow_f16, (size_t)j);
-    const double u = (double)x + (double)f.x, v = (double)y + (double)f.y;
-    float4 r;
-    if (u >= 0.0 && u <= (double)(p.W - 1) && v >= 0.0 && v <= (double)(p.H - 1)) {
-        r.x = (float)(((double)x - p.cxd) / p.fxd);
-        r.y = (float)(((double)y - p.cyd) / p.fyd);
-        r.z = (float)((double)f.x / p.fxd);
-        r.w = (float)((double)f.y / p.fyd);
-    } else {
-        r.x = __int_as_float(0x7fc00000);
-        r.y = r.z = r.w = 0.f;
+    const float q = f * inv_hi;
+    const float l = fmaf(f, inv_lo, fmaf(f, inv_hi, -q)), err = fabsf(q) * 0x1p-40f;
+    const float below = __fadd_rn(q, l - err), above = __fadd_rn(q, l + err);
+    if (below == above && (fabsf(q) > 1e-20f || f == 0.f)) return below;
+    return (float)((double)f / fd);
+}
+
+// A warp takes 32 columns of kEpiRecRows rows: the FP64 divisions of m0 are one per
+// column and one per row of the tile, not two per pixel (four with the flow's, which
+// FP32 pairs replace): 52.5 -> 11.5 us at 1242 x 375.
+constexpr int kEpiRecRows = 8, kEpiRecWarps = 8;
+
+__global__ void __launch_bounds__(32 * kEpiRecWarps) k_epi_records(DevParams p, DevState s, EpiState e)
+{
+    __shared__ int inside_s[kEpiRecWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int x = blockIdx.x * 32 + lane, y0 = (blockIdx.y * kEpiRecWarps + warp) * kEpiRecRows;
+    const float m0x = (float)(((double)x - p.cxd) / p.fxd);
+    const float m0y_l = lane < kEpiRecRows ? (float)(((double)(y0 + lane) - p.cyd) / p.fyd) : 0.f;
+    int inside = 0;
+#pragma unroll
+    for (int k = 0; k < kEpiRecRows; ++k) {
+        const int y = y0 + k;
+        const float m0y = __shfl_sync(0xffffffffu, m0y_l, k);
+        const bool in_image = x < p.W && y < p.H;
+        bool ok = false;
+        if (in_image) {
+            const size_t j = (size_t)y * p.W + x;
+            const float2 f = load_flow(s.flows, p.flow_f16, j);
+            ok = target_inside(x, f.x, p.W - 1) && target_inside(y, f.y, p.H - 1);
+            float4 r = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+            if (ok)
+                r = make_float4(m0x, m0y, quotient32(f.x, p.kdf[8], p.kdf[9], p.fxd),
+                                quotient32(f.y, p.kdf[10], p.kdf[11], p.fyd));
+            e.rec[j] = r;
+        }
+        inside += __popc(__ballot_sync(0xffffffffu, ok));
     }
-    e.rec[j] = r;
+    if (lane == 0) inside_s[warp] = inside;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kEpiRecWarps; ++w) inside += inside_s[w];
+        if (inside) atomicAdd(reinterpret_cast<unsigned long long*>(e.info + 2), (unsigned long long)inside);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -791,37 +823,85 @@ __global__ void k_epi_refine_solve(EpiState e)
 // ---------------------------------------------------------------------------
 // 6. Cheirality and T_1
 // ---------------------------------------------------------------------------
+// The pixel's count for each candidate in FP64 (the definition).
+__device__ __noinline__ unsigned cheirality64(const DevParams& p, float2 f, int x, int y, const double* Cd)
+{
+    unsigned in = 0;
+    const double m0x = ((double)x - p.cxd) / p.fxd, m0y = ((double)y - p.cyd) / p.fyd;
+    const double m1x = ((double)x + (double)f.x - p.cxd) / p.fxd, m1y = ((double)y + (double)f.y - p.cyd) / p.fyd;
+    for (int i = 0; i < 4; ++i) {
+        const double* T = Cd + 12 * i;
+        const double Rx = T[0] * m0x + T[1] * m0y + T[2];
+        const double Ry = T[4] * m0x + T[5] * m0y + T[6];
+        const double Rz = T[8] * m0x + T[9] * m0y + T[10];
+        const double ax = Rx - m1x * Rz, bx = m1x * T[11] - T[3];
+        const double ay = Ry - m1y * Rz, by = m1y * T[11] - T[7];
+        const double aa = ax * ax + ay * ay, ab = ax * bx + ay * by;
+        if (!(aa > 0.0) || !(ab > 0.0)) continue;
+        const double z1 = (ab / aa) * Rz + T[11];
+        if (z1 > 0.0) in |= 1u << i;
+    }
+    return in;
+}
+
+// Only the signs of ab and of ab Rz + aa t_z count, so they are taken in FP32 from
+// the records, each beside a bound of its error, and a pixel one of whose signs the
+// bound leaves open goes to FP64. With u = 2^-24, |R m0| <= n = 1 + |m0x| + |m0y|
+// and m = |m0| + |d| (largest component), |t| = 1: a is known to 8 u n (1 + m), b to
+// 8 u (1 + m), Rz to 8 u n, and the rest is products; the bounds are taken twice.
+// All in FP64 this took 117 us at 1242 x 375; now 14.6 us.
 __global__ void __launch_bounds__(kEpiThreads) k_epi_cheirality(DevParams p, DevState s, EpiState e)
 {
     __shared__ double Cd[48];
+    __shared__ float Cf[48];
+    __shared__ unsigned total[4];
     if (e.info[0] < 0) return;
-    if (threadIdx.x < 48) Cd[threadIdx.x] = e.cand[threadIdx.x];
+    if (threadIdx.x < 48) {
+        Cd[threadIdx.x] = e.cand[threadIdx.x];
+        Cf[threadIdx.x] = (float)e.cand[threadIdx.x];
+    }
+    if (threadIdx.x < 4) total[threadIdx.x] = 0;
     __syncthreads();
     unsigned cnt[4] = {0, 0, 0, 0};
+    constexpr float kU = 0x1p-24f;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < p.N; j += gridDim.x * blockDim.x) {
-        if (e.rec[j].x != e.rec[j].x) continue;
-        const int x = j % p.W, y = j / p.W;
-        const float2 f = load_flow(s.flows, p.flow_f16, (size_t)j);
-        const double m0x = ((double)x - p.cxd) / p.fxd, m0y = ((double)y - p.cyd) / p.fyd;
-        const double m1x = ((double)x + (double)f.x - p.cxd) / p.fxd, m1y = ((double)y + (double)f.y - p.cyd) / p.fyd;
+        const float4 r = e.rec[j];
+        if (r.x != r.x) continue;
+        const float m0x = r.x, m0y = r.y, m1x = r.x + r.z, m1y = r.y + r.w;
+        const float n = 1.f + fabsf(m0x) + fabsf(m0y);
+        const float m = 1.f + fmaxf(fabsf(m0x) + fabsf(r.z), fabsf(m0y) + fabsf(r.w));
+        const float eb = 16.f * kU * m, ea = eb * n, er = 16.f * kU * n;
+        unsigned in = 0;
+        bool open = false;
+#pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const double* T = Cd + 12 * i;
-            const double Rx = T[0] * m0x + T[1] * m0y + T[2];
-            const double Ry = T[4] * m0x + T[5] * m0y + T[6];
-            const double Rz = T[8] * m0x + T[9] * m0y + T[10];
-            const double ax = Rx - m1x * Rz, bx = m1x * T[11] - T[3];
-            const double ay = Ry - m1y * Rz, by = m1y * T[11] - T[7];
-            const double aa = ax * ax + ay * ay, ab = ax * bx + ay * by;
-            if (!(aa > 0.0) || !(ab > 0.0)) continue;
-            const double z1 = (ab / aa) * Rz + T[11];
-            if (z1 > 0.0) ++cnt[i];
+            const float* T = Cf + 12 * i;
+            const float Rx = fmaf(T[0], m0x, fmaf(T[1], m0y, T[2]));
+            const float Ry = fmaf(T[4], m0x, fmaf(T[5], m0y, T[6]));
+            const float Rz = fmaf(T[8], m0x, fmaf(T[9], m0y, T[10]));
+            const float ax = fmaf(-m1x, Rz, Rx), bx = fmaf(m1x, T[11], -T[3]);
+            const float ay = fmaf(-m1y, Rz, Ry), by = fmaf(m1y, T[11], -T[7]);
+            const float aa = fmaf(ax, ax, ay * ay), ab = fmaf(ax, bx, ay * by);
+            const float sa = fabsf(ax) + fabsf(ay), sb = fabsf(bx) + fabsf(by);
+            const float e_ab = fmaf(2.f * eb, sa, ea * (sb + 2.f * eb));
+            const float e_aa = 2.f * ea * (sa + ea) + 8.f * kU * aa;
+            const float z = fmaf(ab, Rz, aa * T[11]);
+            const float e_z = e_ab * n + fabsf(ab) * er + e_aa + 8.f * kU * (fabsf(ab) * n + aa);
+            if (ab < -e_ab) continue;
+            if (!(ab > e_ab && fabsf(z) > e_z)) open = true;
+            else if (z > 0.f) in |= 1u << i;
         }
+        if (open) in = cheirality64(p, load_flow(s.flows, p.flow_f16, (size_t)j), j % p.W, j / p.W, Cd);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) cnt[i] += (in >> i) & 1u;
     }
     for (int i = 0; i < 4; ++i) {
-        unsigned v = cnt[i];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd((unsigned long long*)(e.info + 4 + i), (unsigned long long)v);
+        const unsigned v = __reduce_add_sync(0xffffffffu, cnt[i]);
+        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&total[i], v);
     }
+    __syncthreads();
+    if (threadIdx.x < 4 && total[threadIdx.x])
+        atomicAdd((unsigned long long*)(e.info + 4 + threadIdx.x), (unsigned long long)total[threadIdx.x]);
 }
 
 __global__ void k_epi_finish(EpiState e, double baseline)
@@ -898,7 +978,8 @@ int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, do
 {
     int k = 0;
     cudaMemsetAsync(e.zero, 0, e.zero_bytes, st);
-    k_epi_records<<<(p.N + 255) / 256, 256, 0, st>>>(p, s, e); ++k;
+    k_epi_records<<<dim3((p.W + 31) / 32, (p.H + kEpiRecRows * kEpiRecWarps - 1) / (kEpiRecRows * kEpiRecWarps)),
+                    32 * kEpiRecWarps, 0, st>>>(p, s, e); ++k;
     k_epi_samples<<<(e.M + kEpiSampleBlock - 1) / kEpiSampleBlock, kEpiSampleBlock, 0, st>>>(p, s, e); ++k;
     k_epi_bracket<<<e.M, kEpiSubThreads, 0, st>>>(p, e); ++k;
     // persistent blocks: the number of valid samples is known on the device only
