@@ -19,12 +19,12 @@
 //     and R m0 = m0 + Q m0, the epipolar residual is
 //         t . (m0 x d + (Q m0) x m1),
 //     a sum of small terms, where m1^T E m0 would cancel O(1) products.
-//  4. k_epi_argmin: the smallest median (lowest sample on ties).
-//  5. Reweighted least squares: inliers of the winner (error <= (2.5 s)^2,
+//     The last block takes the smallest median (lowest sample on ties).
+//  4. Reweighted least squares: inliers of the winner (error <= (2.5 s)^2,
 //     s = 1.4826 (1 + 5 / (n - 8)) sqrt(median)), A^T A of their rows
 //     m1 (x) m0 in FP64 (per-block partials reduced in a fixed order), its
 //     smallest eigenvector by inverse iteration, projected again.
-//  6. The four decompositions; k_epi_cheirality counts the valid pixels whose
+//  5. The four decompositions; k_epi_cheirality counts the valid pixels whose
 //     triangulated depth is positive in both cameras; the first candidate with
 //     the largest count gives T_1, with |t| = the caller's baseline.
 #include <cmath>
@@ -579,12 +579,11 @@ __global__ void __launch_bounds__(kEpiThreads, 3) k_epi_count(DevParams p, EpiSt
 // where they do not hold it, radix passes over all pixels (11 + 11 + 10 bits).
 constexpr int kEpiMedianThreads = 1024;
 
-__global__ void __launch_bounds__(kEpiMedianThreads, 2) k_epi_median(DevParams p, EpiState e)
+__device__ __forceinline__ void epi_median(const DevParams& p, const EpiState& e, int q)
 {
     __shared__ unsigned h[kEpiBins], ws[kEpiMedianThreads / 32];
     __shared__ __align__(16) float F[12];
-    if ((int)blockIdx.x >= *e.n_list) return;
-    const int q = blockIdx.x, m = e.list[q];
+    const int m = e.list[q];
     const long long nv = e.info[2];
     if (nv == 0) {
         if (threadIdx.x == 0) e.median[m] = __int_as_float(0x7f800000);
@@ -638,15 +637,24 @@ __global__ void __launch_bounds__(kEpiMedianThreads, 2) k_epi_median(DevParams p
     if (threadIdx.x == 0) e.median[m] = __uint_as_float(bits);
 }
 
-// ---------------------------------------------------------------------------
-// 4. Winner
-// ---------------------------------------------------------------------------
-__global__ void k_epi_argmin(EpiState e)
+// The last block to finish takes the winner: the smallest median, the lowest sample
+// on ties.
+__global__ void __launch_bounds__(kEpiMedianThreads, 2) k_epi_median(DevParams p, EpiState e)
 {
+    if ((int)blockIdx.x < *e.n_list) epi_median(p, e, blockIdx.x);
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(e.median_done, 1) == (int)gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
     float best = __int_as_float(0x7f800000);
     int bi = 0x7fffffff;
     for (int m = threadIdx.x; m < e.M; m += blockDim.x) {
-        const float v = e.median[m];
+        const float v = __ldcg(e.median + m);
         if (v < best || (v == best && m < bi)) { best = v; bi = m; }
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -667,12 +675,38 @@ __global__ void k_epi_argmin(EpiState e)
 }
 
 // ---------------------------------------------------------------------------
-// 5. Reweighted least squares
+// 4. Reweighted least squares
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kEpiThreads) k_epi_refine_accum(DevParams p, DevState s, EpiState e)
+// Sums of 32 values over the warp in 31 additions a lane: lane l gets value l's.
+__device__ __forceinline__ double warp_sum32d(double (&v)[32])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        const bool up = lane & h;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+        }
+    }
+    return v[0];
+}
+
+// A^T A over the winner's inliers. Its 45 entries are 36 different sums, of a product
+// of two of (x, y, 1) with a product of two of (u, v, 1): pixel and target relative to
+// the principal point; the focal lengths are divided out of the sums. A lane stays in
+// a column and walks kEpiAccRows rows, so it adds y^k {uu, uv, u, vv, v, 1} only,
+// k = 0, 1, 2, and multiplies by x and x^2 at the end. What bounds it: FP64, two lanes
+// a clock, 24 instructions a pixel where the 45 sums with their divisions took 120:
+// 116 -> 44 us at 1242 x 375.
+constexpr int kEpiAccRows = 16, kEpiAccWarps = 4, kEpiSums = 36;
+
+__global__ void __launch_bounds__(32 * kEpiAccWarps) k_epi_refine_accum(DevParams p, DevState s, EpiState e)
 {
     __shared__ float F[12];
     __shared__ float thr;
+    __shared__ double ws[kEpiAccWarps][kEpiSums];
     const long long best = e.info[0];
     if (best < 0) return;
     if (threadIdx.x < 12) F[threadIdx.x] = e.form[best * 12 + threadIdx.x];
@@ -682,122 +716,164 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi_refine_accum(DevParams p, D
         thr = (float)((2.5 * sc) * (2.5 * sc));
     }
     __syncthreads();
-    double acc[46];
-    for (int i = 0; i < 46; ++i) acc[i] = 0.0;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < p.N; j += gridDim.x * blockDim.x) {
-        const float4 r = e.rec[j];
-        if (r.x != r.x || !(sampson32(F, r) <= thr)) continue;
-        const int x = j % p.W, y = j / p.W;
-        const float2 f = load_flow(s.flows, p.flow_f16, (size_t)j);
-        const double m0[3] = {((double)x - p.cxd) / p.fxd, ((double)y - p.cyd) / p.fyd, 1.0};
-        const double m1[3] = {((double)x + (double)f.x - p.cxd) / p.fxd, ((double)y + (double)f.y - p.cyd) / p.fyd, 1.0};
-        double a[9];
-        for (int rr = 0; rr < 3; ++rr)
-            for (int c = 0; c < 3; ++c) a[rr * 3 + c] = m1[rr] * m0[c];
-        int k = 0;
-        for (int u = 0; u < 9; ++u)
-            for (int v = u; v < 9; ++v) acc[k++] += a[u] * a[v];
-        acc[45] += 1.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tiles = (p.W + 31) / 32;
+    const int item = blockIdx.x * kEpiAccWarps + warp;
+    const int x = (item % tiles) * 32 + lane, y0 = (item / tiles) * kEpiAccRows;
+    const double xc = (double)x - p.cxd;
+    double a[3][5], sy = 0.0, syy = 0.0;
+    int count = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int i = 0; i < 5; ++i) a[k][i] = 0.0;
+    constexpr int kAhead = 4;
+    for (int k0 = 0; k0 < kEpiAccRows; k0 += kAhead) {
+        float4 r[kAhead];
+        float2 f[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            const int y = y0 + k0 + k;
+            const bool in_image = x < p.W && y < p.H;
+            r[k] = in_image ? e.rec[(size_t)y * p.W + x] : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+            f[k] = in_image ? load_flow(s.flows, p.flow_f16, (size_t)y * p.W + x) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            if (r[k].x != r[k].x || !(sampson32(F, r[k]) <= thr)) continue;
+            const double y = (double)(y0 + k0 + k) - p.cyd, yy = y * y;
+            const double u = xc + (double)f[k].x, v = y + (double)f[k].y;
+            const double q[5] = {u * u, u * v, u, v * v, v};
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                a[0][i] += q[i];
+                a[1][i] += y * q[i];
+                a[2][i] += yy * q[i];
+            }
+            sy += y;
+            syy += yy;
+            ++count;
+        }
     }
-    // block reduction in a fixed order: warps by shuffles, then warp 0 over warps
-    __shared__ double ws[kEpiThreads / 32][46];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = 0; i < 46; ++i) {
-        double v = acc[i];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) ws[warp][i] = v;
+    const double n = (double)count, xx = xc * xc;
+    double lo[32], hi[3];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const double s0 = i < 5 ? a[0][i % 5] : n, s1 = i < 5 ? a[1][i % 5] : sy, s2 = i < 5 ? a[2][i % 5] : syy;
+        lo[i] = xx * s0;
+        lo[6 + i] = xc * s1;
+        lo[12 + i] = xc * s0;
+        lo[18 + i] = s2;
+        lo[24 + i] = s1;
+        if (i < 2) lo[30 + i] = s0;
+        else if (i < 5) hi[i - 2] = s0;
     }
+    ws[warp][lane] = warp_sum32d(lo);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        for (int o = 16; o > 0; o >>= 1) hi[i] += __shfl_xor_sync(0xffffffffu, hi[i], o);
+        if (lane == 0) ws[warp][32 + i] = hi[i];
+    }
+    const unsigned total = __reduce_add_sync(0xffffffffu, (unsigned)count);
+    if (lane == 0) ws[warp][35] = (double)total;
     __syncthreads();
-    if (threadIdx.x < 46) {
+    if (threadIdx.x < kEpiSums) {
         double t = 0.0;
-        for (int w = 0; w < kEpiThreads / 32; ++w) t += ws[w][threadIdx.x];
-        e.partial[(size_t)blockIdx.x * 46 + threadIdx.x] = t;
+        for (int w = 0; w < kEpiAccWarps; ++w) t += ws[w][threadIdx.x];
+        e.partial[(size_t)blockIdx.x * kEpiSums + threadIdx.x] = t;
     }
 }
 
-// Threads 0..45 sum the partials in block order; thread 0 then takes the
-// eigenvector of the smallest eigenvalue of the 9 x 9 A^T A by inverse
-// iteration started at the winning sample's E, through the Cholesky factor of
-// A^T A + d I (d = 1e-13 trace: the shift keeps the eigenvectors and makes an
-// exactly singular A^T A, as from noiseless flows, factorable), until the
-// iterate moves by less than 1e-15 (at most 40 steps; the error shrinks by the
-// ratio of the two smallest eigenvalues per step, 0.006 on the driving
-// windows). The result is projected again; the four decompositions follow.
-__global__ void k_epi_refine_solve(EpiState e)
+// The partials are summed in a fixed order, eight threads a sum. The eigenvector of
+// the smallest eigenvalue of the 9 x 9 A^T A is taken by inverse iteration started at
+// the winning sample's E, with the inverse of A^T A + d I (d = 1e-13 trace: the shift
+// keeps the eigenvectors and makes an exactly singular A^T A, as from noiseless
+// flows, invertible) from Gauss-Jordan elimination in place, until the iterate moves
+// by less than 1e-15 (at most 40 steps; the error shrinks by the ratio of the two
+// smallest eigenvalues per step, 0.006 on the driving windows). The result is
+// projected again; the four decompositions follow. What bounds it: chains of FP64
+// instructions of ~75 cycles each, so the elimination runs on a thread per entry and
+// the iteration on a lane per row: 93 us on one thread, now 56 us (the projection is half of it).
+constexpr int kEpiSolveParts = 8;
+
+__global__ void __launch_bounds__(kEpiSums * kEpiSolveParts) k_epi_refine_solve(DevParams p, EpiState e)
 {
-    __shared__ double sum[46];
+    __shared__ double part[kEpiSolveParts][kEpiSums], sum[kEpiSums], A[9][9], scale[6], xs[9];
     const long long best = e.info[0];
     if (best < 0) return;
-    if (threadIdx.x < 46) {
+    const int tid = threadIdx.x;
+    {
+        const int i = tid % kEpiSums, c = tid / kEpiSums;
         double t = 0.0;
-        for (int b = 0; b < e.partial_blocks; ++b) t += e.partial[(size_t)b * 46 + threadIdx.x];
-        sum[threadIdx.x] = t;
+        for (int b = c; b < e.partial_blocks; b += kEpiSolveParts) t += e.partial[(size_t)b * kEpiSums + i];
+        part[c][i] = t;
+    }
+    if (tid == 0) {
+        const double ix = 1.0 / p.fxd, iy = 1.0 / p.fyd;
+        scale[0] = ix * ix; scale[1] = ix * iy; scale[2] = ix;
+        scale[3] = iy * iy; scale[4] = iy; scale[5] = 1.0;
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    e.info[3] = (long long)sum[45];
+    if (tid < kEpiSums) {
+        double t = 0.0;
+        for (int c = 0; c < kEpiSolveParts; ++c) t += part[c][tid];
+        sum[tid] = t * (scale[tid / 6] * scale[tid % 6]);
+    }
+    __syncthreads();
+    const double n = sum[kEpiSums - 1];
+    // A[(r, c)][(s, d)] = sum of m1_r m1_s m0_c m0_d
+    const int row = (tid % 81) / 9, col = tid % 9;
+    {
+        auto pair = [](int a, int b) { const int lo = min(a, b), hi = max(a, b); return lo == 0 ? hi : lo + hi + 1; };
+        if (tid < 81) A[row][col] = sum[pair(row % 3, col % 3) * 6 + pair(row / 3, col / 3)];
+    }
+    __syncthreads();
+    double tr = 0.0;
+    for (int i = 0; i < 9; ++i) tr += A[i][i];
+    bool ok = n >= 8.0 && tr > 0.0;                        // the same for all threads
+    __syncthreads();
+    if (tid < 9) A[tid][tid] += 1e-13 * tr;
+    __syncthreads();
+    for (int k = 0; k < 9 && ok; ++k) {
+        const double piv = A[k][k], a = A[row][col], ak = A[row][k], ka = A[k][col];
+        ok = piv > 0.0;
+        if (!ok) break;
+        const double inv = 1.0 / piv;
+        const double v = row == k ? (col == k ? inv : ka * inv) : (col == k ? -(ak * inv) : a - ak * (ka * inv));
+        __syncthreads();
+        if (tid < 81) A[row][col] = v;
+        __syncthreads();
+    }
+    if (tid >= 32) return;
+    if (ok) {
+        const int i = min(tid, 8);
+        double B[9], x = tid < 9 ? e.E[best * 9 + tid] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) B[k] = A[i][k];
+        for (int it = 0; it < 40; ++it) {
+            double z[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int k = 0; k < 9; ++k) z[k % 3] += B[k] * __shfl_sync(0xffffffffu, x, k);
+            const double y = tid < 9 ? (z[0] + z[1]) + z[2] : 0.0;
+            double nz = y * y;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) nz += __shfl_xor_sync(0xffffffffu, nz, o);
+            const double zi = y * (1.0 / sqrt(nz));
+            double step = (zi - x) * (zi - x);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) step += __shfl_xor_sync(0xffffffffu, step, o);
+            x = zi;
+            if (__shfl_sync(0xffffffffu, step, 0) < 1e-30) break;
+        }
+        if (tid < 9) xs[tid] = x;
+    }
+    __syncwarp();
+    if (tid != 0) return;
+    e.info[3] = (long long)n;
     double E[9], U[9], Vv[9];
-    bool ok = false;
-    if (sum[45] >= 8.0) {
-        double A[81];
-        {
-            int k = 0;
-            for (int u = 0; u < 9; ++u)
-                for (int v = u; v < 9; ++v) { A[u * 9 + v] = sum[k]; A[v * 9 + u] = sum[k]; ++k; }
-        }
-        double tr = 0.0;
-        for (int i = 0; i < 9; ++i) tr += A[i * 9 + i];
-        const double shift = 1e-13 * tr;
-        // Cholesky: A + shift I = L L^T (lower), with the reciprocals of its diagonal
-        double L[81], inv[9];
-        bool chol = tr > 0.0;
-        for (int i = 0; i < 9 && chol; ++i) {
-            for (int j = 0; j <= i; ++j) {
-                double acc = A[i * 9 + j] + (i == j ? shift : 0.0);
-                for (int k = 0; k < j; ++k) acc -= L[i * 9 + k] * L[j * 9 + k];
-                if (i == j) {
-                    if (!(acc > 0.0)) { chol = false; break; }
-                    L[i * 9 + i] = sqrt(acc);
-                    inv[i] = 1.0 / L[i * 9 + i];
-                } else {
-                    L[i * 9 + j] = acc * inv[j];
-                }
-            }
-        }
-        if (chol) {
-            double x[9];
-            for (int i = 0; i < 9; ++i) x[i] = e.E[best * 9 + i];
-            for (int it = 0; it < 40; ++it) {
-                double y[9], z[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {                  // L y = x
-                    double acc = x[i];
-#pragma unroll
-                    for (int k = 0; k < i; ++k) acc -= L[i * 9 + k] * y[k];
-                    y[i] = acc * inv[i];
-                }
-#pragma unroll
-                for (int i = 8; i >= 0; --i) {                 // L^T z = y
-                    double acc = y[i];
-#pragma unroll
-                    for (int k = i + 1; k < 9; ++k) acc -= L[k * 9 + i] * z[k];
-                    z[i] = acc * inv[i];
-                }
-                double nz = 0.0;
-#pragma unroll
-                for (int i = 0; i < 9; ++i) nz += z[i] * z[i];
-                nz = 1.0 / sqrt(nz);
-                double step = 0.0;
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    const double zi = z[i] * nz;
-                    step += (zi - x[i]) * (zi - x[i]);
-                    x[i] = zi;
-                }
-                if (step < 1e-30) break;
-            }
-            ok = essential_project(x, E, U, Vv);
-        }
+    if (ok) {
+        double x[9];
+        for (int i = 0; i < 9; ++i) x[i] = xs[i];
+        ok = essential_project(x, E, U, Vv);
     }
     if (!ok)
         for (int i = 0; i < 9; ++i) {
@@ -817,11 +893,10 @@ __global__ void k_epi_refine_solve(EpiState e)
             }
         }
     }
-    for (int i = 0; i < 4; ++i) e.info[4 + i] = 0;
 }
 
 // ---------------------------------------------------------------------------
-// 6. Cheirality and T_1
+// 5. Cheirality and T_1
 // ---------------------------------------------------------------------------
 // The pixel's count for each candidate in FP64 (the definition).
 __device__ __noinline__ unsigned cheirality64(const DevParams& p, float2 f, int x, int y, const double* Cd)
@@ -850,7 +925,8 @@ __device__ __noinline__ unsigned cheirality64(const DevParams& p, float2 f, int 
 // and m = |m0| + |d| (largest component), |t| = 1: a is known to 8 u n (1 + m), b to
 // 8 u (1 + m), Rz to 8 u n, and the rest is products; the bounds are taken twice.
 // All in FP64 this took 117 us at 1242 x 375; now 14.6 us.
-__global__ void __launch_bounds__(kEpiThreads) k_epi_cheirality(DevParams p, DevState s, EpiState e)
+// The last block to finish takes the candidate with the largest count.
+__global__ void __launch_bounds__(kEpiThreads) k_epi_cheirality(DevParams p, DevState s, EpiState e, double baseline)
 {
     __shared__ double Cd[48];
     __shared__ float Cf[48];
@@ -902,26 +978,25 @@ __global__ void __launch_bounds__(kEpiThreads) k_epi_cheirality(DevParams p, Dev
     __syncthreads();
     if (threadIdx.x < 4 && total[threadIdx.x])
         atomicAdd((unsigned long long*)(e.info + 4 + threadIdx.x), (unsigned long long)total[threadIdx.x]);
-}
-
-__global__ void k_epi_finish(EpiState e, double baseline)
-{
-    if (threadIdx.x != 0 || e.info[0] < 0) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(e.cheirality_done, 1) != (int)gridDim.x - 1) return;
+    __threadfence();
     int c = 0;
     for (int i = 1; i < 4; ++i)
-        if (e.info[4 + i] > e.info[4 + c]) c = i;
+        if (__ldcg(e.info + 4 + i) > __ldcg(e.info + 4 + c)) c = i;
     e.info[1] = c;
-    const double* T = e.cand + 12 * c;
     for (int r = 0; r < 3; ++r) {
-        for (int q = 0; q < 3; ++q) e.T1[r * 4 + q] = T[r * 4 + q];
-        e.T1[r * 4 + 3] = baseline * T[r * 4 + 3];
+        for (int q = 0; q < 3; ++q) e.T1[r * 4 + q] = Cd[12 * c + r * 4 + q];
+        e.T1[r * 4 + 3] = baseline * Cd[12 * c + r * 4 + 3];
     }
 }
 
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-static int epi_refine_blocks() { return 2 * 152; }
+constexpr int kEpiCheiralityBlocks = 2 * 152;
 
 // Collected errors a sample has room for: a sixteenth of the pixels (the bracket
 // holds a few percent), within these bounds.
@@ -929,8 +1004,9 @@ constexpr int kEpiCapMin = 4096, kEpiCapMax = 65536;
 
 // Carves the scratch for M samples out of `base` (which may be null to measure)
 // and returns the bytes it spans; every piece starts on a 256-byte boundary.
-size_t epi_layout(void* base, int M, int N, float4* rec, EpiState* e)
+size_t epi_layout(void* base, int M, int W, int H, float4* rec, EpiState* e)
 {
+    const int N = W * H;
     const uintptr_t start = reinterpret_cast<uintptr_t>(base);
     size_t off = 0;
     auto take = [&](size_t n) {
@@ -956,21 +1032,23 @@ size_t epi_layout(void* base, int M, int N, float4* rec, EpiState* e)
     e->inside = static_cast<unsigned*>(take((size_t)M * 4));
     e->n_list = static_cast<int*>(take(4));
     e->done = static_cast<int*>(take(4));
+    e->median_done = static_cast<int*>(take(4));
+    e->cheirality_done = static_cast<int*>(take(4));
     e->info = static_cast<long long*>(take(8 * 8));
     e->zero_bytes = off - z0;
     e->median = static_cast<float*>(take((size_t)M * 4));
-    e->partial_blocks = epi_refine_blocks();
-    e->partial = static_cast<double*>(take((size_t)e->partial_blocks * 46 * 8));
+    e->partial_blocks = (((W + 31) / 32) * ((H + kEpiAccRows - 1) / kEpiAccRows) + kEpiAccWarps - 1) / kEpiAccWarps;
+    e->partial = static_cast<double*>(take((size_t)e->partial_blocks * kEpiSums * 8));
     e->refined = static_cast<double*>(take(27 * 8));
     e->cand = static_cast<double*>(take(48 * 8));
     e->T1 = static_cast<double*>(take(12 * 8));
     return off;
 }
 
-size_t epi_scratch_bytes(int M, int N)
+size_t epi_scratch_bytes(int M, int W, int H)
 {
     EpiState e;
-    return epi_layout(nullptr, M, N, nullptr, &e);
+    return epi_layout(nullptr, M, W, H, nullptr, &e);
 }
 
 // Enqueues the whole estimate on st; returns the number of kernels launched.
@@ -985,11 +1063,9 @@ int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, do
     // persistent blocks: the number of valid samples is known on the device only
     k_epi_count<<<3 * 152, kEpiThreads, 0, st>>>(p, e); ++k;
     k_epi_median<<<e.M, kEpiMedianThreads, 0, st>>>(p, e); ++k;
-    k_epi_argmin<<<1, 1024, 0, st>>>(e); ++k;
-    k_epi_refine_accum<<<e.partial_blocks, kEpiThreads, 0, st>>>(p, s, e); ++k;
-    k_epi_refine_solve<<<1, 64, 0, st>>>(e); ++k;
-    k_epi_cheirality<<<epi_refine_blocks(), kEpiThreads, 0, st>>>(p, s, e); ++k;
-    k_epi_finish<<<1, 32, 0, st>>>(e, baseline); ++k;
+    k_epi_refine_accum<<<e.partial_blocks, 32 * kEpiAccWarps, 0, st>>>(p, s, e); ++k;
+    k_epi_refine_solve<<<1, kEpiSums * kEpiSolveParts, 0, st>>>(p, e); ++k;
+    k_epi_cheirality<<<kEpiCheiralityBlocks, kEpiThreads, 0, st>>>(p, s, e, baseline); ++k;
     return k;
 }
 

@@ -492,7 +492,7 @@ voldor_status voldor_bootstrap_epipolar(voldor_ctx* c, int n_samples, double bas
         if (c->epi_base && !cuda_ok(c, cudaFree(c->epi_base))) return kCuda;
         c->epi_base = nullptr;
         c->epi_cap = 0;
-        if (cudaMalloc(&c->epi_base, epi_scratch_bytes(n_samples, c->N)) != cudaSuccess) {
+        if (cudaMalloc(&c->epi_base, epi_scratch_bytes(n_samples, c->W, c->H)) != cudaSuccess) {
             cudaGetLastError();
             c->epi_base = nullptr;
             return VOLDOR_ERR_OOM;
@@ -500,7 +500,7 @@ voldor_status voldor_bootstrap_epipolar(voldor_ctx* c, int n_samples, double bas
         c->epi_cap = n_samples;
     }
     EpiState e;
-    epi_layout(c->epi_base, n_samples, c->N, c->ds.sc_cst, &e);
+    epi_layout(c->epi_base, n_samples, c->W, c->H, c->ds.sc_cst, &e);
     c->launches += launch_epipolar(c->dp, c->ds, e, baseline, c->stream);
     if (!launched(c)) return kCuda;
     c->epi_M = n_samples;
@@ -750,7 +750,7 @@ static bool buffer_of(voldor_ctx* c, int which, void** dev, size_t* bytes, bool*
         case VOLDOR_BUF_EPI_REFINED: {
             if (!c->epi_base || c->epi_M < 1) return false;
             EpiState e;
-            epi_layout(c->epi_base, c->epi_M, c->N, c->ds.sc_cst, &e);
+            epi_layout(c->epi_base, c->epi_M, c->W, c->H, c->ds.sc_cst, &e);
             const size_t M = (size_t)c->epi_M;
             if (which == VOLDOR_BUF_EPI_E) { *dev = e.E; *bytes = M * 9 * 8; }
             else if (which == VOLDOR_BUF_EPI_MEDIANS) { *dev = e.median; *bytes = M * 4; }

@@ -308,16 +308,18 @@ struct EpiState {
     unsigned* inside;         // [M] errors inside it
     int* n_list;              // [1] valid samples
     int* done;                // [1] blocks of the sample kernel done
+    int* median_done;         // [1] blocks of the median kernel done
+    int* cheirality_done;     // [1] blocks of the cheirality kernel done
     float* median;            // [M]
     long long* info;          // [8]: chosen, candidate, n_valid, n_inliers, count[4]
-    double* partial;          // [blocks][46] A^T A partials (45) + inlier count
+    double* partial;          // [partial_blocks][36] sums of the least squares
     double* refined;          // [9 E][9 U][9 V]
     double* cand;             // [4][12] [R | t]
     double* T1;               // [12]
     int partial_blocks;
 };
-size_t epi_scratch_bytes(int M, int N);
-size_t epi_layout(void* base, int M, int N, float4* rec, EpiState* e);
+size_t epi_scratch_bytes(int M, int W, int H);
+size_t epi_layout(void* base, int M, int W, int H, float4* rec, EpiState* e);
 int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, double baseline, cudaStream_t st);
 // Ground-plane scale: hist [4096] and out [3] are device scratch; returns the
 // number of kernels launched.
