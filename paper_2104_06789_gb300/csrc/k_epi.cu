@@ -4,7 +4,7 @@
 //  1. k_epi_records: per pixel, the calibrated correspondence of X_1 as
 //     {m0x, m0y, u/fx, v/fy} (FP32), m0 = K^-1 [x y 1]; NaN marks a pixel whose
 //     flow target leaves I_1 (the test and the values are those of FP64).
-//  2. k_epi_samples: one thread per minimal sample: 8 Philox-drawn pixels,
+//  2. k_epi_samples: eight lanes per minimal sample: 8 Philox-drawn pixels,
 //     the 8-point essential matrix (null vector of the 8 x 9 system by Gaussian
 //     elimination with complete pivoting, FP64), its projection onto the
 //     essential matrices (eigen-decomposition of E^T E by Jacobi rotations),
@@ -225,83 +225,114 @@ __device__ void scoring_form(const double* U, const double* V, float* f)
 // ---------------------------------------------------------------------------
 // 2. Minimal samples
 // ---------------------------------------------------------------------------
+// Eight lanes per sample, a lane per correspondence and row of the 8 x 9 system.
+// What bounds it is the chain of one sample's FP64 instructions (~75 cycles each), so
+// a step of the elimination costs a row's update and a search over the lanes instead
+// of the whole matrix: on one thread per sample, the matrix in local memory, 512
+// samples took 119 us; now 75 us, most of it the projection's Jacobi rotations.
+// Every entry sees the operations of row-by-row elimination in the same order.
+constexpr int kEpiSampleLanes = 8;
+
 __device__ void epi_sample(const DevParams& p, const DevState& s, const EpiState& e, int m)
 {
-    int ok = 1, why = 1;
-    long long j[8];
-    for (int q = 0; q < 2; ++q) {
-        const U64x4 r = philox4x64_10((uint64_t)m, (uint64_t)q, 0, (uint64_t)kStreamEpi, p.seed, p.window_id);
-        for (int i = 0; i < 4; ++i) j[4 * q + i] = (long long)__umul64hi(r.v[i], (uint64_t)p.N);
-    }
-    for (int a = 0; a < 8; ++a)
-        for (int b = a + 1; b < 8; ++b)
-            if (j[a] == j[b]) { ok = 0; why = -1; }
-    double A[8][9];
-    for (int i = 0; i < 8 && ok; ++i) {
-        const int x = (int)(j[i] % p.W), y = (int)(j[i] / p.W);
-        const float2 f = load_flow(s.flows, p.flow_f16, (size_t)j[i]);
-        const double u = (double)x + (double)f.x, v = (double)y + (double)f.y;
-        if (!(u >= 0.0 && u <= (double)(p.W - 1) && v >= 0.0 && v <= (double)(p.H - 1))) { ok = 0; why = -2; break; }
-        const double m0[3] = {((double)x - p.cxd) / p.fxd, ((double)y - p.cyd) / p.fyd, 1.0};
-        const double m1[3] = {(u - p.cxd) / p.fxd, (v - p.cyd) / p.fyd, 1.0};
-        for (int r = 0; r < 3; ++r)
-            for (int c = 0; c < 3; ++c) A[i][r * 3 + c] = m1[r] * m0[c];
-    }
-    double Ev[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    if (ok) {
-        // Gaussian elimination with complete pivoting; col[] tracks the column order
-        int col[9];
-        for (int c = 0; c < 9; ++c) col[c] = c;
-        double piv0 = 0.0;
-        for (int k = 0; k < 8 && ok; ++k) {
-            int br = k, bc = k;
-            double best = -1.0;
-            for (int r = k; r < 8; ++r)
-                for (int c = k; c < 9; ++c)
-                    if (fabs(A[r][c]) > best) { best = fabs(A[r][c]); br = r; bc = c; }
-            if (k == 0) piv0 = best;
-            if (!(best > 1e-12 * piv0) || !(best > 0.0)) { ok = 0; why = -3; break; }
-            if (br != k)
-                for (int c = 0; c < 9; ++c) { const double t = A[k][c]; A[k][c] = A[br][c]; A[br][c] = t; }
-            if (bc != k) {
-                for (int r = 0; r < 8; ++r) { const double t = A[r][k]; A[r][k] = A[r][bc]; A[r][bc] = t; }
-                const int t = col[k]; col[k] = col[bc]; col[bc] = t;
-            }
-            const double inv = 1.0 / A[k][k];
-            for (int r = k + 1; r < 8; ++r) {
-                const double f = A[r][k] * inv;
-                if (f == 0.0) continue;
-                for (int c = k; c < 9; ++c) A[r][c] -= f * A[k][c];
-            }
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, row = lane & 7;
+    const U64x4 rnd = philox4x64_10((uint64_t)m, (uint64_t)(row >> 2), 0, (uint64_t)kStreamEpi, p.seed, p.window_id);
+    uint64_t draw = rnd.v[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i)
+        if ((row & 3) == i) draw = rnd.v[i];
+    const long long j = (long long)__umul64hi(draw, (uint64_t)p.N);
+    bool dup = false;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) dup |= __shfl_xor_sync(kAll, j, i) == j;
+    const int x = (int)(j % p.W), y = (int)(j / p.W);
+    const float2 f = load_flow(s.flows, p.flow_f16, (size_t)j);
+    const double u = (double)x + (double)f.x, v = (double)y + (double)f.y;
+    const bool inside = u >= 0.0 && u <= (double)(p.W - 1) && v >= 0.0 && v <= (double)(p.H - 1);
+    const unsigned group = 0xffu << (lane & 24);
+    const unsigned dups = __ballot_sync(kAll, dup), insides = __ballot_sync(kAll, inside);
+    int why = dups & group ? -1 : (~insides & group ? -2 : 1);
+    // (lanes of a sample agree on `why`; the warp's samples run the same code, a
+    // rejected one on values that go nowhere)
+    const double m0[3] = {((double)x - p.cxd) / p.fxd, ((double)y - p.cyd) / p.fyd, 1.0};
+    const double m1[3] = {(u - p.cxd) / p.fxd, (v - p.cyd) / p.fyd, 1.0};
+    double A[9];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) A[r * 3 + c] = m1[r] * m0[c];
+
+    // Gaussian elimination with complete pivoting. Rows stay in their lanes: `pos` is
+    // the row's place, `holder` and `col` (four bits each) the lane of each place
+    // that is done and the order of the columns.
+    int pos = row;
+    unsigned holder = 0;
+    unsigned long long col = 0x876543210ull;
+    double piv0 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        double best = pos >= k ? -1.0 : -2.0;
+        int bc = k, at = pos, from = row;
+        if (pos >= k) {
+#pragma unroll
+            for (int c = k; c < 9; ++c)
+                if (fabs(A[c]) > best) { best = fabs(A[c]); bc = c; }
         }
-        if (ok) {
-            double z[9];
-            z[8] = 1.0;
-            for (int k = 7; k >= 0; --k) {
-                double acc = 0.0;
-                for (int c = k + 1; c < 9; ++c) acc += A[k][c] * z[c];
-                z[k] = -acc / A[k][k];
-            }
-            double nn = 0.0;
-            for (int c = 0; c < 9; ++c) nn += z[c] * z[c];
-            nn = 1.0 / sqrt(nn);
-            for (int c = 0; c < 9; ++c) Ev[col[c]] = z[c] * nn;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            const double ob = __shfl_xor_sync(kAll, best, o);
+            const int packed = __shfl_xor_sync(kAll, bc | at << 8 | from << 16, o), oat = packed >> 8 & 255;
+            if (ob > best || (ob == best && oat < at)) { best = ob; bc = packed & 255; at = oat; from = packed >> 16; }
+        }
+        if (k == 0) piv0 = best;
+        if (why == 1 && (!(best > 1e-12 * piv0) || !(best > 0.0))) why = -3;
+        if (pos == k) pos = at;                       // rows k and `at` change places
+        if (row == from) pos = k;
+        holder |= (unsigned)from << (4 * k);
+#pragma unroll
+        for (int c = k + 1; c < 9; ++c)
+            if (c == bc) { const double t = A[k]; A[k] = A[c]; A[c] = t; }
+        const unsigned long long d = (col >> 4 * k ^ col >> 4 * bc) & 15;
+        col ^= d << 4 * k;
+        col ^= d << 4 * bc;
+        const double inv = 1.0 / __shfl_sync(kAll, A[k], from, 8);
+        const double fr = pos > k ? A[k] * inv : 0.0;
+#pragma unroll
+        for (int c = k + 1; c < 9; ++c) {
+            const double pc = __shfl_sync(kAll, A[c], from, 8);
+            if (fr != 0.0) A[c] = fma(-fr, pc, A[c]);
         }
     }
-    double E[9], U[9], V[9];
-    if (ok && !essential_project(Ev, E, U, V)) { ok = 0; why = -4; }
+    double z[9];
+    z[8] = 1.0;
+#pragma unroll
+    for (int k = 7; k >= 0; --k) {
+        double acc = 0.0;
+#pragma unroll
+        for (int c = k + 1; c < 9; ++c) acc = fma(A[c], z[c], acc);
+        z[k] = __shfl_sync(kAll, -acc / A[k], (int)(holder >> (4 * k)) & 7, 8);
+    }
+    if (row != 0 || m >= e.M) return;
+    double Ev[9], E[9], U[9], V[9];
+    double nn = 0.0;
+    for (int c = 0; c < 9; ++c) nn += z[c] * z[c];
+    nn = 1.0 / sqrt(nn);
+    for (int c = 0; c < 9; ++c) Ev[(int)(col >> 4 * c) & 15] = z[c] * nn;
+    if (why == 1 && !essential_project(Ev, E, U, V)) why = -4;
     e.valid[m] = why;
-    float* f = e.form + (size_t)m * 12;
-    if (ok) {
+    float* form = e.form + (size_t)m * 12;
+    if (why == 1) {
         for (int i = 0; i < 9; ++i) {
             e.E[(size_t)m * 9 + i] = E[i];
             e.UV[(size_t)m * 18 + i] = U[i];
             e.UV[(size_t)m * 18 + 9 + i] = V[i];
         }
-        scoring_form(U, V, f);
+        scoring_form(U, V, form);
     } else {
         for (int i = 0; i < 9; ++i) e.E[(size_t)m * 9 + i] = 0.0;
-        for (int i = 0; i < 12; ++i) f[i] = 0.f;
+        for (int i = 0; i < 12; ++i) form[i] = 0.f;
+        e.median[m] = __int_as_float(0x7f800000);
     }
 }
 
@@ -310,11 +341,8 @@ __device__ void epi_sample(const DevParams& p, const DevState& s, const EpiState
 // pixel whose target leaves the image).
 __global__ void __launch_bounds__(kEpiSampleBlock) k_epi_samples(DevParams p, DevState s, EpiState e)
 {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < e.M) {
-        epi_sample(p, s, e, m);
-        if (e.valid[m] <= 0) e.median[m] = __int_as_float(0x7f800000);
-    }
+    const int m = (blockIdx.x * blockDim.x + threadIdx.x) / kEpiSampleLanes;
+    if ((m & ~3) < e.M) epi_sample(p, s, e, m);        // whole warps; samples past M are not written
     __threadfence();
     __shared__ bool last;
     __shared__ int wsum[kEpiSampleBlock / 32];
@@ -1058,7 +1086,7 @@ int launch_epipolar(const DevParams& p, const DevState& s, const EpiState& e, do
     cudaMemsetAsync(e.zero, 0, e.zero_bytes, st);
     k_epi_records<<<dim3((p.W + 31) / 32, (p.H + kEpiRecRows * kEpiRecWarps - 1) / (kEpiRecRows * kEpiRecWarps)),
                     32 * kEpiRecWarps, 0, st>>>(p, s, e); ++k;
-    k_epi_samples<<<(e.M + kEpiSampleBlock - 1) / kEpiSampleBlock, kEpiSampleBlock, 0, st>>>(p, s, e); ++k;
+    k_epi_samples<<<(e.M * kEpiSampleLanes + kEpiSampleBlock - 1) / kEpiSampleBlock, kEpiSampleBlock, 0, st>>>(p, s, e); ++k;
     k_epi_bracket<<<e.M, kEpiSubThreads, 0, st>>>(p, e); ++k;
     // persistent blocks: the number of valid samples is known on the device only
     k_epi_count<<<3 * 152, kEpiThreads, 0, st>>>(p, e); ++k;
