@@ -3,9 +3,8 @@
 // flow stack of a window and predicts, per pixel of I_0, a log-depth and a
 // rigidness logit used in place of the triangulation bootstrap. BF16
 // activations and weights, FP32 accumulation: the convolutions of the forward
-// pass and of the input gradient on tcgen05 (TMEM accumulators, TMA row
-// loads), the weight gradient on tcgen05 too (operands transposed into
-// shared memory with ldmatrix / stmatrix); FP32 Adam on master weights.
+// pass, of the input gradient and of the weight gradient on tcgen05 (TMEM
+// accumulators, TMA row loads); FP32 Adam on master weights.
 //
 // Input: the flows of each frame divided by that frame's mean flow magnitude
 // (the network sees the shape of the flow field, not its overall size).
@@ -41,12 +40,6 @@ constexpr int kNetLayers = 6;
 constexpr int kNetWidth = 32;
 constexpr int kAlignBins = 2048;                // histogram bins per level of the median search
 constexpr float kAlignRange = 16.f;             // first level covers log-ratios in [-16, 16)
-
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
-}
 
 // ---------------------------------------------------------------------------
 // 3x3 convolution on the fifth-generation tensor cores (implicit GEMM):
@@ -130,6 +123,30 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, volatile 
     }
     *bad = 1;
     return false;
+}
+
+// The same for a converged warp, with one answer for all its lanes.
+__device__ __forceinline__ bool tc_wait_warp(uint32_t bar, uint32_t parity, volatile int* bad)
+{
+    for (long long i = 0; i < kTcWaitLimit; ++i) {
+        if (__all_sync(0xffffffffu, tc_try_wait(bar, parity))) return true;
+        if ((i & 1023) == 1023 && __any_sync(0xffffffffu, *bad)) return false;
+    }
+    *bad = 1;
+    return false;
+}
+
+__device__ __forceinline__ void tc_tma_row_elect(uint32_t dst, const CUtensorMap* map, int c, int x, int y, int b, uint32_t bar)
+{
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
+                 " @q cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n}"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void tc_expect_tx_elect(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
+                 " @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 __device__ __forceinline__ void tc_tma_row(uint32_t dst, const CUtensorMap* map, int c, int x, int y, int b, uint32_t bar)
@@ -394,7 +411,9 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode_tiled = nullptr;
 static std::once_flag g_encode_once;
 
-static bool tensor_map_rows(CUtensorMap* m, const bf16* base, int C, int W, int H, int B)
+// NHWC activations with C channels as boxes of box_c channels x box_cols columns of a row.
+static bool tensor_map_rows(CUtensorMap* m, const bf16* base, int C, int W, int H, int B, int box_c, int box_cols,
+                            CUtensorMapSwizzle swizzle)
 {
     std::call_once(g_encode_once, [] {
         void* fn = nullptr;
@@ -406,10 +425,10 @@ static bool tensor_map_rows(CUtensorMap* m, const bf16* base, int C, int W, int 
     if (!g_encode_tiled) return false;
     const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
     const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-    const cuuint32_t box[4] = {8, (cuuint32_t)kTcCols, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)box_c, (cuuint32_t)box_cols, 1, 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     return g_encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(base), dims, strides, box, es,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -442,7 +461,7 @@ static bool launch_conv_tc(const ConvArgs& a, cudaStream_t st)
         sms = g_tc_sms[dev];
     }
     CUtensorMap m;
-    if (!tensor_map_rows(&m, a.in, CIN, a.W, a.H, a.B)) return false;
+    if (!tensor_map_rows(&m, a.in, CIN, a.W, a.H, a.B, 8, kTcCols, CU_TENSOR_MAP_SWIZZLE_NONE)) return false;
     const int items = a.B * ((a.H + kTcRows - 1) / kTcRows) * ((a.W + kTcM - 1) / kTcM);
     const int grid = std::min(items, kTcCtasPerSm * sms);
     k_conv_tc<CIN, N><<<grid, kTcThreads, S::kSmemBytes, st>>>(m, a);
@@ -458,7 +477,6 @@ struct WgradArgs {
     float* dw;              // [n_out][9][cin_real]
     float* db;              // [n_out]
     float* part;            // [gridDim.x][9 CIN + 1][NCO] each CTA's sums
-    float* part2;           // [ceil(gridDim.x / kWgGroup)][9 CIN + 1][NCO] their group sums
     int n_out, cin_real;
     int H, W, B;
     int* err;               // set to 1 if a bounded wait expired
@@ -467,83 +485,113 @@ struct WgradArgs {
 // ---------------------------------------------------------------------------
 // Weight gradient on the fifth-generation tensor cores:
 // dw[co][tap][ci] += sum_p dout[p][co] in[p + off(tap)][ci] and
-// db[co] += sum_p dout[p][co], as one GEMM per layer: D[m][n] =
-// sum_k A[m][k] B[n][k] with
-// m = tap * CIN + ci (the 9 CIN rows of the layer's input, shifted by the
-// tap), n = output channel, k = pixel; one extra row of ones (m = 9 CIN)
-// gives the bias gradient sum_p dout[p][n]. Rows are cut into 128-row M tiles
-// (tcgen05.mma M = 128, N = NCO, K = 16, BF16 in, FP32 accumulators in TMEM
-// that persist over all of a CTA's work items).
+// db[co] += sum_p dout[p][co], as one GEMM per layer with the pixels as K:
+// D[m][n] = sum_k A[m][k] B[n][k], k = input pixel (x, y of a row segment),
+// m = (kx, co): dout at column x + 1 - kx, n = (ky, ci): the input row y - 1 + ky
+// for dout's row y.
 //
-// A work item is KP = 64 consecutive output pixels of one image row. Its
-// three input rows (66 pixels each, zero outside the image) and its output
-// gradients are staged pixel-major in shared memory, then transposed 8 x 8 at
-// a time (ldmatrix .trans, then stmatrix) into the K-major, unswizzled
-// core-matrix layout of the two operands: element (m, k) of an M tile at
-// (k / 8) * 2048 + (m / 8) * 128 + (m % 8) * 16 + (k % 8) * 2 bytes, and
-// (n, k) of B at (k / 8) * (NCO / 8) * 128 + (n / 8) * 128 + (n % 8) * 16 +
-// (k % 8) * 2. One thread issues the item's MMAs and commits them to an
-// mbarrier; the next item's pixel-major staging overlaps them, and every
-// thread waits on the commit (bounded) before overwriting the operands. At
-// the end each thread reads its TMEM row (tcgen05.ld) and adds it to the
-// FP32 gradients with atomics.
+// The activations are channel-last, so both operands have their M / N index
+// contiguous: the MN-major swizzled layouts (64 bytes a pixel for 32 channels, 32
+// for 16) are what TMA writes, and no thread touches an operand. A CTA walks down
+// the rows of 64-column strips:
+//   warp 4, one lane: TMA loads of a ring of input rows and a ring of dout rows, a
+//     dout row three times (columns x0 + 1, x0, x0 - 1: kx = 0, 1, 2; zero fill
+//     outside the image). M groups of NCO channels are a dout copy apart, N groups
+//     of CIN channels an input row of the ring.
+//   warp 5, one lane: per row four tcgen05.mma (M = 128, of which 3 NCO rows count;
+//     N = 3 CIN, K = 16 pixels), in two parts where the three rows wrap around the
+//     ring. Even and odd rows accumulate in two sets of TMEM columns (shorter sums).
+//   warps 0-3: the bias sums from the dout rows in shared memory, FP32; at the end
+//     each reads its TMEM lanes and writes the CTA's partial.
+// The rows of all strips are dealt to the CTAs in contiguous runs of equal length.
+// Every mbarrier wait is bounded as in k_conv_tc.
+//
+// What bounds it: HBM in the long run (22 us per 119 MB of operands at 1242 x 375 x 2;
+// the MMAs read 7 KB of shared memory per 16 pixels, 15 us), and here the start and
+// the partials, ~6 us. The kernel before, which transposed 64-pixel tiles through
+// ldmatrix / stmatrix into K-major operands (nine shifted copies of the input per
+// tile), took 177 us for 32 x 32 channels; this one 28.8 us. 42 us of it were left
+// while one lane of a diverged warp issued the MMAs and loads (see tc.cuh); threads
+// that load the rows through registers and store the copies instead of TMA took 48.
+// One CTA per SM with rings twice as deep is slower (53 against 46 us with the
+// reduction): a row's round trip between the roles takes ~800 cycles.
 // ---------------------------------------------------------------------------
-constexpr int kWgKP = 64;                                 // pixels per work item (K)
-constexpr int kWgThreads = 128;
-constexpr int kWgCtasPerSm = 3;                          // weight-gradient grid: at most this many CTAs per SM
+constexpr int kWgKP = 64;                                 // pixels per row segment (K)
+constexpr int kWgThreads = 192;
+constexpr int kWgCtasPerSm = 2;                           // weight-gradient grid: at most this many CTAs per SM
+constexpr int kWgInSlots = 8, kWgDoSlots = 4;             // ring slots
 constexpr int kWgPartRows = 9 * 32 + 1;                   // largest per-CTA partial: rows x 32 columns
 
 template <int CIN, int NCO>
 struct WgShape {
-    static constexpr int kRows = 9 * CIN + 1;                           // + the ones row
-    static constexpr int kMT = (kRows + 127) / 128;
-    static constexpr int kInRowBytes = (kWgKP + 2) * CIN * 2;
-    static constexpr int kInBytes = 3 * kInRowBytes;
-    static constexpr int kDoBytes = kWgKP * NCO * 2;
-    static constexpr int kATileBytes = (kWgKP / 8) * 2048;
-    static constexpr int kBLbo = (NCO / 8) * 128;
-    static constexpr int kBBytes = (kWgKP / 8) * kBLbo;
-    static constexpr int kInOff = 0;
-    static constexpr int kDoOff = kInOff + kInBytes;
-    static constexpr int kAOff = (kDoOff + kDoBytes + 1023) / 1024 * 1024;
-    static constexpr int kBOff = kAOff + kMT * kATileBytes;
-    static constexpr int kBarOff = kBOff + kBBytes;
-    static constexpr int kSmemBytes = kBarOff + 32;
-    static constexpr int kTmemCols = kMT * NCO <= 32 ? 32 : (kMT * NCO <= 64 ? 64 : 128);
-    static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NCO >> 3) << 17) |
-                                       ((uint32_t)(128 >> 4) << 24);
+    static constexpr int kRows = 9 * CIN + 1;                           // a partial's rows: (tap, ci), then the bias
+    static constexpr int kInSlot = kWgKP * CIN * 2;
+    static constexpr int kDoCopy = kWgKP * NCO * 2;                     // a dout row at one shift
+    static constexpr int kDoSlot = 3 * kDoCopy;
+    // dout ring | input ring | barriers. The M = 128 operand reads on past a dout slot's
+    // three copies, at most into the input ring.
+    static constexpr int kInOff = kWgDoSlots * kDoSlot;
+    static constexpr int kBarOff = kInOff + kWgInSlots * kInSlot;
+    static constexpr int kBars = 2 * kWgInSlots + 2 * kWgDoSlots + 1;
+    // then the TMEM address, the abort flag and the warps' bias sums
+    static constexpr int kSmemBytes = kBarOff + kBars * 8 + 8 + 4 * NCO * 4;
+    static constexpr int kSetCols = 3 * CIN;
+    static constexpr int kTmemCols = 2 * kSetCols <= 128 ? 128 : 256;
+    static_assert(128 / NCO * kDoCopy - kDoSlot <= kWgInSlots * kInSlot, "operand reads stay in the rings");
 };
 
-__device__ __forceinline__ void stsm_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3)
+// Descriptor of an MN-major operand of C channels per pixel (C = 32: 64-byte swizzle,
+// 16: 32-byte): groups of C channels `group` bytes apart, 8 pixels = 16 C bytes.
+template <int C>
+__device__ __forceinline__ uint64_t tc_desc_mn(uint32_t addr, uint32_t group)
 {
-    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1),
-                 "r"(r2), "r"(r3) : "memory");
+    return tc_desc(addr, group, 16 * C) | ((uint64_t)(C == 32 ? 4 : 6) << 61);
+}
+
+__host__ __device__ constexpr uint32_t tc_idesc_mn(int n) { return tc_idesc(n) | (1u << 15) | (1u << 16); }
+
+// Run segment: rows y0 .. y0 + rows - 1 of the 64 columns from x0 of image b.
+struct WgSegment {
+    int b, x0, y0, rows;
+};
+
+__device__ __forceinline__ WgSegment wg_segment(int i, int end, int H, int strips)
+{
+    WgSegment t;
+    const int strip = i / H;
+    t.y0 = i - strip * H;
+    t.rows = min(H - t.y0, end - i);
+    t.b = strip / strips;
+    t.x0 = (strip % strips) * kWgKP;
+    return t;
 }
 
 template <int CIN, int NCO>
-__global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __grid_constant__ WgradArgs a)
+__global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
+    k_wgrad_tc(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tdo, const WgradArgs a)
 {
     using S = WgShape<CIN, NCO>;
     extern __shared__ __align__(1024) unsigned char smem[];
     const uint32_t sbase = smem_addr(smem);
-    const uint32_t in_s = sbase + S::kInOff, do_s = sbase + S::kDoOff, A_s = sbase + S::kAOff, B_s = sbase + S::kBOff;
-    const uint32_t bar = sbase + S::kBarOff, done = bar + 8;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + S::kBarOff + 16);
-    volatile int& bad = *reinterpret_cast<volatile int*>(smem + S::kBarOff + 20);
+    const uint32_t in_s = sbase + S::kInOff;
+    const uint32_t in_full = sbase + S::kBarOff, in_empty = in_full + 8 * kWgInSlots, do_full = in_empty + 8 * kWgInSlots,
+                   do_empty = do_full + 8 * kWgDoSlots, done = do_empty + 8 * kWgDoSlots;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + S::kBarOff + S::kBars * 8);
+    volatile int& bad = *reinterpret_cast<volatile int*>(smem + S::kBarOff + S::kBars * 8 + 4);
+    float(*bias_s)[NCO] = reinterpret_cast<float(*)[NCO]>(smem + S::kBarOff + S::kBars * 8 + 8);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int segs = (a.W + kWgKP - 1) / kWgKP;
-    const int n_items = a.B * a.H * segs;
+    const int strips = (a.W + kWgKP - 1) / kWgKP, total = a.B * strips * a.H;
+    const int r0 = (int)((long long)total * blockIdx.x / gridDim.x), r1 = (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
 
-    // constant rows of A in every M tile: the ones row (bias gradient) and zero padding
-    for (int i = tid; i < S::kMT * 128 * kWgKP; i += blockDim.x) {
-        const int m = i / kWgKP, k = i % kWgKP;
-        if (m < 9 * CIN) continue;
-        const int mt = m / 128, mm = m % 128;
-        const uint32_t off = S::kAOff + mt * S::kATileBytes + (k / 8) * 2048 + (mm / 8) * 128 + (mm % 8) * 16 + (k % 8) * 2;
-        *reinterpret_cast<bf16*>(smem + off) = __float2bfloat16_rn(m == 9 * CIN ? 1.f : 0.f);
-    }
     if (tid == 0) {
-        tc_mbar_init(bar, 1);
+        for (int i = 0; i < kWgInSlots; ++i) {
+            tc_mbar_init(in_full + 8 * i, 1);
+            tc_mbar_init(in_empty + 8 * i, 1);
+        }
+        for (int i = 0; i < kWgDoSlots; ++i) {
+            tc_mbar_init(do_full + 8 * i, 1);
+            tc_mbar_init(do_empty + 8 * i, 1 + 4);
+        }
         tc_mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         bad = 0;
@@ -553,185 +601,161 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __grid_constant__
                      "r"((uint32_t)S::kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    float bias[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
-    // an item's input rows and output gradients, loaded into registers one
-    // item ahead (the loads of item i + 1 are in flight while item i is
-    // transposed and multiplied) and stored pixel-major at the top of the loop
-    constexpr int kInVec = 3 * (kWgKP + 2) * (CIN / 8), kDoVec = kWgKP * (NCO / 8);
-    constexpr int kInPer = (kInVec + kWgThreads - 1) / kWgThreads, kDoPer = (kDoVec + kWgThreads - 1) / kWgThreads;
-    uint4 pin[kInPer], pdo[kDoPer];
-    auto fetch = [&](int it) {
-        const int b = it / (a.H * segs), rem = it % (a.H * segs);
-        const int y = rem / segs, x0 = (rem % segs) * kWgKP;
+    if (warp == 4) {
+        uint32_t li = 0, ld = 0;                           // input and dout rows loaded
+        bool go = true;
+        for (int i = r0; i < r1 && go;) {
+            const WgSegment t = wg_segment(i, r1, a.H, strips);
+            for (int r = t.y0 - 1; r <= t.y0 + t.rows; ++r) {
+                const uint32_t si = li % kWgInSlots, sd = ld % kWgDoSlots;
+                if (li >= kWgInSlots) go = tc_wait_warp(in_empty + 8 * si, ((li / kWgInSlots) - 1) & 1, &bad);
+                if (!go) break;
+                tc_expect_tx_elect(in_full + 8 * si, (uint32_t)S::kInSlot);
+                tc_tma_row_elect(in_s + si * S::kInSlot, &tin, 0, t.x0, r, t.b, in_full + 8 * si);
+                ++li;
+                if (r <= t.y0) continue;
+                if (ld >= kWgDoSlots) go = tc_wait_warp(do_empty + 8 * sd, ((ld / kWgDoSlots) - 1) & 1, &bad);
+                if (!go) break;
+                tc_expect_tx_elect(do_full + 8 * sd, (uint32_t)S::kDoSlot);
 #pragma unroll
-        for (int j = 0; j < kInPer; ++j) {
-            const int i = tid + j * kWgThreads;
-            pin[j] = make_uint4(0, 0, 0, 0);
-            if (i < kInVec) {
-                const int v = i % (CIN / 8), q = i / (CIN / 8);
-                const int ky = q / (kWgKP + 2), xx = q % (kWgKP + 2);
-                const int gy = y + ky - 1, gx = x0 + xx - 1;
-                if (gy >= 0 && gy < a.H && gx >= 0 && gx < a.W)
-                    pin[j] = *reinterpret_cast<const uint4*>(a.in + (((size_t)b * a.H + gy) * a.W + gx) * a.cin_g + v * 8);
+                for (int kx = 0; kx < 3; ++kx)
+                    tc_tma_row_elect(sbase + sd * S::kDoSlot + kx * S::kDoCopy, &tdo, 0, t.x0 + 1 - kx, r - 1, t.b, do_full + 8 * sd);
+                ++ld;
             }
+            i += t.rows;
         }
+        // the last loads may still be landing when another role gave up
+        for (uint32_t j = li > kWgInSlots ? li - kWgInSlots : 0; j < li; ++j)
+            for (long long k = 0; k < kTcWaitLimit; ++k)
+                if (tc_try_wait(in_full + 8 * (j % kWgInSlots), (j / kWgInSlots) & 1)) break;
+        for (uint32_t j = ld > kWgDoSlots ? ld - kWgDoSlots : 0; j < ld; ++j)
+            for (long long k = 0; k < kTcWaitLimit; ++k)
+                if (tc_try_wait(do_full + 8 * (j % kWgDoSlots), (j / kWgDoSlots) & 1)) break;
+    } else if (warp == 5) {
+        uint32_t gi = 0, gd = 0, seen = 0;             // input row y - 1, dout row y, input rows waited for
+        bool go = true;
+        for (int i = r0; i < r1 && go;) {
+            const WgSegment t = wg_segment(i, r1, a.H, strips);
+            for (int k = 0; k < t.rows; ++k, ++gi, ++gd) {
+                for (; go && seen < gi + 3; ++seen)
+                    go = tc_wait_warp(in_full + 8 * (seen % kWgInSlots), (seen / kWgInSlots) & 1, &bad);
+                const uint32_t sd = gd % kWgDoSlots, si = gi % kWgInSlots;
+                go = go && tc_wait_warp(do_full + 8 * sd, (gd / kWgDoSlots) & 1, &bad);
+                if (!go) break;
+                tc_fence_after();
+                const int nb = min(3, kWgInSlots - (int)si);             // rows before the ring wraps
+                const uint32_t d = tmem + (gd & 1) * S::kSetCols, i1 = tc_idesc_mn(nb * CIN), i2 = tc_idesc_mn((3 - nb) * CIN);
 #pragma unroll
-        for (int j = 0; j < kDoPer; ++j) {
-            const int i = tid + j * kWgThreads;
-            pdo[j] = make_uint4(0, 0, 0, 0);
-            if (i < kDoVec) {
-                const int v = i % (NCO / 8), px = i / (NCO / 8), gx = x0 + px;
-                if (gx < a.W && v * 8 < a.n_out) {
-                    pdo[j] = *reinterpret_cast<const uint4*>(a.dout + (((size_t)b * a.H + y) * a.W + gx) * a.cout_g + v * 8);
-                    if (v * 8 + 8 > a.n_out) {                // channels past n_out are zero
-                        bf16* e = reinterpret_cast<bf16*>(&pdo[j]);
-                        for (int c = a.n_out - v * 8; c < 8; ++c) e[c] = __float2bfloat16_rn(0.f);
-                    }
+                for (int ks = 0; ks < kWgKP / 16; ++ks) {
+                    const uint64_t ad = tc_desc_mn<NCO>(sbase + sd * S::kDoSlot + ks * 32 * NCO, S::kDoCopy);
+                    const uint32_t acc = gd >= 2 || ks > 0;
+                    tc_mma_elect(d, ad, tc_desc_mn<CIN>(in_s + si * S::kInSlot + ks * 32 * CIN, S::kInSlot), i1, acc);
+                    if (nb < 3) tc_mma_elect(d + nb * CIN, ad, tc_desc_mn<CIN>(in_s + ks * 32 * CIN, S::kInSlot), i2, acc);
                 }
+                tc_commit_elect(do_empty + 8 * sd);
+                tc_commit_elect(in_empty + 8 * si);
             }
+            if (!go) break;
+            tc_commit_elect(in_empty + 8 * (gi % kWgInSlots));                 // the segment's last two rows
+            tc_commit_elect(in_empty + 8 * ((gi + 1) % kWgInSlots));
+            gi += 2;
+            i += t.rows;
         }
-    };
-    if (blockIdx.x < n_items) fetch(blockIdx.x);
-    int local = 0;                                            // items of this CTA so far
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x, ++local) {
-        // pixel-major staging of this item (the operands of the previous item
-        // may still be read by its MMAs; these buffers are not)
-#pragma unroll
-        for (int j = 0; j < kInPer; ++j) {
-            const int i = tid + j * kWgThreads;
-            if (i < kInVec) {
-                const int v = i % (CIN / 8), q = i / (CIN / 8);
-                const int ky = q / (kWgKP + 2), xx = q % (kWgKP + 2);
-                *reinterpret_cast<uint4*>(smem + S::kInOff + ky * S::kInRowBytes + xx * CIN * 2 + v * 16) = pin[j];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < kDoPer; ++j) {
-            const int i = tid + j * kWgThreads;
-            if (i < kDoVec) {
-                const int v = i % (NCO / 8), px = i / (NCO / 8);
-                *reinterpret_cast<uint4*>(smem + S::kDoOff + px * NCO * 2 + v * 16) = pdo[j];
-            }
-        }
-        if (it + (int)gridDim.x < n_items) fetch(it + gridDim.x);
-        // the previous item's MMAs have read A and B; a wait that expires sets
-        // `bad`, which every thread reads after the same barrier
-        if (local > 0) tc_wait(bar, (uint32_t)((local - 1) & 1), &bad);
-        __syncthreads();
-        if (bad) break;
-        // 8 x 8 transposes into the K-major operands: A blocks (tap, ci group, k group), then B blocks
-        constexpr int kABlocks = 9 * (CIN / 8) * (kWgKP / 8), kBBlocks = (NCO / 8) * (kWgKP / 8);
-        static_assert((kABlocks + kBBlocks) % 16 == 0, "four x4 transposes per round, one per warp");
-        for (int q0 = warp * 4; q0 < kABlocks + kBBlocks; q0 += 16) {
-            const int blk = q0 + (lane >> 3), r = lane & 7;
-            uint32_t src, dst;
-            if (blk < kABlocks) {
-                const int kg = blk % (kWgKP / 8), g = (blk / (kWgKP / 8)) % (CIN / 8), tap = blk / ((kWgKP / 8) * (CIN / 8));
-                const int ky = tap / 3, kx = tap % 3;
-                const int m = tap * CIN + g * 8 + r, mt = m / 128, mm = m % 128;
-                src = in_s + ky * S::kInRowBytes + (8 * kg + r + kx) * CIN * 2 + g * 16;
-                dst = A_s + mt * S::kATileBytes + kg * 2048 + (mm / 8) * 128 + r * 16;
-            } else {
-                const int bb = blk - kABlocks, kg = bb % (kWgKP / 8), g = bb / (kWgKP / 8);
-                src = do_s + (8 * kg + r) * NCO * 2 + g * 16;
-                dst = B_s + kg * S::kBLbo + g * 128 + r * 16;
-            }
-            // lane l gives row l % 8 of block l / 8: the transposing load, then the
-            // plain store, writes each block's transpose to the destination rows
-            uint32_t r0, r1, r2, r3;
-            ldsm_x4_t(src, r0, r1, r2, r3);
-            stsm_x4(dst, r0, r1, r2, r3);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-            for (int mt = 0; mt < S::kMT; ++mt)
-#pragma unroll
-                for (int s16 = 0; s16 < kWgKP / 16; ++s16) {
-                    const uint64_t ad = tc_desc(A_s + mt * S::kATileBytes + s16 * 2 * 2048, 2048, 128);
-                    const uint64_t bd = tc_desc(B_s + s16 * 2 * S::kBLbo, S::kBLbo, 128);
-                    tc_mma(tmem + mt * NCO, ad, bd, S::kIdesc, (local > 0 || s16 > 0) ? 1u : 0u);
-                }
-            tc_commit(bar);
-        }
-    }
-    if (tid == 0) {
-        tc_commit(done);                                      // arrives once every MMA issued has completed
+        tc_commit_elect(done);                          // arrives once every MMA issued has completed
         bool drained = false;
         for (long long i = 0; i < kTcWaitLimit && !drained; ++i) drained = tc_try_wait(done, 0);
         if (!drained) bad = 1;
-    }
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!bad) {
-        // this CTA's sums, row m (tap * CIN + ci, then the bias row) of its partial
+    } else {
+        // thread: 16-byte chunk c (channels 8 c ..) of pixels tid / kC, ...; chunks are permuted by the swizzle
+        constexpr int kC = NCO / 8, kStep = 128 / kC;
+        const int c = tid % kC, px = tid / kC;
+        for (int g = 0; g < r1 - r0; ++g) {
+            const uint32_t sd = g % kWgDoSlots;
+            if (!__all_sync(0xffffffffu, tc_wait(do_full + 8 * sd, (g / kWgDoSlots) & 1, &bad))) break;
 #pragma unroll
-        for (int mt = 0; mt < S::kMT; ++mt) {
-            float v[NCO];
-            tc_ld<NCO>(tmem + ((uint32_t)(warp * 32) << 16) + mt * NCO, v);
-            if (local == 0) {
+            for (int x = 0; x < kWgKP; x += kStep) {
+                const int p = x + px, at = NCO == 32 ? (c ^ ((p >> 1) & 3)) : (c ^ ((p >> 2) & 1));
+                const uint4 v = *reinterpret_cast<const uint4*>(smem + sd * S::kDoSlot + S::kDoCopy + p * NCO * 2 + at * 16);
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                for (int co = 0; co < NCO; ++co) v[co] = 0.f;
+                for (int q = 0; q < 4; ++q) {
+                    bias[2 * q] += __uint_as_float(w[q] << 16);
+                    bias[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
+                }
             }
-            const int m = mt * 128 + warp * 32 + lane;
-            if (m < S::kRows) {
-                float4* o = reinterpret_cast<float4*>(a.part + ((size_t)blockIdx.x * S::kRows + m) * NCO);
+            __syncwarp();
+            if (lane == 0) tc_arrive(do_empty + 8 * sd);
+        }
 #pragma unroll
-                for (int q = 0; q < NCO / 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            }
+        for (int q = 0; q < 8; ++q) {
+            for (int o = kC; o < 32; o <<= 1) bias[q] += __shfl_xor_sync(0xffffffffu, bias[q], o);
+            if (lane < kC) bias_s[warp][8 * lane + q] = bias[q];
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    tc_fence_after();
+    if (!bad) {
+        // this CTA's sums: row tap * CIN + ci, then the bias row, of its partial
+        float* part = a.part + (size_t)blockIdx.x * S::kRows * NCO;
+        if (warp * 32 < 3 * NCO) {
+            const int m = warp * 32 + lane, kx = m / NCO, co = m % NCO;
+            const bool two = r1 - r0 > 1;
+            const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky) {
+                float v[CIN], u[CIN];
+                tc_ld<CIN>(row + ky * CIN, v);
+                tc_ld<CIN>(row + S::kSetCols + ky * CIN, u);
+                if (m < 3 * NCO) {
+#pragma unroll
+                    for (int ci = 0; ci < CIN; ++ci)
+                        part[((ky * 3 + kx) * CIN + ci) * NCO + co] = two ? v[ci] + u[ci] : v[ci];
+                }
+            }
+        }
+        if (tid < NCO) part[9 * CIN * NCO + tid] = (bias_s[0][tid] + bias_s[1][tid]) + (bias_s[2][tid] + bias_s[3][tid]);
+    }
+    tc_fence_before();
     __syncthreads();
     if (warp == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)S::kTmemCols));
     }
     if (tid == 0 && bad) atomicExch(a.err, 1);
 }
 
-// The layer's gradients from the CTAs' partial sums, in a fixed order (so
-// that a training run is bit-reproducible, unlike with floating-point
-// atomics), in two levels: k_wgrad_group sums groups of kWgGroup consecutive
-// CTAs (grid.y = group), k_wgrad_reduce the groups in order and writes
-// dw[co][tap][ci] (row m = tap * CIN + ci) or db[co] (m = 9 CIN). Entry
-// i = m * NCO + co.
-constexpr int kWgGroup = 16;
+// The layer's gradients from the CTAs' partial sums, in a fixed order (so that a
+// training run is bit-reproducible, unlike with floating-point atomics): a block
+// takes 32 entries, warp w sums every kWgReduceWarps-th CTA from w, and the warps'
+// sums are added in order. Entry i = m * NCO + co: dw[co][tap][ci] (row m = tap *
+// CIN + ci) or db[co] (m = 9 CIN).
+constexpr int kWgReduceWarps = 16;
 
 template <int CIN, int NCO>
-__global__ void k_wgrad_group(const float* part, int n_cta, float* part2)
+__global__ void __launch_bounds__(32 * kWgReduceWarps)
+    k_wgrad_reduce(const float* part, int n_cta, float* dw, float* db, int n_out, int cin_real)
 {
     constexpr int R = 9 * CIN + 1;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, g = blockIdx.y;
-    if (i >= R * NCO) return;
-    const size_t cs = (size_t)R * NCO;
-    const int c0 = g * kWgGroup, c1 = min(n_cta, c0 + kWgGroup);
-    float v[kWgGroup];
-#pragma unroll
-    for (int u = 0; u < kWgGroup; ++u) v[u] = c0 + u < c1 ? part[(size_t)(c0 + u) * cs + i] : 0.f;
+    __shared__ float sums[kWgReduceWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     float sum = 0.f;
-#pragma unroll
-    for (int u = 0; u < kWgGroup; ++u) sum += v[u];
-    part2[(size_t)g * cs + i] = sum;
-}
-
-template <int CIN, int NCO>
-__global__ void k_wgrad_reduce(const float* part2, int n_groups, float* dw, float* db, int n_out, int cin_real)
-{
-    constexpr int R = 9 * CIN + 1;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= R * NCO) return;
+    if (i < R * NCO) {
+#pragma unroll 8
+        for (int c = warp; c < n_cta; c += kWgReduceWarps) sum += part[(size_t)c * R * NCO + i];
+    }
+    sums[warp][lane] = sum;
+    __syncthreads();
     const int m = i / NCO, co = i % NCO;
-    if (co >= n_out) return;
-    const size_t cs = (size_t)R * NCO;
-    float sum = 0.f;
-    for (int g = 0; g < n_groups; ++g) sum += part2[(size_t)g * cs + i];
+    if (warp != 0 || i >= R * NCO || co >= n_out) return;
+    sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWgReduceWarps; ++w) sum += sums[w][lane];
     if (m < 9 * CIN) {
         const int tap = m / CIN, ci = m % CIN;
         if (ci < cin_real) dw[((size_t)co * 9 + tap) * cin_real + ci] = sum;
@@ -1024,8 +1048,7 @@ struct voldor_net {
     float* pred = nullptr;          // [pix][8]
     bf16* g16 = nullptr;            // [pix][16] gradient at the output
     bf16 *ga = nullptr, *gb = nullptr;   // [pix][32] gradient ping-pong
-    float* wpart = nullptr;         // weight-gradient partial sums: [kWgCtasPerSm * SMs][kWgPartRows][32],
-                                    // then their group sums (the same layout, one entry per group of CTAs)
+    float* wpart = nullptr;         // weight-gradient partial sums: [kWgCtasPerSm * SMs][kWgPartRows][32]
 };
 
 namespace {
@@ -1145,31 +1168,33 @@ static bool launch_wgrad_tc(const WgradArgs& a, cudaStream_t st)
             g_tc_sms[dev] = 152;
         sms = g_tc_sms[dev];
     }
-    const int items = a.B * a.H * ((a.W + kWgKP - 1) / kWgKP);
-    const int grid = std::min(items, kWgCtasPerSm * sms);
-    k_wgrad_tc<CIN, NCO><<<grid, kWgThreads, S::kSmemBytes, st>>>(a);
-    const int n_groups = (grid + kWgGroup - 1) / kWgGroup;
-    const unsigned blocks = (unsigned)((S::kRows * NCO + 255) / 256);
-    k_wgrad_group<CIN, NCO><<<dim3(blocks, n_groups), 256, 0, st>>>(a.part, grid, a.part2);
-    k_wgrad_reduce<CIN, NCO><<<blocks, 256, 0, st>>>(a.part2, n_groups, a.dw, a.db, a.n_out, a.cin_real);
+    CUtensorMap in, dout;
+    if (!tensor_map_rows(&in, a.in, CIN, a.W, a.H, a.B, CIN, kWgKP, CIN == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !tensor_map_rows(&dout, a.dout, NCO, a.W, a.H, a.B, NCO, kWgKP, NCO == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B))
+        return false;
+    const int rows = a.B * a.H * ((a.W + kWgKP - 1) / kWgKP);
+    const int grid = std::min(rows, kWgCtasPerSm * sms);
+    k_wgrad_tc<CIN, NCO><<<grid, kWgThreads, S::kSmemBytes, st>>>(in, dout, a);
+    k_wgrad_reduce<CIN, NCO><<<(S::kRows * NCO + 31) / 32, 32 * kWgReduceWarps, 0, st>>>(a.part, grid, a.dw, a.db, a.n_out, a.cin_real);
     return true;
 }
 
-void wgrad(voldor_net* n, int l, const bf16* in, int cin_g, const bf16* dout, int cout_g, int B, int H, int W, cudaStream_t st)
+bool wgrad(voldor_net* n, int l, const bf16* in, int cin_g, const bf16* dout, int cout_g, int B, int H, int W, cudaStream_t st)
 {
     WgradArgs a{};
     a.in = in; a.cin_g = cin_g; a.dout = dout; a.cout_g = cout_g;
     a.dw = n->grad + n->L.w_off[l]; a.db = n->grad + n->L.b_off[l];
     a.part = n->wpart;
-    a.part2 = n->wpart + (size_t)kWgCtasPerSm * net_sms() * kWgPartRows * 32;
     a.n_out = n->L.cout[l]; a.cin_real = n->L.cin[l];
     a.H = H; a.W = W; a.B = B;
     a.err = n->tc_err;
     const int cinp = n->L.cin_pad[l];
     const bool wide = n->L.cout[l] > 16;
-    if (cinp == 16 && wide) launch_wgrad_tc<16, 32>(a, st);
-    else if (cinp == 32 && wide) launch_wgrad_tc<32, 32>(a, st);
-    else if (cinp == 32 && !wide) launch_wgrad_tc<32, 16>(a, st);
+    const int coutp = wide ? 32 : 16;
+    if (cin_g != cinp || cout_g != coutp) return false;
+    if (cinp == 16 && wide) return launch_wgrad_tc<16, 32>(a, st);
+    if (cinp == 32) return wide ? launch_wgrad_tc<32, 32>(a, st) : launch_wgrad_tc<32, 16>(a, st);
+    return false;
 }
 
 // Backward pass after forward(); target [pix][2] (log-depth, rigidness).
@@ -1185,7 +1210,7 @@ bool backward(voldor_net* n, const float* tgt, int B, int H, int W, float lam_r,
     for (int l = kNetLayers - 1; l >= 0; --l) {
         const bf16* in = l == 0 ? n->in0 : n->act[l - 1];
         const int cin_g = l == 0 ? 16 : 32;
-        wgrad(n, l, in, cin_g, dout, dout_g, B, H, W, st);
+        if (!wgrad(n, l, in, cin_g, dout, dout_g, B, H, W, st)) return false;
         if (l == 0) break;
         // input gradient: forward conv of dout with the flipped transpose, masked by ReLU'(act[l-1])
         ConvArgs a{};
@@ -1239,8 +1264,7 @@ voldor_status voldor_net_create(int T, voldor_net** out)
               net_ok(cudaMalloc(&n->grad, P * 4)) && net_ok(cudaMalloc(&n->fw, n->L.n_fw * sizeof(bf16))) &&
               net_ok(cudaMalloc(&n->bw, n->L.n_bw * sizeof(bf16))) && net_ok(cudaMalloc(&n->fbias, kNetLayers * kNetWidth * 4)) &&
               net_ok(cudaMalloc(&n->loss, 4)) && net_ok(cudaMalloc(&n->align, 8 * sizeof(float))) &&
-              net_ok(cudaMalloc(&n->wpart, (size_t)(kWgCtasPerSm * net_sms() + (kWgCtasPerSm * net_sms() + 15) / 16) *
-                                               kWgPartRows * 32 * sizeof(float))) &&
+              net_ok(cudaMalloc(&n->wpart, (size_t)kWgCtasPerSm * net_sms() * kWgPartRows * 32 * sizeof(float))) &&
               net_ok(cudaMalloc(&n->hist, 2 * kAlignBins * sizeof(unsigned))) && net_ok(cudaMalloc(&n->tc_err, sizeof(int)));
     if (ok) ok = net_ok(cudaMemset(n->master, 0, P * 4)) && net_ok(cudaMemset(n->m, 0, P * 4)) &&
                  net_ok(cudaMemset(n->v, 0, P * 4)) && net_ok(cudaMemset(n->grad, 0, P * 4)) &&
