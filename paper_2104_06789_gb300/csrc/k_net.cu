@@ -45,16 +45,16 @@ constexpr float kAlignRange = 16.f;             // first level covers log-ratios
 // 3x3 convolution on the fifth-generation tensor cores (implicit GEMM):
 // out[p][n] = sum_{tap, c} in[p + off(tap)][c] w[n][tap][c] (+ bias[n]).
 //
-// A CTA owns a strip of kTcM = 128 output pixels of a row and walks down
-// kTcRows rows of it (persistent over strips). Warp roles:
-//   warp 4, one lane: TMA loads of input rows (box 8 channels x 130 columns,
+// A CTA owns a strip of kTcM = 128 output pixels of a row and walks down its run of
+// rows (persistent over strips). Warp roles:
+//   warp 4, an elected lane: TMA loads of input rows (box 8 channels x 130 columns,
 //     zero fill outside the image) into a ring of kTcSlots row slots laid out
 //     [channel block][column][8 channels], which is the K-major, unswizzled
 //     core-matrix layout of the A operand: an A tile of 128 pixels x 16
 //     channels is a descriptor into the slot (8-pixel groups 128 B apart,
 //     the two 8-channel halves one channel-block row apart), and the taps'
 //     column shift kx is 16 kx bytes on its start address.
-//   warp 5, one lane: per output row, 9 taps x CIN/16 tcgen05.mma
+//   warp 5, an elected lane: per output row, 9 taps x CIN/16 tcgen05.mma
 //     (M = 128, N, K = 16, BF16 in, FP32 accumulators in TMEM), cycling
 //     through kTcAcc accumulators, committed to mbarriers that release the
 //     accumulator to the epilogue and the oldest input row to the loader.
@@ -64,6 +64,11 @@ constexpr float kAlignRange = 16.f;             // first level covers log-ratios
 // Weights [N][9][CIN] are staged once per CTA in the B operand's core-matrix
 // layout. Every mbarrier wait is bounded: on expiry the CTA raises *err,
 // drains its own copies and MMAs, frees its TMEM and returns.
+//
+// 32 x 32 channels over eight 1242 x 375 images, where HBM needs 72 us: 102 us; 129 us
+// with 16-row work items (up to 7 to a CTA, 6.3 on average, each with its two rows of
+// halo), MMAs and loads issued by one lane of a diverged warp and 16-byte stores 64
+// bytes apart. Two images: 35 us, before 46 (1.6 items to a CTA).
 // ---------------------------------------------------------------------------
 struct ConvArgs {
     const bf16* in;
@@ -71,11 +76,9 @@ struct ConvArgs {
     const bf16* w;          // [w_rows][9][CIN] bf16; rows w_rows..N-1 are taken as zero
     int w_rows;
     const float* bias;      // N or null
-    bf16* out;              // bf16 output (channel stride cout_g) or null
-    float* out_f;           // fp32 output (channel stride cout_g) or null
-    int cout_g;
-    int n_out;              // real output channels written
-    const bf16* mask;       // zero the output where mask <= 0 (channel stride cout_g), or null
+    bf16* out;              // N = 32: bf16 output, 32 channels a pixel
+    float* out_f;           // N = 16: fp32 output, the first 8 channels
+    const bf16* mask;       // N = 32: zero the output where mask is not above zero (32 channels a pixel), or null
     int relu;
     int H, W, B;
     int* err;               // set to 1 if a wait expired
@@ -87,7 +90,6 @@ constexpr int kTcRowBytes = 2176;                // one channel block of a slot:
 constexpr int kTcSlots = 6;                      // input-row ring slots
 constexpr int kTcAcc = 8;                        // TMEM accumulator slots (output rows in flight)
 constexpr int kTcCtasPerSm = 2;
-constexpr int kTcRows = 16;                      // output rows per work item
 constexpr int kTcThreads = 192;
 constexpr long long kTcWaitLimit = 1ll << 24;    // polls of one mbarrier phase before giving up
 
@@ -104,7 +106,8 @@ struct TcShape {
     // tmem address | abort flag
     static constexpr int kBarOff = kRingBytes + kWBytes;
     static constexpr int kBarBytes = ((2 * kTcSlots + 2 * kTcAcc + 1) * 8 + 15) / 16 * 16;
-    static constexpr int kSmemBytes = kBarOff + kBarBytes + 16;
+    static constexpr int kStageOff = kBarOff + kBarBytes + 16;       // 2 KB per epilogue warp
+    static constexpr int kSmemBytes = kStageOff + 4 * 2048;
     static constexpr int kTmemCols = kTcAcc * N <= 32 ? 32 : (kTcAcc * N <= 64 ? 64 : (kTcAcc * N <= 128 ? 128 : 256));
 };
 
@@ -187,21 +190,30 @@ __device__ __forceinline__ void tc_ld<16>(uint32_t taddr, float* v)
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Work item i: image b, strip sx (128 columns), row chunk cy (kTcRows rows).
-struct TcItem {
+// The rows of all strips (128 columns of an image) are dealt to the CTAs in contiguous
+// runs of equal length; a segment is the part of a run in one strip: rows y0 ..
+// y0 + rows - 1 of the columns from x0 of image b.
+struct TcSegment {
     int b, x0, y0, rows;
 };
 
-__device__ __forceinline__ TcItem tc_item(int i, int H, int W)
+template <int COLS>
+__device__ __forceinline__ TcSegment tc_segment(int i, int end, int H, int strips)
 {
-    const int strips = (W + kTcM - 1) / kTcM, chunks = (H + kTcRows - 1) / kTcRows;
-    TcItem t;
-    t.b = i / (strips * chunks);
-    const int r = i % (strips * chunks);
-    t.x0 = (r % strips) * kTcM;
-    t.y0 = (r / strips) * kTcRows;
-    t.rows = min(kTcRows, H - t.y0);
+    TcSegment t;
+    const int strip = i / H;
+    t.y0 = i - strip * H;
+    t.rows = min(H - t.y0, end - i);
+    t.b = strip / strips;
+    t.x0 = (strip % strips) * COLS;
     return t;
+}
+
+// All ones in each half of a pair of bf16 values that is above zero.
+__device__ __forceinline__ uint32_t positive2(uint32_t v)
+{
+    const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&v);
+    return __hgt2_mask(p, __float2bfloat162_rn(0.f));
 }
 
 // Zero 8 * X consecutive TMEM columns of the warp's 32 lanes.
@@ -227,7 +239,8 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + S::kBarOff + S::kBarBytes);
     volatile int& bad = *reinterpret_cast<volatile int*>(smem + S::kBarOff + S::kBarBytes + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_items = a.B * ((a.H + kTcRows - 1) / kTcRows) * ((a.W + kTcM - 1) / kTcM);
+    const int strips = (a.W + kTcM - 1) / kTcM, total = a.B * strips * a.H;
+    const int r0 = (int)((long long)total * blockIdx.x / gridDim.x), r1 = (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
 
     // weights -> B operand layout: [K step][n group][k half][8 rows][8 channels] with
     // K step s = kx * (CIN / 16) + cp and n = blk * N + co, blk = 2 - ky
@@ -272,129 +285,149 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     if (warp == 4) {
-        if (lane == 0) {
-            // loader
-            uint32_t ld = 0;
-            for (int it = blockIdx.x; it < n_items && !bad; it += gridDim.x) {
-                const TcItem t = tc_item(it, a.H, a.W);
-                for (int r = t.y0 - 1; r <= t.y0 + t.rows && !bad; ++r, ++ld) {
-                    const uint32_t slot = ld % kTcSlots;
-                    if (ld >= kTcSlots && !tc_wait(empty + 8 * slot, ((ld / kTcSlots) - 1) & 1, &bad)) break;
-                    tc_expect_tx(full + 8 * slot, (uint32_t)S::kSlotTxBytes);
-                    for (int cb = 0; cb < S::kCB; ++cb)
-                        tc_tma_row(ring + slot * S::kSlotBytes + cb * kTcRowBytes, &tin, cb * 8, t.x0 - 1, r, t.b,
-                                   full + 8 * slot);
-                }
+        // loader
+        uint32_t ld = 0;
+        bool go = true;
+        for (int i = r0; i < r1 && go;) {
+            const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
+            for (int r = t.y0 - 1; r <= t.y0 + t.rows; ++r, ++ld) {
+                const uint32_t slot = ld % kTcSlots;
+                if (ld >= kTcSlots) go = tc_wait_warp(empty + 8 * slot, ((ld / kTcSlots) - 1) & 1, &bad);
+                if (!go) break;
+                tc_expect_tx_elect(full + 8 * slot, (uint32_t)S::kSlotTxBytes);
+#pragma unroll
+                for (int cb = 0; cb < S::kCB; ++cb)
+                    tc_tma_row_elect(ring + slot * S::kSlotBytes + cb * kTcRowBytes, &tin, cb * 8, t.x0 - 1, r, t.b, full + 8 * slot);
             }
-            // the last loads may still be landing when another role gave up
-            for (uint32_t j = ld > kTcSlots ? ld - kTcSlots : 0; j < ld; ++j) {
-                for (long long i = 0; i < kTcWaitLimit; ++i)
-                    if (tc_try_wait(full + 8 * (j % kTcSlots), (j / kTcSlots) & 1)) break;
-            }
+            i += t.rows;
+        }
+        // the last loads may still be landing when another role gave up
+        for (uint32_t j = ld > kTcSlots ? ld - kTcSlots : 0; j < ld; ++j) {
+            for (long long i = 0; i < kTcWaitLimit; ++i)
+                if (tc_try_wait(full + 8 * (j % kTcSlots), (j / kTcSlots) & 1)) break;
         }
     } else if (warp == 5) {
-        if (lane == 0) {
-            // MMA issuer: tick k of an item consumes input row y0 - 1 + k (all three
-            // kx shifts, N = 3 N columns: ky = 2, 1, 0 for output rows k - 2, k - 1,
-            // k of the item), so output row j accumulates ky = 0, 1, 2 over ticks
-            // j, j + 1, j + 2; output row g of the CTA's work sits in TMEM slot
-            // g % kTcAcc, zeroed by the epilogue after it reads it out
-            uint32_t ld = 0, G = 0;
-            for (int it = blockIdx.x; it < n_items && !bad; it += gridDim.x) {
-                const TcItem t = tc_item(it, a.H, a.W);
-                for (int k = 0; k < t.rows + 2; ++k, ++ld) {
-                    const uint32_t slot = ld % kTcSlots;
-                    if (!tc_wait(full + 8 * slot, (ld / kTcSlots) & 1, &bad)) break;
-                    const int b0 = max(0, 2 - k), b1 = min(3, t.rows - k + 2);
-                    if (b1 == 3) {                               // first contribution to row k
-                        const uint32_t gn = G + k;
-                        if (gn >= kTcAcc && !tc_wait(acc_empty + 8 * (gn % kTcAcc), ((gn / kTcAcc) - 1) & 1, &bad)) break;
+        // MMA issuer: tick k of a segment consumes input row y0 - 1 + k (all three
+        // kx shifts, N = 3 N columns: ky = 2, 1, 0 for output rows k - 2, k - 1,
+        // k of the segment), so output row j accumulates ky = 0, 1, 2 over ticks
+        // j, j + 1, j + 2; output row g of the CTA's work sits in TMEM slot
+        // g % kTcAcc, zeroed by the epilogue after it reads it out
+        uint32_t ld = 0, G = 0;
+        bool go = true;
+        for (int i = r0; i < r1 && go;) {
+            const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
+            for (int k = 0; k < t.rows + 2; ++k, ++ld) {
+                const uint32_t slot = ld % kTcSlots;
+                go = tc_wait_warp(full + 8 * slot, (ld / kTcSlots) & 1, &bad);
+                const int b0 = max(0, 2 - k), b1 = min(3, t.rows - k + 2);
+                const uint32_t gn = G + k;
+                if (go && b1 == 3 && gn >= kTcAcc)               // first contribution to row k
+                    go = tc_wait_warp(acc_empty + 8 * (gn % kTcAcc), ((gn / kTcAcc) - 1) & 1, &bad);
+                if (!go) break;
+                tc_fence_after();
+                const uint32_t g0 = G + k - 2 + b0;
+                const int s0 = g0 % kTcAcc, nb = b1 - b0, nb1 = min(nb, kTcAcc - s0);
+                const uint32_t d1 = tmem + s0 * N, i1 = tc_idesc(nb1 * N), i2 = tc_idesc((nb - nb1) * N);
+                const uint32_t row = ring + slot * S::kSlotBytes;
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+                    for (int cp = 0; cp < CIN / 16; ++cp) {
+                        const int st = kx * (CIN / 16) + cp;
+                        const uint64_t ad = tc_desc(row + cp * 2 * kTcRowBytes + kx * 16, kTcRowBytes, 128);
+                        const uint32_t bb = wsm + st * S::kWStepBytes + b0 * N * 32;
+                        tc_mma_elect(d1, ad, tc_desc(bb, 128, 256), i1, 1u);
+                        if (nb1 < nb) tc_mma_elect(tmem, ad, tc_desc(bb + nb1 * N * 32, 128, 256), i2, 1u);
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t g0 = G + k - 2 + b0;
-                    const int s0 = g0 % kTcAcc, nb = b1 - b0, nb1 = min(nb, kTcAcc - s0);
-                    const uint32_t d1 = tmem + s0 * N, i1 = tc_idesc(nb1 * N), i2 = tc_idesc((nb - nb1) * N);
-                    const uint32_t row = ring + slot * S::kSlotBytes;
-#pragma unroll
-                    for (int kx = 0; kx < 3; ++kx)
-#pragma unroll
-                        for (int cp = 0; cp < CIN / 16; ++cp) {
-                            const int st = kx * (CIN / 16) + cp;
-                            const uint64_t ad = tc_desc(row + cp * 2 * kTcRowBytes + kx * 16, kTcRowBytes, 128);
-                            const uint32_t bb = wsm + st * S::kWStepBytes + b0 * N * 32;
-                            tc_mma(d1, ad, tc_desc(bb, 128, 256), i1, 1u);
-                            if (nb1 < nb) tc_mma(tmem, ad, tc_desc(bb + nb1 * N * 32, 128, 256), i2, 1u);
-                        }
-                    tc_commit(empty + 8 * slot);                 // the input row is free once these are done
-                    if (b0 == 0) tc_commit(acc_full + 8 * ((G + k - 2) % kTcAcc));   // row k - 2 complete
-                }
-                if (bad) break;
-                G += t.rows;
+                tc_commit_elect(empty + 8 * slot);               // the input row is free once these are done
+                if (b0 == 0) tc_commit_elect(acc_full + 8 * ((G + k - 2) % kTcAcc));   // row k - 2 complete
             }
-            tc_commit(done);                  // arrives once every MMA issued above has completed
-            for (long long i = 0; i < kTcWaitLimit; ++i)
-                if (tc_try_wait(done, 0)) break;
+            G += t.rows;
+            i += t.rows;
         }
+        tc_commit_elect(done);                // arrives once every MMA issued above has completed
+        for (long long i = 0; i < kTcWaitLimit; ++i)
+            if (tc_try_wait(done, 0)) break;
     } else {
-        // epilogue: warp w reads TMEM lanes 32w .. 32w + 31 = pixels x0 + 32w + lane
+        // epilogue: warp w reads TMEM lanes 32w .. 32w + 31 = pixels x0 + 32w + lane, a
+        // pixel's channels per thread; through its 2 KB of shared memory the warp
+        // stores (and reads the mask) in whole 16-byte chunks of consecutive pixels
+        constexpr int kChunks = N == 32 ? 4 : 2;                 // of a pixel: 32 bf16 or 8 fp32
+        constexpr int kPix = 32 / kChunks;                       // pixels a warp-wide access covers
+        unsigned char* stage = smem + S::kStageOff + warp * 2048;
+        const int cpx = lane / kChunks, cc = lane % kChunks;
+        auto at = [](int p, int c) {                             // chunk c of pixel p, free of bank conflicts
+            return p * 16 * kChunks + ((kChunks == 4 ? c ^ ((p >> 1) & 3) : c ^ ((p >> 2) & 1)) << 4);
+        };
         float bias[N];
 #pragma unroll
         for (int n = 0; n < N; ++n) bias[n] = a.bias ? __ldg(a.bias + n) : 0.f;
         uint32_t g = 0;
         bool go = true;
-        for (int it = blockIdx.x; it < n_items && go; it += gridDim.x) {
-            const TcItem t = tc_item(it, a.H, a.W);
+        for (int i = r0; i < r1 && go;) {
+            const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
+            const int px0 = t.x0 + warp * 32;
             for (int k = 0; k < t.rows; ++k, ++g) {
                 const uint32_t buf = g % kTcAcc;
-                // every lane polls; the warp proceeds only together (tcgen05.ld is warp-wide)
-                go = __all_sync(0xffffffffu, tc_wait(acc_full + 8 * buf, (g / kTcAcc) & 1, &bad));
+                const size_t pix = ((size_t)t.b * a.H + t.y0 + k) * a.W + px0;
+                uint4 m[kChunks];
+                if (N == 32 && a.mask) {
+#pragma unroll
+                    for (int q = 0; q < kChunks; ++q)
+                        if (px0 + q * kPix + cpx < a.W)
+                            m[q] = *reinterpret_cast<const uint4*>(a.mask + (pix + q * kPix + cpx) * 32 + 8 * cc);
+                }
+                go = tc_wait_warp(acc_full + 8 * buf, (g / kTcAcc) & 1, &bad);
                 if (!go) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tc_fence_after();
                 float v[N];
                 const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + buf * N;
                 tc_ld<N>(taddr, v);
                 tc_zero<N / 8>(taddr);
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                tc_fence_before();
                 tc_arrive(acc_empty + 8 * buf);
-                const int px = t.x0 + warp * 32 + lane, py = t.y0 + k;
-                if (px >= a.W) continue;
-                const size_t o = (((size_t)t.b * a.H + py) * a.W + px) * a.cout_g;
 #pragma unroll
                 for (int n = 0; n < N; ++n) v[n] += bias[n];
                 if (a.relu) {
 #pragma unroll
                     for (int n = 0; n < N; ++n) v[n] = fmaxf(v[n], 0.f);
                 }
-                if (a.mask) {
+                __syncwarp();                                    // the row before has been read out
 #pragma unroll
-                    for (int q = 0; q < N / 8; ++q) {
-                        const uint4 m = *reinterpret_cast<const uint4*>(a.mask + o + 8 * q);
-                        const bf16* mb = reinterpret_cast<const bf16*>(&m);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (!(__bfloat162float(mb[e]) > 0.f)) v[8 * q + e] = 0.f;
-                    }
-                }
-                if (a.out) {
-#pragma unroll
-                    for (int q = 0; q < N / 8; ++q) {
-                        if (8 * q >= a.n_out) break;
+                for (int c = 0; c < kChunks; ++c) {
+                    uint4 o;
+                    if (N == 32) {
                         __align__(16) bf16 h[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) h[e] = __float2bfloat16_rn(v[8 * q + e]);
-                        *reinterpret_cast<uint4*>(a.out + o + 8 * q) = *reinterpret_cast<const uint4*>(h);
+                        for (int e = 0; e < 8; ++e) h[e] = __float2bfloat16_rn(v[(8 * c + e) % N]);
+                        o = *reinterpret_cast<const uint4*>(h);
+                    } else {
+                        o = make_uint4(__float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]), __float_as_uint(v[4 * c + 2]),
+                                       __float_as_uint(v[4 * c + 3]));
                     }
+                    *reinterpret_cast<uint4*>(stage + at(lane, c)) = o;
                 }
-                if (a.out_f) {
+                __syncwarp();
 #pragma unroll
-                    for (int q = 0; q < N / 4; ++q) {
-                        if (4 * q >= a.n_out) break;
-                        *reinterpret_cast<float4*>(a.out_f + o + 4 * q) =
-                            make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                for (int q = 0; q < kChunks; ++q) {
+                    const int p = q * kPix + cpx;
+                    uint4 o = *reinterpret_cast<const uint4*>(stage + at(p, cc));
+                    if (px0 + p >= a.W) continue;
+                    if (N == 32) {
+                        if (a.mask) {
+                            o.x &= positive2(m[q].x);
+                            o.y &= positive2(m[q].y);
+                            o.z &= positive2(m[q].z);
+                            o.w &= positive2(m[q].w);
+                        }
+                        *reinterpret_cast<uint4*>(a.out + (pix + p) * 32 + 8 * cc) = o;
+                    } else {
+                        *reinterpret_cast<uint4*>(a.out_f + (pix + p) * 8 + 4 * cc) = o;
                     }
                 }
             }
+            i += t.rows;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -462,8 +495,7 @@ static bool launch_conv_tc(const ConvArgs& a, cudaStream_t st)
     }
     CUtensorMap m;
     if (!tensor_map_rows(&m, a.in, CIN, a.W, a.H, a.B, 8, kTcCols, CU_TENSOR_MAP_SWIZZLE_NONE)) return false;
-    const int items = a.B * ((a.H + kTcRows - 1) / kTcRows) * ((a.W + kTcM - 1) / kTcM);
-    const int grid = std::min(items, kTcCtasPerSm * sms);
+    const int grid = std::min(a.B * a.H * ((a.W + kTcM - 1) / kTcM), kTcCtasPerSm * sms);
     k_conv_tc<CIN, N><<<grid, kTcThreads, S::kSmemBytes, st>>>(m, a);
     return true;
 }
@@ -494,11 +526,11 @@ struct WgradArgs {
 // contiguous: the MN-major swizzled layouts (64 bytes a pixel for 32 channels, 32
 // for 16) are what TMA writes, and no thread touches an operand. A CTA walks down
 // the rows of 64-column strips:
-//   warp 4, one lane: TMA loads of a ring of input rows and a ring of dout rows, a
+//   warp 4, an elected lane: TMA loads of a ring of input rows and a ring of dout rows, a
 //     dout row three times (columns x0 + 1, x0, x0 - 1: kx = 0, 1, 2; zero fill
 //     outside the image). M groups of NCO channels are a dout copy apart, N groups
 //     of CIN channels an input row of the ring.
-//   warp 5, one lane: per row four tcgen05.mma (M = 128, of which 3 NCO rows count;
+//   warp 5, an elected lane: per row four tcgen05.mma (M = 128, of which 3 NCO rows count;
 //     N = 3 CIN, K = 16 pixels), in two parts where the three rows wrap around the
 //     ring. Even and odd rows accumulate in two sets of TMEM columns (shorter sums).
 //   warps 0-3: the bias sums from the dout rows in shared memory, FP32; at the end
@@ -550,22 +582,6 @@ __device__ __forceinline__ uint64_t tc_desc_mn(uint32_t addr, uint32_t group)
 
 __host__ __device__ constexpr uint32_t tc_idesc_mn(int n) { return tc_idesc(n) | (1u << 15) | (1u << 16); }
 
-// Run segment: rows y0 .. y0 + rows - 1 of the 64 columns from x0 of image b.
-struct WgSegment {
-    int b, x0, y0, rows;
-};
-
-__device__ __forceinline__ WgSegment wg_segment(int i, int end, int H, int strips)
-{
-    WgSegment t;
-    const int strip = i / H;
-    t.y0 = i - strip * H;
-    t.rows = min(H - t.y0, end - i);
-    t.b = strip / strips;
-    t.x0 = (strip % strips) * kWgKP;
-    return t;
-}
-
 template <int CIN, int NCO>
 __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
     k_wgrad_tc(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tdo, const WgradArgs a)
@@ -611,7 +627,7 @@ __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
         uint32_t li = 0, ld = 0;                           // input and dout rows loaded
         bool go = true;
         for (int i = r0; i < r1 && go;) {
-            const WgSegment t = wg_segment(i, r1, a.H, strips);
+            const TcSegment t = tc_segment<kWgKP>(i, r1, a.H, strips);
             for (int r = t.y0 - 1; r <= t.y0 + t.rows; ++r) {
                 const uint32_t si = li % kWgInSlots, sd = ld % kWgDoSlots;
                 if (li >= kWgInSlots) go = tc_wait_warp(in_empty + 8 * si, ((li / kWgInSlots) - 1) & 1, &bad);
@@ -641,7 +657,7 @@ __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
         uint32_t gi = 0, gd = 0, seen = 0;             // input row y - 1, dout row y, input rows waited for
         bool go = true;
         for (int i = r0; i < r1 && go;) {
-            const WgSegment t = wg_segment(i, r1, a.H, strips);
+            const TcSegment t = tc_segment<kWgKP>(i, r1, a.H, strips);
             for (int k = 0; k < t.rows; ++k, ++gi, ++gd) {
                 for (; go && seen < gi + 3; ++seen)
                     go = tc_wait_warp(in_full + 8 * (seen % kWgInSlots), (seen / kWgInSlots) & 1, &bad);
@@ -1136,7 +1152,7 @@ bool forward(voldor_net* n, const void* flows, int f16, int B, int H, int W, cud
         ConvArgs a{};
         a.in = in; a.cin_g = cin_g; a.w = n->fw + n->L.fw_off[l]; a.bias = n->fbias + l * kNetWidth;
         a.out = last ? nullptr : n->act[l]; a.out_f = last ? (out ? out : n->pred) : nullptr;
-        a.cout_g = last ? 8 : 32; a.n_out = last ? 8 : 32; a.mask = nullptr; a.relu = last ? 0 : 1; a.H = H; a.W = W;
+        a.mask = nullptr; a.relu = last ? 0 : 1; a.H = H; a.W = W;
         a.B = B; a.w_rows = n->L.cout_pad[l]; a.err = n->tc_err;
         if (!conv(n->L.cin_pad[l], last ? 16 : 32, a, st)) return false;
         if (last) break;
@@ -1216,7 +1232,7 @@ bool backward(voldor_net* n, const float* tgt, int B, int H, int W, float lam_r,
         ConvArgs a{};
         a.in = dout; a.cin_g = dout_g; a.w = n->bw + n->L.bw_off[l]; a.bias = nullptr;
         bf16* o = bufs[l & 1];
-        a.out = o; a.out_f = nullptr; a.cout_g = 32; a.n_out = 32; a.mask = n->act[l - 1]; a.relu = 0; a.H = H; a.W = W;
+        a.out = o; a.out_f = nullptr; a.mask = n->act[l - 1]; a.relu = 0; a.H = H; a.W = W;
         a.B = B; a.w_rows = n->L.cin_pad[l]; a.err = n->tc_err;
         const int cout_b = n->L.cout_pad[l] < 16 ? 16 : n->L.cout_pad[l];
         if (!conv(cout_b, 32, a, st)) return false;
