@@ -47,19 +47,19 @@ constexpr float kAlignRange = 16.f;             // first level covers log-ratios
 //
 // A CTA owns a strip of kTcM = 128 output pixels of a row and walks down its run of
 // rows (persistent over strips). Warp roles:
-//   warp 4, an elected lane: TMA loads of input rows (box 8 channels x 130 columns,
+//   warp 8, an elected lane: TMA loads of input rows (box 8 channels x 130 columns,
 //     zero fill outside the image) into a ring of kTcSlots row slots laid out
 //     [channel block][column][8 channels], which is the K-major, unswizzled
 //     core-matrix layout of the A operand: an A tile of 128 pixels x 16
 //     channels is a descriptor into the slot (8-pixel groups 128 B apart,
 //     the two 8-channel halves one channel-block row apart), and the taps'
 //     column shift kx is 16 kx bytes on its start address.
-//   warp 5, an elected lane: per output row, 9 taps x CIN/16 tcgen05.mma
+//   warp 9, an elected lane: per output row, 9 taps x CIN/16 tcgen05.mma
 //     (M = 128, N, K = 16, BF16 in, FP32 accumulators in TMEM), cycling
 //     through kTcAcc accumulators, committed to mbarriers that release the
 //     accumulator to the epilogue and the oldest input row to the loader.
-//   warps 0-3: epilogue: tcgen05.ld of the accumulator rows of their 32 TMEM
-//     lanes (one pixel per thread), bias, ReLU, the ReLU mask of a previous
+//   warps 0-3 (even rows) and 4-7 (odd): epilogue: tcgen05.ld of the accumulator
+//     rows of their 32 TMEM lanes (one pixel per thread), bias, ReLU, the ReLU mask of a previous
 //     activation (input gradient), bf16 or fp32 stores.
 // Weights [N][9][CIN] are staged once per CTA in the B operand's core-matrix
 // layout. Every mbarrier wait is bounded: on expiry the CTA raises *err,
@@ -68,7 +68,10 @@ constexpr float kAlignRange = 16.f;             // first level covers log-ratios
 // 32 x 32 channels over eight 1242 x 375 images, where HBM needs 72 us: 102 us; 129 us
 // with 16-row work items (up to 7 to a CTA, 6.3 on average, each with its two rows of
 // halo), MMAs and loads issued by one lane of a diverged warp and 16-byte stores 64
-// bytes apart. Two images: 35 us, before 46 (1.6 items to a CTA).
+// bytes apart. Two images: 35 us, before 46 (1.6 items to a CTA); with the mask eight
+// epilogue warps instead of four take 4 us off. What bounds it: TMA, ~1.4 cycles per
+// 16-byte row of its boxes (one box per row instead of four is no faster), beside
+// shared memory at two thirds of its rate; cp.async by four warps took 119 us.
 // ---------------------------------------------------------------------------
 struct ConvArgs {
     const bf16* in;
@@ -90,7 +93,8 @@ constexpr int kTcRowBytes = 2176;                // one channel block of a slot:
 constexpr int kTcSlots = 6;                      // input-row ring slots
 constexpr int kTcAcc = 8;                        // TMEM accumulator slots (output rows in flight)
 constexpr int kTcCtasPerSm = 2;
-constexpr int kTcThreads = 192;
+constexpr int kTcEpi = 8;                         // epilogue warps: four read the even output rows, four the odd
+constexpr int kTcThreads = 32 * kTcEpi + 64;
 constexpr long long kTcWaitLimit = 1ll << 24;    // polls of one mbarrier phase before giving up
 
 template <int CIN, int N>
@@ -106,8 +110,9 @@ struct TcShape {
     // tmem address | abort flag
     static constexpr int kBarOff = kRingBytes + kWBytes;
     static constexpr int kBarBytes = ((2 * kTcSlots + 2 * kTcAcc + 1) * 8 + 15) / 16 * 16;
-    static constexpr int kStageOff = kBarOff + kBarBytes + 16;       // 2 KB per epilogue warp
-    static constexpr int kSmemBytes = kStageOff + 4 * 2048;
+    static constexpr int kStageOff = kBarOff + kBarBytes + 16;       // 2 KB per epilogue warp, then the bias
+    static constexpr int kBiasOff = kStageOff + kTcEpi * 2048;
+    static constexpr int kSmemBytes = kBiasOff + N * 4;
     static constexpr int kTmemCols = kTcAcc * N <= 32 ? 32 : (kTcAcc * N <= 64 ? 64 : (kTcAcc * N <= 128 ? 128 : 256));
 };
 
@@ -253,6 +258,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
         if (co < a.w_rows) v = *reinterpret_cast<const uint4*>(a.w + ((size_t)co * 9 + ky * 3 + kx) * CIN + cp * 16 + kh * 8);
         *reinterpret_cast<uint4*>(smem + S::kRingBytes + st * S::kWStepBytes + (n >> 3) * 256 + kh * 128 + (n & 7) * 16) = v;
     }
+    if (threadIdx.x < N) reinterpret_cast<float*>(smem + S::kBiasOff)[threadIdx.x] = a.bias ? __ldg(a.bias + threadIdx.x) : 0.f;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kTcSlots; ++i) {
             tc_mbar_init(full + 8 * i, 1);
@@ -284,7 +290,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-    if (warp == 4) {
+    if (warp == kTcEpi) {
         // loader
         uint32_t ld = 0;
         bool go = true;
@@ -306,7 +312,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
             for (long long i = 0; i < kTcWaitLimit; ++i)
                 if (tc_try_wait(full + 8 * (j % kTcSlots), (j / kTcSlots) & 1)) break;
         }
-    } else if (warp == 5) {
+    } else if (warp == kTcEpi + 1) {
         // MMA issuer: tick k of a segment consumes input row y0 - 1 + k (all three
         // kx shifts, N = 3 N columns: ky = 2, 1, 0 for output rows k - 2, k - 1,
         // k of the segment), so output row j accumulates ky = 0, 1, 2 over ticks
@@ -349,7 +355,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
         for (long long i = 0; i < kTcWaitLimit; ++i)
             if (tc_try_wait(done, 0)) break;
     } else {
-        // epilogue: warp w reads TMEM lanes 32w .. 32w + 31 = pixels x0 + 32w + lane, a
+        // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = pixels x0 + 32 (w % 4) + lane, a
         // pixel's channels per thread; through its 2 KB of shared memory the warp
         // stores (and reads the mask) in whole 16-byte chunks of consecutive pixels
         constexpr int kChunks = N == 32 ? 4 : 2;                 // of a pixel: 32 bf16 or 8 fp32
@@ -359,15 +365,14 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
         auto at = [](int p, int c) {                             // chunk c of pixel p, free of bank conflicts
             return p * 16 * kChunks + ((kChunks == 4 ? c ^ ((p >> 1) & 3) : c ^ ((p >> 2) & 1)) << 4);
         };
-        float bias[N];
-#pragma unroll
-        for (int n = 0; n < N; ++n) bias[n] = a.bias ? __ldg(a.bias + n) : 0.f;
+        const float4* bias = reinterpret_cast<const float4*>(smem + S::kBiasOff);
         uint32_t g = 0;
         bool go = true;
         for (int i = r0; i < r1 && go;) {
             const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
-            const int px0 = t.x0 + warp * 32;
+            const int px0 = t.x0 + (warp & 3) * 32;
             for (int k = 0; k < t.rows; ++k, ++g) {
+                if ((g & 1) != (uint32_t)(warp >> 2)) continue;
                 const uint32_t buf = g % kTcAcc;
                 const size_t pix = ((size_t)t.b * a.H + t.y0 + k) * a.W + px0;
                 uint4 m[kChunks];
@@ -381,14 +386,20 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
                 if (!go) break;
                 tc_fence_after();
                 float v[N];
-                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + buf * N;
+                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + buf * N;
                 tc_ld<N>(taddr, v);
                 tc_zero<N / 8>(taddr);
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
                 tc_arrive(acc_empty + 8 * buf);
 #pragma unroll
-                for (int n = 0; n < N; ++n) v[n] += bias[n];
+                for (int n = 0; n < N; n += 4) {
+                    const float4 b = bias[n / 4];
+                    v[n] += b.x;
+                    v[n + 1] += b.y;
+                    v[n + 2] += b.z;
+                    v[n + 3] += b.w;
+                }
                 if (a.relu) {
 #pragma unroll
                     for (int n = 0; n < N; ++n) v[n] = fmaxf(v[n], 0.f);
