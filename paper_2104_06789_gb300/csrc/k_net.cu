@@ -871,15 +871,20 @@ __global__ void k_pack_input(const void* flows, int f16, int T, int N, const flo
 // rigidness logit (weight lam_r); gradients into channels 0, 1 of a 16-channel
 // bf16 buffer, scaled by 1 / n_pix. Targets with a non-finite log-depth are
 // skipped.
-__global__ void k_net_loss(const float* pred, int pred_cs, const float* tgt, size_t n_pix, float lam_r, bf16* dout,
-                           float* loss)
+// The blocks stride over the pixels and add to the loss once each: an addition per
+// warp, 29,000 of them to one address, held the kernel at 55 us for two 1242 x 375
+// images; now 10.5 us. HBM's time for predictions, targets and gradients is 10 us.
+constexpr int kLossThreads = 256, kLossBlocks = 4 * 152;
+
+__global__ void __launch_bounds__(kLossThreads)
+    k_net_loss(const float* pred, int pred_cs, const float* tgt, size_t n_pix, float lam_r, bf16* dout, float* loss)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
-    if (i < n_pix) {
+    const float inv = 1.f / (float)n_pix;
+    float sum = 0.f;
+    for (size_t i = (size_t)blockIdx.x * kLossThreads + threadIdx.x; i < n_pix; i += (size_t)gridDim.x * kLossThreads) {
         const float z0 = pred[i * pred_cs], z1 = pred[i * pred_cs + 1];
         const float t0 = tgt[2 * i], t1 = tgt[2 * i + 1];
-        float g0 = 0.f, g1 = 0.f;
+        float g0 = 0.f, g1 = 0.f, l = 0.f;
         if (isfinite(t0) && isfinite(z0) && isfinite(z1)) {
             const float d = z0 - t0, ad = fabsf(d), delta = 0.1f;
             l = ad < delta ? 0.5f * d * d / delta : ad - 0.5f * delta;
@@ -888,17 +893,20 @@ __global__ void k_net_loss(const float* pred, int pred_cs, const float* tgt, siz
             l += lam_r * (sp - t1 * z1);
             g1 = lam_r * (1.f / (1.f + expf(-z1)) - t1);
         }
-        const float inv = 1.f / (float)n_pix;
-        __align__(16) bf16 v[16];
-        for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
-        v[0] = __float2bfloat16_rn(g0 * inv);
-        v[1] = __float2bfloat16_rn(g1 * inv);
+        sum += l;
+        const __nv_bfloat162 g = __halves2bfloat162(__float2bfloat16_rn(g0 * inv), __float2bfloat16_rn(g1 * inv));
         uint4* o = reinterpret_cast<uint4*>(dout + i * 16);
-        o[0] = *reinterpret_cast<uint4*>(v);
-        o[1] = *reinterpret_cast<uint4*>(v + 8);
+        o[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&g), 0u, 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && l != 0.f) atomicAdd(loss, l / (float)n_pix);
+    __shared__ float warps[kLossThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0) warps[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kLossThreads / 32; ++w) sum += warps[w];
+        if (sum != 0.f) atomicAdd(loss, sum / (float)n_pix);
+    }
 }
 
 struct NetLayout {
@@ -1230,7 +1238,7 @@ bool backward(voldor_net* n, const float* tgt, int B, int H, int W, float lam_r,
     const size_t pix = (size_t)B * H * W;
     cudaMemsetAsync(n->grad, 0, n->L.n_params * sizeof(float), st);
     cudaMemsetAsync(n->loss, 0, sizeof(float), st);
-    k_net_loss<<<(unsigned)((pix + 255) / 256), 256, 0, st>>>(n->pred, 8, tgt, pix, lam_r, n->g16, n->loss);
+    k_net_loss<<<(unsigned)std::min<size_t>((pix + kLossThreads - 1) / kLossThreads, kLossBlocks), kLossThreads, 0, st>>>(n->pred, 8, tgt, pix, lam_r, n->g16, n->loss);
     const bf16* dout = n->g16;
     int dout_g = 16;
     bf16* bufs[2] = {n->ga, n->gb};
