@@ -517,10 +517,7 @@ struct WgradArgs {
     int cin_g;
     const bf16* dout;       // channel stride cout_g
     int cout_g;
-    float* dw;              // [n_out][9][cin_real]
-    float* db;              // [n_out]
     float* part;            // [gridDim.x][9 CIN + 1][NCO] each CTA's sums
-    int n_out, cin_real;
     int H, W, B;
     int* err;               // set to 1 if a bounded wait expired
 };
@@ -757,37 +754,47 @@ __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
     if (tid == 0 && bad) atomicExch(a.err, 1);
 }
 
-// The layer's gradients from the CTAs' partial sums, in a fixed order (so that a
-// training run is bit-reproducible, unlike with floating-point atomics): a block
-// takes 32 entries, warp w sums every kWgReduceWarps-th CTA from w, and the warps'
-// sums are added in order. Entry i = m * NCO + co: dw[co][tap][ci] (row m = tap *
-// CIN + ci) or db[co] (m = 9 CIN).
+// The gradients of all layers from the CTAs' partial sums, in a fixed order (so that
+// a training run is bit-reproducible, unlike with floating-point atomics): grid
+// (blocks of 32 entries, layer); warp w sums every kWgReduceWarps-th CTA from w, and
+// the warps' sums are added in order. Entry i = m * nco + co of a layer: dw[co][tap][ci]
+// (row m = tap * cin + ci) or db[co] (m = 9 cin). A launch per layer took 6 us each.
 constexpr int kWgReduceWarps = 16;
 
-template <int CIN, int NCO>
-__global__ void __launch_bounds__(32 * kWgReduceWarps)
-    k_wgrad_reduce(const float* part, int n_cta, float* dw, float* db, int n_out, int cin_real)
+struct WgLayer {
+    const float* part;                                    // [n_cta][9 cin + 1][nco]
+    float *dw, *db;
+    int n_cta, cin, nco, n_out, cin_real;
+};
+
+struct WgLayers {
+    WgLayer l[kNetLayers];
+};
+
+__global__ void __launch_bounds__(32 * kWgReduceWarps) k_wgrad_reduce(const __grid_constant__ WgLayers layers)
 {
-    constexpr int R = 9 * CIN + 1;
     __shared__ float sums[kWgReduceWarps][32];
+    const WgLayer& g = layers.l[blockIdx.y];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    const int entries = (9 * g.cin + 1) * g.nco;
+    if (blockIdx.x * 32 >= entries) return;
     float sum = 0.f;
-    if (i < R * NCO) {
+    if (i < entries) {
 #pragma unroll 8
-        for (int c = warp; c < n_cta; c += kWgReduceWarps) sum += part[(size_t)c * R * NCO + i];
+        for (int c = warp; c < g.n_cta; c += kWgReduceWarps) sum += g.part[(size_t)c * entries + i];
     }
     sums[warp][lane] = sum;
     __syncthreads();
-    const int m = i / NCO, co = i % NCO;
-    if (warp != 0 || i >= R * NCO || co >= n_out) return;
+    const int m = i / g.nco, co = i % g.nco;
+    if (warp != 0 || i >= entries || co >= g.n_out) return;
     sum = 0.f;
 #pragma unroll
     for (int w = 0; w < kWgReduceWarps; ++w) sum += sums[w][lane];
-    if (m < 9 * CIN) {
-        const int tap = m / CIN, ci = m % CIN;
-        if (ci < cin_real) dw[((size_t)co * 9 + tap) * cin_real + ci] = sum;
+    if (m < 9 * g.cin) {
+        const int tap = m / g.cin, ci = m % g.cin;
+        if (ci < g.cin_real) g.dw[((size_t)co * 9 + tap) * g.cin_real + ci] = sum;
     } else {
-        db[co] = sum;
+        g.db[co] = sum;
     }
 }
 
@@ -1083,7 +1090,7 @@ struct voldor_net {
     float* pred = nullptr;          // [pix][8]
     bf16* g16 = nullptr;            // [pix][16] gradient at the output
     bf16 *ga = nullptr, *gb = nullptr;   // [pix][32] gradient ping-pong
-    float* wpart = nullptr;         // weight-gradient partial sums: [kWgCtasPerSm * SMs][kWgPartRows][32]
+    float* wpart = nullptr;         // weight-gradient partial sums: [layer][kWgCtasPerSm * SMs][kWgPartRows][32]
 };
 
 namespace {
@@ -1181,8 +1188,9 @@ bool forward(voldor_net* n, const void* flows, int f16, int B, int H, int W, cud
     return true;
 }
 
+// Launches a layer's weight gradient; the CTAs' partials go to a.part, their number to grid.
 template <int CIN, int NCO>
-static bool launch_wgrad_tc(const WgradArgs& a, cudaStream_t st)
+static bool launch_wgrad_tc(const WgradArgs& a, cudaStream_t st, int& grid)
 {
     using S = WgShape<CIN, NCO>;
     static bool attr[kTcMaxDevices];
@@ -1208,27 +1216,28 @@ static bool launch_wgrad_tc(const WgradArgs& a, cudaStream_t st)
         !tensor_map_rows(&dout, a.dout, NCO, a.W, a.H, a.B, NCO, kWgKP, NCO == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B))
         return false;
     const int rows = a.B * a.H * ((a.W + kWgKP - 1) / kWgKP);
-    const int grid = std::min(rows, kWgCtasPerSm * sms);
+    grid = std::min(rows, kWgCtasPerSm * sms);
     k_wgrad_tc<CIN, NCO><<<grid, kWgThreads, S::kSmemBytes, st>>>(in, dout, a);
-    k_wgrad_reduce<CIN, NCO><<<(S::kRows * NCO + 31) / 32, 32 * kWgReduceWarps, 0, st>>>(a.part, grid, a.dw, a.db, a.n_out, a.cin_real);
     return true;
 }
 
-bool wgrad(voldor_net* n, int l, const bf16* in, int cin_g, const bf16* dout, int cout_g, int B, int H, int W, cudaStream_t st)
+// A layer's weight gradient, up to its CTAs' partials; g tells k_wgrad_reduce of them.
+bool wgrad(voldor_net* n, int l, const bf16* in, int cin_g, const bf16* dout, int cout_g, int B, int H, int W, cudaStream_t st,
+           WgLayer& g)
 {
     WgradArgs a{};
     a.in = in; a.cin_g = cin_g; a.dout = dout; a.cout_g = cout_g;
-    a.dw = n->grad + n->L.w_off[l]; a.db = n->grad + n->L.b_off[l];
-    a.part = n->wpart;
-    a.n_out = n->L.cout[l]; a.cin_real = n->L.cin[l];
+    a.part = n->wpart + (size_t)l * kWgCtasPerSm * net_sms() * kWgPartRows * 32;
     a.H = H; a.W = W; a.B = B;
     a.err = n->tc_err;
-    const int cinp = n->L.cin_pad[l];
-    const bool wide = n->L.cout[l] > 16;
-    const int coutp = wide ? 32 : 16;
-    if (cin_g != cinp || cout_g != coutp) return false;
-    if (cinp == 16 && wide) return launch_wgrad_tc<16, 32>(a, st);
-    if (cinp == 32) return wide ? launch_wgrad_tc<32, 32>(a, st) : launch_wgrad_tc<32, 16>(a, st);
+    g.part = a.part;
+    g.dw = n->grad + n->L.w_off[l]; g.db = n->grad + n->L.b_off[l];
+    g.n_out = n->L.cout[l]; g.cin_real = n->L.cin[l];
+    g.cin = n->L.cin_pad[l];
+    g.nco = n->L.cout[l] > 16 ? 32 : 16;
+    if (cin_g != g.cin || cout_g != g.nco) return false;
+    if (g.cin == 16 && g.nco == 32) return launch_wgrad_tc<16, 32>(a, st, g.n_cta);
+    if (g.cin == 32) return g.nco == 32 ? launch_wgrad_tc<32, 32>(a, st, g.n_cta) : launch_wgrad_tc<32, 16>(a, st, g.n_cta);
     return false;
 }
 
@@ -1242,10 +1251,11 @@ bool backward(voldor_net* n, const float* tgt, int B, int H, int W, float lam_r,
     const bf16* dout = n->g16;
     int dout_g = 16;
     bf16* bufs[2] = {n->ga, n->gb};
+    WgLayers layers{};
     for (int l = kNetLayers - 1; l >= 0; --l) {
         const bf16* in = l == 0 ? n->in0 : n->act[l - 1];
         const int cin_g = l == 0 ? 16 : 32;
-        if (!wgrad(n, l, in, cin_g, dout, dout_g, B, H, W, st)) return false;
+        if (!wgrad(n, l, in, cin_g, dout, dout_g, B, H, W, st, layers.l[l])) return false;
         if (l == 0) break;
         // input gradient: forward conv of dout with the flipped transpose, masked by ReLU'(act[l-1])
         ConvArgs a{};
@@ -1258,6 +1268,7 @@ bool backward(voldor_net* n, const float* tgt, int B, int H, int W, float lam_r,
         dout = o;
         dout_g = 32;
     }
+    k_wgrad_reduce<<<dim3(kWgPartRows, kNetLayers), 32 * kWgReduceWarps, 0, st>>>(layers);
     return true;
 }
 
@@ -1299,7 +1310,7 @@ voldor_status voldor_net_create(int T, voldor_net** out)
               net_ok(cudaMalloc(&n->grad, P * 4)) && net_ok(cudaMalloc(&n->fw, n->L.n_fw * sizeof(bf16))) &&
               net_ok(cudaMalloc(&n->bw, n->L.n_bw * sizeof(bf16))) && net_ok(cudaMalloc(&n->fbias, kNetLayers * kNetWidth * 4)) &&
               net_ok(cudaMalloc(&n->loss, 4)) && net_ok(cudaMalloc(&n->align, 8 * sizeof(float))) &&
-              net_ok(cudaMalloc(&n->wpart, (size_t)kWgCtasPerSm * net_sms() * kWgPartRows * 32 * sizeof(float))) &&
+              net_ok(cudaMalloc(&n->wpart, (size_t)kNetLayers * kWgCtasPerSm * net_sms() * kWgPartRows * 32 * sizeof(float))) &&
               net_ok(cudaMalloc(&n->hist, 2 * kAlignBins * sizeof(unsigned))) && net_ok(cudaMalloc(&n->tc_err, sizeof(int)));
     if (ok) ok = net_ok(cudaMemset(n->master, 0, P * 4)) && net_ok(cudaMemset(n->m, 0, P * 4)) &&
                  net_ok(cudaMemset(n->v, 0, P * 4)) && net_ok(cudaMemset(n->grad, 0, P * 4)) &&
