@@ -465,13 +465,22 @@ __device__ __forceinline__ int groups_solved(const DevParams& p, const DevState&
     return min(min(*s.p3p_claims, n_chunks) * kP3PChunk, p.G);
 }
 
-// One warp per block spreads the FP64 solves over the SMs. The first wave
-// is sized for about 1.1 S solutions at the yield of driving-like windows
-// (1.4-1.5 solutions per group); further chunks are claimed as needed.
+// One warp per block spreads the FP64 solves over the SMs. The first wave takes S
+// groups (more than one solution each as a rule), so that no warp runs a second chunk
+// after its first, a whole chain later: with 3/4 S groups, enough only above 1.33
+// solutions a group, frames of handheld windows took 78 us on average (54 or 97) at
+// S = 4096 on 640 x 480, now 58, and 79 at S = 2048 on 320 x 240, now 54. An SM solves
+// three and a half chunks in the time of one and no more (5/4 S groups at S = 4096:
+// 68 us, 7/4 S: 77), so beyond kP3PFreeChunks chunks in all it is 3/4 S, as the yield of
+// driving windows (1.4-1.5) allows (S = 8192: 77 us; with 15/16 S 86); further chunks
+// are claimed as needed.
+constexpr int kP3PFreeChunks = 512;
+
 void launch_p3p_groups(const DevParams& p, const DevState& s, int t, cudaStream_t st)
 {
     const int n_chunks = (p.G + kP3PChunk - 1) / kP3PChunk;
-    const int wave = std::max(1, std::min(n_chunks, (3 * p.S + 4 * kP3PChunk - 1) / (4 * kP3PChunk)));
+    const int all = (p.S + kP3PChunk - 1) / kP3PChunk, most = (3 * p.S + 4 * kP3PChunk - 1) / (4 * kP3PChunk);
+    const int wave = std::min(n_chunks, std::max(most, std::min(all, kP3PFreeChunks)));
     k_p3p_groups<<<wave, 32, 0, st>>>(p, s, t);
 }
 
