@@ -40,104 +40,109 @@ __device__ __forceinline__ double horner4(const double* c, double x)
     return (((c[4] * x + c[3]) * x + c[2]) * x + c[1]) * x + c[0];
 }
 
-// x = J^-1 F through the adjugate; false if J is singular.
-__device__ __forceinline__ bool solve3x3(const double* J, const double* F, double* x)
+// a / b, correctly rounded, from y = 1 / b correctly rounded, for quotients and
+// remainders inside the normal range: the first correction brings q within one ulp,
+// and the second then rounds correctly (Markstein, IBM J. Res. Dev. 34, 1990). Five
+// FP64 instructions where the division takes about twelve.
+__device__ __forceinline__ double div_by(double a, double b, double y)
 {
-    const double c00 = J[4] * J[8] - J[5] * J[7];
-    const double c01 = J[5] * J[6] - J[3] * J[8];
-    const double c02 = J[3] * J[7] - J[4] * J[6];
-    const double det = J[0] * c00 + J[1] * c01 + J[2] * c02;
-    if (!(fabs(det) > 0.0)) return false;
-    const double c10 = J[2] * J[7] - J[1] * J[8];
-    const double c11 = J[0] * J[8] - J[2] * J[6];
-    const double c12 = J[1] * J[6] - J[0] * J[7];
-    const double c20 = J[1] * J[5] - J[2] * J[4];
-    const double c21 = J[2] * J[3] - J[0] * J[5];
-    const double c22 = J[0] * J[4] - J[1] * J[3];
-    const double id = 1.0 / det;
-    x[0] = (c00 * F[0] + c10 * F[1] + c20 * F[2]) * id;
-    x[1] = (c01 * F[0] + c11 * F[1] + c21 * F[2]) * id;
-    x[2] = (c02 * F[0] + c12 * F[1] + c22 * F[2]) * id;
-    return true;
+    double q = a * y;
+    q = fma(fma(-b, q, a), y, q);
+    return fma(fma(-b, q, a), y, q);
 }
 
+__device__ __forceinline__ double third(double a) { return div_by(a, 3.0, 1.0 / 3.0); }
+
 // Largest real root of m^3 + A m^2 + B m + C (Cardano or trigonometric form),
-// refined by Newton steps.
+// refined by Newton steps; all lanes of the quad on the same coefficients, the two
+// cube roots on its even and odd lanes. Every lane of the warp takes part.
 __device__ double cubic_max_root(double A, double B, double C)
 {
-    const double A3 = A / 3.0;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, base = lane & ~3;
+    const double A3 = third(A);
     const double pp = B - A * A3;                         // y^3 + pp y + qq = 0, m = y - A/3
     const double qq = 2.0 * A3 * A3 * A3 - A3 * B + C;
-    double y;
-    const double disc = 0.25 * qq * qq + pp * pp * pp / 27.0;
-    if (disc > 0.0) {
+    const double disc = 0.25 * qq * qq + div_by(pp * pp * pp, 27.0, 1.0 / 27.0);
+    const bool one = disc > 0.0;
+    double part = 0.0;
+    if (one) {
         const double sq = sqrt(disc);
-        y = cbrt(-0.5 * qq + sq) + cbrt(-0.5 * qq - sq);
-    } else {
-        const double r = sqrt(fmax(-pp / 3.0, 0.0));
+        part = cbrt(-0.5 * qq + (lane & 1 ? -sq : sq));
+    }
+    double y = __shfl_sync(FULL, part, base) + __shfl_sync(FULL, part, base + 1);
+    if (!one) {
+        const double r = sqrt(fmax(third(-pp), 0.0));
         double arg = (r > 0.0) ? (-0.5 * qq) / (r * r * r) : 0.0;
         arg = fmin(1.0, fmax(-1.0, arg));
-        y = 2.0 * r * cos(acos(arg) / 3.0);
+        y = 2.0 * r * cos(third(acos(arg)));
     }
     double m = y - A3;
+    double f = ((m + A) * m + B) * m + C;
     for (int it = 0; it < 4; ++it) {
-        const double f = ((m + A) * m + B) * m + C;
         const double df = (3.0 * m + 2.0 * A) * m + B;
         if (!(fabs(df) > 0.0)) break;
         const double mn = m - f / df;
         const double fn = ((mn + A) * mn + B) * mn + C;
         if (!(fabs(fn) < fabs(f))) break;
         m = mn;
+        f = fn;
     }
     return m;
 }
 
-// Real root candidates of a quartic (ascending coefficients) by Ferrari's
-// method, before polishing, shifted back by -b/4. Returns the count (<= 4).
-__device__ int quartic_candidates(const double* a, double* roots)
+// Lane r's root candidate of a quartic (ascending coefficients, the same in all lanes
+// of a quad) by Ferrari's method, before polishing, shifted back by -b/4; false if it
+// has none. The quad's candidates, in lane order: the two roots of the first
+// quadratic factor, then those of the second. Every lane of the warp takes part.
+__device__ bool quartic_candidate(const double* a, double& root)
 {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, r = lane & 3, base = lane & ~3;
     double amax = 0.0;
     for (int i = 0; i < 4; ++i) amax = fmax(amax, fabs(a[i]));
-    if (!(fabs(a[4]) > 1e-14 * amax)) return 0;           // degenerate group
-    const double b = a[3] / a[4], c = a[2] / a[4], d = a[1] / a[4], e = a[0] / a[4];
+    const double own = (r == 0 ? a[3] : (r == 1 ? a[2] : (r == 2 ? a[1] : a[0]))) / a[4];
+    const double b = __shfl_sync(FULL, own, base), c = __shfl_sync(FULL, own, base + 1);
+    const double d = __shfl_sync(FULL, own, base + 2), e = __shfl_sync(FULL, own, base + 3);
     const double bb = b * b;
     const double P = c - 0.375 * bb;
     const double Q = d - 0.5 * b * c + 0.125 * bb * b;
     const double R = e - 0.25 * b * d + 0.0625 * bb * c - (3.0 / 256.0) * bb * bb;
-    double y[4];
-    int n = 0;
     // y^4 + P y^2 + Q y + R = (y^2 + P/2 + m)^2 - 2m (y - Q/(4m))^2 for the
     // resolvent root m of m^3 + P m^2 + (P^2/4 - R) m - Q^2/8 = 0
     const double m = cubic_max_root(P, 0.25 * P * P - R, -0.125 * Q * Q);
+    if (!(fabs(a[4]) > 1e-14 * amax)) return false;       // degenerate group
+    double y;
     if (m > 1e-300 && fabs(Q) > 0.0) {
         const double sr = sqrt(2.0 * m);
         const double h = Q / (2.0 * sr);
-        const double c1 = 0.5 * P + m - h, c2 = 0.5 * P + m + h;
-        const double D1 = 2.0 * m - 4.0 * c1, D2 = 2.0 * m - 4.0 * c2;
-        if (D1 >= 0.0) { const double q = sqrt(D1); y[n++] = 0.5 * (-sr + q); y[n++] = 0.5 * (-sr - q); }
-        if (D2 >= 0.0) { const double q = sqrt(D2); y[n++] = 0.5 * (sr + q); y[n++] = 0.5 * (sr - q); }
+        const double cf = 0.5 * P + m + (r < 2 ? -h : h), D = 2.0 * m - 4.0 * cf;
+        if (!(D >= 0.0)) return false;
+        const double q = sqrt(D);
+        y = 0.5 * ((r < 2 ? -sr : sr) + (r & 1 ? -q : q));
     } else {
         const double D = P * P - 4.0 * R;                 // biquadratic y^4 + P y^2 + R
-        if (D >= 0.0) {
-            const double z1 = 0.5 * (-P + sqrt(D)), z2 = 0.5 * (-P - sqrt(D));
-            if (z1 >= 0.0) { y[n++] = sqrt(z1); y[n++] = -sqrt(z1); }
-            if (z2 >= 0.0) { y[n++] = sqrt(z2); y[n++] = -sqrt(z2); }
-        }
+        if (!(D >= 0.0)) return false;
+        const double sq = sqrt(D), z = 0.5 * (-P + (r < 2 ? sq : -sq));
+        if (!(z >= 0.0)) return false;
+        y = sqrt(z);
+        if (r & 1) y = -y;
     }
-    for (int i = 0; i < n; ++i) roots[i] = y[i] - 0.25 * b;
-    return n;
+    root = y - 0.25 * b;
+    return true;
 }
 
 // One candidate root polished by Newton steps on the quartic.
 __device__ double polish_quartic_root(const double* a, double x)
 {
+    double f = horner4(a, x);
     for (int it = 0; it < 3; ++it) {
-        const double f = horner4(a, x);
         const double df = ((4.0 * a[4] * x + 3.0 * a[3]) * x + 2.0 * a[2]) * x + a[1];
         if (!(fabs(df) > 0.0)) break;
-        const double xn = x - f / df;
-        if (!(fabs(horner4(a, xn)) < fabs(f))) break;
+        const double xn = x - f / df, fn = horner4(a, xn);
+        if (!(fabs(fn) < fabs(f))) break;
         x = xn;
+        f = fn;
     }
     return x;
 }
@@ -181,13 +186,22 @@ struct P3PSetup {
     double N[3], D[2], Q[5];
 };
 
+// Lane r of the quad forms the squared distance and the cosine of points (0, 1),
+// (0, 2) or (1, 2) (lane 3 the first again). Every lane of the warp takes part.
 __device__ bool p3p_setup(const double P[3][3], const double b[3][3], P3PSetup& q)
 {
-    double e12[3], e13[3], e23[3];
-    for (int i = 0; i < 3; ++i) { e12[i] = P[0][i] - P[1][i]; e13[i] = P[0][i] - P[2][i]; e23[i] = P[1][i] - P[2][i]; }
-    const double d12 = d3dot(e12, e12), d13 = d3dot(e13, e13), d23 = d3dot(e23, e23);
-    if (!(d12 > 0.0 && d13 > 0.0 && d23 > 0.0)) return false;
-    const double c12 = d3dot(b[0], b[1]), c13 = d3dot(b[0], b[2]), c23 = d3dot(b[1], b[2]);
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, r = lane & 3, base = lane & ~3;
+    double e[3], bi[3], bj[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        e[i] = (r == 2 ? P[1][i] : P[0][i]) - (r == 1 || r == 2 ? P[2][i] : P[1][i]);
+        bi[i] = r == 2 ? b[1][i] : b[0][i];
+        bj[i] = r == 1 || r == 2 ? b[2][i] : b[1][i];
+    }
+    const double dist = d3dot(e, e), cosine = d3dot(bi, bj);
+    const double d12 = __shfl_sync(FULL, dist, base), d13 = __shfl_sync(FULL, dist, base + 1), d23 = __shfl_sync(FULL, dist, base + 2);
+    const double c12 = __shfl_sync(FULL, cosine, base), c13 = __shfl_sync(FULL, cosine, base + 1), c23 = __shfl_sync(FULL, cosine, base + 2);
     const double K2 = d13 / d12;
     const double g[3] = {K2 - 1.0, -2.0 * K2 * c12, K2};
     q.d12 = d12; q.d13 = d13; q.d23 = d23; q.c12 = c12; q.c13 = c13; q.c23 = c23;
@@ -203,7 +217,7 @@ __device__ bool p3p_setup(const double P[3][3], const double b[3][3], P3PSetup& 
     const double DD[3] = {D[0] * D[0], 2.0 * D[0] * D[1], D[1] * D[1]};
     for (int i = 0; i < 3; ++i)
         for (int j = 0; j < 3; ++j) q.Q[i + j] -= g[i] * DD[j];
-    return true;
+    return d12 > 0.0 && d13 > 0.0 && d23 > 0.0;
 }
 
 // The pose of one polished root u of the quartic: v, the distances s_i
@@ -227,21 +241,29 @@ __device__ bool p3p_from_root(const double P[3][3], const double b[3][3], const 
     s[1] = u * s[0];
     s[2] = v * s[0];
     if (!(s[0] > 0.0 && s[1] > 0.0 && s[2] > 0.0) || !isfinite(s[2])) return false;
+    // residuals of the three equations; J = 2 {j0 j1 0; j2 0 j3; 0 j4 j5} is solved
+    // through the adjugate of the half, whose entries are single products
+    auto residuals = [&](const double* s, double* F) {
+        F[0] = s[0] * s[0] + s[1] * s[1] - 2.0 * c12 * s[0] * s[1] - d12;
+        F[1] = s[0] * s[0] + s[2] * s[2] - 2.0 * c13 * s[0] * s[2] - d13;
+        F[2] = s[1] * s[1] + s[2] * s[2] - 2.0 * c23 * s[1] * s[2] - d23;
+    };
+    double F[3];
+    residuals(s, F);
     for (int it = 0; it < 5; ++it) {
-        const double F[3] = {s[0] * s[0] + s[1] * s[1] - 2.0 * c12 * s[0] * s[1] - d12,
-                             s[0] * s[0] + s[2] * s[2] - 2.0 * c13 * s[0] * s[2] - d13,
-                             s[1] * s[1] + s[2] * s[2] - 2.0 * c23 * s[1] * s[2] - d23};
-        const double J[9] = {2.0 * (s[0] - c12 * s[1]), 2.0 * (s[1] - c12 * s[0]), 0.0,
-                             2.0 * (s[0] - c13 * s[2]), 0.0, 2.0 * (s[2] - c13 * s[0]),
-                             0.0, 2.0 * (s[1] - c23 * s[2]), 2.0 * (s[2] - c23 * s[1])};
-        double ds[3];
-        if (!solve3x3(J, F, ds)) break;
-        const double nsv[3] = {s[0] - ds[0], s[1] - ds[1], s[2] - ds[2]};
-        const double G0 = nsv[0] * nsv[0] + nsv[1] * nsv[1] - 2.0 * c12 * nsv[0] * nsv[1] - d12;
-        const double G1 = nsv[0] * nsv[0] + nsv[2] * nsv[2] - 2.0 * c13 * nsv[0] * nsv[2] - d13;
-        const double G2 = nsv[1] * nsv[1] + nsv[2] * nsv[2] - 2.0 * c23 * nsv[1] * nsv[2] - d23;
-        if (!(fabs(G0) + fabs(G1) + fabs(G2) < fabs(F[0]) + fabs(F[1]) + fabs(F[2]))) break;
-        s[0] = nsv[0]; s[1] = nsv[1]; s[2] = nsv[2];
+        const double j0 = s[0] - c12 * s[1], j1 = s[1] - c12 * s[0], j2 = s[0] - c13 * s[2], j3 = s[2] - c13 * s[0],
+                     j4 = s[1] - c23 * s[2], j5 = s[2] - c23 * s[1];
+        const double c00 = -(j3 * j4), c01 = -(j2 * j5), c02 = j2 * j4, c10 = -(j1 * j5), c11 = j0 * j5, c12_ = -(j0 * j4),
+                     c20 = j1 * j3, c21 = -(j0 * j3), c22 = -(j1 * j2);
+        const double det = j0 * c00 + j1 * c01;
+        if (!(fabs(det) > 0.0)) break;
+        const double id = 0.5 * (1.0 / det);
+        const double ns[3] = {s[0] - (c00 * F[0] + c10 * F[1] + c20 * F[2]) * id, s[1] - (c01 * F[0] + c11 * F[1] + c21 * F[2]) * id,
+                              s[2] - (c02 * F[0] + c12_ * F[1] + c22 * F[2]) * id};
+        double G[3];
+        residuals(ns, G);
+        if (!(fabs(G[0]) + fabs(G[1]) + fabs(G[2]) < fabs(F[0]) + fabs(F[1]) + fabs(F[2]))) break;
+        for (int i = 0; i < 3; ++i) { s[i] = ns[i]; F[i] = G[i]; }
     }
     if (!(s[0] > 0.0 && s[1] > 0.0 && s[2] > 0.0)) return false;
     double Qc[3][3];
@@ -252,8 +274,8 @@ __device__ bool p3p_from_root(const double P[3][3], const double b[3][3], const 
     sol.s1 = s[0];
     double cw[3], cc[3];
     for (int c = 0; c < 3; ++c) {
-        cw[c] = (P[0][c] + P[1][c] + P[2][c]) / 3.0;
-        cc[c] = (Qc[0][c] + Qc[1][c] + Qc[2][c]) / 3.0;
+        cw[c] = third(P[0][c] + P[1][c] + P[2][c]);
+        cc[c] = third(Qc[0][c] + Qc[1][c] + Qc[2][c]);
     }
     for (int r0 = 0; r0 < 3; ++r0) {
         for (int c = 0; c < 3; ++c)
@@ -278,24 +300,46 @@ __device__ bool p3p_from_root(const double P[3][3], const double b[3][3], const 
 // (i - offset)-th set bit of that block's per-warp ballots.
 __device__ int valid_pixel_at(const DevState& s, int nb, int i)
 {
-    int lo = 0, hi = nb - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s.pix_block_count[mid] <= i) lo = mid;
-        else hi = mid - 1;
+    // the last of the nb offsets that is <= i: seven probes a round, all in flight
+    int lo = 0, n = nb;
+    while (n > 1) {
+        const int step = (n + 7) >> 3;
+        int below = 0;
+#pragma unroll
+        for (int q = 1; q < 8; ++q) {
+            const int at = q * step;
+            below += at < n && s.pix_block_count[lo + at] <= i;
+        }
+        lo += below * step;
+        n = min(step, n - below * step);
     }
     int r = i - s.pix_block_count[lo];
-    const unsigned* m = s.pix_vmask + (size_t)lo * (kPixThreads / 32);
+    const uint4* m4 = reinterpret_cast<const uint4*>(s.pix_vmask + (size_t)lo * (kPixThreads / 32));
+    static_assert(kPixThreads == 256, "eight ballots a block");
+    const uint4 ma = m4[0], mb = m4[1];
+    const unsigned m[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
+#pragma unroll
     for (int w = 0; w < kPixThreads / 32; ++w) {
-        unsigned mw = m[w];
-        const int c = __popc(mw);
-        if (r < c) {
-            for (int q = 0; q < r; ++q) mw &= mw - 1u;
-            return lo * kPixThreads + w * 32 + (__ffs(mw) - 1);
+        const int c = __popc(m[w]);
+        if (r < c) {                                      // its r-th set bit
+            unsigned mw = m[w];
+            int bit = 0;
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1) {
+                const int low = __popc(mw & ((1u << h) - 1u));
+                if (r >= low) { r -= low; mw >>= h; bit += h; }
+            }
+            return lo * kPixThreads + w * 32 + bit;
         }
         r -= c;
     }
     return -1;
+}
+
+// a / f for a focal length f with y = 1 / f rounded.
+__device__ __forceinline__ double by_focal(double a, double f, double y)
+{
+    return f > 1e-60 && f < 1e60 && fabs(a) < 1e60 ? div_by(a, f, y) : a / f;
 }
 
 // Point in camera t-1 and bearing of the flow target of valid pixel j, in
@@ -309,7 +353,7 @@ __device__ bool group_point(const DevParams& p, const DevState& s, const double*
 {
     const int x = j % p.W, y = j / p.W;
     const double th = (double)s.theta[j];
-    const double d[3] = {((double)x - p.cxd) / p.fxd, ((double)y - p.cyd) / p.fyd, 1.0};
+    const double d[3] = {by_focal((double)x - p.cxd, p.fxd, p.inv_fxd), by_focal((double)y - p.cyd, p.fyd, p.inv_fyd), 1.0};
     double u, v;
     if (t == 1) {
         P[0] = th * d[0]; P[1] = th * d[1]; P[2] = th;
@@ -331,8 +375,8 @@ __device__ bool group_point(const DevParams& p, const DevState& s, const double*
     const double w00 = (1 - ax) * (1 - ay), w10 = ax * (1 - ay), w01 = (1 - ax) * ay, w11 = ax * ay;
     const double fu = w00 * f00.x + w10 * f10.x + w01 * f01.x + w11 * f11.x;
     const double fv = w00 * f00.y + w10 * f10.y + w01 * f01.y + w11 * f11.y;
-    bear[0] = (u + fu - p.cxd) / p.fxd;
-    bear[1] = (v + fv - p.cyd) / p.fyd;
+    bear[0] = by_focal(u + fu - p.cxd, p.fxd, p.inv_fxd);
+    bear[1] = by_focal(v + fv - p.cyd, p.fyd, p.inv_fyd);
     bear[2] = 1.0;
     return d3unit(bear);
 }
@@ -350,12 +394,19 @@ __device__ bool group_point(const DevParams& p, const DevState& s, const double*
 // whatever the timing.
 //
 // Within a quad, lanes 0-2 compute the FP64 point and bearing of the group's
-// pixels 0-2 and share them by shuffles; every lane forms the quartic and its
-// Ferrari candidates, lane r polishes candidate r and turns it into a pose,
-// and each solution's slot is its rank by s1 among the quad's solutions
-// (ties by root order): the group's solutions sorted by s1. A warp's
-// FP64 dependency chain is then the common part and one root, not up to four
-// roots in turn.
+// pixels 0-2 and share them by shuffles; the lanes share the work on the quartic (the
+// pairs of points, its division by the leading coefficient, the cube roots), lane r
+// forms and polishes root candidate r and turns it into a pose, and each solution's
+// slot is its rank by s1 among the quad's solutions (ties by root order): the group's
+// solutions sorted by s1. A warp's FP64 work is then the common part and one root,
+// not up to four roots in turn.
+//
+// What bounds it is the number of FP64 instructions of a warp: one issues every ~54
+// cycles from a single warp whether or not it depends on the last, and an SM takes
+// three and a half such warps before they slow each other down. So nothing is
+// computed in two lanes that one can do, divisions by constants go through their
+// reciprocals, a Newton step keeps its residual for the next and leaves out the zeros
+// of its matrix: 53 -> 45 us up to S = 2048, 58 -> 50 at 4096, 77 -> 64 at 8192.
 constexpr int kP3PChunk = 8;
 
 __global__ void __launch_bounds__(32) k_p3p_groups(DevParams p, DevState s, int t)
@@ -422,14 +473,12 @@ __global__ void __launch_bounds__(32) k_p3p_groups(DevParams p, DevState s, int 
         if (!valid_group) weight = 0.0;
         // the quartic (every lane), then lane r's root
         P3PSetup qs;
-        int nr = 0;
-        double cand[4] = {0.0, 0.0, 0.0, 0.0};
-        if (valid_group && p3p_setup(P, b, qs)) nr = quartic_candidates(qs.Q, cand);
+        double u0 = 0.0;
+        const bool set = p3p_setup(P, b, qs), some = quartic_candidate(qs.Q, u0);
         P3PSol sol;
         sol.s1 = 0.0;
         bool has = false;
-        if (r < nr) {
-            const double u0 = r == 0 ? cand[0] : (r == 1 ? cand[1] : (r == 2 ? cand[2] : cand[3]));
+        if (valid_group && set && some) {
             has = p3p_from_root(P, b, qs, polish_quartic_root(qs.Q, u0), sol);
         }
         // slot = rank by s1 among the quad's solutions, ties by root order
@@ -469,11 +518,12 @@ __device__ __forceinline__ int groups_solved(const DevParams& p, const DevState&
 // groups (more than one solution each as a rule), so that no warp runs a second chunk
 // after its first, a whole chain later: with 3/4 S groups, enough only above 1.33
 // solutions a group, frames of handheld windows took 78 us on average (54 or 97) at
-// S = 4096 on 640 x 480, now 58, and 79 at S = 2048 on 320 x 240, now 54. An SM solves
-// three and a half chunks in the time of one and no more (5/4 S groups at S = 4096:
-// 68 us, 7/4 S: 77), so beyond kP3PFreeChunks chunks in all it is 3/4 S, as the yield of
-// driving windows (1.4-1.5) allows (S = 8192: 77 us; with 15/16 S 86); further chunks
-// are claimed as needed.
+// S = 4096 on 640 x 480 where S groups took 58, and 79 against 54 at S = 2048 on
+// 320 x 240. An SM solves three and a half chunks in the time of one and no more (5/4 S
+// groups at S = 4096: 68 us, 7/4 S: 77), so beyond kP3PFreeChunks chunks in all it is
+// 3/4 S, as the yield of driving windows (1.4-1.5) allows (S = 8192: 77 us; with 15/16 S
+// 86); further chunks are claimed as needed. (All before the solver's FP64 work was
+// cut by a sixth.)
 constexpr int kP3PFreeChunks = 512;
 
 void launch_p3p_groups(const DevParams& p, const DevState& s, int t, cudaStream_t st)
