@@ -279,9 +279,13 @@ __device__ __forceinline__ float depth_ell_fast(const DevParams& p, const float*
 //   runs     per pixel r (in parallel): test own_r at r+1, r+2, ... until it
 //            loses, at most kRunCap positions (speculation);
 //   resolve  per chain: follow r -> end of run from the chain start; a run
-//            that reached the cap is continued on the fly.
+//            that reached the cap is continued there.
 // ---------------------------------------------------------------------------
-constexpr int kRunCap = 8;
+// Speculation pays where neighbouring pixels' tests share a warp's time, and costs where
+// one lane of it goes on alone: runs + resolve take 43 + 137 us with a cap of 1, 71 + 108
+// with 2, 97 + 95 with 3, 120 + 88 with 4 and 140 + 57 with 8 (1242 x 375, T = 8), and
+// 31, 29, 29, 31 and 39 us together on 160 x 120.
+constexpr int kRunCap = 2;
 
 __device__ __forceinline__ float nan_to_ninf(float v) { return isnan(v) ? -INFINITY : v; }
 
@@ -292,6 +296,32 @@ __device__ __forceinline__ float mie_score(const DevParams& p, const DevState& s
     for (int t = 1; t <= p.T; ++t) {
         const float q = s.qs[(size_t)(t - 1) * p.N + j];
         acc = __fadd_rn(acc, __fmul_rn(q, depth_ell_fast(p, f.v[t - 1], s.flows, t, x, y, d)));
+    }
+    return nan_to_ninf(acc);
+}
+
+// Under MIE no term of S is positive (log rho / (rho + mu), weights >= 0), so a partial
+// sum only falls: once it is at most `limit` the whole is too. True if pixel j's
+// weights allow that conclusion.
+__device__ __forceinline__ bool falling(const DevParams& p, const DevState& s, int j)
+{
+    bool ok = p.criterion != VOLDOR_CRITERION_MLE;
+    for (int t = 0; t < p.T; ++t) ok &= s.qs[(size_t)t * p.N + j] >= 0.f;
+    return ok;
+}
+
+// S(d), or some partial sum at most `limit` where S(d) is at most `limit` too (then
+// only that it loses against `limit` is of interest).
+__device__ __forceinline__ float mie_score_above(const DevParams& p, const DevState& s, const FramesF& f, int x, int y, float d,
+                                                 float limit)
+{
+    const int j = y * p.W + x;
+    const bool stop = falling(p, s, j);
+    float acc = 0.f;
+    for (int t = 1; t <= p.T; ++t) {
+        const float q = s.qs[(size_t)(t - 1) * p.N + j];
+        acc = __fadd_rn(acc, __fmul_rn(q, depth_ell_fast(p, f.v[t - 1], s.flows, t, x, y, d)));
+        if (stop && acc <= limit) break;
     }
     return nan_to_ninf(acc);
 }
@@ -323,9 +353,10 @@ __global__ void k_mie_prepare(DevParams p, DevState s)
     const U64x4 r = philox4x64_10((uint64_t)j, 0ull, (uint64_t)k, (uint64_t)kStreamDepth, p.seed, p.window_id);
     const float u = (float)(r.v[0] >> 40) * (1.f / 16777216.f);
     const float smp = 1.f / fmaf(u, p.inv_depth_max - p.inv_depth_min, p.inv_depth_min);
-    s.mie_prev_score[j] = mie_score(p, s, f, x, y, s.theta[j]);
+    const float prev = mie_score(p, s, f, x, y, s.theta[j]);
+    s.mie_prev_score[j] = prev;
     s.mie_smp[j] = smp;
-    s.mie_smp_score[j] = mie_score(p, s, f, x, y, smp);
+    s.mie_smp_score[j] = mie_score_above(p, s, f, x, y, smp, prev);   // below S(prev) its value has no effect
 }
 
 // own value of pixel j (before the sweep overwrites theta)
@@ -360,80 +391,128 @@ __global__ void k_mie_runs(DevParams p, DevState s)
     s.mie_next[j] = (steps == kRunCap && e < len) ? -e : e;
 }
 
-constexpr int kResolveThreads = 128;
+constexpr int kResolveWarps = 16, kResolveThreads = 32 * kResolveWarps;
 constexpr int kMaxChain = kMaxImageSide;
 
-// Resolution of one chain per block. All threads walk the run ends in
-// lockstep from the chain start (uniform control flow); a run whose
-// speculation reached the cap is continued kResolveThreads positions at a
-// time, each thread testing one position; the run's positions are filled in
-// parallel.
+// End of the run of own_r, which survived up to position `pos` of chain c: a warp tests
+// 32 / G positions at a time, G lanes to a position, a frame each (two from T = 9 on);
+// the frames' terms are independent, only their sum is in order.
+__device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, float v)
+{
+    const int lane = threadIdx.x & 31, G = p.T > 4 ? 8 : (p.T > 2 ? 4 : p.T), sub = lane % G, first = lane - sub;
+    for (;; pos += 32 / G) {
+        const int q = pos + lane / G;
+        int x, y;
+        chain_xy(p, dir, c, min(q, len - 1), x, y);
+        const int j = y * p.W + x;
+        float term[2] = {0.f, 0.f};
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int t = u * G + sub + 1;
+            if (t <= p.T) term[u] = __fmul_rn(s.qs[(size_t)(t - 1) * p.N + j], depth_ell_fast(p, f.v[t - 1], s.flows, t, x, y, v));
+        }
+        float acc = 0.f;
+        for (int t = 0; t < p.T; ++t) acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, t < G ? term[0] : term[1], first + t % G));
+        const unsigned lost = __ballot_sync(0xffffffffu, q >= len || !survives(s, j, nan_to_ninf(acc)));
+        if (lost) return min(pos + (__ffs(lost) - 1) / G, len);
+    }
+}
+
+// Resolution of one chain per block. The walk r -> end of r's run depends on nothing
+// but r, so walks from different positions join at the first reset they share. Each
+// warp first walks its own part of the chain from the part's first position, and
+// whatever a run that reached the cap costs is paid by the warps side by side; then
+// warp 0 follows the true walk from one part to the next, step by step until it meets
+// the part's own walk, from there on by its result. A chain's runs one after another,
+// tested by the whole block, took 212 us at 1242 x 375, T = 8; with the parts 57, and
+// 108 with a cap of 2 instead of 8 (see kRunCap). 8 parts: 101, 32: 146.
 __global__ void __launch_bounds__(kResolveThreads) k_mie_resolve(DevParams p, DevState s)
 {
     __shared__ FramesF f;
     __shared__ short origin[kMaxChain];
     __shared__ int next_s[kMaxChain];
-    __shared__ int first_fail;
+    __shared__ float own_s[kMaxChain];
+    __shared__ unsigned char reset[kMaxChain];             // 1: on the part's own walk, 2: on the true one before they meet
+    __shared__ int part_end[kResolveWarps], part_from[kResolveWarps], last_s[kResolveWarps];
     load_frames32(p, s, f);
     const int dir = (*s.iter) & 3;
     const bool rows = (dir == 0 || dir == 2);
     const int n_chains = rows ? p.H : p.W;
     const int len = rows ? p.W : p.H;
-    const int c = blockIdx.x;
+    const int c = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (c >= n_chains) return;
     for (int q = threadIdx.x; q < len; q += kResolveThreads) {
         int x, y;
         chain_xy(p, dir, c, q, x, y);
         next_s[q] = s.mie_next[y * p.W + x];
+        own_s[q] = own_value(s, y * p.W + x);
+        reset[q] = 0;
     }
     __syncthreads();
-    int r = 0;
-    while (r < len) {
+    // the end of r's run, kept for the next to ask
+    auto end_of = [&](int r) {
         int e = next_s[r];
-        if (e < 0) {                           // speculation capped: continue block-parallel
-            int xr, yr;
-            chain_xy(p, dir, c, r, xr, yr);
-            const float v = own_value(s, yr * p.W + xr);
-            int pos = -e;
-            while (true) {
-                if (threadIdx.x == 0) first_fail = len;
-                __syncthreads();
-                const int q = pos + (int)threadIdx.x;
-                if (q < len) {
-                    int xe, ye;
-                    chain_xy(p, dir, c, q, xe, ye);
-                    if (!survives(s, ye * p.W + xe, mie_score(p, s, f, xe, ye, v))) atomicMin(&first_fail, q);
-                }
-                __syncthreads();
-                const int ff = first_fail;
-                __syncthreads();
-                if (ff < len || pos + kResolveThreads >= len) { e = ff < len ? ff : len; break; }
-                pos += kResolveThreads;
-            }
+        if (e < 0) {
+            e = mie_run_end(p, s, f, dir, c, len, -e, own_s[r]);
+            __syncwarp();
+            if (lane == 0) next_s[r] = e;
+            __syncwarp();
         }
-        for (int q = r + (int)threadIdx.x; q < e; q += kResolveThreads) origin[q] = (short)r;
-        r = e;
+        return e;
+    };
+    const int part = (len + kResolveWarps - 1) / kResolveWarps;
+    {
+        const int stop = min((warp + 1) * part, len);
+        int r = min(warp * part, len);
+        while (r < stop) {
+            if (lane == 0) reset[r] = 1;
+            r = end_of(r);
+        }
+        if (lane == 0) part_end[warp] = r;
     }
     __syncthreads();
-    // new depths and labels; read every own value before any theta is written
-    float vals[kMaxChain / kResolveThreads];
-    unsigned char labs[kMaxChain / kResolveThreads];
-    int n = 0;
-    for (int q = threadIdx.x; q < len; q += kResolveThreads, ++n) {
-        int x, y;
-        chain_xy(p, dir, c, origin[q], x, y);
-        const int jo = y * p.W + x;
-        vals[n] = own_value(s, jo);
-        labs[n] = (origin[q] != q) ? 1 : (s.mie_smp_score[jo] > s.mie_prev_score[jo] ? 2 : 0);
+    if (warp == 0) {
+        int r = 0;
+        for (int k = 0; k < kResolveWarps; ++k) {
+            const int stop = min((k + 1) * part, len);
+            while (r < stop && reset[r] != 1) {
+                if (lane == 0) reset[r] = 2;
+                r = end_of(r);
+            }
+            if (lane == 0) part_from[k] = r < stop ? r : len;
+            if (r < stop) r = part_end[k];
+        }
     }
     __syncthreads();
-    n = 0;
-    for (int q = threadIdx.x; q < len; q += kResolveThreads, ++n) {
+    // origin of each position: the last reset of the true walk up to it, a contiguous
+    // piece per thread, then a scan over the pieces
+    const int per = (len + kResolveThreads - 1) / kResolveThreads, q0 = threadIdx.x * per, q1 = min(q0 + per, len);
+    auto is_reset = [&](int q) { return reset[q] == 2 || (reset[q] == 1 && q >= part_from[q / part]); };
+    int last = -1;
+    for (int q = q0; q < q1; ++q)
+        if (is_reset(q)) last = q;
+    int before = last;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before = max(before, v);
+    }
+    if (lane == 31) last_s[warp] = before;
+    before = __shfl_up_sync(0xffffffffu, before, 1);
+    if (lane == 0) before = -1;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) before = max(before, last_s[w]);
+    for (int q = q0; q < q1; ++q) {
+        if (is_reset(q)) before = q;
+        origin[q] = (short)before;
+    }
+    __syncthreads();
+    // new depths and labels (the chain's own values are in shared memory)
+    for (int q = threadIdx.x; q < len; q += kResolveThreads) {
         int x, y;
         chain_xy(p, dir, c, q, x, y);
         const int j = y * p.W + x;
-        s.theta[j] = vals[n];
-        s.labels[j] = labs[n];
+        s.theta[j] = own_s[origin[q]];
+        s.labels[j] = origin[q] != q ? 1 : (s.mie_smp_score[j] > s.mie_prev_score[j] ? 2 : 0);
     }
 }
 
