@@ -322,7 +322,21 @@ void launch_emissions(const DevParams& p, const DevState& s, float* out, cudaStr
 // product of the segments before it (forward) or after it (backward), and
 // each lane then walks its own segment with the step-by-step recursion from
 // the message entering it.
+//
+// A block stages kFbChains neighbouring chains in shared memory, emissions and forward
+// messages, and moves them between there and global memory in whole rows (or, along
+// columns, kFbChains columns of a row at a time): with the lanes' strided accesses in
+// global memory the kernel took 107 us at 1242 x 375, T = 8; now 73. What bounds it
+// now: the latency of a step (up to two divisions) times four passes over a segment,
+// with the twelve chains an SM holds.
 // ---------------------------------------------------------------------------
+constexpr int kFbChains = 4;
+
+// Floats of a chain's row in shared memory: 32 segments, padded to an odd length so
+// that the lanes' steps fall into different banks.
+__host__ __device__ constexpr int fb_segment(int len) { return (len + 31) / 32; }
+__host__ __device__ constexpr int fb_row(int len) { return 32 * (fb_segment(len) | 1); }
+
 struct M22 {
     float a, b, c, d;   // [[a, b], [c, d]]
 };
@@ -351,29 +365,20 @@ __device__ __forceinline__ M22 m22_shfl(const M22& x, int src_delta, bool up)
     return r;
 }
 
-__global__ void __launch_bounds__(256) k_forward_backward(DevParams p, DevState s)
+// One chain by a warp: its emissions in shared memory are replaced by q. e, fw: the
+// lane's segment (e[LP] is the next lane's first element).
+__device__ __forceinline__ void fb_chain(const DevParams& p, int len, float* e, float2* fw, const float* chain)
 {
-    const int dir = (*s.iter) & 3;
-    const bool rows = (dir == 0 || dir == 2);
-    const int n_chains = rows ? p.H : p.W;
-    const int len = rows ? p.W : p.H;
-    const int stride = rows ? 1 : p.W;
     const int lane = threadIdx.x & 31;
-    const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (id >= p.T * n_chains) return;                // whole warps leave together
-    const int t = id / n_chains, c = id % n_chains;
-    const size_t base = (size_t)t * p.N + (rows ? (size_t)c * p.W : (size_t)c);
-    float* e = s.qs + base;
-    float2* fw = reinterpret_cast<float2*>(s.fb_fwd) + base;
     const float g = p.gamma, h = 1.f - p.gamma;
-    const int L = (len + 31) / 32;
+    const int L = fb_segment(len), LP = L | 1;
     const int i0 = min(lane * L, len), i1 = min(i0 + L, len);    // this lane's segment [i0, i1)
     const bool has = i0 < i1;
 
     // ---- forward: segment products of diag(e_i) A for i in [max(i0, 1), i1)
     M22 P{1.f, 0.f, 0.f, 1.f};
     for (int i = (i0 > 0 ? i0 : 1); i < i1; ++i) {
-        const float w = e[(size_t)i * stride];
+        const float w = e[i - i0];
         const M22 Mi{(1.f - w) * g, (1.f - w) * h, w * h, w * g};
         P = m22_mul(Mi, P);
     }
@@ -386,7 +391,7 @@ __global__ void __launch_bounds__(256) k_forward_backward(DevParams p, DevState 
     const M22 Sprev = m22_shfl(S, 1, true);          // S_{k-1}
     float f0, f1;
     {
-        const float w = e[0];
+        const float w = chain[0];
         const float a0 = 1.f - w, a1 = w, sum = a0 + a1;
         f0 = a0 / sum;
         f1 = a1 / sum;
@@ -403,12 +408,12 @@ __global__ void __launch_bounds__(256) k_forward_backward(DevParams p, DevState 
             i = 1;
         }
         for (; i < i1; ++i) {
-            const float w = e[(size_t)i * stride];
+            const float w = e[i - i0];
             const float p0 = g * f0 + h * f1, p1 = h * f0 + g * f1;
             const float a0 = (1.f - w) * p0, a1 = w * p1, sum = a0 + a1;
             f0 = a0 / sum;
             f1 = a1 / sum;
-            fw[(size_t)i * stride] = make_float2(f0, f1);
+            fw[i - i0] = make_float2(f0, f1);
         }
     }
 
@@ -416,12 +421,12 @@ __global__ void __launch_bounds__(256) k_forward_backward(DevParams p, DevState 
     const int j1 = min(i1, len - 1);
     M22 R{1.f, 0.f, 0.f, 1.f};
     for (int i = j1 - 1; i >= i0; --i) {
-        const float w = e[(size_t)(i + 1) * stride];
+        const float w = i + 1 < i1 ? e[i + 1 - i0] : e[LP];
         const M22 Ni{g * (1.f - w), h * w, h * (1.f - w), g * w};
         R = m22_mul(Ni, R);                           // N_i ... N_{j1 - 1}
     }
     // the emission just past this segment, read before any lane writes q
-    const float w_after = i1 < len ? e[(size_t)i1 * stride] : 0.f;
+    const float w_after = i1 < len ? e[LP] : 0.f;
     // suffix scan: U_k = R_k R_{k+1} ... R_31
     M22 U = R;
     for (int d = 1; d < 32; d <<= 1) {
@@ -440,10 +445,10 @@ __global__ void __launch_bounds__(256) k_forward_backward(DevParams p, DevState 
         float w_next = w_after;
         int i = i1 - 1;
         if (i1 == len) {                               // the chain's last element: b = 1
-            w_next = e[(size_t)i * stride];
-            const float2 f = fw[(size_t)i * stride];
+            w_next = e[i - i0];
+            const float2 f = fw[i - i0];
             const float q0 = f.x * b0, q1 = f.y * b1;
-            e[(size_t)i * stride] = q1 / (q0 + q1);
+            e[i - i0] = q1 / (q0 + q1);
             --i;
         }
         for (; i >= i0; --i) {
@@ -451,18 +456,55 @@ __global__ void __launch_bounds__(256) k_forward_backward(DevParams p, DevState 
             const float n0 = g * c0 + h * c1, n1 = h * c0 + g * c1, sum = n0 + n1;
             b0 = n0 / sum;
             b1 = n1 / sum;
-            w_next = e[(size_t)i * stride];
-            const float2 f = fw[(size_t)i * stride];
+            w_next = e[i - i0];
+            const float2 f = fw[i - i0];
             const float q0 = f.x * b0, q1 = f.y * b1;
-            e[(size_t)i * stride] = q1 / (q0 + q1);
+            e[i - i0] = q1 / (q0 + q1);
         }
     }
 }
 
+// grid (groups of chains, frame)
+__global__ void __launch_bounds__(32 * kFbChains) k_forward_backward(DevParams p, DevState s)
+{
+    extern __shared__ float fb_smem[];
+    const int dir = (*s.iter) & 3;
+    const bool rows = (dir == 0 || dir == 2);
+    const int n_chains = rows ? p.H : p.W;
+    const int len = rows ? p.W : p.H;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * kFbChains, here = min(kFbChains, n_chains - c0);
+    if (here <= 0) return;
+    const int L = fb_segment(len), LP = L | 1, row = fb_row(len);
+    float* q = s.qs + (size_t)blockIdx.y * p.N + (rows ? (size_t)c0 * p.W : (size_t)c0);
+    // element i of chain k: es(k)[i + (i / L) (LP - L)]
+    auto for_all = [&](auto&& f) {
+        if (rows) {
+            if (warp < here)
+                for (int i = lane; i < len; i += 32) f(q + (size_t)warp * p.W + i, fb_smem + 3 * row * warp + i + i / L * (LP - L));
+        } else {
+            for (int n = threadIdx.x; n < len * kFbChains; n += 32 * kFbChains) {
+                const int i = n / kFbChains, k = n % kFbChains;
+                if (k < here) f(q + (size_t)i * p.W + k, fb_smem + 3 * row * k + i + i / L * (LP - L));
+            }
+        }
+    };
+    for_all([](float* g, float* m) { *m = *g; });
+    __syncthreads();
+    if (warp < here) {
+        float* es = fb_smem + 3 * row * warp;
+        fb_chain(p, len, es + lane * LP, reinterpret_cast<float2*>(es + row) + lane * LP, es);
+    }
+    __syncthreads();
+    for_all([](float* g, float* m) { *g = *m; });
+}
+
 void launch_forward_backward(const DevParams& p, const DevState& s, cudaStream_t st)
 {
-    const int n = p.T * (p.H > p.W ? p.H : p.W);      // chains (warps) of the longer count
-    k_forward_backward<<<(n + 7) / 8, 256, 0, st>>>(p, s);
+    const int most = p.H > p.W ? p.H : p.W;               // chains in one direction, their length in the other
+    const int smem = kFbChains * 3 * fb_row(most) * (int)sizeof(float);
+    cudaFuncSetAttribute(k_forward_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_forward_backward<<<dim3((most + kFbChains - 1) / kFbChains, p.T), 32 * kFbChains, smem, st>>>(p, s);
 }
 
 }  // namespace vd

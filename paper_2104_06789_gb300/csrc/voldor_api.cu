@@ -175,7 +175,6 @@ size_t layout(voldor_ctx& c, char* base)
     s.mie_smp_score = (float*)take(N * 4);
     s.mie_next = (int*)take(N * 4);
     s.labels = (unsigned char*)take(N);
-    s.fb_fwd = (float*)take(T * N * 8);
     s.score_log = (long long*)take((size_t)kScoreLogMax * 2 * 8);
     s.n_chunks = chunks;
     s.score_hpt = kScoreDefaultHpt;

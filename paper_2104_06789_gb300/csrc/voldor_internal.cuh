@@ -111,7 +111,6 @@ struct DevState {
     float* mie_smp_score;     // [N]
     int* mie_next;            // [N] end of each pixel's speculative run (chain position), negative if capped
     unsigned char* labels;    // [N]
-    float* fb_fwd;            // [T][H][W] forward messages
     long long* score_log;     // [kScoreLogMax][2] (n_hyp, n_pix) of timed scoring launches
     int n_chunks;             // dense scoring pixel chunks
     int score_hpt;            // hypotheses a scoring thread takes from tensor memory at a time (2, 4 or 8)
