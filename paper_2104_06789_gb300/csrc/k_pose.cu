@@ -608,16 +608,20 @@ __device__ void se3_exp_vec(const double* p6, double* Rt)
     Rt[11] = rho[2] + B * a[2] + C * b[2];
 }
 
-// Hypothesis collection: one thread per (group, solution slot) writes its
+// Hypothesis collection: four lanes per (group, solution slot), one for each row of
+// [R | t], write its
 // solution h = offset + slot < S with its scoring form and tensor-core operand.
-// A block covers 32 groups and finds its offset itself, as the sum of all earlier
+// A block covers 8 groups and finds its offset itself, as the sum of all earlier
 // groups' counts: up to 24 KB of counts read from L2 per block take less time than
 // a scan kernel before this one (4 us and a launch per frame).
-constexpr int kHypGroups = 32;             // groups per block
+// A lane per solution, with all of its FP64 work, took 10.7 us at S = 256 (14.6 at
+// 8192), four lanes with 32 groups to a block, all on one SM, 12.2 (19.1); now 7.5 (14.5).
+constexpr int kHypGroups = 8;              // groups per block
+constexpr int kHypThreads = kHypGroups * kMaxSols * 4;
 
-__global__ void __launch_bounds__(kHypGroups * kMaxSols) k_hyp_write(DevParams p, DevState s, int t)
+__global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState s, int t)
 {
-    __shared__ int wsum[kHypGroups * kMaxSols / 32], off_s[kHypGroups];
+    __shared__ int wsum[kHypThreads / 32], off_s[kHypGroups];
     __shared__ double e0[12];
     const int tid = threadIdx.x, lane = tid & 31;
     const int G = groups_solved(p, s), g0 = blockIdx.x * kHypGroups;
@@ -626,8 +630,10 @@ __global__ void __launch_bounds__(kHypGroups * kMaxSols) k_hyp_write(DevParams p
     const double sc[3] = {1.0, q, 1.0};
     if (tid < 12) {                                       // the frame's current pose in scaled form, {E, t}
         const double* T0 = s.poses + 12 * (t - 1);
-        const int r = tid / 3, c = tid % 3;
-        e0[tid] = tid < 9 ? sc[r] * (T0[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c] : sc[tid - 9] * T0[(tid - 9) * 4 + 3];
+        const int r = tid < 9 ? tid / 3 : tid - 9, c = tid < 9 ? tid % 3 : 3;
+        double v = T0[r * 4 + c] - (r == c ? 1.0 : 0.0);
+        if (q != 1.0) v = c < 3 ? sc[r] * v / sc[c] : sc[r] * v;     // square pixels need no scaling
+        e0[r * 4 + c] = v;
     }
     int before = 0;
     for (int i = tid; i < g0 / 4; i += blockDim.x) {
@@ -639,44 +645,46 @@ __global__ void __launch_bounds__(kHypGroups * kMaxSols) k_hyp_write(DevParams p
     __syncthreads();
     if (tid < 32) {
         int base = 0;
-        for (int w = 0; w < kHypGroups * kMaxSols / 32; ++w) base += wsum[w];
-        const int c = g0 + tid < G ? s.grp_count[g0 + tid] : 0;
+        for (int w = 0; w < kHypThreads / 32; ++w) base += wsum[w];
+        const int c = tid < kHypGroups && g0 + tid < G ? s.grp_count[g0 + tid] : 0;
         int incl = c;
         for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
         }
-        off_s[tid] = base + incl - c;
+        if (tid < kHypGroups) off_s[tid] = base + incl - c;
         if (tid == 31 && g0 + kHypGroups >= G) *s.n_hyp = min(base + incl, p.S);   // the last block with groups
     }
     __syncthreads();
-    const int g = g0 + tid / kMaxSols, i = tid % kMaxSols;
-    if (g >= G || i >= s.grp_count[g]) return;
-    const int h = off_s[tid / kMaxSols] + i;
+    const int item = tid >> 2, r = min(tid & 3, 2), g = g0 + item / kMaxSols, i = item % kMaxSols;
+    if (g >= G || i >= s.grp_count[g]) return;            // whole quads leave together
+    const int h = off_s[item / kMaxSols] + i;
     if (h >= p.S) return;
-    const double* Rt = s.grp_sols + ((size_t)g * kMaxSols + i) * 12;
-    double* oR = s.hyp_Rt + (size_t)h * 12;
-    float* f = s.hyp_f32 + (size_t)h * 12;
-    double e[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) {
-            oR[r * 3 + c] = Rt[r * 4 + c];
-            e[r * 3 + c] = Rt[r * 4 + c] - (r == c ? 1.0 : 0.0);
-        }
-        oR[9 + r] = Rt[r * 4 + 3];
-        e[9 + r] = Rt[r * 4 + 3];
+    const double* Rt = s.grp_sols + ((size_t)g * kMaxSols + i) * 12 + r * 4;
+    double v[4], e[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        v[c] = Rt[c];
+        e[c] = v[c] - (r == c ? 1.0 : 0.0);
     }
     if (q != 1.0) {                        // square pixels need no scaling, and FP64 divisions are long here
-        for (int r = 0; r < 3; ++r) {
-            for (int c = 0; c < 3; ++c) e[r * 3 + c] = sc[r] * e[r * 3 + c] / sc[c];
-            e[9 + r] = sc[r] * e[9 + r];
-        }
+        for (int c = 0; c < 3; ++c) e[c] = sc[r] * e[c] / sc[c];
+        e[3] = sc[r] * e[3];
     }
-    for (int c = 0; c < 12; ++c) f[c] = (float)e[c];
-    if (write_hyp_operand(s.sc_hyp, h, e, e0)) atomicOr(s.sc_wild, 1);
-    s.hyp_w[h] = s.grp_weight[g];
-    s.hyp_info[(size_t)h * 2 + 0] = g;
-    s.hyp_info[(size_t)h * 2 + 1] = i;
+    if ((tid & 3) < 3) {
+        double* oR = s.hyp_Rt + (size_t)h * 12;
+        float* f = s.hyp_f32 + (size_t)h * 12;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            oR[c < 3 ? r * 3 + c : 9 + r] = v[c];
+            f[c < 3 ? r * 3 + c : 9 + r] = (float)e[c];
+        }
+    } else {
+        s.hyp_w[h] = s.grp_weight[g];
+        s.hyp_info[(size_t)h * 2 + 0] = g;
+        s.hyp_info[(size_t)h * 2 + 1] = i;
+    }
+    if (write_hyp_operand(s.sc_hyp, h, e, e0 + 4 * r)) atomicOr(s.sc_wild, 1);
 }
 
 // The meanshift's form of hypothesis h (after k_hyp_write): its se(3)
@@ -710,37 +718,36 @@ void launch_hyp_log(const DevParams& p, const DevState& s, cudaStream_t st)
 void launch_hyp_collect(const DevParams& p, const DevState& s, int t, cudaStream_t st)
 {
     // sized for the budget; blocks past the solved prefix return at once
-    k_hyp_write<<<(p.G + kHypGroups - 1) / kHypGroups, kHypGroups * kMaxSols, 0, st>>>(p, s, t);
+    k_hyp_write<<<(p.G + kHypGroups - 1) / kHypGroups, kHypThreads, 0, st>>>(p, s, t);
 }
 
 // Scoring form of caller-given hypotheses already copied to hyp_Rt.
 __global__ void k_hyp_from_rt(DevParams p, DevState s, int t, int n)
 {
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h == 0) *s.n_hyp = n;
-    if (h >= n) return;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x, h = id >> 2, r = min(id & 3, 2);
+    if (id == 0) *s.n_hyp = n;
+    if (h >= n) return;                                   // whole quads leave together
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};
     const double* R = s.hyp_Rt + (size_t)h * 12;
-    const double* T0 = s.poses + 12 * (t - 1);
-    float* f = s.hyp_f32 + (size_t)h * 12;
-    double e[12], e0[12];
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) {
-            e[r * 3 + c] = sc[r] * (R[r * 3 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
-            e0[r * 3 + c] = sc[r] * (T0[r * 4 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
-            f[r * 3 + c] = (float)e[r * 3 + c];
-        }
-        e[9 + r] = sc[r] * R[9 + r];
-        e0[9 + r] = sc[r] * T0[r * 4 + 3];
-        f[9 + r] = (float)e[9 + r];
+    const double* T0 = s.poses + 12 * (t - 1) + r * 4;
+    double e[4], e0[4];
+    for (int c = 0; c < 3; ++c) {
+        e[c] = sc[r] * (R[r * 3 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
+        e0[c] = sc[r] * (T0[c] - (r == c ? 1.0 : 0.0)) / sc[c];
+    }
+    e[3] = sc[r] * R[9 + r];
+    e0[3] = sc[r] * T0[3];
+    if ((id & 3) < 3) {
+        float* f = s.hyp_f32 + (size_t)h * 12;
+        for (int c = 0; c < 4; ++c) f[c < 3 ? r * 3 + c : 9 + r] = (float)e[c];
     }
     if (write_hyp_operand(s.sc_hyp, h, e, e0)) atomicOr(s.sc_wild, 1);
 }
 
 void score_hyps_from_host(const DevParams& p, const DevState& s, int t, int n, cudaStream_t st)
 {
-    k_hyp_from_rt<<<(n + 127) / 128 + 1, 128, 0, st>>>(p, s, t, n);
+    k_hyp_from_rt<<<(4 * n + 127) / 128 + 1, 128, 0, st>>>(p, s, t, n);
 }
 
 // ---------------------------------------------------------------------------

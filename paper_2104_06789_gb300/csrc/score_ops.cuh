@@ -91,12 +91,11 @@ __device__ __forceinline__ void pixel_block_s(const Slice3* f, const Slice3& ref
     o[k++] = ref.h;
 }
 
-// Coefficients of block S: c of (x, y, w), c1 of 1, g (0 or 1) of a_z0; kLarge: the
-// large ones too (else 0: they are in XU / XV).
-template <bool kLarge>
-__device__ __forceinline__ void hyp_block_s(const Slice3* c, const Slice3& c1, float g, __nv_bfloat16* o)
+// Coefficients of block S: c of (x, y, w), c1 of 1, and 1 or 0 of a_z0; a_z's row has
+// the large ones too (else 0: they are in XU / XV).
+__device__ __forceinline__ void hyp_block_s(const Slice3* c, const Slice3& c1, bool az, __nv_bfloat16* o)
 {
-    const __nv_bfloat16 r = __float2bfloat16_rn(g), zero = __float2bfloat16_rn(0.f);
+    const __nv_bfloat16 r = __float2bfloat16_rn(az ? 1.f : 0.f), zero = __float2bfloat16_rn(0.f);
     int k = 0;
 #pragma unroll
     for (; k < 8; ++k) o[k] = zero;
@@ -109,8 +108,8 @@ __device__ __forceinline__ void hyp_block_s(const Slice3* c, const Slice3& c1, f
     o[k++] = c1.m;
     o[k++] = r;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) o[k++] = kLarge ? c[i].h : zero;
-    o[k++] = kLarge ? c1.h : zero;
+    for (int i = 0; i < 3; ++i) o[k++] = az ? c[i].h : zero;
+    o[k++] = az ? c1.h : zero;
     o[k++] = r;
 }
 
@@ -167,45 +166,52 @@ constexpr double kScUntruncate = 1.0 + 4.3e-8;
 constexpr float kScWild = 1073741824.f;                  // 2^30
 
 // Operand row of hypothesis h from its scaled form (E, t) and the frame's current
-// pose (E0, t0), both FP64, as {E row-major (9), t (3)}. True if it is wild.
+// pose (E0, t0), both FP64, by a quad of lanes: lane r < 3 is given row r, {E_r0, E_r1,
+// E_r2, t_r}, and lane 3 row 2 again. Rows 0 and 1 make U's and V's coefficients, row 2
+// those of a_z, which U and V need too. A warp issues an FP64 instruction every ~54
+// cycles, so a lane per hypothesis would take three times as long. True in the lane
+// that finds the hypothesis wild.
 __device__ __forceinline__ bool write_hyp_operand(unsigned char* base, int h, const double* e, const double* e0)
 {
-    Slice3 x[3], y[3], z[3], cx, cy, cz;
-    bool wild = false;
-    auto cut = [](double d) {
+    const int lane = threadIdx.x & 31, r = lane & 3;
+    const unsigned quad = 0xfu << (lane & 28);
+    const bool az = r >= 2;
+    auto cut = [&](double v, double v0) {
+        double d = az ? v - v0 : v0 - v;
         d *= kScUntruncate;
         const float hi = (float)d;
         return slice3(hi, (float)(d - (double)hi));
     };
+    const Slice3 c[3] = {cut(e[0], e0[0]), cut(e[1], e0[1]), cut(e[3], e0[3])};      // of x, y, w
+    const Slice3 c1 = cut(e[2], e0[2]);
+    bool wild = false;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {                        // coefficients of x, y, w
-        const int q = i < 2 ? i : 9;
-        x[i] = cut(i < 2 ? e0[q] - e[q] : e0[9] - e[9]);
-        y[i] = cut(i < 2 ? e0[3 + q] - e[3 + q] : e0[10] - e[10]);
-        z[i] = cut(i < 2 ? e[6 + q] - e0[6 + q] : e[11] - e0[11]);
-        wild |= !(fabs(i < 2 ? e[6 + q] : e[11]) < (double)kScWild) || !(fabs(i < 2 ? e0[6 + q] : e0[11]) < (double)kScWild);
+    for (int i = 0; i < 4; ++i) wild |= !(fabs(e[i]) < (double)kScWild) || !(fabs(e0[i]) < (double)kScWild);
+    // row 2's slices to all lanes
+    Slice3 z[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const Slice3& own = i < 3 ? c[i] : c1;
+        const unsigned hm = (unsigned)__bfloat16_as_ushort(own.h) | (unsigned)__bfloat16_as_ushort(own.m) << 16;
+        const unsigned a = __shfl_sync(quad, hm, 2, 4), b = __shfl_sync(quad, (unsigned)__bfloat16_as_ushort(own.l), 2, 4);
+        z[i].h = __ushort_as_bfloat16((unsigned short)(a & 0xffffu));
+        z[i].m = __ushort_as_bfloat16((unsigned short)(a >> 16));
+        z[i].l = __ushort_as_bfloat16((unsigned short)b);
     }
-    cx = cut(e0[2] - e[2]);
-    cy = cut(e0[5] - e[5]);
-    cz = cut(e[8] - e0[8]);
-    const Slice3 zz[4] = {z[0], z[1], z[2], cz};
+    if (r == 3) return false;
     __align__(16) __nv_bfloat16 o[32];
     unsigned char* d = base + (size_t)(h / kScStageHyps) * kScStageBytes + ((h % kScStageHyps) / 8) * 128 + (h % 8) * 16;
     auto put = [&](unsigned char* dst, int stride) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(dst + q * stride) = *reinterpret_cast<const uint4*>(o + 8 * q);
     };
-    hyp_block_s<false>(x, cx, 0.f, o);
-    put(d, kScHypSBlock);
-    hyp_block_s<false>(y, cy, 0.f, o);
-    put(d + kScStageHyps * 16, kScHypSBlock);
-    hyp_block_s<true>(z, cz, 1.f, o);
-    put(d + 2 * kScStageHyps * 16, kScHypSBlock);
-    hyp_block_x(zz, x, cx, o);
-    put(d + kScHypUOff, kScHypXBlock);
-    hyp_block_x(zz, y, cy, o);
-    put(d + kScHypVOff, kScHypXBlock);
-    return wild || !(fabs(e[8]) < (double)kScWild) || !(fabs(e0[8]) < (double)kScWild);
+    hyp_block_s(c, c1, az, o);
+    put(d + r * kScStageHyps * 16, kScHypSBlock);
+    if (!az) {
+        hyp_block_x(z, c, c1, o);
+        put(d + (r == 0 ? kScHypUOff : kScHypVOff), kScHypXBlock);
+    }
+    return az && wild;
 }
 
 }  // namespace vd
