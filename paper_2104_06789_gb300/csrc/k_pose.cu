@@ -609,8 +609,7 @@ __device__ void se3_exp_vec(const double* p6, double* Rt)
 }
 
 // Hypothesis collection: four lanes per (group, solution slot), one for each row of
-// [R | t], write its
-// solution h = offset + slot < S with its scoring form and tensor-core operand.
+// [R | t], write its solution h = offset + slot < S with its scoring form and tensor-core operand.
 // A block covers 8 groups and finds its offset itself, as the sum of all earlier
 // groups' counts: up to 24 KB of counts read from L2 per block take less time than
 // a scan kernel before this one (4 us and a launch per frame).
