@@ -503,7 +503,9 @@ void launch_forward_backward(const DevParams& p, const DevState& s, cudaStream_t
 {
     const int most = p.H > p.W ? p.H : p.W;               // chains in one direction, their length in the other
     const int smem = kFbChains * 3 * fb_row(most) * (int)sizeof(float);
-    cudaFuncSetAttribute(k_forward_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the longest chain's, whatever this window's: the attribute belongs to all windows and threads
+    constexpr int kSmemMax = kFbChains * 3 * fb_row(kMaxImageSide) * (int)sizeof(float);
+    cudaFuncSetAttribute(k_forward_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     k_forward_backward<<<dim3((most + kFbChains - 1) / kFbChains, p.T), 32 * kFbChains, smem, st>>>(p, s);
 }
 
