@@ -43,14 +43,14 @@ ALGO_MUFU_MIX = {("mie", "fisk"): (1, 2, 1), ("mle", "fisk"): (1, 2, 1),
                  ("mie", "gaussian"): (1, 1, 1), ("mle", "gaussian"): (1, 0, 0)}
 NOMINAL_SMS, NOMINAL_MAX_MHZ = 152, 2070.0
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per k_score launch,
-# mean over the 40 launches of one driving-window step (S = 8192 on every frame,
-# 5 iterations), from one ncu capture of the current default MIE / Fisk kernel
-# (2 hypotheses per thread, three blocks per SM), over two complete iterations:
-# 14.19 MB read, < 1 KB written, against 48 B per valid record + 48 B per
-# hypothesis of algorithmic bytes (13.8 MB at the mean of ~280k valid pixels
-# per frame; frame 1: 23.32 MB read for 22.75 MB). The other
-# variants and hypothesis counts were not captured: their traffic is null.
-SCORE_TRAFFIC_BYTES = {("mie", "fisk", 8192): 14.19e6}
+# mean over the 40 launches of one driving window (S = 8192 on every frame, 5
+# iterations), from one ncu capture of the MIE / Fisk kernel with the projection
+# on the tensor cores: 64.52 MB read, 0.30 MB written, against 212 B per valid
+# pixel (operand columns, constants) + 320 B per hypothesis of algorithmic bytes
+# (62 MB at the mean of ~280k valid pixels per frame; frame 1: 101.7 MB read for
+# 101.4 MB). The other variants and hypothesis counts were not captured: their
+# traffic is null.
+SCORE_TRAFFIC_BYTES = {("mie", "fisk", 8192): 64.82e6}
 
 
 def parse_args():
