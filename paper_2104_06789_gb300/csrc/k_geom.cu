@@ -8,6 +8,8 @@
 // with another kernel's, and fused FP64 multiply-adds cut the FP64
 // instructions of the geometry (this GPU's FP64 rate is a small fraction of
 // its FP32 rate).
+#include <algorithm>
+
 #include "df32.cuh"
 #include "score_ops.cuh"
 #include "voldor_internal.cuh"
@@ -323,19 +325,28 @@ void launch_emissions(const DevParams& p, const DevState& s, float* out, cudaStr
 // each lane then walks its own segment with the step-by-step recursion from
 // the message entering it.
 //
-// A block stages kFbChains neighbouring chains in shared memory, emissions and forward
-// messages, and moves them between there and global memory in whole rows (or, along
-// columns, kFbChains columns of a row at a time): with the lanes' strided accesses in
-// global memory the kernel took 107 us at 1242 x 375, T = 8; now 73. What bounds it
+// A block stages neighbouring chains in shared memory, emissions and forward messages,
+// and moves them between there and global memory in whole rows (or, along columns, some
+// columns of a row at a time): kFbChains of the longer direction's chains, and of the
+// shorter ones what fits in the same room, up to a chain per warp. With the lanes'
+// strided accesses in global memory the kernel took 107 us at 1242 x 375, T = 8; now
+// 66 (58 along rows, 74 along columns; 90 with four chains there too). What bounds it
 // now: the latency of a step (up to two divisions) times four passes over a segment,
-// with the twelve chains an SM holds.
+// with the chains an SM has room for.
 // ---------------------------------------------------------------------------
-constexpr int kFbChains = 4;
+constexpr int kFbChains = 4, kFbWarps = 8;
 
 // Floats of a chain's row in shared memory: 32 segments, padded to an odd length so
 // that the lanes' steps fall into different banks.
 __host__ __device__ constexpr int fb_segment(int len) { return (len + 31) / 32; }
 __host__ __device__ constexpr int fb_row(int len) { return 32 * (fb_segment(len) | 1); }
+
+// Chains of length len to a block whose room is kFbChains chains of length most.
+__host__ __device__ inline int fb_chains(int len, int most)
+{
+    const int fit = kFbChains * fb_row(most) / fb_row(len);
+    return fit < kFbWarps ? fit : kFbWarps;
+}
 
 struct M22 {
     float a, b, c, d;   // [[a, b], [c, d]]
@@ -465,7 +476,7 @@ __device__ __forceinline__ void fb_chain(const DevParams& p, int len, float* e, 
 }
 
 // grid (groups of chains, frame)
-__global__ void __launch_bounds__(32 * kFbChains) k_forward_backward(DevParams p, DevState s)
+__global__ void __launch_bounds__(32 * kFbWarps) k_forward_backward(DevParams p, DevState s)
 {
     extern __shared__ float fb_smem[];
     const int dir = (*s.iter) & 3;
@@ -473,7 +484,7 @@ __global__ void __launch_bounds__(32 * kFbChains) k_forward_backward(DevParams p
     const int n_chains = rows ? p.H : p.W;
     const int len = rows ? p.W : p.H;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c0 = blockIdx.x * kFbChains, here = min(kFbChains, n_chains - c0);
+    const int per = fb_chains(len, max(p.W, p.H)), c0 = blockIdx.x * per, here = min(per, n_chains - c0);
     if (here <= 0) return;
     const int L = fb_segment(len), LP = L | 1, row = fb_row(len);
     float* q = s.qs + (size_t)blockIdx.y * p.N + (rows ? (size_t)c0 * p.W : (size_t)c0);
@@ -483,8 +494,8 @@ __global__ void __launch_bounds__(32 * kFbChains) k_forward_backward(DevParams p
             if (warp < here)
                 for (int i = lane; i < len; i += 32) f(q + (size_t)warp * p.W + i, fb_smem + 3 * row * warp + i + i / L * (LP - L));
         } else {
-            for (int n = threadIdx.x; n < len * kFbChains; n += 32 * kFbChains) {
-                const int i = n / kFbChains, k = n % kFbChains;
+            for (int n = threadIdx.x; n < len * per; n += 32 * kFbWarps) {
+                const int i = n / per, k = n % per;
                 if (k < here) f(q + (size_t)i * p.W + k, fb_smem + 3 * row * k + i + i / L * (LP - L));
             }
         }
@@ -506,7 +517,9 @@ void launch_forward_backward(const DevParams& p, const DevState& s, cudaStream_t
     // the longest chain's, whatever this window's: the attribute belongs to all windows and threads
     constexpr int kSmemMax = kFbChains * 3 * fb_row(kMaxImageSide) * (int)sizeof(float);
     cudaFuncSetAttribute(k_forward_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    k_forward_backward<<<dim3((most + kFbChains - 1) / kFbChains, p.T), 32 * kFbChains, smem, st>>>(p, s);
+    const int rows = fb_chains(p.W, most), cols = fb_chains(p.H, most);   // chains to a block, along rows and columns
+    const int blocks = std::max((p.H + rows - 1) / rows, (p.W + cols - 1) / cols);
+    k_forward_backward<<<dim3(blocks, p.T), 32 * kFbWarps, smem, st>>>(p, s);
 }
 
 }  // namespace vd
