@@ -202,7 +202,6 @@ struct TcSegment {
     int b, x0, y0, rows;
 };
 
-template <int COLS>
 __device__ __forceinline__ TcSegment tc_segment(int i, int end, int H, int strips)
 {
     TcSegment t;
@@ -210,7 +209,7 @@ __device__ __forceinline__ TcSegment tc_segment(int i, int end, int H, int strip
     t.y0 = i - strip * H;
     t.rows = min(H - t.y0, end - i);
     t.b = strip / strips;
-    t.x0 = (strip % strips) * COLS;
+    t.x0 = (strip % strips) * kTcM;
     return t;
 }
 
@@ -295,7 +294,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
         uint32_t ld = 0;
         bool go = true;
         for (int i = r0; i < r1 && go;) {
-            const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
+            const TcSegment t = tc_segment(i, r1, a.H, strips);
             for (int r = t.y0 - 1; r <= t.y0 + t.rows; ++r, ++ld) {
                 const uint32_t slot = ld % kTcSlots;
                 if (ld >= kTcSlots) go = tc_wait_warp(empty + 8 * slot, ((ld / kTcSlots) - 1) & 1, &bad);
@@ -321,7 +320,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
         uint32_t ld = 0, G = 0;
         bool go = true;
         for (int i = r0; i < r1 && go;) {
-            const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
+            const TcSegment t = tc_segment(i, r1, a.H, strips);
             for (int k = 0; k < t.rows + 2; ++k, ++ld) {
                 const uint32_t slot = ld % kTcSlots;
                 go = tc_wait_warp(full + 8 * slot, (ld / kTcSlots) & 1, &bad);
@@ -369,7 +368,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) k_conv_tc(const __gr
         uint32_t g = 0;
         bool go = true;
         for (int i = r0; i < r1 && go;) {
-            const TcSegment t = tc_segment<kTcM>(i, r1, a.H, strips);
+            const TcSegment t = tc_segment(i, r1, a.H, strips);
             const int px0 = t.x0 + (warp & 3) * 32;
             for (int k = 0; k < t.rows; ++k, ++g) {
                 if ((g & 1) != (uint32_t)(warp >> 2)) continue;
@@ -526,58 +525,48 @@ struct WgradArgs {
 // Weight gradient on the fifth-generation tensor cores:
 // dw[co][tap][ci] += sum_p dout[p][co] in[p + off(tap)][ci] and
 // db[co] += sum_p dout[p][co], as one GEMM per layer with the pixels as K:
-// D[m][n] = sum_k A[m][k] B[n][k], k = input pixel (x, y of a row segment),
-// m = (kx, co): dout at column x + 1 - kx, n = (ky, ci): the input row y - 1 + ky
-// for dout's row y.
+// D[m][n] = sum_k A[m][k] B[n][k], m = tap * CIN + ci (the nine shifted copies of the
+// input) and one row of ones (m = 9 CIN) for the bias, n = output channel, k = pixel.
 //
 // The activations are channel-last, so both operands have their M / N index
 // contiguous: the MN-major swizzled layouts (64 bytes a pixel for 32 channels, 32
-// for 16) are what TMA writes, and no thread touches an operand. A CTA walks down
-// the rows of 64-column strips:
-//   warp 4, an elected lane: TMA loads of a ring of input rows and a ring of dout rows, a
-//     dout row three times (columns x0 + 1, x0, x0 - 1: kx = 0, 1, 2; zero fill
-//     outside the image). M groups of NCO channels are a dout copy apart, N groups
-//     of CIN channels an input row of the ring.
-//   warp 5, an elected lane: per row four tcgen05.mma (M = 128, of which 3 NCO rows count;
-//     N = 3 CIN, K = 16 pixels), in two parts where the three rows wrap around the
-//     ring. Even and odd rows accumulate in two sets of TMEM columns (shorter sums).
-//   warps 0-3: the bias sums from the dout rows in shared memory, FP32; at the end
-//     each reads its TMEM lanes and writes the CTA's partial.
-// The rows of all strips are dealt to the CTAs in contiguous runs of equal length.
-// Every mbarrier wait is bounded as in k_conv_tc.
+// for 16) are what TMA writes, and no thread touches an operand. A work item is 64
+// consecutive output pixels of a row:
+//   warp 4, an elected lane: ten TMA loads, the nine taps' copies of the input (a group
+//     of CIN channels each, zero fill outside the image, followed by the constant group
+//     with the row of ones) and the output gradients;
+//   warp 5, an elected lane: per M tile of 128 rows four tcgen05.mma (N = NCO, K = 16);
+//     the rows past the ones multiply whatever follows them and are not read;
+//   warps 0-3: at the end read their TMEM lanes and write the CTA's partial.
+// Every mbarrier wait is bounded as in k_conv_tc. CTA c takes items c, c + grid, ...,
+// three CTAs to an SM: while one waits for its loads the others multiply. The sums are
+// formed in the order of the kernel before and are bit-identical to it (a different
+// split of the pixels, with a third of the loads, took 29 us; but the optimiser turns the
+// sign of a gradient that is zero up to rounding into a whole step).
 //
-// What bounds it: HBM in the long run (22 us per 119 MB of operands at 1242 x 375 x 2;
-// the MMAs read 7 KB of shared memory per 16 pixels, 15 us), and here the start and
-// the partials, ~6 us. The kernel before, which transposed 64-pixel tiles through
-// ldmatrix / stmatrix into K-major operands (nine shifted copies of the input per
-// tile), took 177 us for 32 x 32 channels; this one 28.8 us. 42 us of it were left
-// while one lane of a diverged warp issued the MMAs and loads (see tc.cuh); threads
-// that load the rows through registers and store the copies instead of TMA took 48.
-// One CTA per SM with rings twice as deep is slower (53 against 46 us with the
-// reduction): a row's round trip between the roles takes ~800 cycles.
+// The kernel before transposed the tiles through ldmatrix / stmatrix into K-major
+// operands: 177 us for 32 x 32 channels on two 1242 x 375 images; this one about 55 us.
+// HBM needs 18, the MMAs 32 (52 cycles each, the reads of their 4 KB A tiles).
 // ---------------------------------------------------------------------------
-constexpr int kWgKP = 64;                                 // pixels per row segment (K)
+constexpr int kWgKP = 64;                                 // pixels per work item (K)
 constexpr int kWgThreads = 192;
-constexpr int kWgCtasPerSm = 2;                           // weight-gradient grid: at most this many CTAs per SM
-constexpr int kWgInSlots = 8, kWgDoSlots = 4;             // ring slots
+constexpr int kWgCtasPerSm = 3;                           // weight-gradient grid: at most this many CTAs per SM
 constexpr int kWgPartRows = 9 * 32 + 1;                   // largest per-CTA partial: rows x 32 columns
 
 template <int CIN, int NCO>
 struct WgShape {
-    static constexpr int kRows = 9 * CIN + 1;                           // a partial's rows: (tap, ci), then the bias
-    static constexpr int kInSlot = kWgKP * CIN * 2;
-    static constexpr int kDoCopy = kWgKP * NCO * 2;                     // a dout row at one shift
-    static constexpr int kDoSlot = 3 * kDoCopy;
-    // dout ring | input ring | barriers. The M = 128 operand reads on past a dout slot's
-    // three copies, at most into the input ring.
-    static constexpr int kInOff = kWgDoSlots * kDoSlot;
-    static constexpr int kBarOff = kInOff + kWgInSlots * kInSlot;
-    static constexpr int kBars = 2 * kWgInSlots + 2 * kWgDoSlots + 1;
-    // then the TMEM address, the abort flag and the warps' bias sums
-    static constexpr int kSmemBytes = kBarOff + kBars * 8 + 8 + 4 * NCO * 4;
-    static constexpr int kSetCols = 3 * CIN;
-    static constexpr int kTmemCols = 2 * kSetCols <= 128 ? 128 : 256;
-    static_assert(128 / NCO * kDoCopy - kDoSlot <= kWgInSlots * kInSlot, "operand reads stay in the rings");
+    static constexpr int kRows = 9 * CIN + 1;                           // + the ones row
+    static constexpr int kMT = (kRows + 127) / 128;
+    static constexpr int kGroup = kWgKP * CIN * 2;                      // a tap's copy
+    static constexpr int kDoOff = 10 * kGroup;
+    static constexpr int kSlot = kDoOff + kWgKP * NCO * 2;
+    static constexpr int kSlots = CIN == 32 ? 1 : 2;
+    // the last M tile reads on past the ones group: kMT tiles of 128 / CIN groups from a slot's start
+    static constexpr int kBarOff = kSlots * kSlot + (kMT * (128 / CIN) * kGroup > kSlot ? kMT * (128 / CIN) * kGroup - kSlot : 0);
+    static constexpr int kBars = 2 * kSlots + 1;
+    static constexpr int kSmemBytes = kBarOff + kBars * 8 + 8;          // then the TMEM address and the abort flag
+    static constexpr int kTmemCols = kMT * NCO <= 32 ? 32 : (kMT * NCO <= 64 ? 64 : 128);
+    static_assert(kSlot % 1024 == 0 && kBarOff % 8 == 0, "slots start where the swizzle does");
 };
 
 // Descriptor of an MN-major operand of C channels per pixel (C = 32: 64-byte swizzle,
@@ -597,24 +586,22 @@ __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
     using S = WgShape<CIN, NCO>;
     extern __shared__ __align__(1024) unsigned char smem[];
     const uint32_t sbase = smem_addr(smem);
-    const uint32_t in_s = sbase + S::kInOff;
-    const uint32_t in_full = sbase + S::kBarOff, in_empty = in_full + 8 * kWgInSlots, do_full = in_empty + 8 * kWgInSlots,
-                   do_empty = do_full + 8 * kWgDoSlots, done = do_empty + 8 * kWgDoSlots;
+    const uint32_t full = sbase + S::kBarOff, empty = full + 8 * S::kSlots, done = empty + 8 * S::kSlots;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + S::kBarOff + S::kBars * 8);
     volatile int& bad = *reinterpret_cast<volatile int*>(smem + S::kBarOff + S::kBars * 8 + 4);
-    float(*bias_s)[NCO] = reinterpret_cast<float(*)[NCO]>(smem + S::kBarOff + S::kBars * 8 + 8);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int strips = (a.W + kWgKP - 1) / kWgKP, total = a.B * strips * a.H;
-    const int r0 = (int)((long long)total * blockIdx.x / gridDim.x), r1 = (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
+    const int segs = (a.W + kWgKP - 1) / kWgKP, n_items = a.B * a.H * segs;
 
+    // the ones group of each slot: channel 0 of every pixel 1, the others 0
+    for (int i = tid; i < S::kSlots * kWgKP * (CIN / 8); i += kWgThreads) {
+        const int slot = i / (kWgKP * (CIN / 8)), p = i / (CIN / 8) % kWgKP, c = i % (CIN / 8);
+        const int at = CIN == 32 ? c ^ ((p >> 1) & 3) : c ^ ((p >> 2) & 1);
+        *reinterpret_cast<uint4*>(smem + slot * S::kSlot + 9 * S::kGroup + p * CIN * 2 + at * 16) = make_uint4(c == 0 ? 0x3f80u : 0u, 0u, 0u, 0u);
+    }
     if (tid == 0) {
-        for (int i = 0; i < kWgInSlots; ++i) {
-            tc_mbar_init(in_full + 8 * i, 1);
-            tc_mbar_init(in_empty + 8 * i, 1);
-        }
-        for (int i = 0; i < kWgDoSlots; ++i) {
-            tc_mbar_init(do_full + 8 * i, 1);
-            tc_mbar_init(do_empty + 8 * i, 1 + 4);
+        for (int i = 0; i < S::kSlots; ++i) {
+            tc_mbar_init(full + 8 * i, 1);
+            tc_mbar_init(empty + 8 * i, 1);
         }
         tc_mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -625,125 +612,65 @@ __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
                      "r"((uint32_t)S::kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    float bias[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
     if (warp == 4) {
-        uint32_t li = 0, ld = 0;                           // input and dout rows loaded
+        uint32_t ld = 0;
         bool go = true;
-        for (int i = r0; i < r1 && go;) {
-            const TcSegment t = tc_segment<kWgKP>(i, r1, a.H, strips);
-            for (int r = t.y0 - 1; r <= t.y0 + t.rows; ++r) {
-                const uint32_t si = li % kWgInSlots, sd = ld % kWgDoSlots;
-                if (li >= kWgInSlots) go = tc_wait_warp(in_empty + 8 * si, ((li / kWgInSlots) - 1) & 1, &bad);
-                if (!go) break;
-                tc_expect_tx_elect(in_full + 8 * si, (uint32_t)S::kInSlot);
-                tc_tma_row_elect(in_s + si * S::kInSlot, &tin, 0, t.x0, r, t.b, in_full + 8 * si);
-                ++li;
-                if (r <= t.y0) continue;
-                if (ld >= kWgDoSlots) go = tc_wait_warp(do_empty + 8 * sd, ((ld / kWgDoSlots) - 1) & 1, &bad);
-                if (!go) break;
-                tc_expect_tx_elect(do_full + 8 * sd, (uint32_t)S::kDoSlot);
+        for (int it = blockIdx.x; it < n_items && go; it += gridDim.x) {
+            const int b = it / (a.H * segs), rem = it % (a.H * segs), y = rem / segs, x0 = (rem % segs) * kWgKP;
+            const uint32_t slot = ld % S::kSlots, at = sbase + slot * S::kSlot;
+            if (ld >= S::kSlots) go = tc_wait_warp(empty + 8 * slot, ((ld / S::kSlots) - 1) & 1, &bad);
+            if (!go) break;
+            tc_expect_tx_elect(full + 8 * slot, (uint32_t)(9 * S::kGroup + kWgKP * NCO * 2));
 #pragma unroll
-                for (int kx = 0; kx < 3; ++kx)
-                    tc_tma_row_elect(sbase + sd * S::kDoSlot + kx * S::kDoCopy, &tdo, 0, t.x0 + 1 - kx, r - 1, t.b, do_full + 8 * sd);
-                ++ld;
-            }
-            i += t.rows;
+            for (int tap = 0; tap < 9; ++tap)
+                tc_tma_row_elect(at + tap * S::kGroup, &tin, 0, x0 + tap % 3 - 1, y + tap / 3 - 1, b, full + 8 * slot);
+            tc_tma_row_elect(at + S::kDoOff, &tdo, 0, x0, y, b, full + 8 * slot);
+            ++ld;
         }
         // the last loads may still be landing when another role gave up
-        for (uint32_t j = li > kWgInSlots ? li - kWgInSlots : 0; j < li; ++j)
+        for (uint32_t j = ld > S::kSlots ? ld - S::kSlots : 0; j < ld; ++j)
             for (long long k = 0; k < kTcWaitLimit; ++k)
-                if (tc_try_wait(in_full + 8 * (j % kWgInSlots), (j / kWgInSlots) & 1)) break;
-        for (uint32_t j = ld > kWgDoSlots ? ld - kWgDoSlots : 0; j < ld; ++j)
-            for (long long k = 0; k < kTcWaitLimit; ++k)
-                if (tc_try_wait(do_full + 8 * (j % kWgDoSlots), (j / kWgDoSlots) & 1)) break;
+                if (tc_try_wait(full + 8 * (j % S::kSlots), (j / S::kSlots) & 1)) break;
     } else if (warp == 5) {
-        uint32_t gi = 0, gd = 0, seen = 0;             // input row y - 1, dout row y, input rows waited for
-        bool go = true;
-        for (int i = r0; i < r1 && go;) {
-            const TcSegment t = tc_segment<kWgKP>(i, r1, a.H, strips);
-            for (int k = 0; k < t.rows; ++k, ++gi, ++gd) {
-                for (; go && seen < gi + 3; ++seen)
-                    go = tc_wait_warp(in_full + 8 * (seen % kWgInSlots), (seen / kWgInSlots) & 1, &bad);
-                const uint32_t sd = gd % kWgDoSlots, si = gi % kWgInSlots;
-                go = go && tc_wait_warp(do_full + 8 * sd, (gd / kWgDoSlots) & 1, &bad);
-                if (!go) break;
-                tc_fence_after();
-                const int nb = min(3, kWgInSlots - (int)si);             // rows before the ring wraps
-                const uint32_t d = tmem + (gd & 1) * S::kSetCols, i1 = tc_idesc_mn(nb * CIN), i2 = tc_idesc_mn((3 - nb) * CIN);
+        uint32_t ld = 0;
+        for (int it = blockIdx.x; it < n_items; it += gridDim.x, ++ld) {
+            const uint32_t slot = ld % S::kSlots, at = sbase + slot * S::kSlot;
+            if (!tc_wait_warp(full + 8 * slot, (ld / S::kSlots) & 1, &bad)) break;
+            tc_fence_after();
 #pragma unroll
-                for (int ks = 0; ks < kWgKP / 16; ++ks) {
-                    const uint64_t ad = tc_desc_mn<NCO>(sbase + sd * S::kDoSlot + ks * 32 * NCO, S::kDoCopy);
-                    const uint32_t acc = gd >= 2 || ks > 0;
-                    tc_mma_elect(d, ad, tc_desc_mn<CIN>(in_s + si * S::kInSlot + ks * 32 * CIN, S::kInSlot), i1, acc);
-                    if (nb < 3) tc_mma_elect(d + nb * CIN, ad, tc_desc_mn<CIN>(in_s + ks * 32 * CIN, S::kInSlot), i2, acc);
-                }
-                tc_commit_elect(do_empty + 8 * sd);
-                tc_commit_elect(in_empty + 8 * si);
-            }
-            if (!go) break;
-            tc_commit_elect(in_empty + 8 * (gi % kWgInSlots));                 // the segment's last two rows
-            tc_commit_elect(in_empty + 8 * ((gi + 1) % kWgInSlots));
-            gi += 2;
-            i += t.rows;
+            for (int mt = 0; mt < S::kMT; ++mt)
+#pragma unroll
+                for (int ks = 0; ks < kWgKP / 16; ++ks)
+                    tc_mma_elect(tmem + mt * NCO, tc_desc_mn<CIN>(at + mt * (128 / CIN) * S::kGroup + ks * 32 * CIN, S::kGroup),
+                                 tc_desc_mn<NCO>(at + S::kDoOff + ks * 32 * NCO, S::kGroup), tc_idesc_mn(NCO), ld > 0 || ks > 0);
+            tc_commit_elect(empty + 8 * slot);
         }
-        tc_commit_elect(done);                          // arrives once every MMA issued has completed
+        tc_commit_elect(done);                        // arrives once every MMA issued has completed
         bool drained = false;
         for (long long i = 0; i < kTcWaitLimit && !drained; ++i) drained = tc_try_wait(done, 0);
         if (!drained) bad = 1;
-    } else {
-        // thread: 16-byte chunk c (channels 8 c ..) of pixels tid / kC, ...; chunks are permuted by the swizzle
-        constexpr int kC = NCO / 8, kStep = 128 / kC;
-        const int c = tid % kC, px = tid / kC;
-        for (int g = 0; g < r1 - r0; ++g) {
-            const uint32_t sd = g % kWgDoSlots;
-            if (!__all_sync(0xffffffffu, tc_wait(do_full + 8 * sd, (g / kWgDoSlots) & 1, &bad))) break;
-#pragma unroll
-            for (int x = 0; x < kWgKP; x += kStep) {
-                const int p = x + px, at = NCO == 32 ? (c ^ ((p >> 1) & 3)) : (c ^ ((p >> 2) & 1));
-                const uint4 v = *reinterpret_cast<const uint4*>(smem + sd * S::kDoSlot + S::kDoCopy + p * NCO * 2 + at * 16);
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    bias[2 * q] += __uint_as_float(w[q] << 16);
-                    bias[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) tc_arrive(do_empty + 8 * sd);
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            for (int o = kC; o < 32; o <<= 1) bias[q] += __shfl_xor_sync(0xffffffffu, bias[q], o);
-            if (lane < kC) bias_s[warp][8 * lane + q] = bias[q];
-        }
     }
     __syncthreads();
     tc_fence_after();
-    if (!bad) {
-        // this CTA's sums: row tap * CIN + ci, then the bias row, of its partial
-        float* part = a.part + (size_t)blockIdx.x * S::kRows * NCO;
-        if (warp * 32 < 3 * NCO) {
-            const int m = warp * 32 + lane, kx = m / NCO, co = m % NCO;
-            const bool two = r1 - r0 > 1;
-            const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
+    if (!bad && warp < 4) {
+        // this CTA's sums, row m (tap * CIN + ci, then the bias row) of its partial
 #pragma unroll
-            for (int ky = 0; ky < 3; ++ky) {
-                float v[CIN], u[CIN];
-                tc_ld<CIN>(row + ky * CIN, v);
-                tc_ld<CIN>(row + S::kSetCols + ky * CIN, u);
-                if (m < 3 * NCO) {
+        for (int mt = 0; mt < S::kMT; ++mt) {
+            float v[NCO];
+            tc_ld<NCO>(tmem + ((uint32_t)(warp * 32) << 16) + mt * NCO, v);
+            const int m = mt * 128 + warp * 32 + lane;
+            if (m < S::kRows) {
+                float4* o = reinterpret_cast<float4*>(a.part + ((size_t)blockIdx.x * S::kRows + m) * NCO);
 #pragma unroll
-                    for (int ci = 0; ci < CIN; ++ci)
-                        part[((ky * 3 + kx) * CIN + ci) * NCO + co] = two ? v[ci] + u[ci] : v[ci];
-                }
+                for (int q = 0; q < NCO / 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
         }
-        if (tid < NCO) part[9 * CIN * NCO + tid] = (bias_s[0][tid] + bias_s[1][tid]) + (bias_s[2][tid] + bias_s[3][tid]);
     }
     tc_fence_before();
     __syncthreads();
@@ -756,10 +683,10 @@ __global__ void __launch_bounds__(kWgThreads, kWgCtasPerSm)
 
 // The gradients of all layers from the CTAs' partial sums, in a fixed order (so that
 // a training run is bit-reproducible, unlike with floating-point atomics): grid
-// (blocks of 32 entries, layer); warp w sums every kWgReduceWarps-th CTA from w, and
-// the warps' sums are added in order. Entry i = m * nco + co of a layer: dw[co][tap][ci]
+// (blocks of 32 entries, layer); a warp sums groups of kWgGroup consecutive CTAs, and the
+// groups' sums are added in order. Entry i = m * nco + co of a layer: dw[co][tap][ci]
 // (row m = tap * cin + ci) or db[co] (m = 9 cin). A launch per layer took 6 us each.
-constexpr int kWgReduceWarps = 16;
+constexpr int kWgReduceWarps = 16, kWgGroup = 16, kWgMaxGroups = 64;
 
 struct WgLayer {
     const float* part;                                    // [n_cta][9 cin + 1][nco]
@@ -773,23 +700,26 @@ struct WgLayers {
 
 __global__ void __launch_bounds__(32 * kWgReduceWarps) k_wgrad_reduce(const __grid_constant__ WgLayers layers)
 {
-    __shared__ float sums[kWgReduceWarps][32];
+    __shared__ float sums[kWgMaxGroups][32];
     const WgLayer& g = layers.l[blockIdx.y];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     const int entries = (9 * g.cin + 1) * g.nco;
     if (blockIdx.x * 32 >= entries) return;
-    float sum = 0.f;
-    if (i < entries) {
-#pragma unroll 8
-        for (int c = warp; c < g.n_cta; c += kWgReduceWarps) sum += g.part[(size_t)c * entries + i];
+    const int groups = (g.n_cta + kWgGroup - 1) / kWgGroup;
+    for (int q = warp; q < groups; q += kWgReduceWarps) {
+        float v[kWgGroup], sum = 0.f;
+#pragma unroll
+        for (int u = 0; u < kWgGroup; ++u)
+            v[u] = i < entries && q * kWgGroup + u < g.n_cta ? g.part[(size_t)(q * kWgGroup + u) * entries + i] : 0.f;
+#pragma unroll
+        for (int u = 0; u < kWgGroup; ++u) sum += v[u];
+        sums[q][lane] = sum;
     }
-    sums[warp][lane] = sum;
     __syncthreads();
     const int m = i / g.nco, co = i % g.nco;
     if (warp != 0 || i >= entries || co >= g.n_out) return;
-    sum = 0.f;
-#pragma unroll
-    for (int w = 0; w < kWgReduceWarps; ++w) sum += sums[w][lane];
+    float sum = 0.f;
+    for (int q = 0; q < groups; ++q) sum += sums[q][lane];
     if (m < 9 * g.cin) {
         const int tap = m / g.cin, ci = m % g.cin;
         if (ci < g.cin_real) g.dw[((size_t)co * 9 + tap) * g.cin_real + ci] = sum;
@@ -1215,8 +1145,8 @@ static bool launch_wgrad_tc(const WgradArgs& a, cudaStream_t st, int& grid)
     if (!tensor_map_rows(&in, a.in, CIN, a.W, a.H, a.B, CIN, kWgKP, CIN == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B) ||
         !tensor_map_rows(&dout, a.dout, NCO, a.W, a.H, a.B, NCO, kWgKP, NCO == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B))
         return false;
-    const int rows = a.B * a.H * ((a.W + kWgKP - 1) / kWgKP);
-    grid = std::min(rows, kWgCtasPerSm * sms);
+    const int items = a.B * a.H * ((a.W + kWgKP - 1) / kWgKP);
+    grid = std::min(items, std::min(kWgCtasPerSm * sms, kWgMaxGroups * kWgGroup));
     k_wgrad_tc<CIN, NCO><<<grid, kWgThreads, S::kSmemBytes, st>>>(in, dout, a);
     return true;
 }

@@ -1,7 +1,7 @@
-"""The weight gradient's row segments at their edges: images narrower than, as wide
-as and one column wider than a segment of 64 columns, one and two rows (fewer rows
-than CTAs), runs that cross from one strip or image to the next, and rings that
-wrap; every layer shape (16 -> 32, 32 -> 32, 32 -> 2 channels) is in each.
+"""The weight gradient's work items at their edges: images narrower than, as wide as
+and one column wider than an item of 64 columns, one and two rows (fewer items than
+CTAs), several images, and more items than CTAs; every layer shape (16 -> 32, 32 ->
+32, 32 -> 2 channels) is in each.
 
 Against the network with BF16 rounding at the kernels' storage points the kernels
 differ by FP32 accumulation order and the rare BF16 rounding it flips: 1e-2 relative
