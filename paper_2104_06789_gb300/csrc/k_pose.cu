@@ -620,7 +620,7 @@ constexpr int kHypThreads = kHypGroups * kMaxSols * 4;
 
 __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState s, int t)
 {
-    __shared__ int wsum[kHypThreads / 32], off_s[kHypGroups];
+    __shared__ int wsum[kHypThreads / 32], off_s[kHypGroups], n_s;
     __shared__ double e0[12];
     const int tid = threadIdx.x, lane = tid & 31;
     const int G = groups_solved(p, s), g0 = blockIdx.x * kHypGroups;
@@ -652,9 +652,13 @@ __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState
             if (lane >= o) incl += v;
         }
         if (tid < kHypGroups) off_s[tid] = base + incl - c;
-        if (tid == 31 && g0 + kHypGroups >= G) *s.n_hyp = min(base + incl, p.S);   // the last block with groups
+        if (tid == 31) {
+            n_s = 0;
+            if (g0 + kHypGroups >= G) *s.n_hyp = n_s = min(base + incl, p.S);      // the last block with groups
+        }
     }
     __syncthreads();
+    if ((n_s & 1) && tid < kScHypChunks) clear_hyp_operand(s.sc_hyp, n_s, tid);   // the last hypothesis's partner
     const int item = tid >> 2, r = min(tid & 3, 2), g = g0 + item / kMaxSols, i = item % kMaxSols;
     if (g >= G || i >= s.grp_count[g]) return;            // whole quads leave together
     const int h = off_s[item / kMaxSols] + i;
@@ -725,6 +729,7 @@ __global__ void k_hyp_from_rt(DevParams p, DevState s, int t, int n)
 {
     const int id = blockIdx.x * blockDim.x + threadIdx.x, h = id >> 2, r = min(id & 3, 2);
     if (id == 0) *s.n_hyp = n;
+    if ((n & 1) && id < kScHypChunks) clear_hyp_operand(s.sc_hyp, n, id);   // the last hypothesis's partner
     if (h >= n) return;                                   // whole quads leave together
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};

@@ -160,6 +160,19 @@ __device__ __forceinline__ void hyp_block_x(const Slice3* z, const Slice3* a, co
 // of the scores was 4e-8 to 9e-8 larger without it.
 constexpr double kScUntruncate = 1.0 + 4.3e-8;
 
+// Sixteen bytes i < kScHypChunks of hypothesis h's operand row set to zero: a_z = U = V = 0 for
+// every pixel. A pair of hypotheses shares a reciprocal, so with an odd count the row after
+// the last one enters its score and may not hold what an earlier frame left there.
+constexpr int kScHypChunks = 20;
+
+__device__ __forceinline__ void clear_hyp_operand(unsigned char* base, int h, int i)
+{
+    unsigned char* d = base + (size_t)(h / kScStageHyps) * kScStageBytes + ((h % kScStageHyps) / 8) * 128 + (h % 8) * 16;
+    if (i < 12) d += i / 4 * (kScStageHyps * 16) + i % 4 * kScHypSBlock;
+    else d += (i < 16 ? kScHypUOff : kScHypVOff) + i % 4 * kScHypXBlock;
+    *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // Values beyond this size in a hypothesis's a_z coefficients or a pixel's x, y,
 // w send a frame to the scoring's path without shared reciprocals: below it
 // the product of two (1 + a_z) stays under 2^124.
