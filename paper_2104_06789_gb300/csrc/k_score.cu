@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
         auto tiles = [&](auto is_wild, int t0, int t1, int stages) {
             constexpr bool kWild = decltype(is_wild)::value;
             int j = t0 * kScTilePix + quarter * 32 + lane;
-            // a lane past the last pixel: weight 0 and a finite term (whatever its operand row holds)
+            // a lane past the last pixel: weight 0 and a finite term, whatever its operand row holds
             float4 cst;
             float xmu;
             auto load_const = [&]() {

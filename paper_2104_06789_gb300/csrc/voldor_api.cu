@@ -1,6 +1,7 @@
 // C ABI of the VOLDOR library (declared in include/voldor.h): context
 // lifetime, argument checking, the Table 1 iteration as a sequence of kernel
 // launches, CUDA-graph capture of voldor_em_step, and host readout.
+#include <cfloat>
 #include <cmath>
 #include <cstdio>
 #include <algorithm>
@@ -99,8 +100,10 @@ DevParams make_dev_params(const voldor_ctx& c)
     d.b1 = (float)p.b1; d.b2 = (float)p.b2; d.beta_min = (float)p.beta_min;
     d.lambda2 = (float)(p.lambda_ * p.lambda_);
     d.x_min = (float)p.x_min; d.x_max = (float)p.x_max;
-    d.xs_min = (float)(p.x_min / (c.K.fx * c.K.fx));
-    d.xs_max = (float)(p.x_max / (c.K.fx * c.K.fx));
+    // within FP32's normal range: the scoring's lanes past the last pixel multiply a term of a residual
+    // anywhere between the two by a weight of zero, and that term has to be finite
+    d.xs_min = std::max((float)(p.x_min / (c.K.fx * c.K.fx)), FLT_MIN);
+    d.xs_max = std::min((float)(p.x_max / (c.K.fx * c.K.fx)), 0x1p120f);
     d.log2_fx2 = (float)std::log2(c.K.fx * c.K.fx);
     d.inv_depth_min = (float)p.inv_depth_min; d.inv_depth_max = (float)p.inv_depth_max;
     d.gamma = (float)p.gamma;
