@@ -151,12 +151,6 @@ __device__ __forceinline__ void tc_tma_row_elect(uint32_t dst, const CUtensorMap
                  ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void tc_expect_tx_elect(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
-                 " @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(bar), "r"(bytes) : "memory");
-}
-
 __device__ __forceinline__ void tc_tma_row(uint32_t dst, const CUtensorMap* map, int c, int x, int y, int b, uint32_t bar)
 {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"

@@ -289,6 +289,14 @@ __device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t* r)
                  : "r"(taddr));
 }
 
+// Keeps what reads loaded columns behind the wait for them.
+template <int NC>
+__device__ __forceinline__ void tmem_hold(uint32_t* r)
+{
+#pragma unroll
+    for (int i = 0; i < NC; ++i) asm volatile("" : "+r"(r[i]));
+}
+
 // Bounded wait on an mbarrier phase: false (and *bad set, if given) on expiry or
 // when another role of the CTA already gave up. The loop is out of line: the
 // first try nearly always succeeds, and the hot loop holds only that.
@@ -309,13 +317,19 @@ __device__ __forceinline__ bool score_wait(uint32_t bar, uint32_t parity, volati
     return tc_try_wait(bar, parity) || score_wait_loop(bar, parity, bad, kWaitLimit);
 }
 
+// The same for a converged warp, with one answer for all its lanes.
+__device__ __forceinline__ bool score_wait_warp(uint32_t bar, uint32_t parity, volatile int* bad)
+{
+    return __all_sync(0xffffffffu, score_wait(bar, parity, bad));
+}
+
 // ---------------------------------------------------------------------------
 // The scoring kernel: one persistent CTA per SM over work items (pixel chunk,
 // group of 128 hypotheses), chunk-major so that the CTAs running at one time
 // share the pixel tiles in L2. Warp roles:
-//   warp 16, one lane: bulk copies of an item's hypothesis operand (40 KB, two
+//   warp 16, an elected lane: bulk copies of an item's hypothesis operand (40 KB, two
 //     buffers) and pixel tiles (128 pixels, 24 KB, kScSlots slots);
-//   warp 17, one lane: per tile and stage of 32 hypotheses six MMAs of M = 128
+//   warp 17, an elected lane: per tile and stage of 32 hypotheses six MMAs of M = 128
 //     pixels, K = 16 (N = 96: S by US, VS, ZS; N = 32: U by XU, V by XV) into one of
 //     five TMEM buffers of 96 columns U, V, a_z;
 //   warps 0-15: warp w takes the 32 pixels of TMEM lane quarter w % 4 and stage
@@ -333,7 +347,13 @@ __device__ __forceinline__ bool score_wait(uint32_t bar, uint32_t parity, volati
 // tensor pipe 10 %. With the contractions in FP32 on the CUDA cores the term
 // needed 28 packed instructions and five shared-memory loads per pixel and was
 // bound by dispatch: 88 cycles. 8192 hypotheses x 465,750 pixels: 4.38 -> 3.64 ms.
-// Measured and not kept: 8 or 12 compute warps with more registers (101 and 91
+// The two issuing warps run converged: with their loops inside an `if (lane == 0)` a
+// stage's six MMAs, descriptors, waits and commit took longer than the arithmetic of the
+// light variants, and MLE with the Gaussian residual (one rcp a pair) took 1977 us a frame
+// on average there, now 1587, MIE with it 2198, now 2055; MIE / Fisk 2334, now 2318.
+// Measured and not kept: the next columns' loads from tensor memory issued before the
+// arithmetic on the present ones (24 more registers: MIE / Fisk 1 % faster, MLE / Fisk 1 %
+// and MIE / Gaussian 5 % slower), 8 or 12 compute warps with more registers (101 and 91
 // cycles against 88 with 16 at the first version), all arithmetic scalar (79
 // against 73), two 64-hypothesis buffers (76), lg2(1 + r) as a polynomial on the
 // FMA pipe (115 in the FP32 kernel), and a shortened register share for the two
@@ -412,77 +432,76 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
     const uint32_t tmem = *tmem_slot;
 
     if (warp == kScWarps) {
-        if (lane == 0) {
-            // loader: n counts tiles, w work items (those with pixels)
-            uint32_t n = 0, w = 0;
-            for (int u = blockIdx.x; u < n_items && !bad; u += gridDim.x) {
-                const ScItem it = item(u);
-                if (it.cnt == 0) continue;
-                const uint32_t hb = w & 1, bytes = (it.hyps + kScStageHyps - 1) / kScStageHyps * kScStageBytes;
-                if (w >= 2 && !score_wait(hempty + 8 * hb, ((w >> 1) - 1) & 1, &bad)) break;
-                tc_expect_tx(hfull + 8 * hb, bytes);
-                tc_bulk_g2s(hyp_s + hb * kScGroupBytes, s.sc_hyp + (size_t)(u % n_groups) * kScGroupBytes, bytes, hfull + 8 * hb);
-                ++w;
-                for (int k = 0; k < it.cnt && !bad; ++k, ++n) {
-                    const uint32_t slot = n % kScSlots;
-                    if (n >= kScSlots && !score_wait(empty + 8 * slot, ((n / kScSlots) - 1) & 1, &bad)) break;
-                    tc_expect_tx(full + 8 * slot, kScTileBytes);
-                    tc_bulk_g2s(ring + slot * kScTileBytes, s.sc_pix + (size_t)(it.t0 + k) * kScTileBytes, kScTileBytes, full + 8 * slot);
-                }
+        // loader: n counts tiles, w work items (those with pixels)
+        uint32_t n = 0, w = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < n_items && ok; u += gridDim.x) {
+            const ScItem it = item(u);
+            if (it.cnt == 0) continue;
+            const uint32_t hb = w & 1, bytes = (it.hyps + kScStageHyps - 1) / kScStageHyps * kScStageBytes;
+            if (w >= 2) ok = score_wait_warp(hempty + 8 * hb, ((w >> 1) - 1) & 1, &bad);
+            if (!ok) break;
+            tc_expect_tx_elect(hfull + 8 * hb, bytes);
+            tc_bulk_g2s_elect(hyp_s + hb * kScGroupBytes, s.sc_hyp + (size_t)(u % n_groups) * kScGroupBytes, bytes, hfull + 8 * hb);
+            ++w;
+            for (int k = 0; k < it.cnt; ++k, ++n) {
+                const uint32_t slot = n % kScSlots;
+                if (n >= kScSlots) ok = score_wait_warp(empty + 8 * slot, ((n / kScSlots) - 1) & 1, &bad);
+                if (!ok) break;
+                tc_expect_tx_elect(full + 8 * slot, kScTileBytes);
+                tc_bulk_g2s_elect(ring + slot * kScTileBytes, s.sc_pix + (size_t)(it.t0 + k) * kScTileBytes, kScTileBytes, full + 8 * slot);
             }
-            // the last copies may still be landing when another role gave up
-            for (uint32_t j = n > kScSlots ? n - kScSlots : 0; j < n; ++j)
-                score_wait(full + 8 * (j % kScSlots), (j / kScSlots) & 1, nullptr);
-            for (uint32_t j = w > 2 ? w - 2 : 0; j < w; ++j) score_wait(hfull + 8 * (j & 1), (j >> 1) & 1, nullptr);
         }
+        // the last copies may still be landing when another role gave up
+        for (uint32_t j = n > kScSlots ? n - kScSlots : 0; j < n; ++j)
+            score_wait(full + 8 * (j % kScSlots), (j / kScSlots) & 1, nullptr);
+        for (uint32_t j = w > 2 ? w - 2 : 0; j < w; ++j) score_wait(hfull + 8 * (j & 1), (j >> 1) & 1, nullptr);
     } else if (warp == kScWarps + 1) {
-        if (lane == 0) {
-            // MMA issuer: m counts stages (stage m in TMEM buffer m % kScBufs)
-            constexpr uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kScTilePix >> 4) << 24);
-            constexpr uint32_t idS = id | ((uint32_t)(3 * kScStageHyps >> 3) << 17), idX = id | ((uint32_t)(kScStageHyps >> 3) << 17);
-            constexpr uint32_t kA = kScTilePix * 16;                   // bytes of a column block of A
-            uint32_t n = 0, w = 0, m = 0;
-            for (int u = blockIdx.x; u < n_items && !bad; u += gridDim.x) {
-                const ScItem it = item(u);
-                if (it.cnt == 0) continue;
-                const uint32_t hb = w & 1;
-                if (!score_wait(hfull + 8 * hb, (w >> 1) & 1, &bad)) break;
-                const int stages = (it.hyps + kScStageHyps - 1) / kScStageHyps;
-                for (int k = 0; k < it.cnt && !bad; ++k, ++n) {
-                    const uint32_t slot = n % kScSlots, a = ring + slot * kScTileBytes;
-                    if (!score_wait(full + 8 * slot, (n / kScSlots) & 1, &bad)) break;
-                    for (int st = 0; st < stages; ++st, ++m) {
-                        const uint32_t tb = m % kScBufs;
-                        if (m >= kScBufs && !score_wait(aempty + 8 * tb, ((m / kScBufs) - 1) & 1, &bad)) break;
-                        tc_fence_after();
-                        const uint32_t b = hyp_s + hb * kScGroupBytes + st * kScStageBytes, d = tmem + tb * kScStageCols;
-                        // column blocks of A: S at 0, U at 4, V at 8; each block's small products are in its
-                        // first two column blocks, the large ones of U and V in the last two of U and V
-                        auto mma_s = [&](int half, uint32_t acc) {
-                            tc_mma(d, tc_desc(a + 2 * half * kA, kA, 128), tc_desc(b + 2 * half * kScHypSBlock, kScHypSBlock, 128), idS, acc);
-                        };
-                        auto mma_x = [&](int v, int half) {
-                            tc_mma(d + v * kScStageHyps, tc_desc(a + (4 + 4 * v + 2 * half) * kA, kA, 128),
-                                   tc_desc(b + (v ? kScHypVOff : kScHypUOff) + 2 * half * kScHypXBlock, kScHypXBlock, 128), idX, 1u);
-                        };
-                        mma_s(0, 0u);
-                        mma_s(1, 1u);
-                        mma_x(0, 0);
-                        mma_x(1, 0);
-                        mma_x(0, 1);
-                        mma_x(1, 1);
-                        tc_commit(afull + 8 * tb);
-                    }
-                    if (bad) break;
-                    tc_commit(empty + 8 * slot);
+        // MMA issuer: stages in TMEM buffers 0 .. kScBufs - 1 in turn, tb the next one's
+        constexpr uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kScTilePix >> 4) << 24);
+        constexpr uint32_t idS = id | ((uint32_t)(3 * kScStageHyps >> 3) << 17), idX = id | ((uint32_t)(kScStageHyps >> 3) << 17);
+        constexpr uint32_t kA = kScTilePix * 16;                       // bytes of a column block of A
+        uint32_t n = 0, w = 0, m = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < n_items && ok; u += gridDim.x) {
+            const ScItem it = item(u);
+            if (it.cnt == 0) continue;
+            const uint32_t hb = w & 1;
+            ok = score_wait_warp(hfull + 8 * hb, (w >> 1) & 1, &bad);
+            const int stages = (it.hyps + kScStageHyps - 1) / kScStageHyps;
+            for (int k = 0; k < it.cnt && ok; ++k, ++n) {
+                const uint32_t slot = n % kScSlots, a = ring + slot * kScTileBytes;
+                ok = score_wait_warp(full + 8 * slot, (n / kScSlots) & 1, &bad);
+                for (int st = 0; st < stages && ok; ++st, ++m) {
+                    const uint32_t tb = m % kScBufs;
+                    if (m >= kScBufs) ok = score_wait_warp(aempty + 8 * tb, ((m / kScBufs) - 1) & 1, &bad);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t b = hyp_s + hb * kScGroupBytes + st * kScStageBytes, d = tmem + tb * kScStageCols;
+                    // column blocks of A: S at 0, U at 4, V at 8; each block's small products are in its
+                    // first two column blocks, the large ones of U and V in the last two of U and V
+                    auto mma_s = [&](int half, uint32_t acc) {
+                        tc_mma_elect(d, tc_desc(a + 2 * half * kA, kA, 128), tc_desc(b + 2 * half * kScHypSBlock, kScHypSBlock, 128), idS, acc);
+                    };
+                    auto mma_x = [&](int v, int half) {
+                        tc_mma_elect(d + v * kScStageHyps, tc_desc(a + (4 + 4 * v + 2 * half) * kA, kA, 128),
+                                     tc_desc(b + (v ? kScHypVOff : kScHypUOff) + 2 * half * kScHypXBlock, kScHypXBlock, 128), idX, 1u);
+                    };
+                    mma_s(0, 0u);
+                    mma_s(1, 1u);
+                    mma_x(0, 0);
+                    mma_x(1, 0);
+                    mma_x(0, 1);
+                    mma_x(1, 1);
+                    tc_commit_elect(afull + 8 * tb);
                 }
-                if (bad) break;
-                tc_commit(hempty + 8 * hb);
-                ++w;
+                if (ok) tc_commit_elect(empty + 8 * slot);
             }
-            tc_commit(done);                  // arrives once every MMA issued above has completed
-            score_wait(done, 0, nullptr);
+            if (ok) tc_commit_elect(hempty + 8 * hb);
+            ++w;
         }
+        tc_commit_elect(done);                // arrives once every MMA issued above has completed
+        score_wait(done, 0, nullptr);
     } else {
         const int quarter = warp & 3, wg = warp >> 2;
         const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -527,6 +546,9 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
                     tmem_ld<kL>(cols + part * kL + kScStageHyps, V);
                     tmem_ld<kL>(cols + part * kL + 2 * kScStageHyps, Z);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tmem_hold<kL>(U);
+                    tmem_hold<kL>(V);
+                    tmem_hold<kL>(Z);
                     if (part == kScStageHyps / kL - 1) {      // the warp's columns are in registers
                         tc_fence_before();
                         __syncwarp();
