@@ -289,14 +289,6 @@ __device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t* r)
                  : "r"(taddr));
 }
 
-// Keeps what reads loaded columns behind the wait for them.
-template <int NC>
-__device__ __forceinline__ void tmem_hold(uint32_t* r)
-{
-#pragma unroll
-    for (int i = 0; i < NC; ++i) asm volatile("" : "+r"(r[i]));
-}
-
 // Bounded wait on an mbarrier phase: false (and *bad set, if given) on expiry or
 // when another role of the CTA already gave up. The loop is out of line: the
 // first try nearly always succeeds, and the hot loop holds only that.
@@ -546,9 +538,9 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
                     tmem_ld<kL>(cols + part * kL + kScStageHyps, V);
                     tmem_ld<kL>(cols + part * kL + 2 * kScStageHyps, Z);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    tmem_hold<kL>(U);
-                    tmem_hold<kL>(V);
-                    tmem_hold<kL>(Z);
+                    tc_hold<kL>(U);
+                    tc_hold<kL>(V);
+                    tc_hold<kL>(Z);
                     if (part == kScStageHyps / kL - 1) {      // the warp's columns are in registers
                         tc_fence_before();
                         __syncwarp();

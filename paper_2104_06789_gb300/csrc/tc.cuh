@@ -71,6 +71,14 @@ __device__ __forceinline__ void tc_bulk_g2s_elect(uint32_t dst, const void* src,
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// Keeps what reads columns loaded from tensor memory behind the wait for them.
+template <int NC>
+__device__ __forceinline__ void tc_hold(uint32_t* r)
+{
+#pragma unroll
+    for (int i = 0; i < NC; ++i) asm volatile("" : "+r"(r[i]));
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
