@@ -608,6 +608,19 @@ __device__ void se3_exp_vec(const double* p6, double* Rt)
     Rt[11] = rho[2] + B * a[2] + C * b[2];
 }
 
+// What the scoring needs beside n hypotheses' own rows, by the first 32 of the threads:
+// zeros as the partner of an odd last one, and the pixel chunks of a frame with few.
+__device__ __forceinline__ void finish_hypotheses(const DevParams& p, const DevState& s, int n, int id)
+{
+    if (id >= 32) return;
+    if ((n & 1) && id < kScHypChunks) clear_hyp_operand(s.sc_hyp, n, id);
+    const int groups = (n + kScGroupHyps - 1) / kScGroupHyps, all = (p.S + kScGroupHyps - 1) / kScGroupHyps;
+    int chunks = 0;
+    if (groups > 0 && groups < all)
+        chunks = chunks_for_groups(groups, max(1, (*s.pix_count + kScTilePix - 1) / kScTilePix), s.chunks_max, s.score_ctas);
+    if (id == 0) *s.few_chunks = chunks;
+}
+
 // Hypothesis collection: four lanes per (group, solution slot), one for each row of
 // [R | t], write its solution h = offset + slot < S with its scoring form and tensor-core operand.
 // A block covers 8 groups and finds its offset itself, as the sum of all earlier
@@ -653,12 +666,12 @@ __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState
         }
         if (tid < kHypGroups) off_s[tid] = base + incl - c;
         if (tid == 31) {
-            n_s = 0;
+            n_s = -1;
             if (g0 + kHypGroups >= G) *s.n_hyp = n_s = min(base + incl, p.S);      // the last block with groups
         }
     }
     __syncthreads();
-    if ((n_s & 1) && tid < kScHypChunks) clear_hyp_operand(s.sc_hyp, n_s, tid);   // the last hypothesis's partner
+    if (n_s >= 0) finish_hypotheses(p, s, n_s, tid);
     const int item = tid >> 2, r = min(tid & 3, 2), g = g0 + item / kMaxSols, i = item % kMaxSols;
     if (g >= G || i >= s.grp_count[g]) return;            // whole quads leave together
     const int h = off_s[item / kMaxSols] + i;
@@ -729,7 +742,7 @@ __global__ void k_hyp_from_rt(DevParams p, DevState s, int t, int n)
 {
     const int id = blockIdx.x * blockDim.x + threadIdx.x, h = id >> 2, r = min(id & 3, 2);
     if (id == 0) *s.n_hyp = n;
-    if ((n & 1) && id < kScHypChunks) clear_hyp_operand(s.sc_hyp, n, id);   // the last hypothesis's partner
+    finish_hypotheses(p, s, n, id);
     if (h >= n) return;                                   // whole quads leave together
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};

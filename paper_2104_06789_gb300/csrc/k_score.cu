@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kScThreads, 1) k_score(DevParams p, DevState s
         s.score_log[2 * log_idx + 1] = n_pix;
     }
     const int n_tiles = (n_pix + kScTilePix - 1) / kScTilePix;
-    const int n_groups = (n_hyp + kScGroupHyps - 1) / kScGroupHyps, n_chunks = s.n_chunks;
+    const int few = *s.few_chunks, n_groups = (n_hyp + kScGroupHyps - 1) / kScGroupHyps, n_chunks = few ? few : s.n_chunks;
     const int n_items = n_groups * n_chunks;
     if (blockIdx.x >= n_items) return;
     auto item = [&](int u) {
@@ -672,6 +672,8 @@ int score_chunks_for(int S, int N, int waves)
     return best;
 }
 
+int score_ctas() { return num_sms(); }
+
 int score_chunks(int S, int N) { return score_chunks_for(S, N, kScoreDefaultWaves); }
 
 // Largest chunk count a window accepts (and its partial sums are sized for).
@@ -700,8 +702,10 @@ static void launch_score_as(const DevParams& p, const DevState& s, int li, cudaS
             raised[dev] = cudaFuncSetAttribute(k_score<kL, kMLE, kGauss>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                kScSmemBytes) == cudaSuccess;
     }
-    const long long items = (long long)((p.S + kScGroupHyps - 1) / kScGroupHyps) * s.n_chunks;
-    k_score<kL, kMLE, kGauss><<<(unsigned)std::min<long long>(items, num_sms()), kScThreads, kScSmemBytes, st>>>(p, s, li);
+    // a frame with fewer groups may have more items than a full one's
+    const int groups = (p.S + kScGroupHyps - 1) / kScGroupHyps;
+    const long long items = (long long)groups * s.n_chunks, most = groups > 1 ? num_sms() : items;
+    k_score<kL, kMLE, kGauss><<<(unsigned)std::min<long long>(most, num_sms()), kScThreads, kScSmemBytes, st>>>(p, s, li);
 }
 
 template <int kL>

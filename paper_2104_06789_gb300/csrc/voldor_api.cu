@@ -172,6 +172,7 @@ size_t layout(voldor_ctx& c, char* base)
     s.hyp_info = (long long*)take(S * 2 * 8);
     s.partial = (double*)take((size_t)chunks_max * S * 8);
     s.score_done = (int*)take((S + kScGroupHyps - 1) / kScGroupHyps * 4);
+    s.few_chunks = (int*)take(4);
     s.scores = (double*)take(S * 8);
     s.mie_prev_score = (float*)take(N * 4);
     s.mie_smp = (float*)take(N * 4);
@@ -180,6 +181,8 @@ size_t layout(voldor_ctx& c, char* base)
     s.labels = (unsigned char*)take(N);
     s.score_log = (long long*)take((size_t)kScoreLogMax * 2 * 8);
     s.n_chunks = chunks;
+    s.chunks_max = chunks_max;
+    s.score_ctas = score_ctas();
     s.score_hpt = kScoreDefaultHpt;
     return off;
 }
@@ -843,7 +846,8 @@ voldor_status voldor_autotune(voldor_ctx* c, int* hpt_out, int* chunks_out, floa
     launch_pose_prep(c->dp, c->ds, 1, c->stream);
     launch_p3p_groups(c->dp, c->ds, 1, c->stream);
     launch_hyp_collect(c->dp, c->ds, 1, c->stream);
-    if (!launched(c)) return kCuda;
+    // frame 1 stands for a full one here, however few its hypotheses are
+    if (!launched(c) || !cuda_ok(c, cudaMemsetAsync(c->ds.few_chunks, 0, 4, c->stream))) return kCuda;
     cudaEvent_t e0, e1;
     if (!cuda_ok(c, cudaEventCreate(&e0)) || !cuda_ok(c, cudaEventCreate(&e1))) return kCuda;
     const int saved_hpt = c->ds.score_hpt, saved_chunks = c->ds.n_chunks;

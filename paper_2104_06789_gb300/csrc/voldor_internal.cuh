@@ -102,7 +102,7 @@ struct DevState {
     double* hyp_w;            // [S]
     float* hyp_dp;            // [S][8] meanshift scratch: p_h - p_seed (6), w_h, 0
     long long* hyp_info;      // [S][2]
-    double* partial;          // [n_chunks][S]
+    double* partial;          // [chunks_max][S]
     int* score_done;          // [ceil(S / 128)] chunks scored per hypothesis group (0 between launches)
     double* scores;           // [S]
     // depth sweep
@@ -112,7 +112,10 @@ struct DevState {
     int* mie_next;            // [N] end of each pixel's speculative run (chain position), negative if capped
     unsigned char* labels;    // [N]
     long long* score_log;     // [kScoreLogMax][2] (n_hyp, n_pix) of timed scoring launches
-    int n_chunks;             // dense scoring pixel chunks
+    int n_chunks;             // dense scoring pixel chunks of a frame with all its hypotheses
+    int chunks_max;           // chunks that `partial` holds
+    int score_ctas;           // SMs: the scoring's largest grid
+    int* few_chunks;          // [1] pixel chunks of a frame with fewer groups of hypotheses, 0 for n_chunks
     int score_hpt;            // hypotheses a scoring thread takes from tensor memory at a time (2, 4 or 8)
 };
 
@@ -327,6 +330,7 @@ int launch_ground_scale(const DevParams& p, const DevState& s, double camera_hei
                         double dmax, int apply, unsigned* hist, double* out, cudaStream_t st);
 int score_chunks_for(int S, int N, int waves);
 int score_chunks_max(int S, int N);
+int score_ctas();
 void score_hyps_from_host(const DevParams& p, const DevState& s, int t, int n, cudaStream_t st);
 
 }  // namespace vd
