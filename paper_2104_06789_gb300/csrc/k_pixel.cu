@@ -383,28 +383,39 @@ __global__ void k_mie_runs(DevParams p, DevState s)
 constexpr int kResolveWarps = 16, kResolveThreads = 32 * kResolveWarps;
 constexpr int kMaxChain = kMaxImageSide;
 
-// End of the run of own_r, which survived up to position `pos` of chain c: a warp tests
-// 32 / G positions at a time, G lanes to a position, a frame each (two from T = 9 on);
-// the frames' terms are independent, only their sum is in order.
-__device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, float v)
+// Positions of a chain a warp tests at a time with G lanes to a position, a frame each
+// (two from T = 9 on); the frames' terms are independent, only their sum is in order.
+__device__ __forceinline__ int test_lanes(const DevParams& p) { return p.T > 4 ? 8 : (p.T > 2 ? 4 : p.T); }
+
+// The lanes of a warp at which v is lost, tested at positions pos, pos + 1, ... of chain c.
+__device__ unsigned mie_test(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, int G, float v)
 {
-    const int lane = threadIdx.x & 31, G = p.T > 4 ? 8 : (p.T > 2 ? 4 : p.T), sub = lane % G, first = lane - sub;
-    for (;; pos += 32 / G) {
-        const int q = pos + lane / G;
-        int x, y;
-        chain_xy(p, dir, c, min(q, len - 1), x, y);
-        const int j = y * p.W + x;
-        float term[2] = {0.f, 0.f};
+    const int lane = threadIdx.x & 31, sub = lane % G, first = lane - sub, q = pos + lane / G;
+    int x, y;
+    chain_xy(p, dir, c, min(q, len - 1), x, y);
+    const int j = y * p.W + x;
+    float term[2] = {0.f, 0.f};
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int t = u * G + sub + 1;
-            if (t <= p.T) term[u] = __fmul_rn(s.qs[(size_t)(t - 1) * p.N + j], depth_ell_fast(p, f.v[t - 1], s.flows, t, x, y, v));
-        }
-        float acc = 0.f;
-        for (int t = 0; t < p.T; ++t) acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, t < G ? term[0] : term[1], first + t % G));
-        const unsigned lost = __ballot_sync(0xffffffffu, q >= len || !survives(s, j, nan_to_ninf(acc)));
-        if (lost) return min(pos + (__ffs(lost) - 1) / G, len);
+    for (int u = 0; u < 2; ++u) {
+        const int t = u * G + sub + 1;
+        if (t <= p.T) term[u] = __fmul_rn(s.qs[(size_t)(t - 1) * p.N + j], depth_ell_fast(p, f.v[t - 1], s.flows, t, x, y, v));
     }
+    float acc = 0.f;
+    for (int t = 0; t < p.T; ++t) acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, t < G ? term[0] : term[1], first + t % G));
+    return __ballot_sync(0xffffffffu, q >= len || !survives(s, j, nan_to_ninf(acc)));
+}
+
+// End of the run of v, which survived up to position `pos` of chain c, by one warp; -q if
+// it is alive at a position q >= limit, not tested yet.
+__device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, int limit, float v)
+{
+    const int G = test_lanes(p);
+    do {
+        const unsigned lost = mie_test(p, s, f, dir, c, len, pos, G, v);
+        if (lost) return min(pos + (__ffs(lost) - 1) / G, len);
+        pos += 32 / G;
+    } while (pos < limit);
+    return pos < len ? -pos : len;
 }
 
 // Resolution of one chain per block. The walk r -> end of r's run depends on nothing
@@ -415,14 +426,27 @@ __device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF&
 // the part's own walk, from there on by its result. A chain's runs one after another,
 // tested by the whole block, took 212 us at 1242 x 375, T = 8; with the parts 57, and
 // 108 with a cap of 2 instead of 8 (see kRunCap). 8 parts: 101, 32: 146.
-__global__ void __launch_bounds__(kResolveThreads) k_mie_resolve(DevParams p, DevState s)
+//
+// A run that goes on kOver positions past its warp's part is left open: the true walk may
+// never come by it, and where it does (or meets a run of its own that outlives kAlone
+// positions) the whole block tests the next positions at once. Followed to their ends by
+// the parts' warps, runs of hundreds of positions, as over a plane whose depth was poor
+// and whose flows are quiet, made the sweep 955 us at 1242 x 375, T = 8; now 464, with
+// every test by the block (before there were parts) 545. Scenes of short runs lose 1 to 3 %.
+// Tried: all warps walking (421 there, but 3 to 8 % on short runs), long runs a lane per
+// position instead of a frame per lane (no change), two more blocks per SM (40 registers,
+// spills).
+constexpr int kOver = 32, kAlone = 16;
+
+__global__ void __launch_bounds__(kResolveThreads, 2) k_mie_resolve(DevParams p, DevState s)
 {
     __shared__ FramesF f;
     __shared__ short origin[kMaxChain];
     __shared__ int next_s[kMaxChain];
     __shared__ float own_s[kMaxChain];
     __shared__ unsigned char reset[kMaxChain];             // 1: on the part's own walk, 2: on the true one before they meet
-    __shared__ int part_end[kResolveWarps], part_from[kResolveWarps], last_s[kResolveWarps];
+    __shared__ int part_end[kResolveWarps], part_last[kResolveWarps], part_from[kResolveWarps], last_s[kResolveWarps];
+    __shared__ int first_lost[3];
     load_frames32(p, s, f);
     const int dir = (*s.iter) & 3;
     const bool rows = (dir == 0 || dir == 2);
@@ -438,38 +462,80 @@ __global__ void __launch_bounds__(kResolveThreads) k_mie_resolve(DevParams p, De
         reset[q] = 0;
     }
     __syncthreads();
-    // the end of r's run, kept for the next to ask
-    auto end_of = [&](int r) {
-        int e = next_s[r];
-        if (e < 0) {
-            e = mie_run_end(p, s, f, dir, c, len, -e, own_s[r]);
-            __syncwarp();
-            if (lane == 0) next_s[r] = e;
-            __syncwarp();
-        }
-        return e;
-    };
     const int part = (len + kResolveWarps - 1) / kResolveWarps;
     {
         const int stop = min((warp + 1) * part, len);
-        int r = min(warp * part, len);
-        while (r < stop) {
+        int r = min(warp * part, len), last = 0;
+        while (r >= 0 && r < stop) {
+            last = r;
+            int e = next_s[r];
+            if (e < 0) {
+                e = mie_run_end(p, s, f, dir, c, len, -e, stop + kOver, own_s[r]);
+                __syncwarp();
+                if (lane == 0) next_s[r] = e;
+            }
             if (lane == 0) reset[r] = 1;
-            r = end_of(r);
+            r = e;
         }
-        if (lane == 0) part_end[warp] = r;
+        if (lane == 0) {
+            part_end[warp] = r;
+            part_last[warp] = last;
+        }
     }
+    if (threadIdx.x == 0) first_lost[0] = kMaxChain;
     __syncthreads();
+    // the end of an open run of v, alive at `pos`, by the whole block
+    int step = 0;
+    auto follow = [&](int pos, float v) {
+        const int G = test_lanes(p), wide = 32 / G;
+        for (;; pos += wide * kResolveWarps) {
+            const unsigned lost = mie_test(p, s, f, dir, c, len, pos + warp * wide, G, v);
+            const int slot = step % 3;
+            step += 1;
+            if (lane == 0 && lost) atomicMin(&first_lost[slot], pos + warp * wide + (__ffs(lost) - 1) / G);
+            if (threadIdx.x == 0) first_lost[step % 3] = kMaxChain;     // read for the last time two steps ago
+            __syncthreads();
+            const int at = first_lost[slot];
+            if (at < kMaxChain) return min(at, len);
+            if (pos + wide * kResolveWarps >= len) return len;
+        }
+    };
+    // warp 0 walks; the others wait for the open runs it meets
+    __shared__ int open_pos[2];
+    __shared__ float open_v[2];
+    int call = 0;
     if (warp == 0) {
+        auto ask = [&](int pos, float v) {
+            pos = mie_run_end(p, s, f, dir, c, len, pos, pos + kAlone, v);
+            if (pos >= 0) return pos;
+            pos = -pos;
+            if (lane == 0) { open_pos[call & 1] = pos; open_v[call & 1] = v; }
+            call += 1;
+            __syncthreads();
+            return follow(pos, v);
+        };
         int r = 0;
         for (int k = 0; k < kResolveWarps; ++k) {
             const int stop = min((k + 1) * part, len);
             while (r < stop && reset[r] != 1) {
                 if (lane == 0) reset[r] = 2;
-                r = end_of(r);
+                const int e = next_s[r];
+                r = e < 0 ? ask(-e, own_s[r]) : e;
             }
             if (lane == 0) part_from[k] = r < stop ? r : len;
-            if (r < stop) r = part_end[k];
+            if (r < stop) {
+                r = part_end[k];
+                if (r < 0) r = ask(-r, own_s[part_last[k]]);
+            }
+        }
+        if (lane == 0) open_pos[call & 1] = -1;
+        __syncthreads();
+    } else {
+        for (;; ++call) {
+            __syncthreads();
+            const int pos = open_pos[call & 1];
+            if (pos < 0) break;
+            follow(pos, open_v[call & 1]);
         }
     }
     __syncthreads();
