@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
     const int cnt = __syncthreads_count(valid);
     // the last block to finish turns the block counts into block offsets
     // (exclusive scan, in place), sets the record count and clears the P3P
-    // claim counters of the frame; no block waits
+    // claim counters and coarse counts of the frame; no block waits
     __shared__ bool last;
     if (threadIdx.x == 0) {
         s.pix_block_count[blockIdx.x] = cnt;
@@ -120,6 +120,8 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
         counts[b] = off;
         off += c;
     }
+    static_assert(kP3PMaxBlocks <= kPixThreads, "one count a thread");
+    if (threadIdx.x < kP3PMaxBlocks) s.block_sols[threadIdx.x] = 0;
     if (threadIdx.x == blockDim.x - 1) {
         *s.pix_count = off;
         *s.prep_done = 0u;

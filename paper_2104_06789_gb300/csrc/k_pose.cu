@@ -407,8 +407,6 @@ __device__ bool group_point(const DevParams& p, const DevState& s, const double*
 // computed in two lanes that one can do, divisions by constants go through their
 // reciprocals, a Newton step keeps its residual for the next and leaves out the zeros
 // of its matrix: 53 -> 45 us up to S = 2048, 58 -> 50 at 4096, 77 -> 64 at 8192.
-constexpr int kP3PChunk = 8;
-
 __global__ void __launch_bounds__(32) k_p3p_groups(DevParams p, DevState s, int t)
 {
     const int lane = threadIdx.x, quad = lane >> 2, r = lane & 3, base = lane & ~3;
@@ -503,7 +501,11 @@ __global__ void __launch_bounds__(32) k_p3p_groups(DevParams p, DevState s, int 
         int tot = (r == 0) ? cnt : 0;
         for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(FULL, tot, o);
         __threadfence();
-        if (lane == 0) atomicAdd(s.p3p_done, (1ull << 32) | (unsigned long long)tot);
+        if (lane == 0) {
+            s.chunk_sols[c] = tot;
+            if (tot) atomicAdd(s.block_sols + c / kP3PBlock, tot);
+            atomicAdd(s.p3p_done, (1ull << 32) | (unsigned long long)tot);
+        }
     }
 }
 
@@ -623,12 +625,13 @@ __device__ __forceinline__ void finish_hypotheses(const DevParams& p, const DevS
 
 // Hypothesis collection: four lanes per (group, solution slot), one for each row of
 // [R | t], write its solution h = offset + slot < S with its scoring form and tensor-core operand.
-// A block covers 8 groups and finds its offset itself, as the sum of all earlier
-// groups' counts: up to 24 KB of counts read from L2 per block take less time than
-// a scan kernel before this one (4 us and a launch per frame).
+// A block covers the 8 groups of a P3P chunk and finds its offset itself, from the chunks'
+// and the coarse counts that P3P leaves (at most 255 and 128 of them): a scan kernel
+// before this one took 4 us and a launch per frame, and the sum of all earlier groups'
+// counts, G^2 / 16 of them in all, 0.4 of 2.0 ms of a frame with 262144 groups solved.
 // A lane per solution, with all of its FP64 work, took 10.7 us at S = 256 (14.6 at
 // 8192), four lanes with 32 groups to a block, all on one SM, 12.2 (19.1); now 7.5 (14.5).
-constexpr int kHypGroups = 8;              // groups per block
+constexpr int kHypGroups = kP3PChunk;      // groups per block
 constexpr int kHypThreads = kHypGroups * kMaxSols * 4;
 
 __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState s, int t)
@@ -648,10 +651,9 @@ __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState
         e0[r * 4 + c] = v;
     }
     int before = 0;
-    for (int i = tid; i < g0 / 4; i += blockDim.x) {
-        const int4 c = *reinterpret_cast<const int4*>(s.grp_count + 4 * i);
-        before += c.x + c.y + c.z + c.w;
-    }
+    const int full = blockIdx.x / kP3PBlock;              // coarse counts before this block's groups
+    for (int i = tid; i < full; i += kHypThreads) before += s.block_sols[i];
+    for (int i = full * kP3PBlock + tid; i < blockIdx.x; i += kHypThreads) before += s.chunk_sols[i];
     for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
     if (lane == 0) wsum[tid >> 5] = before;
     __syncthreads();

@@ -76,7 +76,7 @@ bool params_ok(const voldor_params& p)
     if (!finite_pos(p.x_min) || !finite_pos(p.x_max) || !(p.x_max > p.x_min)) return false;
     if (!finite_pos(p.beta_min) || !(p.ms_tol >= 0.0) || !std::isfinite(p.ms_tol)) return false;
     if (p.hyps_per_frame < 1 || p.hyps_per_frame > 65536) return false;
-    if (p.groups_per_frame < 1 || p.groups_per_frame > 262144) return false;
+    if (p.groups_per_frame < 1 || p.groups_per_frame > kMaxGroups) return false;
     if (p.ms_max_iter < 1 || p.ms_max_iter > 100000) return false;
     if (p.criterion != VOLDOR_CRITERION_MIE && p.criterion != VOLDOR_CRITERION_MLE) return false;
     if (p.residual != VOLDOR_RESIDUAL_FISK && p.residual != VOLDOR_RESIDUAL_GAUSSIAN) return false;
@@ -163,6 +163,8 @@ size_t layout(voldor_ctx& c, char* base)
     s.grp_sols = (double*)take(G * kMaxSols * 12 * 8);
     s.grp_weight = (double*)take(G * 8);
     s.grp_count = (int*)take(G * 4);
+    s.chunk_sols = (int*)take((G + kP3PChunk - 1) / kP3PChunk * 4);
+    s.block_sols = (int*)take(kP3PMaxBlocks * 4);
     s.n_hyp = (int*)take(4);
     s.hyp_Rt = (double*)take(S * 12 * 8);
     s.hyp_f32 = (float*)take(S * 12 * 4);

@@ -23,6 +23,10 @@ constexpr int kScoreHypsPerBlock = kScoreThreads * kScoreHypsPerThread;
 constexpr int kMeanshiftCtas = 8;      // thread-block cluster of the meanshift
 constexpr int kMeanshiftThreads = 256;
 constexpr int kPixThreads = 256;
+constexpr int kP3PChunk = 8;           // minimal groups a P3P warp solves at a time
+constexpr int kP3PBlock = 256;         // chunks to a coarse count of solutions
+constexpr int kMaxGroups = 262144;     // largest group budget of a frame
+constexpr int kP3PMaxBlocks = kMaxGroups / (kP3PChunk * kP3PBlock);
 constexpr int kScoreLogMax = 1024;
 // Status word 3 of a window: a count of frames whose pose update was
 // degenerate, plus this bit when a bounded device-side wait gave up.
@@ -90,11 +94,13 @@ struct DevState {
     int* pix_count;           // [1]
     unsigned* pix_vmask;      // [ceil(N / kPixThreads) * kPixThreads / 32] per-warp ballots of the valid pixels
     // P3P
-    int* p3p_claims;          // [1] 32-group chunks claimed by the P3P warps of the current frame
+    int* p3p_claims;          // [1] chunks of kP3PChunk groups claimed by the P3P warps of the current frame
     unsigned long long* p3p_done;   // [1] chunks solved (high 32 bits) and their solutions (low 32 bits)
     double* grp_sols;         // [G][4][12]
     double* grp_weight;       // [G]
     int* grp_count;           // [G]
+    int* chunk_sols;          // [ceil(G / 8)] solutions of each chunk of kP3PChunk groups
+    int* block_sols;          // [kP3PMaxBlocks] their sums over kP3PBlock chunks
     int* n_hyp;               // [1]
     double* hyp_Rt;           // [S][12]
     float* hyp_f32;           // [S][12] scoring form
