@@ -24,6 +24,7 @@ struct voldor_ctx {
     cudaStream_t stream = nullptr;
     void* arena = nullptr;
     size_t arena_bytes = 0;
+    size_t cleared_bytes = 0;         // of the arena, from its start: set to zero
     size_t flows_bytes = 0;
     int* flag_dev = nullptr;          // inside the arena: counter of rejected flow blocks
     bool bootstrapped = false;
@@ -149,7 +150,6 @@ size_t layout(voldor_ctx& c, char* base)
     s.iter = (int*)take(4);
     s.status = (int*)take(16);
     c.flag_dev = (int*)take(4);
-    s.sc_pix = (unsigned char*)take((N + kScTilePix - 1) / kScTilePix * kScTileBytes);
     s.sc_cst = (float4*)take(N * sizeof(float4));
     s.sc_xmu = (float*)take(N * sizeof(float));
     s.sc_hyp = (unsigned char*)take((S + kScGroupHyps - 1) / kScGroupHyps * kScGroupBytes);
@@ -182,6 +182,9 @@ size_t layout(voldor_ctx& c, char* base)
     s.mie_next = (int*)take(N * 4);
     s.labels = (unsigned char*)take(N);
     s.score_log = (long long*)take((size_t)kScoreLogMax * 2 * 8);
+    // last, and not cleared: what no pixel has written enters no result
+    c.cleared_bytes = off;
+    s.sc_pix = (unsigned char*)take((N + kScTilePix - 1) / kScTilePix * kScTileBytes);
     s.n_chunks = chunks;
     s.chunks_max = chunks_max;
     s.score_ctas = score_ctas();
@@ -461,7 +464,7 @@ voldor_status voldor_init_window(voldor_ctx** out, int width, int height, int T,
         voldor_destroy(c);
         return kCuda;
     }
-    if (!cuda_ok(c, cudaMemsetAsync(c->arena, 0, bytes, c->stream))) { voldor_destroy(c); return kCuda; }
+    if (!cuda_ok(c, cudaMemsetAsync(c->arena, 0, c->cleared_bytes, c->stream))) { voldor_destroy(c); return kCuda; }
     voldor_status st = upload_flows(c, flows, flows_on_device);
     if (st != VOLDOR_OK) { voldor_destroy(c); return st; }
     *out = c;
