@@ -122,18 +122,8 @@ __host__ __device__ constexpr uint32_t tc_idesc(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
 }
 
-// Bounded wait; false (and *bad set) on expiry or when another role already gave up.
-__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, volatile int* bad)
-{
-    for (long long i = 0; i < kTcWaitLimit; ++i) {
-        if (tc_try_wait(bar, parity)) return true;
-        if ((i & 1023) == 1023 && *bad) return false;
-    }
-    *bad = 1;
-    return false;
-}
-
-// The same for a converged warp, with one answer for all its lanes.
+// Bounded wait of a converged warp, with one answer for all its lanes; false (and *bad set)
+// on expiry or when another role already gave up.
 __device__ __forceinline__ bool tc_wait_warp(uint32_t bar, uint32_t parity, volatile int* bad)
 {
     for (long long i = 0; i < kTcWaitLimit; ++i) {
@@ -148,12 +138,6 @@ __device__ __forceinline__ void tc_tma_row_elect(uint32_t dst, const CUtensorMap
 {
     asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
                  " @q cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n}"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tc_tma_row(uint32_t dst, const CUtensorMap* map, int c, int x, int y, int b, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
                  ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(bar) : "memory");
 }
 
@@ -508,10 +492,8 @@ static bool launch_conv_tc(const ConvArgs& a, cudaStream_t st)
 
 // Arguments of the weight-gradient kernel below.
 struct WgradArgs {
-    const bf16* in;
-    int cin_g;
-    const bf16* dout;       // channel stride cout_g
-    int cout_g;
+    const bf16* in;         // CIN channels a pixel
+    const bf16* dout;       // NCO channels a pixel
     float* part;            // [gridDim.x][9 CIN + 1][NCO] each CTA's sums
     int H, W, B;
     int* err;               // set to 1 if a bounded wait expired
@@ -1173,7 +1155,7 @@ bool wgrad(voldor_net* n, int l, const bf16* in, int cin_g, const bf16* dout, in
            WgLayer& g)
 {
     WgradArgs a{};
-    a.in = in; a.cin_g = cin_g; a.dout = dout; a.cout_g = cout_g;
+    a.in = in; a.dout = dout;
     a.part = n->wpart + n->wpart_off[l];
     a.H = H; a.W = W; a.B = B;
     a.err = n->tc_err;

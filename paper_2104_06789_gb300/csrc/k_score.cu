@@ -74,12 +74,9 @@ __device__ __forceinline__ float log2_1p_pos(float r)
     return r < kL1pMax ? small : big;
 }
 
-// Scalar pair term (the allocation-free entry point's form): -ell / ln2 =
-// log2(1 + mu/rho) of one (hypothesis, pixel) pair (MIE, Eq. 10), or with kMLE
-// log2(r) (MLE, Eq. 9: log rho - log mu = -ln2 * this); behind camera t,
-// rho := mu (r = 1). The checked form tests 1 + a_z > 0 and caps the squared
-// residual at xs_max.
-template <bool kChecked, bool kMLE = false>
+// Scalar pair term of the allocation-free entry point: -ell / ln2 = log2(1 + mu/rho)
+// of one (hypothesis, pixel) pair (MIE, Eq. 10), the projection in FP32 and a
+// reciprocal to each pair; behind camera t (1 + a_z <= 0) rho := mu (r = 1).
 __device__ __forceinline__ float pair_term2(const HypF& h, const float4 a, const float4 b, float xs_min, float xs_max)
 {
     const float xb = a.x, yb2 = a.y, w = a.z, ut = a.w;
@@ -91,15 +88,11 @@ __device__ __forceinline__ float pair_term2(const HypF& h, const float4 a, const
     const float rd = mufu_rcp(den);
     const float ru = fmaf(fmaf(-xb, az, ax), rd, -ut);
     const float rv = fmaf(fmaf(-yb2, az, ay), rd, -vt);
-    float xs = fmaxf(fmaf(ru, ru, rv * rv), xs_min);
-    if (kChecked) xs = fminf(xs, xs_max);
+    const float xs = fminf(fmaxf(fmaf(ru, ru, rv * rv), xs_min), xs_max);
     const float sg = fabsf(fmaf(beta, mufu_lg2(xs), beta_k));
     const float r = Cp * xs * (mufu_ex2(sg) + (2.f + mufu_ex2(-sg)));
-    const float v = kMLE ? mufu_lg2(r) : log2_1p_pos(r);
-    if (kChecked) return den > 0.f ? v : (kMLE ? 0.f : 1.f);
-    return v;
+    return den > 0.f ? log2_1p_pos(r) : 1.f;
 }
-
 
 // ---------------------------------------------------------------------------
 // Packed pair arithmetic (.f32x2).
@@ -772,7 +765,7 @@ k_score_records(const float4* __restrict__ pix, int n_pix, const float* __restri
             const float wq = __ldg(reinterpret_cast<const float*>(pix + 3 * j + 2));
 #pragma unroll
             for (int i = 0; i < kScoreHypsPerThread; ++i)
-                facc[i] = fmaf(wq, pair_term2<true>(hy[i], a, b, xs_min, xs_max), facc[i]);
+                facc[i] = fmaf(wq, pair_term2(hy[i], a, b, xs_min, xs_max), facc[i]);
         }
 #pragma unroll
         for (int i = 0; i < kScoreHypsPerThread; ++i) { acc[i] += (double)facc[i]; facc[i] = 0.f; }
