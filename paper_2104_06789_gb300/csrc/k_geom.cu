@@ -187,19 +187,22 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevStat
         const DF up{1.f, (float)(kScUntruncate - 1.0)};
         const Slice3 fs[3] = {slice3(xn), slice3(yn), slice3(iz)};
         pixel_block_s(fs, slice3(df_mul(az0, up)), o);
+        // under the Gaussian model the scoring adds the references itself, up to what FP32 leaves of them
+        const bool gauss = p.residual == VOLDOR_RESIDUAL_GAUSSIAN;
         const Slice3 fu4[4] = {slice3(df_mul(X, xn)), slice3(df_mul(X, yn)), slice3(df_mul(X, iz)), slice3(X)};
-        pixel_block_x(fu4, slice3(df_mul(U0, up)), fs, o + 32);
+        pixel_block_x(fu4, gauss ? slice3(U0.lo, 0.f) : slice3(df_mul(U0, up)), fs, o + 32);
         const Slice3 fv4[4] = {slice3(df_mul(Y, xn)), slice3(df_mul(Y, yn)), slice3(df_mul(Y, iz)), slice3(Y)};
-        pixel_block_x(fv4, slice3(df_mul(V0, up)), fs, o + 64);
+        pixel_block_x(fv4, gauss ? slice3(V0.lo, 0.f) : slice3(df_mul(V0, up)), fs, o + 64);
         const int i = base + rank;
         unsigned char* d = s.sc_pix + (size_t)(i / kScTilePix) * kScTileBytes + ((i % kScTilePix) / 8) * 128 + (i % 8) * 16;
 #pragma unroll
         for (int q = 0; q < kScPixCols / 8; ++q)
             *reinterpret_cast<uint4*>(d + q * (kScTilePix * 16)) = *reinterpret_cast<const uint4*>(o + 8 * q);
         float4 cst;
-        if (p.residual == VOLDOR_RESIDUAL_GAUSSIAN) {
+        if (gauss) {
             const GaussConst gc = gauss_const(p, n);
-            cst = make_float4(fx2 * gc.inv_alpha, -gc.x_mu * gc.inv_alpha, 0.f, 0.f);
+            cst = make_float4(fx2 * gc.inv_alpha, -gc.x_mu * gc.inv_alpha, U0.hi, 0.f);
+            s.sc_xmu[i] = V0.hi;
         } else {
             const FiskConst fc = fisk_const(p, n);
             cst = make_float4(fc.beta, fc.beta * (p.log2_fx2 - fc.log2_alpha), fx2 * fc.mu_over_beta, 0.f);

@@ -156,8 +156,8 @@ __device__ __forceinline__ f2 f2_lg2(f2 v) { return f2_pack(mufu_lg2(f2_lo(v)), 
 // Terms of P hypothesis pairs against the lane's pixel, added to acc.
 // ---------------------------------------------------------------------------
 struct PixConst {
-    f2 beta, beta_k, Cp, wq;
-    float xmu;                       // x_mu / fx^2: the squared residual at which rho = mu
+    f2 beta, beta_k, Cp, wq;         // Gaussian: Cp is the pixel's U0
+    float xmu;                       // x_mu / fx^2: the squared residual at which rho = mu; Gaussian: V0
 };
 
 // The polynomial of log2_1p_pos for r < 1/8.
@@ -183,8 +183,12 @@ __device__ __forceinline__ float lg2_if_large(float small, float r, float r1)
 // lanes of a pair, 1 / d0 = d1 / (d0 d1), d = 1 + a_z: a nonzero d is at least 2^-25
 // in size (the spacing of a_z near -1), so adding 2^-40 moves no d beyond its own
 // rounding and keeps an exact 0 from spoiling its partner; above, kWild frames (the
-// only ones where |d| may reach 2^62) take a reciprocal per lane. Behind the
-// camera (d <= 0) rho := mu. The loops over P keep P independent chains side by
+// only ones where |d| may reach 2^62) take a reciprocal per lane. So does the Gaussian
+// model, whose terms grow with the squared residual itself and carry every rounding of
+// it, and it adds U0 and V0 here, rounded, instead of in the tensor core, which
+// truncates: the error of its scores near the current pose, rms over 60 sets of
+// hypotheses against 64 bits, is 0.99 of what it was with the projection in FP32, 1.17
+// without the two. Behind the camera (d <= 0) rho := mu. The loops over P keep P independent chains side by
 // side for the in-order issue.
 template <int P, bool kMLE, bool kGauss, bool kWild>
 __device__ __forceinline__ void score_pairs(const uint32_t* U, const uint32_t* V, const uint32_t* Z, const PixConst& q,
@@ -198,14 +202,15 @@ __device__ __forceinline__ void score_pairs(const uint32_t* U, const uint32_t* V
 #pragma unroll
     for (int i = 0; i < P; ++i) {
         f2 rd;                                            // -1 / (1 + a_z): squared below
-        if (kWild) {
+        if (kWild || kGauss) {
             rd = f2_pack(mufu_rcp(f2_lo(nden[i])), mufu_rcp(f2_hi(nden[i])));
         } else {
             const f2 d = f2_add(nden[i], f2_both(9.094947e-13f));
             const float inv = mufu_rcp(f2_lo(d) * f2_hi(d));
             rd = f2_pack(inv * f2_hi(d), inv * f2_lo(d));
         }
-        const f2 ru = f2_mul(at(U, i), rd), rv = f2_mul(at(V, i), rd);
+        const f2 u = kGauss ? f2_add(at(U, i), q.Cp) : at(U, i), w = kGauss ? f2_add(at(V, i), f2_both(q.xmu)) : at(V, i);
+        const f2 ru = f2_mul(u, rd), rv = f2_mul(w, rd);
         const f2 x = f2_fma(ru, ru, f2_mul(rv, rv));
         float x0 = fminf(fmaxf(f2_lo(x), xs_min), xs_max), x1 = fminf(fmaxf(f2_hi(x), xs_min), xs_max);
         if (!kGauss && !kMLE) {
@@ -335,7 +340,8 @@ __device__ __forceinline__ bool score_wait_warp(uint32_t bar, uint32_t parity, v
 // The two issuing warps run converged: with their loops inside an `if (lane == 0)` a
 // stage's six MMAs, descriptors, waits and commit took longer than the arithmetic of the
 // light variants, and MLE with the Gaussian residual (one rcp a pair) took 1977 us a frame
-// on average there, now 1587, MIE with it 2198, now 2055; MIE / Fisk 2334, now 2318.
+// on average there, then 1587, MIE with it 2198, then 2055 (1599 and 2128 with what
+// score_pairs does for their precision); MIE / Fisk 2334, now 2306, MLE / Fisk 2190.
 // Measured and not kept: the next columns' loads from tensor memory issued before the
 // arithmetic on the present ones (24 more registers: MIE / Fisk 1 % faster, MLE / Fisk 1 %
 // and MIE / Gaussian 5 % slower), 8 or 12 compute warps with more registers (101 and 91

@@ -85,8 +85,8 @@ struct DevState {
     unsigned char* sc_pix;    // tensor-core operand of the current frame's valid pixels, compacted in pixel order:
                               // [ceil(N / 128)] tiles of 24 KB (score_ops.cuh)
     float4* sc_cst;           // [N] their Fisk constants {beta, beta log2(fx^2 / alpha), fx^2 mu / beta, W}, under the
-                              // Gaussian model {fx^2 / alpha, -x_mu / alpha, 0, W}
-    float* sc_xmu;            // [N] their x_mu / fx^2 (Fisk)
+                              // Gaussian model {fx^2 / alpha, -x_mu / alpha, U0, W}
+    float* sc_xmu;            // [N] their x_mu / fx^2, under the Gaussian model V0
     unsigned char* sc_hyp;    // tensor-core operand of the hypotheses: [ceil(S / 128)] groups of 40 KB
     int* sc_wild;             // [1] nonzero if a pixel or hypothesis of the frame is beyond kScWild
     int* pix_block_count;     // [ceil(N / kPixThreads)] valid pixels per block, then the blocks' record offsets
