@@ -131,6 +131,9 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
     }
 }
 
+// The two residual models apart: with the choice at run time the kernel needs 62 registers
+// instead of 40, and the P3P beside it starts later (50 to 65 us a frame at 640 x 480).
+template <bool kGauss>
 __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevState s, int t)
 {
     __shared__ DF C[12], T0[12];
@@ -188,18 +191,17 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevStat
         const Slice3 fs[3] = {slice3(xn), slice3(yn), slice3(iz)};
         pixel_block_s(fs, slice3(df_mul(az0, up)), o);
         // under the Gaussian model the scoring adds the references itself, up to what FP32 leaves of them
-        const bool gauss = p.residual == VOLDOR_RESIDUAL_GAUSSIAN;
         const Slice3 fu4[4] = {slice3(df_mul(X, xn)), slice3(df_mul(X, yn)), slice3(df_mul(X, iz)), slice3(X)};
-        pixel_block_x(fu4, gauss ? slice3(U0.lo, 0.f) : slice3(df_mul(U0, up)), fs, o + 32);
+        pixel_block_x(fu4, kGauss ? slice3(U0.lo, 0.f) : slice3(df_mul(U0, up)), fs, o + 32);
         const Slice3 fv4[4] = {slice3(df_mul(Y, xn)), slice3(df_mul(Y, yn)), slice3(df_mul(Y, iz)), slice3(Y)};
-        pixel_block_x(fv4, gauss ? slice3(V0.lo, 0.f) : slice3(df_mul(V0, up)), fs, o + 64);
+        pixel_block_x(fv4, kGauss ? slice3(V0.lo, 0.f) : slice3(df_mul(V0, up)), fs, o + 64);
         const int i = base + rank;
         unsigned char* d = s.sc_pix + (size_t)(i / kScTilePix) * kScTileBytes + ((i % kScTilePix) / 8) * 128 + (i % 8) * 16;
 #pragma unroll
         for (int q = 0; q < kScPixCols / 8; ++q)
             *reinterpret_cast<uint4*>(d + q * (kScTilePix * 16)) = *reinterpret_cast<const uint4*>(o + 8 * q);
         float4 cst;
-        if (gauss) {
+        if (kGauss) {
             const GaussConst gc = gauss_const(p, n);
             cst = make_float4(fx2 * gc.inv_alpha, -gc.x_mu * gc.inv_alpha, U0.hi, 0.f);
             s.sc_xmu[i] = V0.hi;
@@ -223,7 +225,8 @@ void launch_prep_count(const DevParams& p, const DevState& s, int t, cudaStream_
 void launch_prep_write(const DevParams& p, const DevState& s, int t, cudaStream_t st)
 {
     const int nb = (p.N + kPixThreads - 1) / kPixThreads;
-    k_prep_write<<<nb, kPixThreads, 0, st>>>(p, s, t);
+    if (p.residual == VOLDOR_RESIDUAL_GAUSSIAN) k_prep_write<true><<<nb, kPixThreads, 0, st>>>(p, s, t);
+    else k_prep_write<false><<<nb, kPixThreads, 0, st>>>(p, s, t);
 }
 
 void launch_pose_prep(const DevParams& p, const DevState& s, int t, cudaStream_t st)
