@@ -383,39 +383,41 @@ __global__ void k_mie_runs(DevParams p, DevState s)
 constexpr int kResolveWarps = 16, kResolveThreads = 32 * kResolveWarps;
 constexpr int kMaxChain = kMaxImageSide;
 
-// Positions of a chain a warp tests at a time with G lanes to a position, a frame each
+// A warp tests 32 >> lg positions of a chain at a time, 2^lg lanes to a position, a frame each
 // (two from T = 9 on); the frames' terms are independent, only their sum is in order.
-__device__ __forceinline__ int test_lanes(const DevParams& p) { return p.T > 4 ? 8 : (p.T > 2 ? 4 : p.T); }
+__device__ __forceinline__ int test_lanes_log2(const DevParams& p) { return p.T > 4 ? 3 : (p.T > 2 ? 2 : p.T - 1); }
 
-// The lanes of a warp at which v is lost, tested at positions pos, pos + 1, ... of chain c.
-__device__ unsigned mie_test(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, int G, float v)
+// The first of the positions pos, pos + 1, ... of chain c at which the warp finds v lost, or
+// pos + (32 >> lg) if it survives them all. Positions past the chain's end are lost.
+__device__ int mie_test(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, int lg, float v)
 {
-    const int lane = threadIdx.x & 31, sub = lane % G, first = lane - sub, q = pos + lane / G;
+    const int lane = threadIdx.x & 31, mask = (1 << lg) - 1, sub = lane & mask, first = lane - sub, q = pos + (lane >> lg);
     int x, y;
     chain_xy(p, dir, c, min(q, len - 1), x, y);
     const int j = y * p.W + x;
     float term[2] = {0.f, 0.f};
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const int t = u * G + sub + 1;
+        const int t = (u << lg) + sub + 1;
         if (t <= p.T) term[u] = __fmul_rn(s.qs[(size_t)(t - 1) * p.N + j], depth_ell_fast(p, f.v[t - 1], s.flows, t, x, y, v));
     }
     float acc = 0.f;
-    for (int t = 0; t < p.T; ++t) acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, t < G ? term[0] : term[1], first + t % G));
-    return __ballot_sync(0xffffffffu, q >= len || !survives(s, j, nan_to_ninf(acc)));
+    for (int t = 0; t < p.T; ++t) acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, t <= mask ? term[0] : term[1], first + (t & mask)));
+    const unsigned lost = __ballot_sync(0xffffffffu, q >= len || !survives(s, j, nan_to_ninf(acc)));
+    return pos + (lost ? (__ffs(lost) - 1) >> lg : 32 >> lg);
 }
 
 // End of the run of v, which survived up to position `pos` of chain c, by one warp; -q if
 // it is alive at a position q >= limit, not tested yet.
-__device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, int limit, float v)
+__device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF& f, int dir, int c, int len, int pos, int limit, int lg,
+                           float v)
 {
-    const int G = test_lanes(p);
-    do {
-        const unsigned lost = mie_test(p, s, f, dir, c, len, pos, G, v);
-        if (lost) return min(pos + (__ffs(lost) - 1) / G, len);
-        pos += 32 / G;
-    } while (pos < limit);
-    return pos < len ? -pos : len;
+    for (;;) {
+        const int end = pos + (32 >> lg);
+        pos = mie_test(p, s, f, dir, c, len, pos, lg, v);
+        if (pos < end) return min(pos, len);
+        if (pos >= limit) return pos < len ? -pos : len;
+    }
 }
 
 // Resolution of one chain per block. The walk r -> end of r's run depends on nothing
@@ -431,14 +433,16 @@ __device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF&
 // never come by it, and where it does (or meets a run of its own that outlives kAlone
 // positions) the whole block tests the next positions at once. Followed to their ends by
 // the parts' warps, runs of hundreds of positions, as over a plane whose depth was poor
-// and whose flows are quiet, made the sweep 955 us at 1242 x 375, T = 8; now 464, with
-// every test by the block (before there were parts) 545. Scenes of short runs lose 1 to 3 %.
-// Tried: all warps walking (421 there, but 3 to 8 % on short runs), long runs a lane per
-// position instead of a frame per lane (no change), two more blocks per SM (40 registers,
-// spills).
+// and whose flows are quiet, made a sweep 958 us at 1242 x 375, T = 8; now 396, with
+// every test by the block (before there were parts) 545. With short runs 250 us along
+// rows and 291 along columns (266 and 388). The lanes' shares are shifts and masks: with
+// divisions by the lanes per position a sweep took 9 % longer. Tried: all warps walking
+// (3 % longer on short runs), long runs a lane per position instead of a frame per lane
+// (no change), two blocks per SM instead of three (56 registers instead of 40 and a few
+// spills: 2 % longer at this size, 4 % shorter at 320 x 240).
 constexpr int kOver = 32, kAlone = 16;
 
-__global__ void __launch_bounds__(kResolveThreads, 2) k_mie_resolve(DevParams p, DevState s)
+__global__ void __launch_bounds__(kResolveThreads, 3) k_mie_resolve(DevParams p, DevState s)
 {
     __shared__ FramesF f;
     __shared__ short origin[kMaxChain];
@@ -462,7 +466,7 @@ __global__ void __launch_bounds__(kResolveThreads, 2) k_mie_resolve(DevParams p,
         reset[q] = 0;
     }
     __syncthreads();
-    const int part = (len + kResolveWarps - 1) / kResolveWarps;
+    const int part = (len + kResolveWarps - 1) / kResolveWarps, lg = test_lanes_log2(p);
     {
         const int stop = min((warp + 1) * part, len);
         int r = min(warp * part, len), last = 0;
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(kResolveThreads, 2) k_mie_resolve(DevParams p,
             last = r;
             int e = next_s[r];
             if (e < 0) {
-                e = mie_run_end(p, s, f, dir, c, len, -e, stop + kOver, own_s[r]);
+                e = mie_run_end(p, s, f, dir, c, len, -e, stop + kOver, lg, own_s[r]);
                 __syncwarp();
                 if (lane == 0) next_s[r] = e;
             }
@@ -484,58 +488,59 @@ __global__ void __launch_bounds__(kResolveThreads, 2) k_mie_resolve(DevParams p,
     }
     if (threadIdx.x == 0) first_lost[0] = kMaxChain;
     __syncthreads();
-    // the end of an open run of v, alive at `pos`, by the whole block
-    int step = 0;
-    auto follow = [&](int pos, float v) {
-        const int G = test_lanes(p), wide = 32 / G;
+    // warp 0 walks until it meets an open run that it leaves to the block, or the chain's end
+    __shared__ int open_pos;
+    __shared__ float open_v;
+    const int wide = 32 >> lg;
+    int r = 0, k = 0, step = 0;
+    for (;;) {
+        if (warp == 0) {
+            int pos = 0;
+            float v = 0.f;
+            while (k < kResolveWarps) {
+                if (r >= min((k + 1) * part, len)) {         // the walk passes the part by
+                    if (lane == 0) part_from[k] = len;
+                    ++k;
+                    continue;
+                }
+                int e;
+                if (reset[r] == 1) {                          // it goes on as the part's own
+                    if (lane == 0) part_from[k] = r;
+                    e = part_end[k];
+                    v = own_s[part_last[k]];
+                    ++k;
+                } else {
+                    if (lane == 0) reset[r] = 2;
+                    e = next_s[r];
+                    v = own_s[r];
+                }
+                if (e < 0) e = mie_run_end(p, s, f, dir, c, len, -e, kAlone - e, lg, v);
+                if (e < 0) {
+                    pos = -e;
+                    break;
+                }
+                r = e;
+            }
+            if (lane == 0) {
+                open_pos = pos;
+                open_v = v;
+            }
+        }
+        __syncthreads();
+        int pos = open_pos;
+        if (pos == 0) break;
+        const float v = open_v;
+        // the run's end, tested by the whole block
         for (;; pos += wide * kResolveWarps) {
-            const unsigned lost = mie_test(p, s, f, dir, c, len, pos + warp * wide, G, v);
-            const int slot = step % 3;
+            const int mine = pos + warp * wide, slot = step % 3;
+            const int end = mie_test(p, s, f, dir, c, len, mine, lg, v);
             step += 1;
-            if (lane == 0 && lost) atomicMin(&first_lost[slot], pos + warp * wide + (__ffs(lost) - 1) / G);
+            if (lane == 0 && end < mine + wide) atomicMin(&first_lost[slot], end);
             if (threadIdx.x == 0) first_lost[step % 3] = kMaxChain;     // read for the last time two steps ago
             __syncthreads();
             const int at = first_lost[slot];
-            if (at < kMaxChain) return min(at, len);
-            if (pos + wide * kResolveWarps >= len) return len;
-        }
-    };
-    // warp 0 walks; the others wait for the open runs it meets
-    __shared__ int open_pos[2];
-    __shared__ float open_v[2];
-    int call = 0;
-    if (warp == 0) {
-        auto ask = [&](int pos, float v) {
-            pos = mie_run_end(p, s, f, dir, c, len, pos, pos + kAlone, v);
-            if (pos >= 0) return pos;
-            pos = -pos;
-            if (lane == 0) { open_pos[call & 1] = pos; open_v[call & 1] = v; }
-            call += 1;
-            __syncthreads();
-            return follow(pos, v);
-        };
-        int r = 0;
-        for (int k = 0; k < kResolveWarps; ++k) {
-            const int stop = min((k + 1) * part, len);
-            while (r < stop && reset[r] != 1) {
-                if (lane == 0) reset[r] = 2;
-                const int e = next_s[r];
-                r = e < 0 ? ask(-e, own_s[r]) : e;
-            }
-            if (lane == 0) part_from[k] = r < stop ? r : len;
-            if (r < stop) {
-                r = part_end[k];
-                if (r < 0) r = ask(-r, own_s[part_last[k]]);
-            }
-        }
-        if (lane == 0) open_pos[call & 1] = -1;
-        __syncthreads();
-    } else {
-        for (;; ++call) {
-            __syncthreads();
-            const int pos = open_pos[call & 1];
-            if (pos < 0) break;
-            follow(pos, open_v[call & 1]);
+            r = min(at, len);
+            if (at < kMaxChain || pos + wide * kResolveWarps >= len) break;
         }
     }
     __syncthreads();

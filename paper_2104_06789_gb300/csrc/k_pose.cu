@@ -673,11 +673,10 @@ __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState
         }
     }
     __syncthreads();
-    if (n_s >= 0) finish_hypotheses(p, s, n_s, tid);
     const int item = tid >> 2, r = min(tid & 3, 2), g = g0 + item / kMaxSols, i = item % kMaxSols;
-    if (g >= G || i >= s.grp_count[g]) return;            // whole quads leave together
     const int h = off_s[item / kMaxSols] + i;
-    if (h >= p.S) return;
+    if (n_s >= 0) finish_hypotheses(p, s, n_s, kHypThreads - 1 - tid);    // the last warp, whose slots are seldom all filled
+    if (g >= G || i >= s.grp_count[g] || h >= p.S) return;                // whole quads leave together
     const double* Rt = s.grp_sols + ((size_t)g * kMaxSols + i) * 12 + r * 4;
     double v[4], e[4];
 #pragma unroll
