@@ -701,10 +701,10 @@ static void launch_score_as(const DevParams& p, const DevState& s, int li, cudaS
             raised[dev] = cudaFuncSetAttribute(k_score<kL, kMLE, kGauss>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                kScSmemBytes) == cudaSuccess;
     }
-    // a frame with fewer groups may have more items than a full one's
-    const int groups = (p.S + kScGroupHyps - 1) / kScGroupHyps;
-    const long long items = (long long)groups * s.n_chunks, most = groups > 1 ? num_sms() : items;
-    k_score<kL, kMLE, kGauss><<<(unsigned)std::min<long long>(most, num_sms()), kScThreads, kScSmemBytes, st>>>(p, s, li);
+    // a frame with fewer groups may have more items than a full one
+    const int groups = (p.S + kScGroupHyps - 1) / kScGroupHyps, tiles = (p.N + kScTilePix - 1) / kScTilePix;
+    const long long items = std::max((long long)groups * s.n_chunks, (long long)(groups - 1) * std::min(s.chunks_max, tiles));
+    k_score<kL, kMLE, kGauss><<<(unsigned)std::min<long long>(items, num_sms()), kScThreads, kScSmemBytes, st>>>(p, s, li);
 }
 
 template <int kL>
