@@ -342,18 +342,27 @@ void launch_emissions(const DevParams& p, const DevState& s, float* out, cudaStr
 // now: the latency of a step (up to two divisions) times four passes over a segment,
 // with the chains an SM has room for.
 // ---------------------------------------------------------------------------
-constexpr int kFbChains = 4, kFbWarps = 8;
+constexpr int kFbChains = 4, kFbMaxWarps = 32;
 
 // Floats of a chain's row in shared memory: 32 segments, padded to an odd length so
 // that the lanes' steps fall into different banks.
 __host__ __device__ constexpr int fb_segment(int len) { return (len + 31) / 32; }
 __host__ __device__ constexpr int fb_row(int len) { return 32 * (fb_segment(len) | 1); }
 
-// Chains of length len to a block whose room is kFbChains chains of length most.
-__host__ __device__ inline int fb_chains(int len, int most)
+// Warps of a block: 8, but of a strip whose longer chains leave an SM room for two blocks or
+// one, as many as the shorter chains fill (4096 x 16, T = 8, columns: 77 us, 136 with 8).
+__host__ inline int fb_warps(int most, int least)
+{
+    const int room = 227 * 1024 / (kFbChains * 3 * fb_row(most) * (int)sizeof(float));
+    const int fit = kFbChains * fb_row(most) / fb_row(least);
+    return room > 2 ? 8 : std::max(8, std::min(fit, kFbMaxWarps / room));
+}
+
+// Chains of length len to a block of `warps` whose room is kFbChains chains of length most.
+__host__ __device__ inline int fb_chains(int len, int most, int warps)
 {
     const int fit = kFbChains * fb_row(most) / fb_row(len);
-    return fit < kFbWarps ? fit : kFbWarps;
+    return fit < warps ? fit : warps;
 }
 
 struct M22 {
@@ -484,7 +493,7 @@ __device__ __forceinline__ void fb_chain(const DevParams& p, int len, float* e, 
 }
 
 // grid (groups of chains, frame)
-__global__ void __launch_bounds__(32 * kFbWarps) k_forward_backward(DevParams p, DevState s)
+__global__ void __launch_bounds__(32 * kFbMaxWarps) k_forward_backward(DevParams p, DevState s)
 {
     extern __shared__ float fb_smem[];
     const int dir = (*s.iter) & 3;
@@ -492,7 +501,7 @@ __global__ void __launch_bounds__(32 * kFbWarps) k_forward_backward(DevParams p,
     const int n_chains = rows ? p.H : p.W;
     const int len = rows ? p.W : p.H;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per = fb_chains(len, max(p.W, p.H)), c0 = blockIdx.x * per, here = min(per, n_chains - c0);
+    const int per = fb_chains(len, max(p.W, p.H), blockDim.x >> 5), c0 = blockIdx.x * per, here = min(per, n_chains - c0);
     if (here <= 0) return;
     const int L = fb_segment(len), LP = L | 1, row = fb_row(len);
     float* q = s.qs + (size_t)blockIdx.y * p.N + (rows ? (size_t)c0 * p.W : (size_t)c0);
@@ -502,7 +511,7 @@ __global__ void __launch_bounds__(32 * kFbWarps) k_forward_backward(DevParams p,
             if (warp < here)
                 for (int i = lane; i < len; i += 32) f(q + (size_t)warp * p.W + i, fb_smem + 3 * row * warp + i + i / L * (LP - L));
         } else {
-            for (int n = threadIdx.x; n < len * per; n += 32 * kFbWarps) {
+            for (int n = threadIdx.x; n < len * per; n += blockDim.x) {
                 const int i = n / per, k = n % per;
                 if (k < here) f(q + (size_t)i * p.W + k, fb_smem + 3 * row * k + i + i / L * (LP - L));
             }
@@ -525,9 +534,10 @@ void launch_forward_backward(const DevParams& p, const DevState& s, cudaStream_t
     // the longest chain's, whatever this window's: the attribute belongs to all windows and threads
     constexpr int kSmemMax = kFbChains * 3 * fb_row(kMaxImageSide) * (int)sizeof(float);
     cudaFuncSetAttribute(k_forward_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    const int rows = fb_chains(p.W, most), cols = fb_chains(p.H, most);   // chains to a block, along rows and columns
+    const int warps = fb_warps(most, std::min(p.W, p.H));
+    const int rows = fb_chains(p.W, most, warps), cols = fb_chains(p.H, most, warps);   // chains to a block, along rows and columns
     const int blocks = std::max((p.H + rows - 1) / rows, (p.W + cols - 1) / cols);
-    k_forward_backward<<<dim3(blocks, p.T), 32 * kFbWarps, smem, st>>>(p, s);
+    k_forward_backward<<<dim3(blocks, p.T), 32 * warps, smem, st>>>(p, s);
 }
 
 }  // namespace vd
