@@ -140,8 +140,10 @@ voldor_status voldor_bootstrap(voldor_ctx* ctx, int mode, const double* T1_rowma
  * both cameras, and |t| = baseline (a monocular window's scale is free).
  * T1_out (host, 16 doubles, may be NULL) receives T_1. Synchronises the
  * context's stream. VOLDOR_ERR_DEGENERATE if no sample is valid (the state is
- * then unchanged). n_samples in [1, VOLDOR_EPI_MAX_SAMPLES]; scratch of about
- * 25 KB per sample is allocated on first use and kept by the context. */
+ * then unchanged). n_samples in [1, VOLDOR_EPI_MAX_SAMPLES]. The first use allocates
+ * scratch, kept by the context: per sample 4 bytes for each sixteenth pixel, but
+ * for no fewer than 4096 and no more than 65536 of them, and about 300 bytes (at
+ * 1242 x 375 0.12 MB a sample, 60 MB for 512; at most 0.27 MB a sample). */
 #define VOLDOR_EPI_MAX_SAMPLES 4096
 voldor_status voldor_bootstrap_epipolar(voldor_ctx* ctx, int n_samples, double baseline, double* T1_out);
 
@@ -261,7 +263,8 @@ const char* voldor_last_error_string(const voldor_ctx* ctx);
  *
  * It computes, on the device and asynchronously on `cuda_stream`,
  *   L[h] = - sum_j records[j].wq * log(1 + mu_j / rho_j(h))
- * for h < n_hyps: the dense score voldor_score_hypotheses returns, but for
+ * for h < n_hyps: the dense score of voldor_score_hypotheses (to within the bound
+ * on dense scores, 1e-5 relative; the projection is plain FP32 here), but for
  * pixel records and hypotheses the caller supplies.
  *  records: device, n_pix records of 12 floats (48 bytes, 16-byte aligned):
  *           {xb, yb2, w, ut, vt, beta, beta_k, Cp, wq, 0, 0, 0} with, for the
@@ -318,7 +321,10 @@ voldor_status voldor_probe_bounded_wait(long long polls, long long* cycles);
  * Synchronises. Outputs may be NULL. */
 voldor_status voldor_autotune(voldor_ctx* ctx, int* hyps_per_thread, int* chunks, float* best_ms);
 
-/* Sets the dense-scoring tile shape directly (hyps_per_thread 2, 4 or 8). */
+/* Sets the dense-scoring shape directly: the hypotheses a thread takes from tensor
+ * memory at a time (2, 4 or 8) and the pixel chunks of a frame. A frame (or a call of
+ * voldor_score_hypotheses) with fewer groups of 128 hypotheses than
+ * hyps_per_frame makes chooses its own chunks. */
 voldor_status voldor_set_score_shape(voldor_ctx* ctx, int hyps_per_thread, int chunks);
 
 /* A batch of windows run as one CUDA graph: every window's n_iters

@@ -523,7 +523,7 @@ struct WgradArgs {
 // sign of a gradient that is zero up to rounding into a whole step).
 //
 // The kernel before transposed the tiles through ldmatrix / stmatrix into K-major
-// operands: 177 us for 32 x 32 channels on two 1242 x 375 images; this one about 55 us.
+// operands: 177 us for 32 x 32 channels on two 1242 x 375 images; this one 59 us (cold).
 // HBM needs 18, the MMAs 32 (52 cycles each, the reads of their 4 KB A tiles).
 // ---------------------------------------------------------------------------
 constexpr int kWgKP = 64;                                 // pixels per work item (K)

@@ -271,9 +271,9 @@ __device__ __forceinline__ float depth_ell_fast(const DevParams& p, const float*
 //            that reached the cap is continued there.
 // ---------------------------------------------------------------------------
 // Speculation pays where neighbouring pixels' tests share a warp's time, and costs where
-// one lane of it goes on alone: runs + resolve take 43 + 137 us with a cap of 1, 71 + 108
-// with 2, 97 + 95 with 3, 120 + 88 with 4 and 140 + 57 with 8 (1242 x 375, T = 8), and
-// 31, 29, 29, 31 and 39 us together on 160 x 120.
+// one lane of it goes on alone: runs + resolve take 43 + 110 us with a cap of 1, 71 + 89
+// with 2, 98 + 79 with 3, 118 + 74 with 4 and 178 + 65 with 8 (the first four sweeps over a
+// driving window of 1242 x 375, T = 8), and 30, 30, 29, 32 and 39 us together on 160 x 120.
 constexpr int kRunCap = 2;
 
 __device__ __forceinline__ float nan_to_ninf(float v) { return isnan(v) ? -INFINITY : v; }
@@ -426,8 +426,9 @@ __device__ int mie_run_end(const DevParams& p, const DevState& s, const FramesF&
 // whatever a run that reached the cap costs is paid by the warps side by side; then
 // warp 0 follows the true walk from one part to the next, step by step until it meets
 // the part's own walk, from there on by its result. A chain's runs one after another,
-// tested by the whole block, took 212 us at 1242 x 375, T = 8; with the parts 57, and
-// 108 with a cap of 2 instead of 8 (see kRunCap). 8 parts: 101, 32: 146.
+// tested by the whole block, took 212 us at 1242 x 375, T = 8 with a cap of 8; the parts
+// take 65 with that cap and 89 with 2 (see kRunCap). With 8 or 32 parts instead of 16 a
+// first version took 101 and 146 us where it took 108.
 //
 // A run that goes on kOver positions past its warp's part is left open: the true walk may
 // never come by it, and where it does (or meets a run of its own that outlives kAlone

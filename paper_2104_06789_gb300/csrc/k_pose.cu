@@ -519,13 +519,12 @@ __device__ __forceinline__ int groups_solved(const DevParams& p, const DevState&
 // One warp per block spreads the FP64 solves over the SMs. The first wave takes S
 // groups (more than one solution each as a rule), so that no warp runs a second chunk
 // after its first, a whole chain later: with 3/4 S groups, enough only above 1.33
-// solutions a group, frames of handheld windows took 78 us on average (54 or 97) at
-// S = 4096 on 640 x 480 where S groups took 58, and 79 against 54 at S = 2048 on
+// solutions a group, frames of handheld windows take 64 us on average (46 or 81) at
+// S = 4096 on 640 x 480 where S groups take 48, and 68 against 45 at S = 2048 on
 // 320 x 240. An SM solves three and a half chunks in the time of one and no more (5/4 S
-// groups at S = 4096: 68 us, 7/4 S: 77), so beyond kP3PFreeChunks chunks in all it is
-// 3/4 S, as the yield of driving windows (1.4-1.5) allows (S = 8192: 77 us; with 15/16 S
-// 86); further chunks are claimed as needed. (All before the solver's FP64 work was
-// cut by a sixth.)
+// groups at S = 4096: 57 us), so beyond kP3PFreeChunks chunks in all it is 3/4 S, as the
+// yield of driving windows (1.4-1.5) allows (S = 8192: 64 us; with S groups 73, with 5/4 S
+// 93); further chunks are claimed as needed.
 constexpr int kP3PFreeChunks = 512;
 
 void launch_p3p_groups(const DevParams& p, const DevState& s, int t, cudaStream_t st)
@@ -630,7 +629,7 @@ __device__ __forceinline__ void finish_hypotheses(const DevParams& p, const DevS
 // before this one took 4 us and a launch per frame, and the sum of all earlier groups'
 // counts, G^2 / 16 of them in all, 0.4 of 2.0 ms of a frame with 262144 groups solved.
 // A lane per solution, with all of its FP64 work, took 10.7 us at S = 256 (14.6 at
-// 8192), four lanes with 32 groups to a block, all on one SM, 12.2 (19.1); now 7.5 (14.5).
+// 8192), four lanes with 32 groups to a block, all on one SM, 12.2 (19.1); now 7.7 (14.7).
 constexpr int kHypGroups = kP3PChunk;      // groups per block
 constexpr int kHypThreads = kHypGroups * kMaxSols * 4;
 

@@ -334,7 +334,7 @@ __device__ __forceinline__ bool score_wait_warp(uint32_t bar, uint32_t parity, v
 // lg2, two ex2 per pair, one lg2 where r >= 1/8; rcp and lg2 take 8 cycles per
 // warp, ex2 4) and 49 issue slots, of which the 17 packed instructions hold the
 // dispatch port two cycles each; it runs in 73 cycles, the SFU 77 % busy, the
-// tensor pipe 10 %. With the contractions in FP32 on the CUDA cores the term
+// tensor pipe 31 %. With the contractions in FP32 on the CUDA cores the term
 // needed 28 packed instructions and five shared-memory loads per pixel and was
 // bound by dispatch: 88 cycles. 8192 hypotheses x 465,750 pixels: 4.38 -> 3.64 ms.
 // The two issuing warps run converged: with their loops inside an `if (lane == 0)` a
@@ -734,8 +734,9 @@ void launch_score(const DevParams& p, const DevState& s, int log_idx, cudaStream
 // nodes, a host that hands the GPU to this library under a fixed memory
 // budget, or a caller whose own allocator owns all device memory. For them,
 // voldor_score_records_noalloc scores caller-given pixel records against
-// caller-given hypotheses with the same per-pair arithmetic as k_score and
-// takes its only scratch (the per-chunk partial sums) from the file-scope
+// caller-given hypotheses by the same formula, in plain FP32 (no tensor cores, a
+// reciprocal to each pair): its scores and k_score's agree within the bound on dense
+// scores, not bit for bit. It takes its only scratch (the per-chunk partial sums) from the file-scope
 // array below, which every GPU that loads this library holds until the
 // process exits.
 // ---------------------------------------------------------------------------
