@@ -159,8 +159,9 @@ __device__ __forceinline__ void hyp_block_x(const Slice3* z, const Slice3* a, co
 // leaves the scores without the bias: measured against 64 bits, the mean relative error
 // of the scores was 4e-8 to 9e-8 larger without it. Over 60 sets of hypotheses within
 // 0.005 rad and 5 cm of the current pose the rms error of the scores is 0.93 to 1.00
-// of what it was with the projection in FP32 (Fisk), between 0.86 and 1.10 of it in a single
-// scene's sets; far from it single pixels beside the camera plane decide, either way.
+// of what it was with the projection in FP32 (Fisk): 1.01 to 1.09 on the driving scenes,
+// 0.89 to 1.04 on the others; farther away single pixels beside the camera plane decide,
+// either way.
 constexpr double kScUntruncate = 1.0 + 4.3e-8;
 
 // Sixteen bytes i < kScHypChunks of hypothesis h's operand row set to zero: a_z = U = V = 0 for
