@@ -74,24 +74,57 @@ __device__ __forceinline__ PrepGeo prep_geometry(const DevParams& p, const DF* C
     return g;
 }
 
+// True if the pose M (hi parts of T_t) leaves a smaller residual at a valid pixel than no
+// motion at all, with the pixel's own flow f instead of the one at its projection (FP32).
+// The scoring's operands are formed around a reference pose that every hypothesis is the
+// difference from; around one far from the hypotheses the differences cancel against it
+// and the scores lose their digits (a translation of 70 in a scene 2 to 20 deep cost
+// 1.2e-5 of them, one of 2e5 cost 7 %). So the current pose is the reference only where
+// it explains more of the pixels than the identity does, whose part of a residual is the
+// flow itself.
+__device__ __forceinline__ bool pose_explains(const DevParams& p, const float* M, const PrepGeo& g, float2 f)
+{
+    const float iz = 1.f / g.Pz.hi, x = g.Px.hi * iz, y = g.Py.hi * iz;
+    const float fu = f.x * p.inv_fx, fv = f.y * p.inv_fy;
+    const float ax = fmaf(M[0] - 1.f, x, fmaf(M[1], y, fmaf(M[3], iz, M[2])));
+    const float ay = fmaf(M[4], x, fmaf(M[5] - 1.f, y, fmaf(M[7], iz, M[6])));
+    const float az = fmaf(M[8], x, fmaf(M[9], y, fmaf(M[11], iz, M[10] - 1.f))), den = 1.f + az;
+    const float U = fmaf(x + fu, az, fu - ax), V = fmaf(y + fv, az, fv - ay);
+    return den > 0.f && fabsf(U) + fabsf(V) <= (fabsf(fu) + fabsf(fv)) * den;
+}
+
 __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevState s, int t)
 {
     __shared__ DF C[12];
+    __shared__ float M[12];
+    __shared__ int votes_s, votes_all;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // one warp of a block votes on the reference pose, another one in each block
+    const bool voter = warp == (blockIdx.x & (kPixThreads / 32 - 1));
+    float2 f = make_float2(0.f, 0.f);
+    if (voter && j < p.N) f = load_flow(s.flows, p.flow_f16, (size_t)(t - 1) * p.N + j);
+    if (threadIdx.x >= 32 && threadIdx.x < 44) M[threadIdx.x - 32] = s.poses_df[24 * (t - 1) + 2 * (threadIdx.x - 32)];
     load_cum_df(s, t, C);
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    bool valid = false;
-    if (j < p.N) valid = prep_geometry(p, C, t, j, s.theta[j]).valid;
+    PrepGeo g;
+    g.valid = false;
+    if (j < p.N) g = prep_geometry(p, C, t, j, s.theta[j]);
+    const bool valid = g.valid;
     // per-warp ballots of the valid pixels: with the block offsets they map
     // the i-th valid pixel (pixel order) to its index for the minimal groups
     const unsigned bal = __ballot_sync(0xffffffffu, valid);
-    if ((threadIdx.x & 31) == 0) s.pix_vmask[j >> 5] = bal;
+    if (lane == 0) s.pix_vmask[j >> 5] = bal;
+    if (voter) {
+        const int votes = __popc(__ballot_sync(0xffffffffu, valid && pose_explains(p, M, g, f)));
+        if (lane == 0) votes_s = (2 * votes - __popc(bal)) * 65536;
+    }
+    if (threadIdx.x == 0) votes_all = 0;
     const int cnt = __syncthreads_count(valid);
     // the last block to finish turns the block counts into block offsets
     // (exclusive scan, in place), sets the record count and clears the P3P
     // claim counters and coarse counts of the frame; no block waits
     __shared__ bool last;
     if (threadIdx.x == 0) {
-        s.pix_block_count[blockIdx.x] = cnt;
+        s.pix_block_count[blockIdx.x] = cnt + votes_s;       // above the count: the votes for less those against
         __threadfence();
         last = atomicAdd(s.prep_done, 1u) == gridDim.x - 1;
     }
@@ -101,10 +134,15 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
     const int nb = gridDim.x, per = (nb + blockDim.x - 1) / blockDim.x;
     const int b0 = min((int)threadIdx.x * per, nb), b1 = min(b0 + per, nb);
     volatile int* counts = s.pix_block_count;
-    int local = 0;
-    for (int b = b0; b < b1; ++b) local += counts[b];
+    int local = 0, votes = 0;
+    for (int b = b0; b < b1; ++b) {
+        const int c = counts[b];
+        local += c & 0xffff;
+        votes += c >> 16;
+    }
+    votes = __reduce_add_sync(0xffffffffu, votes);
+    if (lane == 0) atomicAdd(&votes_all, votes);
     __shared__ int wsum[kPixThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = local;
     for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, incl, o);
@@ -116,7 +154,7 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
     for (int w = 0; w < warp; ++w) before += wsum[w];
     int off = before + incl - local;
     for (int b = b0; b < b1; ++b) {
-        const int c = counts[b];
+        const int c = counts[b] & 0xffff;
         counts[b] = off;
         off += c;
     }
@@ -128,20 +166,24 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_count(DevParams p, DevStat
         *s.p3p_claims = 0;
         *s.p3p_done = 0ull;
         *s.sc_wild = 0;
+        *s.sc_ref = votes_all >= 0;
     }
 }
 
 // What bounds the write: float-float arithmetic at three quarters of the issue slots; it
-// leaves 212 bytes a pixel for the scoring (21 us at 640 x 480). The two residual models apart: with the choice at run time the kernel needs 62 registers
-// instead of 40, and the P3P beside it starts later (50 to 65 us a frame at 640 x 480).
+// leaves 212 bytes a pixel for the scoring (21 us at 640 x 480). The two residual models
+// apart: with the choice at run time the kernel needs 62 registers instead of 40, and
+// the P3P beside it starts later (50 to 65 us a frame at 640 x 480).
 template <bool kGauss>
 __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevState s, int t)
 {
     __shared__ DF C[12], T0[12];
     __shared__ int warp_sum[kPixThreads / 32];
-    if (threadIdx.x < 12) {
+    if (threadIdx.x < 12) {                               // the reference pose (pose_explains)
         const float* c = s.poses_df + 24 * (t - 1) + 2 * threadIdx.x;
-        T0[threadIdx.x] = DF{c[0], c[1]};
+        const float hi = c[0], lo = c[1];
+        const bool current = *s.sc_ref != 0;
+        T0[threadIdx.x] = DF{current ? hi : (threadIdx.x % 5 == 0 ? 1.f : 0.f), current ? lo : 0.f};
     }
     load_cum_df(s, t, C);
     const int base = s.pix_block_count[blockIdx.x];      // this block's offset (set by the count pass)
@@ -178,7 +220,7 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevStat
         // features of the projection (score_ops.cuh), in float-float
         const DF xn = df_mul(g.Px, iz), yu = df_mul(g.Py, iz), yn = df_mul(yu, p.fy_over_fx);
         const DF X = df_add(xn, ut), Y = df_add(yn, vt);
-        // a = (T_t - I) p at the current pose: a_z0, U0 = X a_z0 - a_x0 + ut, V0 alike
+        // a = (T - I) p at the reference pose T: a_z0, U0 = X a_z0 - a_x0 + ut, V0 alike
         auto row = [&](int r) {
             const DF e0 = r == 0 ? df_add(T0[0], -1.f) : T0[4 * r], e1 = r == 1 ? df_add(T0[5], -1.f) : T0[4 * r + 1];
             const DF e2 = r == 2 ? df_add(T0[10], -1.f) : T0[4 * r + 2];

@@ -638,16 +638,17 @@ __global__ void __launch_bounds__(kHypThreads) k_hyp_write(DevParams p, DevState
     __shared__ int wsum[kHypThreads / 32], off_s[kHypGroups], n_s;
     __shared__ double e0[12];
     const int tid = threadIdx.x, lane = tid & 31;
+    const bool current = *s.sc_ref != 0;
     const int G = groups_solved(p, s), g0 = blockIdx.x * kHypGroups;
     if (g0 >= G && blockIdx.x > 0) return;
     const double q = p.fyd / p.fxd;
     const double sc[3] = {1.0, q, 1.0};
-    if (tid < 12) {                                       // the frame's current pose in scaled form, {E, t}
+    if (tid < 12) {                                       // the frame's reference pose in scaled form, {E, t}
         const double* T0 = s.poses + 12 * (t - 1);
         const int r = tid < 9 ? tid / 3 : tid - 9, c = tid < 9 ? tid % 3 : 3;
         double v = T0[r * 4 + c] - (r == c ? 1.0 : 0.0);
         if (q != 1.0) v = c < 3 ? sc[r] * v / sc[c] : sc[r] * v;     // square pixels need no scaling
-        e0[r * 4 + c] = v;
+        e0[r * 4 + c] = current ? v : 0.0;
     }
     int before = 0;
     const int full = blockIdx.x / kP3PBlock;              // coarse counts before this block's groups
@@ -751,10 +752,10 @@ __global__ void k_hyp_from_rt(DevParams p, DevState s, int t, int n)
     double e[4], e0[4];
     for (int c = 0; c < 3; ++c) {
         e[c] = sc[r] * (R[r * 3 + c] - (r == c ? 1.0 : 0.0)) / sc[c];
-        e0[c] = sc[r] * (T0[c] - (r == c ? 1.0 : 0.0)) / sc[c];
+        e0[c] = *s.sc_ref ? sc[r] * (T0[c] - (r == c ? 1.0 : 0.0)) / sc[c] : 0.0;
     }
     e[3] = sc[r] * R[9 + r];
-    e0[3] = sc[r] * T0[3];
+    e0[3] = *s.sc_ref ? sc[r] * T0[3] : 0.0;
     if ((id & 3) < 3) {
         float* f = s.hyp_f32 + (size_t)h * 12;
         for (int c = 0; c < 4; ++c) f[c < 3 ? r * 3 + c : 9 + r] = (float)e[c];

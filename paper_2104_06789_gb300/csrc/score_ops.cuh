@@ -6,8 +6,8 @@
 //   a_z = E_z p + t_z w,   U = X a_z - a_x + ut,   V = Y a_z - a_y + vt
 // with X = x + ut, Y = y + vt: U / (1 + a_z) and V / (1 + a_z) are the residual
 // over fx. All three are linear in the hypothesis once the products X x, X y,
-// X w (and Y's) count as pixel features. Around the frame's current pose
-// (E0, t0), with d = (E, t) - (E0, t0):
+// X w (and Y's) count as pixel features. Around a reference pose (E0, t0), the frame's
+// current one or the identity, with d = (E, t) - (E0, t0):
 //   a_z = a_z0 + (d_z . (x, y, w, 1))
 //   U   = U0   + d_z . (X x, X y, X w, X) - d_x . (x, y, w, 1)
 // so the large terms that cancel in U are formed once per pixel in float-float
@@ -205,7 +205,7 @@ __device__ __forceinline__ int chunks_for_groups(int groups, int tiles, int most
 // the product of two (1 + a_z) stays under 2^124.
 constexpr float kScWild = 1073741824.f;                  // 2^30
 
-// Operand row of hypothesis h from its scaled form (E, t) and the frame's current
+// Operand row of hypothesis h from its scaled form (E, t) and the frame's reference
 // pose (E0, t0), both FP64, by a quad of lanes: lane r < 3 is given row r, {E_r0, E_r1,
 // E_r2, t_r}, and lane 3 row 2 again. Rows 0 and 1 make U's and V's coefficients, row 2
 // those of a_z, which U and V need too. A warp issues an FP64 instruction every ~54

@@ -153,6 +153,7 @@ size_t layout(voldor_ctx& c, char* base)
     s.sc_cst = (float4*)take(N * sizeof(float4));
     s.sc_xmu = (float*)take(N * sizeof(float));
     s.sc_hyp = (unsigned char*)take((S + kScGroupHyps - 1) / kScGroupHyps * kScGroupBytes);
+    s.sc_ref = (int*)take(4);
     s.sc_wild = (int*)take(4);
     s.pix_block_count = (int*)take(((N + kPixThreads - 1) / kPixThreads) * 4);
     s.prep_done = (unsigned*)take(4);

@@ -88,6 +88,7 @@ struct DevState {
                               // Gaussian model {fx^2 / alpha, -x_mu / alpha, U0, W}
     float* sc_xmu;            // [N] their x_mu / fx^2, under the Gaussian model V0
     unsigned char* sc_hyp;    // tensor-core operand of the hypotheses: [ceil(S / 128)] groups of 40 KB
+    int* sc_ref;              // [1] reference pose of the frame's operands: 1 its current pose, 0 the identity
     int* sc_wild;             // [1] nonzero if a pixel or hypothesis of the frame is beyond kScWild
     int* pix_block_count;     // [ceil(N / kPixThreads)] valid pixels per block, then the blocks' record offsets
     unsigned* prep_done;      // [1] blocks of the count pass finished (0 between launches)
