@@ -251,7 +251,14 @@ __global__ void __launch_bounds__(kPixThreads) k_prep_write(DevParams p, DevStat
         } else {
             const FiskConst fc = fisk_const(p, n);
             cst = make_float4(fc.beta, fc.beta * (p.log2_fx2 - fc.log2_alpha), fx2 * fc.mu_over_beta, 0.f);
-            s.sc_xmu[i] = fminf(fmaxf(p.lambda2 * n * n, p.x_min), p.x_max) / fx2;
+            // At x_mu, where a pixel behind the camera is taken, r = Cp xs (2^s + 2 + 2^-s) is 1; with
+            // |s| beyond 128 (flows of thousands of pixels with a shape that is not small) its
+            // factors overflow. Only one power of two counts there: s is moved to 80.
+            if (fabsf(fc.s_mu) > 100.f) {
+                cst.y = copysignf(80.f, fc.s_mu) - fc.beta * (log2f(fc.x_mu) - p.log2_fx2);
+                cst.z = fx2 * 0x1p-80f / fc.x_mu;
+            }
+            s.sc_xmu[i] = fc.x_mu / fx2;
         }
         cst.w = s.wmap[(size_t)(t - 1) * N + j];
         s.sc_cst[i] = cst;

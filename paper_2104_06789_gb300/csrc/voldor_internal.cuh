@@ -223,6 +223,7 @@ __device__ __forceinline__ void load_frames(const DevParams& p, const DevState& 
 // x_mu = lambda^2 n^2 and ys = 2^-|beta log2(x_mu / alpha)|.
 struct FiskConst {
     float beta, log2_alpha, mu_over_beta;
+    float x_mu, s_mu;                   // x_mu and beta log2(x_mu / alpha)
 };
 
 __device__ __forceinline__ FiskConst fisk_const(const DevParams& p, float n)
@@ -230,11 +231,11 @@ __device__ __forceinline__ FiskConst fisk_const(const DevParams& p, float n)
     FiskConst c;
     c.log2_alpha = fmaf(p.a2_log2e, n, p.log2_a1);
     c.beta = fmaxf(fmaf(p.b1, n, p.b2), p.beta_min);
-    const float xmu = fminf(fmaxf(p.lambda2 * n * n, p.x_min), p.x_max);
-    const float smu = c.beta * (log2f(xmu) - c.log2_alpha);
-    const float ys = exp2f(-fabsf(smu));
+    c.x_mu = fminf(fmaxf(p.lambda2 * n * n, p.x_min), p.x_max);
+    c.s_mu = c.beta * (log2f(c.x_mu) - c.log2_alpha);
+    const float ys = exp2f(-fabsf(c.s_mu));
     const float g = 1.f + ys;
-    c.mu_over_beta = ys / (xmu * g * g);
+    c.mu_over_beta = ys / (c.x_mu * g * g);
     return c;
 }
 
