@@ -81,7 +81,8 @@ __device__ __forceinline__ PrepGeo prep_geometry(const DevParams& p, const DF* C
 // and the scores lose their digits (a translation of 70 in a scene 2 to 20 deep cost
 // 1.2e-5 of them, one of 2e5 cost 7 %). So the current pose is the reference only where
 // it explains more of the pixels than the identity does, whose part of a residual is the
-// flow itself.
+// flow itself. The vote takes 0.5 to 1 us of the count; in a kernel of its own, beside P3P,
+// it took one block 8 us, and score_hypotheses, which has no P3P, 10 us a call.
 __device__ __forceinline__ bool pose_explains(const DevParams& p, const float* M, const PrepGeo& g, float2 f)
 {
     const float iz = 1.f / g.Pz.hi, x = g.Px.hi * iz, y = g.Py.hi * iz;
